@@ -242,7 +242,11 @@ __device__ __forceinline__ int pair_index(int b, int c, int L) {
 // Pass 2: y-moments of the column sums over one y-chunk of 32 rows,
 // Y_bc(i) = sum_j y_j^b S_c(i, j), summed over the z-chunks.  Block = 8 warps
 // over (x tile of 32, power c, y-chunk); lanes over x (coalesced), warps over
-// the chunk's rows; the 8 warp partials are added in warp order.
+// the chunk's rows; the 8 warp partials are added in warp order.  A row's
+// z-chunks are added up first and its powers of y applied to the sum, so the
+// FP64 chain of a thread is rows * (z-chunks + powers) additions long and not
+// their product (32^3, 1 plane per z-chunk: 102.6 us under ncu with the powers
+// applied chunk by chunk).
 constexpr int MP_JT = 32;   // rows per y-chunk
 
 template <int L>
@@ -261,16 +265,19 @@ __global__ void __launch_bounds__(256)
 #pragma unroll
   for (int b = 0; b <= L; b++) acc[b] = 0.0;
   if (i < ni) {
-    for (int q = 0; q < nchunk; q++) {
-      const double* src = colmom + ((long long)q * (L + 1) + c) * plane + i;
-      for (int j = jb + w; j < je; j += 8) {
-        const double y = fma((double)(j + 1), hy, y0);
-        double pw = src[(long long)j * ni];
+    const long long cs = (long long)(L + 1) * plane;   // stride between z-chunks
+    const double* src = colmom + c * plane + i;
+    for (int j = jb + w; j < je; j += 8) {
+      const double* p = src + (long long)j * ni;
+      double v = p[0];
+#pragma unroll 4
+      for (int q = 1; q < nchunk; q++) v += p[q * cs];
+      const double y = fma((double)(j + 1), hy, y0);
+      double pw = 1.0;
 #pragma unroll
-        for (int b = 0; b <= L; b++) {
-          if (b < nb) acc[b] += pw;
-          pw *= y;
-        }
+      for (int b = 0; b <= L; b++) {
+        if (b < nb) acc[b] = fma(v, pw, acc[b]);
+        pw *= y;
       }
     }
   }
@@ -408,10 +415,15 @@ __global__ void __launch_bounds__(256)
 }
 
 // ------------------------------------------------------------------ host launchers
-// z-chunks of pass 1: enough columns x chunks for about 1024 threads per SM
+// z-chunks of pass 1: enough columns x chunks for about 1024 threads per SM,
+// but at least MP_KC_MIN planes each: pass 2 reads every chunk of a row in
+// turn, and below that length it took longer than the column pass saved (32^3:
+// 31 one-plane chunks cost 7.5 us in pass 1 and 102.6 us in pass 2).
+constexpr int MP_KC_MIN = 8;
 static int mp_chunks(const Dims& d) {
   const long long cols = (long long)d.ni() * d.nj();
   long long nc = (device_sm_count() * 1024LL + cols - 1) / cols;
+  nc = std::min(nc, (long long)((d.nk() + MP_KC_MIN - 1) / MP_KC_MIN));
   nc = std::max(nc, (long long)((d.nk() + MP_KC_MAX - 1) / MP_KC_MAX));
   return (int)std::max(1LL, std::min(nc, (long long)d.nk()));
 }
