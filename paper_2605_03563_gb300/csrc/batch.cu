@@ -346,7 +346,7 @@ __global__ void __launch_bounds__(BBX* BBY) kb_norm(BArgs a, int list) {
 
 // ------------------------------------------------------------------ norm finisher
 // One block per active solve (its own item): convergence check (mode 2).
-__global__ void __launch_bounds__(1024) kb_finish(BArgs a, int list) {
+__global__ void __launch_bounds__(FINISH_THREADS) kb_finish(BArgs a, int list) {
   const BList L = a.lists[list];
   if ((int)blockIdx.x >= L.count) return;
   const BSlot& sl = a.slots[a.items[L.off + blockIdx.x].slot];
@@ -536,7 +536,7 @@ cudaError_t launch_b_norm(const BArgs& a, int order, int list, cudaStream_t s) {
 }
 
 cudaError_t launch_b_finish(const BArgs& a, int list, int max_blocks, cudaStream_t s) {
-  kb_finish<<<max_blocks, 1024, 0, s>>>(a, list);
+  kb_finish<<<max_blocks, FINISH_THREADS, 0, s>>>(a, list);
   return cudaGetLastError();
 }
 

@@ -103,22 +103,18 @@ __device__ __forceinline__ void store_dt(void* out, int dt, long long p, double 
 // Block reduction of {sum, max} into partials[2*block], partials[2*block+1];
 // m >= 0 (a max of magnitudes), reduced by its bits on the integer pipe.
 __device__ __forceinline__ void block_sum_max(double s, double m, double* partials) {
-  __shared__ double sh[64];
+  __shared__ double sh[BX * BY];
+  __shared__ double shm[32];
   const int tid = threadIdx.x + blockDim.x * threadIdx.y;
-  const int lane = tid & 31, warp = tid >> 5, nw = (blockDim.x * blockDim.y + 31) >> 5;
-  s = warp_sum(s);
   m = warp_absmax(m);
-  if (lane == 0) { sh[warp] = s; sh[32 + warp] = m; }
-  __syncthreads();
-  if (warp == 0) {
-    double a = lane < nw ? sh[lane] : 0.0;
-    double b = lane < nw ? sh[32 + lane] : 0.0;
-    a = warp_sum(a);
-    b = warp_absmax(b);
-    if (lane == 0) {
+  if ((tid & 31) == 0) shm[tid >> 5] = m;
+  s = block_sum_warp0(s, tid, BX * BY, sh);
+  if (tid < 32) {
+    m = warp_absmax(tid < BX * BY / 32 ? shm[tid] : 0.0);
+    if (tid == 0) {
       int bid = block_linear_id();
-      partials[2 * bid] = a;
-      partials[2 * bid + 1] = b;
+      partials[2 * bid] = s;
+      partials[2 * bid + 1] = m;
     }
   }
 }
@@ -1684,7 +1680,7 @@ __global__ void k_finish_norm(const double* __restrict__ partials, int nblocks, 
 
 cudaError_t launch_finish_norm(const double* partials, int nblocks, double dscale, int mode,
                                DevState* st, cudaStream_t s, unsigned long long cond, int chunk) {
-  k_finish_norm<<<1, 1024, 0, s>>>(partials, nblocks, dscale, mode, st, cond, chunk);
+  k_finish_norm<<<1, FINISH_THREADS, 0, s>>>(partials, nblocks, dscale, mode, st, cond, chunk);
   return cudaGetLastError();
 }
 
@@ -1875,17 +1871,16 @@ int pcg_precond_kernels(int order) { return order == 2 ? 3 : 5; }
 // 4: PCG beta = (r.z)/rho, rho = r.z; 5: PCG start, rho = r.z
 __global__ void k_cg_scalar(const double* __restrict__ partials, int nblocks, int which,
                             DevState* __restrict__ st, unsigned long long cond, int chunk) {
-  __shared__ double red[32];
+  __shared__ double red[FINISH_THREADS];
   if (which != 2 && st->done) {
     if ((which == 1 || which == 3) && threadIdx.x == 0) set_loop(st, cond, chunk);
     return;
   }
   double s = 0.0;
-  for (int b = threadIdx.x; b < nblocks; b += blockDim.x) s += partials[2 * b];
-  double a[1] = {s};
-  block_sum<1>(a, red);
+#pragma unroll 4
+  for (int b = threadIdx.x; b < nblocks; b += FINISH_THREADS) s += partials[2 * b];
+  const double S = block_sum_warp0(s, threadIdx.x, FINISH_THREADS, red);
   if (threadIdx.x != 0) return;
-  const double S = a[0];
   if (which == 0) {
     st->pq = S;
     st->alpha = st->rho / S;
@@ -1964,7 +1959,7 @@ cudaError_t launch_cg_pupdate(const Dims& d, const double* r, double* p, const D
 
 cudaError_t launch_cg_scalar(const double* partials, int nblocks, int which, DevState* st,
                              cudaStream_t s, unsigned long long cond, int chunk) {
-  k_cg_scalar<<<1, 1024, 0, s>>>(partials, nblocks, which, st, cond, chunk);
+  k_cg_scalar<<<1, FINISH_THREADS, 0, s>>>(partials, nblocks, which, st, cond, chunk);
   return cudaGetLastError();
 }
 

@@ -136,14 +136,48 @@ struct AbsMax {
   __device__ __forceinline__ double value() const { return __hiloint2double((int)hi, (int)lo); }
 };
 
-// Max over the warp of |v| (the bit order of AbsMax, integer pipe only).
+// Max over the warp of |v| (the bit order of AbsMax, integer pipe only): the
+// largest high word, then the largest low word among its holders.
 __device__ __forceinline__ double warp_absmax(double v) {
-  AbsMax a;
-  a.take(v);
-#pragma unroll
-  for (int o = 16; o > 0; o >>= 1)
-    a.take_bits(__shfl_xor_sync(0xffffffffu, a.hi, o), __shfl_xor_sync(0xffffffffu, a.lo, o));
-  return a.value();
+  const unsigned h = (unsigned)__double2hiint(v) & 0x7fffffffu, l = (unsigned)__double2loint(v);
+  const unsigned mh = __reduce_max_sync(0xffffffffu, h);
+  const unsigned ml = __reduce_max_sync(0xffffffffu, h == mh ? l : 0u);
+  return __hiloint2double((int)mh, (int)ml);
+}
+
+// Sum of v over a block of nthr threads (thread index tid), valid in warp 0.
+// The values go through shared memory (sh: nthr doubles) and warp 0 adds them,
+// nthr / 32 per lane in two chains, then across its lanes: nthr / 32 + 5 FP64
+// instructions per warp-wide step instead of 5 in every warp (a dependent FP64
+// add takes about 63 cycles here and one SM issues 1.7 a cycle, so eight warps'
+// shuffle trees at once take 760 cycles).
+__device__ __forceinline__ double block_sum_warp0(double v, int tid, int nthr, double* sh) {
+  sh[tid] = v;
+  __syncthreads();
+  double a = 0.0;
+  if (tid < 32) {
+    double b = 0.0;
+    for (int i = tid; i < nthr; i += 64) {
+      a += sh[i];
+      if (i + 32 < nthr) b += sh[i + 32];
+    }
+    a = warp_sum(a + b);
+  }
+  return a;
+}
+
+// 2^-rint(log2 m): the power-of-two scale of a residual of magnitude m > 0,
+// from the exponent field (rounded up from sqrt(2) on; log2 and exp2 cost
+// about 600 cycles each on this part's FP64 pipe).  Zeros, subnormals, infinities
+// and NaNs take the functions.
+__device__ __forceinline__ double pow2_scale(double m) {
+  const long long b = __double_as_longlong(m);
+  int e = (int)((b >> 52) & 0x7ff) - 1023;
+  if (b > 0 && e >= -1000 && e <= 1000) {
+    if ((b & 0x000fffffffffffffLL) >= 0x0006a09e667f3bcdLL) e++;
+    return __longlong_as_double((long long)(1023 - e) << 52);
+  }
+  return m > 0.0 ? exp2(-rint(log2(m))) : 1.0;
 }
 
 // Block-wide sum of NV values per thread, result valid in thread 0.
