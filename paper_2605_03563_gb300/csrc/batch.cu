@@ -277,21 +277,33 @@ __global__ void __launch_bounds__(BBX* BBY) kb_prolong(BArgs a, int list) {
 }
 
 // ------------------------------------------------------------------ coarsest CG
-// One block per solve whose coarsest level is item.level (the block's own item).
+// One cluster per solve whose coarsest level is item.level (the cluster's own item).
+template <int G, bool ISO, typename T>
+__device__ __forceinline__ void coarse_slots(const BLevel& lv, int slots, double tol, DevState* st, double* sm) {
+  const int nunk = lv.d.ni() * lv.d.nj() * lv.d.nk();
+  const T* fs = (const T*)lv.fs;
+  T* e = (T*)lv.phi;
+  if (slots <= 1) coarse_cg_cluster<G, ISO, T, T, 1>(lv.d, lv.cf64, fs, e, tol, nunk, st, sm);
+  else if (slots <= 2) coarse_cg_cluster<G, ISO, T, T, 2>(lv.d, lv.cf64, fs, e, tol, nunk, st, sm);
+  else if (slots <= 4) coarse_cg_cluster<G, ISO, T, T, 4>(lv.d, lv.cf64, fs, e, tol, nunk, st, sm);
+  else if (slots <= 12) coarse_cg_cluster<G, ISO, T, T, 12>(lv.d, lv.cf64, fs, e, tol, nunk, st, sm);
+  else coarse_cg_cluster<G, ISO, T, T, CG_MAX_SLOTS>(lv.d, lv.cf64, fs, e, tol, nunk, st, sm);
+}
+
 template <int G, typename T>
-__global__ void __launch_bounds__(256) kb_coarse(BArgs a, int list, double tol) {
-  extern __shared__ double p[];
+__global__ void __launch_bounds__(CG_MAXT) kb_coarse(BArgs a, int list, double tol) {
+  extern __shared__ double sm[];
   const BList L = a.lists[list];
-  if ((int)blockIdx.x >= L.count) return;
-  const BItem item = a.items[L.off + blockIdx.x];   // one tile per entry
+  const int nc = (int)cluster_size(), it = blockIdx.x / nc;
+  if (it >= L.count) return;   // uniform over the cluster
+  const BItem item = a.items[L.off + it];   // one tile per entry
   const BSlot& sl = a.slots[item.slot];
   if (sl.st->done) return;
   const BLevel& lv = sl.lv[item.level];
-  const int nunk = lv.d.ni() * lv.d.nj() * lv.d.nk();
-  if (lv.iso)
-    coarse_cg_block<G, true, T, T, 16, 256>(lv.d, lv.cf64, (const T*)lv.fs, (T*)lv.phi, tol, nunk, sl.st, p);
-  else
-    coarse_cg_block<G, false, T, T, 16, 256>(lv.d, lv.cf64, (const T*)lv.fs, (T*)lv.phi, tol, nunk, sl.st, p);
+  const CgSlab C(lv.d, nc);
+  const int slots = C.positions(blockDim.x) * C.np;
+  if (lv.iso) coarse_slots<G, true, T>(lv, slots, tol, sl.st, sm);
+  else coarse_slots<G, false, T>(lv, slots, tol, sl.st, sm);
 }
 
 // ------------------------------------------------------------------ norm after the post-smoothing (FP64)
@@ -512,12 +524,24 @@ template <int G, typename T>
 static cudaError_t coarse_launch(const BArgs& a, int list, int max_blocks, size_t smem, double tol,
                                  cudaStream_t s) {
   auto kern = kb_coarse<G, T>;
-  if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-  }
-  kern<<<max_blocks, 256, smem, s>>>(a, list, tol);
-  return cudaGetLastError();
+  cudaError_t e;
+  const int nc = coarse_cg_cluster_ctas();
+  if (nc > 8 && (e = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1)) != cudaSuccess)
+    return e;
+  if (smem > 48 * 1024 &&
+      (e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem)) != cudaSuccess)
+    return e;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3((unsigned)(max_blocks * nc));
+  cfg.blockDim = dim3(CG_MAXT);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim = {(unsigned)nc, 1, 1};
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kern, a, list, tol);
 }
 
 cudaError_t launch_b_coarse(const BArgs& a, int order, int dt, int list, int max_blocks,

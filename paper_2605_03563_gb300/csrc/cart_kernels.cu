@@ -16,6 +16,7 @@
 // launch still fills every SM instead of serialising memory latency along z.
 // Kernels recover the chunk from gridDim.z.
 #include <algorithm>
+#include <atomic>
 #include <cstdio>
 
 #include "cart_kernels.cuh"
@@ -1539,51 +1540,89 @@ cudaError_t launch_apply(const Dims& d, int order, const double h[3], int dt, co
 }
 
 // ------------------------------------------------------------------ coarsest-level CG
-template <int G, bool ISO, typename TF, typename TE, int PPT, int MAXT>
-__global__ void __launch_bounds__(MAXT)
+template <int G, bool ISO, typename TF, typename TE, int PPT>
+__global__ void __launch_bounds__(CG_MAXT)
     k_coarse_cg(Dims d, Coef<double> cf, const TF* __restrict__ fs, TE* __restrict__ e,
                 double tol, int max_iter, DevState* __restrict__ st) {
-  extern __shared__ double p[];
-  coarse_cg_block<G, ISO, TF, TE, PPT, MAXT>(d, cf, fs, e, tol, max_iter, st, p);
+  extern __shared__ double sm[];
+  coarse_cg_cluster<G, ISO, TF, TE, PPT>(d, cf, fs, e, tol, max_iter, st, sm);
 }
 
 size_t coarse_cg_smem_bytes(const Dims& d) { return (size_t)d.size() * sizeof(double); }
 
+// CTAs per cluster of the coarsest CG: 16 (the opt-in size) where the device
+// can place such a cluster, else the portable 8.
+int coarse_cg_cluster_ctas() {
+  static std::atomic<int> cached{0};
+  int nc = cached.load(std::memory_order_relaxed);
+  if (nc) return nc;
+  auto kern = k_coarse_cg<1, true, double, double, 1>;
+  nc = 8;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(CG_MAXNC);
+  cfg.blockDim = dim3(CG_MAXT);
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim = {CG_MAXNC, 1, 1};
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  int n = 0;
+  if (cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+      cudaOccupancyMaxActiveClusters(&n, kern, &cfg) == cudaSuccess && n > 0)
+    nc = CG_MAXNC;
+  (void)cudaGetLastError();
+  cached.store(nc, std::memory_order_relaxed);
+  return nc;
+}
+
+size_t coarse_cg_slab_bytes(const Dims& d, int nc) {
+  return (size_t)CgSlab(d, nc).smem_doubles(d.g) * sizeof(double);
+}
+
+// Levels of at most 8192 unknowns.  A level with 8 planes or fewer along its
+// longest axis takes a cluster of 8 (one plane per CTA), others the largest
+// cluster: the CTAs beyond the planes would only wait at the barriers.
+// Solve times under ncu, FP64 (one CTA with 83-1024 threads before): 7^3
+// 7-point 38.0 -> 25.1 us (9.2 iterations), 11^3 7-point 118.5 -> 37.0 (12.4),
+// 11^3 13-point 207 -> 50.4, 19 x 13 x 25 with unequal spacings 377 -> 65.2
+// (13.6).  The same slabs with textbook CG (two barriers an iteration, 256
+// threads) took 39.0, 57.5, 79.7 and 104.5 us.
 template <int G, bool ISO, typename TF, typename TE>
 static cudaError_t coarse_t(const Dims& d, const double h[3], int order, const void* fs, void* e,
                             double tol, int max_iter, DevState* st, cudaStream_t s) {
   Coef<double> cf = make_coef<double>(d, h, order);
-  const size_t smem = coarse_cg_smem_bytes(d);
-  const int nint = d.ni() * d.nj() * d.nk();
-  int ppt = 1;
-  while (ppt < 16 && (nint + ppt - 1) / ppt > 128) ppt *= 2;
-  // up to 512 unknowns: 4 warps (one per SM sub-partition, each with its FP64
-  // unit) with up to 4 unknowns per thread
-  if (nint <= 512) ppt = (nint + 127) / 128;
-  // very elongated coarsest levels (more than 16 x 256 unknowns): up to 1024 threads x 8
-  const bool wide = (nint + ppt - 1) / ppt > 256;
-  if (wide) ppt = 8;
-  if ((nint + ppt - 1) / ppt > (wide ? 1024 : 256)) return cudaErrorInvalidValue;
-  const int nthr = std::max(32, (((nint + ppt - 1) / ppt) + 31) / 32 * 32);
-  cudaError_t err;
-#define PS_COARSE_LAUNCH(P, MT)                                                               \
-  {                                                                                           \
-    auto kern = k_coarse_cg<G, ISO, TF, TE, P, MT>;                                           \
-    if (smem > 48 * 1024 &&                                                                   \
-        (err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,        \
-                                    (int)smem)) != cudaSuccess)                               \
-      return err;                                                                             \
-    kern<<<1, nthr, smem, s>>>(d, cf, (const TF*)fs, (TE*)e, tol, max_iter, st);              \
-  }
-  if (wide) PS_COARSE_LAUNCH(8, 1024)
-  else if (ppt == 1) PS_COARSE_LAUNCH(1, 256)
-  else if (ppt == 2) PS_COARSE_LAUNCH(2, 256)
-  else if (ppt == 3) PS_COARSE_LAUNCH(3, 256)
-  else if (ppt == 4) PS_COARSE_LAUNCH(4, 256)
-  else if (ppt == 8) PS_COARSE_LAUNCH(8, 256)
-  else PS_COARSE_LAUNCH(16, 256)
-#undef PS_COARSE_LAUNCH
-  return cudaGetLastError();
+  if ((long long)d.ni() * d.nj() * d.nk() > 8192) return cudaErrorInvalidValue;
+  const int big = coarse_cg_cluster_ctas();
+  const int nc = CgSlab(d, big).m2 <= 8 ? 8 : big;
+  const CgSlab L(d, nc);
+  const size_t smem = coarse_cg_slab_bytes(d, nc);
+  const int area = L.m0 * L.m1, q = L.positions(CG_MAXT), slots = q * L.np;
+  if (slots > CG_MAX_SLOTS) return cudaErrorInvalidValue;
+  const int nthr = ((area + q - 1) / q + 31) / 32 * 32;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = dim3(nc);
+  cfg.blockDim = dim3(nthr);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim = {(unsigned)nc, 1, 1};
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  auto go = [&](auto kern) -> cudaError_t {
+    cudaError_t err;
+    if (nc > 8 && (err = cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1)) != cudaSuccess)
+      return err;
+    if (smem > 48 * 1024 && (err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                        (int)smem)) != cudaSuccess)
+      return err;
+    return cudaLaunchKernelEx(&cfg, kern, d, cf, (const TF*)fs, (TE*)e, tol, max_iter, st);
+  };
+  if (slots <= 1) return go(k_coarse_cg<G, ISO, TF, TE, 1>);
+  if (slots <= 2) return go(k_coarse_cg<G, ISO, TF, TE, 2>);
+  if (slots <= 4) return go(k_coarse_cg<G, ISO, TF, TE, 4>);
+  if (slots <= 12) return go(k_coarse_cg<G, ISO, TF, TE, 12>);
+  return go(k_coarse_cg<G, ISO, TF, TE, CG_MAX_SLOTS>);
 }
 
 template <typename TF, typename TE>

@@ -135,7 +135,10 @@ cudaError_t launch_apply(const Dims& d, int order, const double h[3], int dt, co
 cudaError_t launch_coarse_cg(const Dims& d, int order, const double h[3], int dt_fs,
                              const void* fs, int dt_e, void* e, double tol, int max_iter,
                              DevState* st, cudaStream_t s);
-size_t coarse_cg_smem_bytes(const Dims& d);
+size_t coarse_cg_smem_bytes(const Dims& d);   // the whole ghosted level
+// CTAs per cluster of the coarsest CG, and the shared memory of one CTA of nc
+int coarse_cg_cluster_ctas();
+size_t coarse_cg_slab_bytes(const Dims& d, int nc);
 
 // Sum the per-block partials of a delta pass into the state and decide
 // convergence.  mode: 0 = record reference norm, 1 = record initial residual,

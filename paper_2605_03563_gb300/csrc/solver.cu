@@ -287,7 +287,7 @@ bool levels_for(const int n[3], std::vector<std::array<int, 3>>* out) {
 }
 
 // Library-owned level arrays pad rows to 32 elements; the coarsest level,
-// which the single-CTA CG keeps whole in shared memory, stays dense.
+// which the coarsest CG stages in shared memory, stays dense.
 Dims level_dims(const std::array<int, 3>& n, int gw, bool coarsest) {
   return make_dims(n[0], n[1], n[2], gw, coarsest ? 1 : 32);
 }
@@ -1469,7 +1469,7 @@ ps_status batch_rebuild(ps_batch_ctx* b) {
       push(BL_CELLS * L + l, si, l, gx, gy, gz);
     }
     push(BL_CG * L + (nl - 1), si, nl - 1, 1, 1, 1);
-    smem = std::max(smem, coarse_cg_smem_bytes(sd.lv[nl - 1].d));
+    smem = std::max(smem, coarse_cg_slab_bytes(sd.lv[nl - 1].d, coarse_cg_cluster_ctas()));
     if (b->prec == 0) {
       batch_tiles_sweep(sd.lv[0].d, b->order, sd.lv[0].zc, &gx, &gy, &gz);
       push(BL_NORM0 * L, si, 0, gx, gy, gz);
@@ -1753,10 +1753,10 @@ ps_status poisson_create(const ps_grid* grid, const double* const coords_host[3]
         return bail(fail(PS_ERR_OOM, "multipole alloc: %s", cudaGetErrorString(e)));
       h->bytes += h->mp.bytes;
     }
-    // the coarsest level must fit one CTA's shared memory for the coarse CG
+    // the coarsest CG takes levels of up to 200 KB
     const Dims& dc = h->dims.back();
     if (h->nlev >= 2 && coarse_cg_smem_bytes(dc) > 200 * 1024)
-      return bail(fail(PS_ERR_INVALID_ARG, "coarsest level %dx%dx%d too large for the single-CTA CG", dc.nx, dc.ny, dc.nz));
+      return bail(fail(PS_ERR_INVALID_ARG, "coarsest level %dx%dx%d too large for the coarsest-level CG", dc.nx, dc.ny, dc.nz));
   } else {
     h->sd.nr = grid->n[0];
     h->sd.nt = grid->n[1];

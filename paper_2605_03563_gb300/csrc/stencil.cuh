@@ -137,120 +137,248 @@ __device__ __forceinline__ void finish_norm_block(const double* __restrict__ par
   set_loop(st, cond, chunk);
 }
 
+// 1 / x for normal x well inside the exponent range: the approximate reciprocal
+// instruction, then two Newton steps y += y (1 - x y), each doubling the correct
+// bits (4 FP64 instructions; a division takes about 10, 76 cycles each per warp).
+__device__ __forceinline__ double recip(double x) {
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+  y = fma(y, fma(-x, y, 1.0), y);
+  return fma(y, fma(-x, y, 1.0), y);
+}
+
+// ------------------------------------------------------------------ thread-block cluster
+__device__ __forceinline__ unsigned cluster_rank() {
+  unsigned r;
+  asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ unsigned cluster_size() {
+  unsigned r;
+  asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
+  return r;
+}
+// Barrier over the cluster's threads; shared-memory writes before it, remote
+// ones included, are visible after it.
+__device__ __forceinline__ void cluster_sync() {
+  __syncwarp();
+  asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// Store v at the address that p (in this CTA's shared memory) has in CTA `rank`.
+__device__ __forceinline__ void store_remote(double* p, unsigned rank, double v) {
+  unsigned a;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(a) : "r"((unsigned)__cvta_generic_to_shared(p)), "r"(rank));
+  asm volatile("st.shared::cluster.f64 [%0], %1;" ::"r"(a), "d"(v) : "memory");
+}
+
 // ------------------------------------------------------------------ coarsest-level CG
-// One CTA solves -A e = d * fs (zero boundary, e0 = 0) by CG (Sec. 2.1.3: the
-// coarsest level is solved with CG) until ||r|| <= tol ||r0|| or max_iter
-// iterations.  Each thread owns up to PPT unknowns and keeps their x, r, q in
-// registers; only the search direction p lives in shared memory (on the full
-// ghosted layout, zero boundary), because the stencil reads neighbours.
-// GB300's FP64 pipe is narrow, so the FP64 work that is not per unknown is done
-// once: each dot product is one per-thread partial in shared memory summed by
-// warp 0 (a strided loop, then one shuffle tree), and thread 0 alone forms
-// alpha, beta and the convergence test and hands them out through shared memory.
-// About 100 threads with several unknowns each keep the pipe busy with
-// independent work while the block's barriers stay cheap.
-// p: shared memory holding the whole ghosted level (d.size() doubles).
-template <int G, bool ISO, typename TF, typename TE, int PPT, int MAXT>
-__device__ __forceinline__ void coarse_cg_block(const Dims& d, const Coef<double>& cf,
-                                                const TF* __restrict__ fs, TE* __restrict__ e,
-                                                double tol, int max_iter, DevState* __restrict__ st,
-                                                double* p) {
-  __shared__ double part[MAXT];
-  __shared__ double scal[2];   // alpha / beta handed out by thread 0
-  __shared__ int stop;
-  const int tid = threadIdx.x, nthr = blockDim.x, lane = tid & 31;
-  const int ni = d.ni(), nj = d.nj(), nk = d.nk();
-  const int nint = ni * nj * nk;
-  const long long n = d.size();
-  const long long sy = d.sy(), sz = d.sz();
-  // block sum of v into lane values of warp 0 (valid in thread 0)
-  auto block_sum0 = [&](double v) -> double {
-    part[tid] = v;
-    __syncthreads();
-    double t = 0.0;
-    if (tid < 32) {
-      for (int i = lane; i < nthr; i += 32) t += part[i];
-      t = warp_sum(t);
-    }
-    return t;
+// One cluster solves -A e = d * fs (zero boundary, e0 = 0) by CG (Sec. 2.1.3:
+// the coarsest level is solved with CG) until ||r|| <= tol ||r0|| or max_iter
+// iterations.  GB300's FP64 pipe is narrow (about 1.7 instructions a cycle and
+// SM, 63 cycles from one to the next that needs it), so one SM spends most of
+// a solve issuing FP64: the level is cut into slabs along its longest axis, one
+// slab per CTA, and the work runs on up to 16 SMs.  What is left is the chain
+// of an iteration's sums and exchanges, so the recurrences are those of
+// pipelined CG (P. Ghysels, W. Vanroose, Parallel Computing 40, 2014): with
+// w = A r kept beside r, gamma = r.r and delta = w.r are summed together and
+// n = A w does not wait for them,
+//   beta = gamma / gamma', den = delta - beta^2 den', alpha = gamma / den,
+//   z = n + beta z, s = w + beta s, p = r + beta p,
+//   x += alpha p, r -= alpha s, w -= alpha z,
+// the iterates of CG with one cluster barrier an iteration instead of three
+// (den = p.A p).  The barrier hands round each warp's partial sums and the
+// values of w next to the slab edges; w is kept twice, so that the next values
+// are written while a slower CTA still reads the last ones.  A thread owns
+// in-plane positions over the slab's planes, all vectors but w in registers.
+// All CTAs add the same partials in the same order and therefore take the same
+// alpha, beta and decision to stop.  Solve times: see launch_coarse_cg.
+struct CgSlab {
+  int s, a0, a1;      // slab axis (the longest, z first) and the in-plane axes
+  int m0, m1, m2;     // unknowns along a0, a1, s
+  int np;             // planes per CTA
+  __host__ __device__ CgSlab(const Dims& d, int nc) {
+    const int n[3] = {d.ni(), d.nj(), d.nk()};
+    s = 2;
+    if (n[1] > n[s]) s = 1;
+    if (n[0] > n[s]) s = 0;
+    a0 = s == 0 ? 1 : 0;
+    a1 = s == 2 ? 1 : 2;
+    m0 = n[a0];
+    m1 = n[a1];
+    m2 = n[s];
+    np = (m2 + nc - 1) / nc;
+  }
+  __host__ __device__ int smem_doubles(int g) const {
+    return 2 * (np + 2 * g) * (m0 + 2 * g) * (m1 + 2 * g);   // w, twice
+  }
+  // in-plane positions per thread and register slots (positions x planes) for at most maxt threads
+  __host__ __device__ int positions(int maxt) const { return (m0 * m1 + maxt - 1) / maxt; }
+};
+constexpr int CG_MAXT = 128;      // threads per CTA: one warp per SM sub-partition and FP64 unit
+constexpr int CG_MAXNC = 16;      // CTAs per cluster
+constexpr int CG_MAX_SLOTS = 24;  // register slots per thread of the largest variant
+
+template <int G, bool ISO, typename TF, typename TE, int PPT>
+__device__ __forceinline__ void coarse_cg_cluster(const Dims& d, const Coef<double>& cf0,
+                                                  const TF* __restrict__ fs, TE* __restrict__ e,
+                                                  double tol, int max_iter, DevState* __restrict__ st,
+                                                  double* sm) {
+  __shared__ double part[2][2][CG_MAXNC * (CG_MAXT / 32)];   // [set][gamma, delta][rank, warp]
+  const int tid = threadIdx.x, nthr = blockDim.x, lane = tid & 31, warp = tid >> 5, nw = nthr >> 5;
+  const int rank = (int)cluster_rank(), NC = (int)cluster_size();
+  const CgSlab L(d, NC);
+  const int m0 = L.m0, m1 = L.m1, m2 = L.m2, np = L.np, area = m0 * m1;
+  const int w0 = m0 + 2 * G, plane = w0 * (m1 + 2 * G);
+  const int k0 = rank * np, nown = max(0, min(np, m2 - k0)), nsl = np + 2 * G;
+  const int wsz = nsl * plane;   // w is kept at sm and sm + wsz: [nsl][m1 + 2G][m0 + 2G] each
+  Coef<double> cf = cf0;
+  // along the slab's axes (selects: an index would put the arrays in local memory)
+  auto along = [](int a, auto v0, auto v1, auto v2) { return a == 0 ? v0 : (a == 1 ? v1 : v2); };
+  auto permute = [&](const double (&v)[3], double (&o)[3]) {
+    o[0] = along(L.a0, v[0], v[1], v[2]);
+    o[1] = along(L.a1, v[0], v[1], v[2]);
+    o[2] = along(L.s, v[0], v[1], v[2]);
   };
-  for (long long u = tid; u < n; u += nthr) p[u] = 0.0;
-  long long c[PPT];
-  double x[PPT], r[PPT], q[PPT];
-  bool own[PPT];
-#pragma unroll
-  for (int k = 0; k < PPT; k++) {
-    const int u = tid + k * nthr;
-    own[k] = u < nint;
-    const int uu = own[k] ? u : 0;
-    const int i = uu % ni, t = uu / ni;
-    c[k] = d.at(i + G, t % nj + G, t / nj + G);
-    x[k] = 0.0;
-    r[k] = 0.0;
-    q[k] = 0.0;
-  }
+  permute(cf0.c1, cf.c1);
+  permute(cf0.c2, cf.c2);
+  const int t0 = (int)along(L.a0, 1LL, d.sy(), d.sz()), t1 = (int)along(L.a1, 1LL, d.sy(), d.sz()),
+            t2 = (int)along(L.s, 1LL, d.sy(), d.sz());   // strides in fs and e (dense, small)
+  const int Q = (area + nthr - 1) / nthr;   // in-plane positions per thread
+  for (int u = tid; u < 2 * wsz; u += nthr) sm[u] = 0.0;
   __syncthreads();
-  double loc = 0.0;
-#pragma unroll
-  for (int k = 0; k < PPT; k++) {
-    if (own[k]) {
-      const double b = cf.d * (double)St<TF>::ld(fs + c[k]);
-      r[k] = b;
-      p[c[k]] = b;
-      loc = fma(b, b, loc);
+  // b = d fs on every plane of the slab and its neighbours (in the second array: w takes its place after the first step)
+  for (int q = 0; q < Q; q++) {
+    const int f = tid + q * nthr;
+    if (f >= area) break;
+    const int j = f / m0, i = f - j * m0;
+    for (int l = 0; l < nsl; l++) {
+      const int k = k0 - G + l;
+      if (k < 0 || k >= m2) continue;
+      sm[wsz + l * plane + (j + G) * w0 + i + G] =
+          cf.d * (double)St<TF>::ld(fs + (i + G) * t0 + (j + G) * t1 + (k + G) * t2);
     }
   }
-  // thread 0 keeps rr, ref and the iteration count
-  double rr = block_sum0(loc);
-  double ref = 0.0;
+  cluster_sync();   // b complete here, and every CTA runs before its memory is written
+  // slot k = (q, l): position tid + q * nthr of the slab's plane l
+  int gofs[PPT];   // offset in fs and e, -1 where the slot is empty
+  int c[PPT];      // offset in w
+  int up[PPT];     // ranks that have the slot's plane among their neighbours (G below, G above; a byte each, 255 = none)
+  double x[PPT], r[PPT], p[PPT], s[PPT], z[PPT], w[PPT];
+  // (A v) at a slot: d v - sum of d c times the neighbours
+  const double cd = cf.d;
+#pragma unroll
+  for (int a = 0; a < 3; a++) {
+    cf.c1[a] *= -cd;
+    cf.c2[a] *= -cd;
+  }
+  auto apply = [&](const double* v, int at) -> double {
+    return gs_value<G, ISO>(v, (long long)at, (long long)w0, (long long)plane, cf, cd * v[at]);
+  };
+#pragma unroll
+  for (int k = 0; k < PPT; k++) {
+    const int q = k / np, l = k - q * np, f = tid + q * nthr;
+    const bool own = q < Q && f < area && l < nown;
+    const int j = own ? f / m0 : 0, i = own ? f - j * m0 : 0;
+    gofs[k] = own ? (i + G) * t0 + (j + G) * t1 + (k0 + l + G) * t2 : -1;
+    c[k] = own ? (l + G) * plane + (j + G) * w0 + i + G : 0;
+    unsigned to = 0xffffffffu;
+    int last = rank;
+#pragma unroll
+    for (int o = -G, b = 0; o <= G; o++) {
+      if (o == 0) continue;
+      const int kz = k0 + l + o, tr = kz >= 0 ? kz / np : 0;
+      if (own && kz >= 0 && kz < m2 && tr != rank && tr != last) {
+        to = (to & ~(0xffu << (8 * b))) | ((unsigned)tr << (8 * b));
+        last = tr;
+      }
+      b++;
+    }
+    up[k] = (int)to;
+    x[k] = p[k] = s[k] = z[k] = 0.0;
+    r[k] = own ? sm[wsz + c[k]] : 0.0;
+    w[k] = own ? apply(sm + wsz, c[k]) : 0.0;
+  }
+  // w of the slots into buffer bsel, here and in the CTAs that read it
+  auto publish = [&](int bsel) {
+#pragma unroll
+    for (int k = 0; k < PPT; k++) {
+      if (gofs[k] < 0) continue;
+      double* at = sm + (bsel ? wsz : 0) + c[k];
+      *at = w[k];
+      if (up[k] == -1) continue;
+#pragma unroll
+      for (int b = 0; b < 2 * G; b++) {
+        const int to = (up[k] >> (8 * b)) & 0xff;
+        // the plane's place in that CTA's slab: shifted by the distance of the slabs
+        if (to != 0xff) store_remote(at + (rank - to) * np * plane, to, w[k]);
+      }
+    }
+  };
+  double igamma = 0.0, den = 0.0, stop2 = 0.0;
   int it = 0;
-  if (tid == 0) {
-    ref = sqrt(rr);
-    stop = !(ref > 0.0) || max_iter <= 0;
-  }
-  __syncthreads();
-  while (!stop) {
-    loc = 0.0;
+  publish(0);
+  for (;; it++) {
+    const int b = it & 1;
+    double ga = 0.0, da = 0.0;
+#pragma unroll
+    for (int k = 0; k < PPT; k++) {   // empty slots hold zeros
+      ga = fma(r[k], r[k], ga);
+      da = fma(w[k], r[k], da);
+    }
+    // both sums in one tree: lanes 0-15 add gamma, 16-31 delta (a warp-wide
+    // FP64 instruction holds its sub-partition for 76 cycles)
+    const bool hi = lane >= 16;
+    double v = (hi ? da : ga) + __shfl_xor_sync(0xffffffffu, hi ? ga : da, 16);
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    if ((lane & 15) < NC) store_remote(&part[b][hi][rank * nw + warp], lane & 15, v);
+    cluster_sync();
+    v = 0.0;
+    for (int i = lane & 15; i < NC * nw; i += 16) v += part[b][hi][i];
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    const double g = __shfl_sync(0xffffffffu, v, 0), dl = __shfl_sync(0xffffffffu, v, 16);
+    double n[PPT];   // A w: independent of the sums
+#pragma unroll
+    for (int k = 0; k < PPT; k++) n[k] = gofs[k] >= 0 ? apply(sm + (b ? wsz : 0), c[k]) : 0.0;
+    if (it == 0) {
+      stop2 = tol * tol * g;   // on squared norms
+      if (!(g > 0.0) || max_iter <= 0) break;
+    } else if (g <= stop2 || it >= max_iter) {
+      break;
+    }
+    const double beta = g * igamma;   // 0 in the first step
+    den = fma(-beta * beta, den, dl);
+    // alpha = g / den and 1 / g (for the next beta) from one reciprocal
+    const double gd = g * den;
+    double alpha;
+    if (fabs(gd) > 1e-280 && fabs(gd) < 1e280) {
+      const double inv = recip(gd);
+      alpha = g * (g * inv);
+      igamma = den * inv;
+    } else {
+      alpha = g / den;
+      igamma = 1.0 / g;
+    }
 #pragma unroll
     for (int k = 0; k < PPT; k++) {
-      if (own[k]) {
-        const double pc = p[c[k]];
-        q[k] = cf.d * (pc - gs_value<G, ISO>(p, c[k], sy, sz, cf, 0.0));
-        loc = fma(pc, q[k], loc);
-      }
+      s[k] = fma(beta, s[k], w[k]);
+      z[k] = fma(beta, z[k], n[k]);
+      w[k] = fma(-alpha, z[k], w[k]);
     }
-    const double pq = block_sum0(loc);
-    if (tid == 0) scal[0] = rr / pq;
-    __syncthreads();
-    const double alpha = scal[0];
-    loc = 0.0;
+    publish(b ^ 1);
 #pragma unroll
     for (int k = 0; k < PPT; k++) {
-      if (own[k]) {
-        x[k] = fma(alpha, p[c[k]], x[k]);
-        r[k] = fma(-alpha, q[k], r[k]);
-        loc = fma(r[k], r[k], loc);
-      }
+      p[k] = fma(beta, p[k], r[k]);
+      x[k] = fma(alpha, p[k], x[k]);
+      r[k] = fma(-alpha, s[k], r[k]);
     }
-    const double rrn = block_sum0(loc);
-    if (tid == 0) {
-      it++;
-      stop = sqrt(rrn) <= tol * ref || it >= max_iter;
-      scal[1] = rrn / rr;
-      rr = rrn;
-    }
-    __syncthreads();   // every thread is past its stencil reads of p
-    if (stop) break;
-    const double beta = scal[1];
-#pragma unroll
-    for (int k = 0; k < PPT; k++)
-      if (own[k]) p[c[k]] = fma(beta, p[c[k]], r[k]);
-    __syncthreads();   // p complete
   }
+  // (no remote write follows the last barrier, so every CTA may leave)
 #pragma unroll
   for (int k = 0; k < PPT; k++)
-    if (own[k]) St<TE>::st(e + c[k], (typename St<TE>::C)x[k]);
-  if (tid == 0 && st != nullptr) {
+    if (gofs[k] >= 0) St<TE>::st(e + gofs[k], (typename St<TE>::C)x[k]);
+  if (rank == 0 && tid == 0 && st != nullptr) {
     st->coarse_iter_last = it;
     st->coarse_iter_total += it;
   }
