@@ -20,6 +20,7 @@
 #include <cstdio>
 
 #include "cart_kernels.cuh"
+#include "fixed.cuh"
 #include "stencil.cuh"
 
 namespace ps {
@@ -222,17 +223,28 @@ __global__ void __launch_bounds__(BX* BY)
   if (RED >= 1) block_sum_max(s2, mx, partials);
 }
 
+// *to = max(*to, v over the block's threads); one atomic per warp, and none
+// where the value is already as large.
+__device__ __forceinline__ void block_atomic_max(unsigned v, unsigned* to) {
+  v = __reduce_max_sync(0xffffffffu, v);
+  const int lane = (threadIdx.x + blockDim.x * threadIdx.y) & 31;
+  if (lane == 0 && v > *(volatile unsigned*)to) atomicMax(to, v);
+}
+
 // Set-up copy of the caller's initial guess (dense rows) into the handle's
 // pitched array, one warp per row.  It records in st->guess_nonzero whether
 // any interior node of the guess is nonzero (+0 and -0 both count as zero):
 // from a zero guess the initial residual f - A phi0 is the reference vector,
-// and the initial residual pass takes the reference norm instead.
+// and the initial residual pass takes the reference norm instead.  The largest
+// |phi| of the interior and of the boundary nodes (high words) go to st->umax
+// and st->bmax, which set the unit of the fixed-point residual passes.
 __global__ void __launch_bounds__(256)
     k_copy_guess(Dims dd, Dims sd, const double* __restrict__ src, double* __restrict__ dst,
                  DevState* __restrict__ st) {
   const long long rows = (long long)sd.ey * sd.ez;
   const long long row = blockIdx.x * 8LL + (threadIdx.x >> 5);
   int nz = 0;
+  unsigned hi = 0u, hb = 0u;
   if (row < rows) {
     const int j = (int)(row % sd.ey), k = (int)(row / sd.ey), g = sd.g;
     const bool inrow = j >= g && j < sd.ey - g && k >= g && k < sd.ez - g;
@@ -242,9 +254,17 @@ __global__ void __launch_bounds__(256)
     for (int i = threadIdx.x & 31; i < sd.ex; i += 32) {
       const double v = a[i];
       b[i] = v;
-      if (inrow && i >= g && i < sd.ex - g && ((unsigned long long)__double_as_longlong(v) << 1) != 0ull) nz = 1;
+      const unsigned h = (unsigned)__double2hiint(v) & 0x7fffffffu;
+      if (inrow && i >= g && i < sd.ex - g) {
+        if (((unsigned long long)__double_as_longlong(v) << 1) != 0ull) nz = 1;
+        hi = max(hi, h);
+      } else {
+        hb = max(hb, h);
+      }
     }
   }
+  block_atomic_max(hi, &st->umax);
+  block_atomic_max(hb, &st->bmax);
   if (__syncthreads_or(nz) && threadIdx.x == 0) st->guess_nonzero = 1;
 }
 
@@ -468,6 +488,10 @@ __global__ void __launch_bounds__(BX* BY)
 // both members of the thread's x pair, each with its carried (N + U) pair sum
 // (5 + 1 FP64 instructions per node; the order of gs_value, so every delta
 // equals k_delta's bit for bit and only the reductions run in another order).
+// The refinement and initial passes of larger grids take k_fx_delta instead
+// (fx_level): this kernel stays for grids below, where a tile's march along z
+// would be the longer chain (32^3: 6 us), and for norms of a potential whose
+// largest value is not known.
 // STORE: the refinement pass of k_delta (the scaled FP32/BF16 inner right-hand
 // side, the FP32 sum of squares and max of the scaled values); otherwise the
 // FP64 sum of delta^2.  Partials {sum, max} per block.  initial: the solve's
@@ -575,13 +599,83 @@ __global__ void __launch_bounds__(BX* BY)
   else block_sum_max(s2, 0.0, partials);
 }
 
+// The same deltas with the neighbour sums on the integer pipe (fixed.cuh), for
+// the passes that know the largest |phi|: the refinement's outer residual
+// (STORE: the scaled FP32/BF16 inner right-hand side, its FP32 sum of squares
+// and max) and the initial residual of every solve.  Two FP64 instructions a
+// node (with the norm three) instead of 6 or 11.
+// Outer residual in the solve: 256^3 7-point 216 -> 79 us, 512^3 13-point
+// 2952 -> 830 us (under ncu 256^3 74.7 us with DRAM 58% and the integer pipe 64%
+// busy; 320^3 13-point 202 us, 40% and 53%).
+template <int KIND, bool STORE>
+__global__ void __launch_bounds__(256, 2)
+    k_fx_delta(const __grid_constant__ CUtensorMap mU, const __grid_constant__ CUtensorMap mB, Dims d, FxOp op, int zc,
+               int dout, void* __restrict__ out, DevState* __restrict__ st, double* __restrict__ partials) {
+  if (!STORE && st->guess_nonzero == 0) return;   // an initial residual from zero: the reference vector
+  struct Epi {
+    double oscale, s2;
+    int oexp, dout;
+    float s2f, mxf;
+    void* out;
+    __device__ __forceinline__ void operator()(long long at, int px, const bool (&in)[4], const double (&v)[4],
+                                               const double (&)[4]) {
+      if (STORE) {
+        float x[4];
+        if (oexp != INT_MIN) fx_to_f32(v, oexp, x);
+        else
+          for (int r = 0; r < 4; r++) x[r] = (float)(v[r] * oscale);
+#pragma unroll
+        for (int r = 0; r < 4; r++) {
+          if (!in[r]) continue;
+          s2f = fmaf(x[r], x[r], s2f);
+          mxf = fmaxf(mxf, fabsf(x[r]));
+          if (dout == DT_F32) ((float*)out)[at + r * px] = x[r];
+          else ((__nv_bfloat16*)out)[at + r * px] = __float2bfloat16_rn(x[r]);
+        }
+      } else {
+#pragma unroll
+        for (int r = 0; r < 4; r++)
+          if (in[r]) s2 = fma(v[r], v[r], s2);
+      }
+    }
+  } epi;
+  epi.oscale = STORE ? st->scale_next : 1.0;
+  epi.s2 = 0.0;
+  epi.oexp = pow2_exponent(epi.oscale);
+  epi.dout = dout;
+  epi.s2f = epi.mxf = 0.0f;
+  epi.out = out;
+  fx_pass<KIND>(mU, mB, d, op, max(st->umax, st->bmax), zc, &st->fault, epi);
+  if (STORE) block_sum_max_scaled(epi.s2f, epi.mxf, epi.oscale, partials);
+  else block_sum_max(epi.s2, 0.0, partials);
+}
+
+template <int KIND, bool STORE>
+static cudaError_t fx_delta_t(const Dims& d, double c, const double* phi, const double* fs, int dout, void* out,
+                              DevState* st, double* partials, int* nblocks, cudaStream_t s) {
+  static std::atomic<int> cached{0};
+  constexpr int smem = FxGeom<KIND>::SMEM;
+  int occ = 0, zc = 0;
+  const cudaError_t e = fx_occupancy(k_fx_delta<KIND, STORE>, smem, cached, &occ);
+  if (e != cudaSuccess) return e;
+  CUtensorMap mU, mB;
+  if (!fx_maps<KIND>(d, phi, fs, &mU, &mB)) return cudaErrorInvalidValue;
+  const dim3 grid = fx_grid<KIND>(d, occ, &zc);
+  if (nblocks) *nblocks = (int)(grid.x * grid.y * grid.z);
+  k_fx_delta<KIND, STORE><<<grid, 256, smem, s>>>(mU, mB, d, FxOp{c, 0, 0, 0}, zc, dout, out, st, partials);
+  return cudaGetLastError();
+}
+
 cudaError_t launch_delta_diag(const Dims& d, const double h[3], const double* phi, const double* fs, int dout,
-                              void* out, const DevState* st, bool initial, double* partials, int* nblocks,
+                              void* out, DevState* st, bool initial, double* partials, int* nblocks,
                               cudaStream_t s) {
   if (!is_iso(h) || d.g != 1 || (out != nullptr && (st == nullptr || (dout != DT_F32 && dout != DT_BF16))) ||
       (initial && st == nullptr))
     return cudaErrorInvalidValue;
   const Coef<double> cf = make_coef<double>(d, h, 2);
+  if (st != nullptr && fx_level(d))
+    return out != nullptr ? fx_delta_t<FX7, true>(d, cf.c1[0], phi, fs, dout, out, st, partials, nblocks, s)
+                          : fx_delta_t<FX7, false>(d, cf.c1[0], phi, fs, dout, out, st, partials, nblocks, s);
   const int dl = diag_walk_len(d.nk());
   const int pairs = (d.ni() + 1) / 2;
   const dim3 grid((pairs + BX - 1) / BX, (d.nj() + dl - 1 + BY - 1) / BY, (d.nk() + dl - 1) / dl);
@@ -752,12 +846,15 @@ int delta_diag13_blocks(const Dims& d) {
 }
 
 cudaError_t launch_delta_diag13(const Dims& d, const double h[3], int mode, const double* phi, const double* fs,
-                                int dout, void* out, const DevState* st, double* partials, int* nblocks,
+                                int dout, void* out, DevState* st, double* partials, int* nblocks,
                                 cudaStream_t s) {
   if (!is_iso(h) || d.g != 2 || mode < 0 || mode > 3 || (mode == 1 && out == nullptr) || (mode < 2 && st != nullptr) ||
       (mode == 3 && (out == nullptr || st == nullptr || (dout != DT_F32 && dout != DT_BF16))))
     return cudaErrorInvalidValue;
   const Coef<double> cf = make_coef<double>(d, h, 4);
+  if (st != nullptr && fx_level(d))   // c1 = 16 c, c2 = -c
+    return mode == 3 ? fx_delta_t<FX13, true>(d, cf.c1[0] / 16.0, phi, fs, dout, out, st, partials, nblocks, s)
+                     : fx_delta_t<FX13, false>(d, cf.c1[0] / 16.0, phi, fs, dout, out, st, partials, nblocks, s);
   int dl = 0;
   const dim3 grid = diag13_grid(d, &dl), blk(BX, BY);
   if (nblocks) *nblocks = (int)(grid.x * grid.y * grid.z);
@@ -1465,30 +1562,35 @@ cudaError_t launch_scale_rhs_any(const Dims& d, double factor, int dt, const voi
 template <typename TE>
 __global__ void __launch_bounds__(BX* BY)
     k_correct(Dims d, const TE* __restrict__ e, double inv_scale, double* __restrict__ phi,
-              const DevState* __restrict__ st) {
+              DevState* __restrict__ st) {
   if (st != nullptr && st->done) return;
   double isc = inv_scale;
   if (st != nullptr) isc = inverse_scale(st->scale_cur);
   const int g = d.g;
   const int i = blockIdx.x * BX + threadIdx.x + g;
   const int j = blockIdx.y * BY + threadIdx.y + g;
-  if (i >= g + d.ni() || j >= g + d.nj()) return;
-  const int zc = zchunk(d.nk());
-  const int k0 = blockIdx.z * zc + g, k1 = min(k0 + zc, g + d.nk());
-  // FP32/BF16 corrections scaled by a power of two: the scaled value is built
-  // on the integer pipe and one DADD remains (the same bits as the FMA)
-  const int ie = sizeof(TE) < sizeof(double) ? pow2_exponent(isc) : INT_MIN;
-  // unrolled: the loads of several planes in flight together
+  unsigned hm = 0u;   // high word of the largest |phi| written
+  if (i < g + d.ni() && j < g + d.nj()) {
+    const int zc = zchunk(d.nk());
+    const int k0 = blockIdx.z * zc + g, k1 = min(k0 + zc, g + d.nk());
+    // FP32/BF16 corrections scaled by a power of two: the scaled value is built
+    // on the integer pipe and one DADD remains (the same bits as the FMA)
+    const int ie = sizeof(TE) < sizeof(double) ? pow2_exponent(isc) : INT_MIN;
+    // unrolled: the loads of several planes in flight together
 #pragma unroll 4
-  for (int k = k0; k < k1; k++) {
-    const long long p = d.at(i, j, k);
-    if (ie != INT_MIN) phi[p] += f32_to_f64_pow2((float)St<TE>::ld(e + p), ie);
-    else phi[p] = fma((double)St<TE>::ld(e + p), isc, phi[p]);
+    for (int k = k0; k < k1; k++) {
+      const long long p = d.at(i, j, k);
+      const double v = ie != INT_MIN ? phi[p] + f32_to_f64_pow2((float)St<TE>::ld(e + p), ie)
+                                     : fma((double)St<TE>::ld(e + p), isc, phi[p]);
+      phi[p] = v;
+      hm = max(hm, (unsigned)__double2hiint(v) & 0x7fffffffu);
+    }
   }
+  if (st != nullptr) block_atomic_max(hm, &st->umax);
 }
 
 cudaError_t launch_correct(const Dims& d, int dt_e, const void* e, double inv_scale, double* phi,
-                           const DevState* st, cudaStream_t s) {
+                           DevState* st, cudaStream_t s) {
   if (dt_e == DT_F64) k_correct<double><<<point_grid(d), dim3(BX, BY), 0, s>>>(d, (const double*)e, inv_scale, phi, st);
   else if (dt_e == DT_F32) k_correct<float><<<point_grid(d), dim3(BX, BY), 0, s>>>(d, (const float*)e, inv_scale, phi, st);
   else k_correct<__nv_bfloat16><<<point_grid(d), dim3(BX, BY), 0, s>>>(d, (const __nv_bfloat16*)e, inv_scale, phi, st);

@@ -59,7 +59,7 @@ cudaError_t launch_scale_rhs_any(const Dims& d, double factor, int dt, const voi
 // delta_diag13_blocks(d).
 int delta_diag13_blocks(const Dims& d);
 cudaError_t launch_delta_diag13(const Dims& d, const double h[3], int mode, const double* phi, const double* fs,
-                                int dout, void* out, const DevState* st, double* partials, int* nblocks,
+                                int dout, void* out, DevState* st, double* partials, int* nblocks,
                                 cudaStream_t s);
 
 // Lagged convergence check of FP64 7-point V-cycles on equal spacings: the
@@ -100,7 +100,7 @@ cudaError_t launch_scale_rhs_ref(const Dims& d, const Dims& du, int order, const
 // == 0 the plain pass writes nothing (finisher mode 4) and the refinement pass
 // takes its deltas from fs and the ghost values alone.
 cudaError_t launch_delta_diag(const Dims& d, const double h[3], const double* phi, const double* fs, int dout,
-                              void* out, const DevState* st, bool initial, double* partials, int* nblocks,
+                              void* out, DevState* st, bool initial, double* partials, int* nblocks,
                               cudaStream_t s);
 
 // fs_coarse = factor * R(delta_fine)  (scaled coarse right-hand side); coarse = layout of fs_c
@@ -124,8 +124,9 @@ cudaError_t launch_scale_rhs(const Dims& d, const Dims& du, double factor, const
                              void* fs, cudaStream_t s);
 
 // phi64 += e * inv_scale on interior nodes
+// (with st: skipped once done, scaled by 1 / st->scale_cur; st->umax takes the largest |phi64| written)
 cudaError_t launch_correct(const Dims& d, int dt_e, const void* e, double inv_scale, double* phi,
-                           const DevState* st, cudaStream_t s);
+                           DevState* st, cudaStream_t s);
 
 // out = A phi (unscaled) on interior nodes, storage dt
 cudaError_t launch_apply(const Dims& d, int order, const double h[3], int dt, const void* phi,

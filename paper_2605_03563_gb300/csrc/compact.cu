@@ -23,12 +23,14 @@
 // serve the rows above and below as well (12.5 FP64 operations per node for
 // a residual instead of 27 multiply-adds).
 #include <algorithm>
+#include <atomic>
 #include <cmath>
 #include <type_traits>
 #include <vector>
 
 #include "cart_kernels.cuh"
 #include "compact.cuh"
+#include "fixed.cuh"
 #include "stencil.cuh"
 #include "tma.cuh"
 
@@ -378,18 +380,133 @@ cudaError_t launch_c27_resid_dt(const Dims& d, const W27& A, const double* u, co
   return cudaGetLastError();
 }
 
-cudaError_t launch_c27_init(const Dims& d, const W27& A, const double* u, const double* b, int dt_r, void* r,
-                            double* partials, cudaStream_t s) {
-  if (d.g != 1) return cudaErrorInvalidValue;
-  const dim3 g = c27_grid(d), b64(CBX, CBY / FRB);
-  const int nb = c27_blocks(d);
-  if (dt_r == DT_F64)
-    k_c27_f64<0, false, double, true, true><<<g, b64, 0, s>>>(d, wts<double>(A), 0.0, u, b, (double*)r, partials, nullptr, nb);
-  else if (dt_r == DT_F32)
-    k_c27_f64<0, false, float, true, true><<<g, b64, 0, s>>>(d, wts<double>(A), 0.0, u, b, (float*)r, partials, nullptr, nb);
-  else
-    return cudaErrorInvalidValue;
+// The finest level's residual r = b - L_h u with the sums over the 26 neighbours
+// on the integer pipe (fixed.cuh): the weights of L_h are integers over 30 h^2
+// (6 h^2, h^2), so three FP64 instructions a node are left with the norm,
+// instead of 13.5.  INIT: also the sum of b^2, which k_c27_shell completes to the
+// reference norm.
+// Under ncu at 256^3: outer residual 532 -> 138 us, initial pass 815 -> 167 us
+// and 29 us for the shell; 512^3 outer residual in the solve 3942 -> 1110 us.
+template <typename TR, bool INIT>
+__global__ void __launch_bounds__(256, 2)
+    k_c27_fx(const __grid_constant__ CUtensorMap mU, const __grid_constant__ CUtensorMap mB, Dims d, FxOp op,
+             TR* __restrict__ dst, int zc, double* __restrict__ partials, DevState* __restrict__ st, int nblocks) {
+  if (!INIT && st->done) return;   // uniform
+  struct Epi {
+    TR* dst;
+    double s2, s0;
+    __device__ __forceinline__ void operator()(long long at, int px, const bool (&in)[4], const double (&v)[4],
+                                               const double (&base)[4]) {
+      TR x[4];
+      if constexpr (std::is_same<TR, float>::value) fx_to_f32(v, 0, x);
+      else
+        for (int r = 0; r < 4; r++) x[r] = v[r];
+#pragma unroll
+      for (int r = 0; r < 4; r++) {
+        if (!in[r]) continue;
+        dst[at + r * px] = x[r];
+        s2 = fma(v[r], v[r], s2);
+        if (INIT) s0 = fma(base[r], base[r], s0);
+      }
+    }
+  } epi{dst, 0.0, 0.0};
+  fx_pass<FX27>(mU, mB, d, op, max(st->umax, st->bmax), zc, &st->fault, epi);
+  if constexpr (INIT) block_partial2_nt<256>(epi.s2, epi.s0, partials, partials + 2 * nblocks);
+  else block_partial_nt<256>(epi.s2, partials);
+}
+
+// What the boundary data add to the reference norm: k_c27_fx<INIT> sums b^2, and
+// the reference residual b - A u0 differs from b on the nodes that have a
+// boundary node among their 26 neighbours, the first and last layer of each
+// axis.  Partials {sum of (b - A u0)^2 - b^2, 0} per block over those nodes.
+__global__ void __launch_bounds__(256)
+    k_c27_shell(Dims d, Wts<double> W, const double* __restrict__ u, const double* __restrict__ b,
+                double* __restrict__ partials) {
+  const int ni = d.ni(), nj = d.nj(), nk = d.nk();
+  const double nw[4] = {-W.w[0], -W.w[1], -W.w[2], -W.w[3]};
+  // faces k = 1, nk whole; j = 1, nj without those; i = 1, ni without both
+  const int lk = nk > 1 ? 2 : 1, lj = nj > 1 ? 2 : 1, li = ni > 1 ? 2 : 1;
+  const int mk = nk - lk, mj = nj - lj;   // planes and rows strictly inside
+  const long long nz = (long long)lk * ni * nj, ny = (long long)lj * ni * mk, nx = (long long)li * mj * mk;
+  double s = 0.0;
+  for (long long t0 = blockIdx.x * 256LL + threadIdx.x; t0 < nz + ny + nx; t0 += gridDim.x * 256LL) {
+    long long t = t0;
+    int i, j, k;
+    if (t < nz) {
+      i = (int)(t % ni) + 1;
+      j = (int)(t / ni % nj) + 1;
+      k = t / ni / nj == 0 ? 1 : nk;
+    } else if ((t -= nz) < ny) {
+      i = (int)(t % ni) + 1;
+      k = (int)(t / ni % mk) + 2;
+      j = t / ni / mk == 0 ? 1 : nj;
+    } else {
+      t -= ny;
+      j = (int)(t % mj) + 2;
+      k = (int)(t / mj % mk) + 2;
+      i = t / mj / mk == 0 ? 1 : ni;
+    }
+    const double f = b[d.at(i, j, k)];
+    const double r0 = plane_p_plus(nw, plane_of(plane_load<true>(d, u, i, j, k)), f,
+                                   plane_q(nw, plane_of(plane_load<true>(d, u, i, j, k - 1))),
+                                   plane_q(nw, plane_of(plane_load<true>(d, u, i, j, k + 1))));
+    s += fma(r0, r0, -(f * f));
+  }
+  block_partial_nt<256>(s, partials);
+}
+
+template <typename TR, bool INIT>
+static cudaError_t c27_fx_t(const Dims& d, int order, double h, const double* u, const double* b, TR* r,
+                            double* partials, DevState* st, int* nb, cudaStream_t s) {
+  static std::atomic<int> cached{0};
+  constexpr int smem = FxGeom<FX27>::SMEM;
+  int occ = 0;
+  const cudaError_t e = fx_occupancy(k_c27_fx<TR, INIT>, smem, cached, &occ);
+  if (e != cudaSuccess) return e;
+  CUtensorMap mU, mB;
+  if (!fx_maps<FX27>(d, u, b, &mU, &mB)) return cudaErrorInvalidValue;
+  FxOp op;   // r = b - T / (den h^2)
+  const double den = order == 2 ? 1.0 : (order == 4 ? 6.0 : 30.0);
+  op.a1 = order == 2 ? 1 : (order == 4 ? 2 : 14);
+  op.a2 = order == 2 ? 0 : (order == 4 ? 1 : 3);
+  op.a3 = order == 6 ? 1 : 0;
+  op.c = -1.0 / (den * h * h);
+  int zc = 0;
+  const dim3 grid = fx_grid<FX27>(d, occ, &zc);
+  *nb = (int)(grid.x * grid.y * grid.z);
+  k_c27_fx<TR, INIT><<<grid, 256, smem, s>>>(mU, mB, d, op, r, zc, partials, st, *nb);
+  if (INIT)
+    k_c27_shell<<<C27_SHELL_BLOCKS, 256, 0, s>>>(d, wts<double>(compact_lhs(order, h)), u, b, partials + 4 * *nb);
   return cudaGetLastError();
+}
+
+cudaError_t launch_c27_init(const Dims& d, int order, double h, const double* u, const double* b, int dt_r, void* r,
+                            double* partials, DevState* st, int* nb, int* nref, int* kernels, cudaStream_t s) {
+  if (d.g != 1 || (dt_r != DT_F64 && dt_r != DT_F32)) return cudaErrorInvalidValue;
+  if (fx_level(d)) {
+    const cudaError_t e = dt_r == DT_F64 ? c27_fx_t<double, true>(d, order, h, u, b, (double*)r, partials, st, nb, s)
+                                         : c27_fx_t<float, true>(d, order, h, u, b, (float*)r, partials, st, nb, s);
+    *nref = *nb + C27_SHELL_BLOCKS;
+    *kernels = 2;
+    return e;
+  }
+  const dim3 g = c27_grid(d), b64(CBX, CBY / FRB);
+  const Wts<double> w = wts<double>(compact_lhs(order, h));
+  *nb = *nref = c27_blocks(d);
+  *kernels = 1;
+  if (dt_r == DT_F64)
+    k_c27_f64<0, false, double, true, true><<<g, b64, 0, s>>>(d, w, 0.0, u, b, (double*)r, partials, nullptr, *nb);
+  else
+    k_c27_f64<0, false, float, true, true><<<g, b64, 0, s>>>(d, w, 0.0, u, b, (float*)r, partials, nullptr, *nb);
+  return cudaGetLastError();
+}
+
+cudaError_t launch_c27_outer(const Dims& d, int order, double h, const double* u, const double* b, float* r,
+                             double* partials, DevState* st, int* nb, cudaStream_t s) {
+  if (d.g != 1) return cudaErrorInvalidValue;
+  if (fx_level(d)) return c27_fx_t<float, false>(d, order, h, u, b, r, partials, st, nb, s);
+  *nb = c27_blocks(d);
+  return launch_c27_resid_dt(d, compact_lhs(order, h), u, b, DT_F32, r, partials, st, s);
 }
 
 cudaError_t launch_c27_spai(const Dims& d, const W27& M, double omega, const double* r, double* u,

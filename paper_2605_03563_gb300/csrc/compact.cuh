@@ -28,12 +28,19 @@ cudaError_t launch_c27_resid(const Dims& d, const W27& A, const double* u, const
 cudaError_t launch_c27_resid_dt(const Dims& d, const W27& A, const double* u, const double* b, int dt_r, void* r,
                                 double* partials, const DevState* st, cudaStream_t s);
 int c27_blocks(const Dims& d);
-// Initial residual of a compact solve: r = b - A u (stored FP64 or FP32 per
-// dt_r) with per-block partials {sum r^2, 0} at partials[0 .. 2 nb) and the
-// reference residual b - A u0 (u0: boundary data of u only) as partials at
-// partials[2 nb .. 4 nb), nb = c27_blocks(d), in one pass.
-cudaError_t launch_c27_init(const Dims& d, const W27& A, const double* u, const double* b, int dt_r, void* r,
-                            double* partials, cudaStream_t s);
+// Initial residual of a compact solve of the given order and spacing: r = b - L_h u
+// (stored FP64 or FP32 per dt_r) with *nb per-block partials {sum r^2, 0} at
+// partials[0 .. 2 nb) and *nref partials of the reference residual b - L_h u0
+// (u0: boundary data of u only) at partials[2 nb .. 2 nb + 2 nref).  nb <=
+// c27_blocks(d), nref <= nb + C27_SHELL_BLOCKS.  st->umax and st->bmax bound |u|.
+// *kernels: launches.
+constexpr int C27_SHELL_BLOCKS = 304;
+cudaError_t launch_c27_init(const Dims& d, int order, double h, const double* u, const double* b, int dt_r, void* r,
+                            double* partials, DevState* st, int* nb, int* nref, int* kernels, cudaStream_t s);
+// r = b - L_h u stored as FP32 with partials {sum r^2, 0} in *nb blocks: the
+// refinement's outer residual after launch_correct (st->umax bounds |u|)
+cudaError_t launch_c27_outer(const Dims& d, int order, double h, const double* u, const double* b, float* r,
+                             double* partials, DevState* st, int* nb, cudaStream_t s);
 // u -= omega M r on the interior (Eq. richardson for A = -L_h with M of Eq. Smoother)
 cudaError_t launch_c27_spai(const Dims& d, const W27& M, double omega, const double* r, double* u,
                             const DevState* st, cudaStream_t s);

@@ -319,6 +319,8 @@ struct DevState {
   int iter_repl;           // BiCGSTAB: iteration of the last replacement
   int discard;             // refinement form: the inner solve failed, drop its increments
   int inner_cap;           // refinement form: most iterations of the current inner solve
+  unsigned umax;      // high word of max |phi| of the finest FP64 potential as last written (set-up copy, correction)
+  unsigned bmax;      // the same over its boundary nodes
   int lag_pending;         // lagged-norm V-cycles: a first colour pass with saved values ran this step
 };
 

@@ -931,18 +931,20 @@ cudaError_t vcycle_compact(ps_ctx* h, Hier* H, const CompactLevels& C, int l, in
 // b = R_h (4 pi G rho), then the initial residual r (stored as dt_r) and the
 // reference norm ||b - A u0|| in one pass; the state takes the reference
 // first, then the initial relative residual.
-static cudaError_t compact_prologue(ps_ctx* h, int order, const W27& A0, const double* rho, const double* phi,
-                                    double* b, int dt_r, void* r, int nb, cudaStream_t s) {
+static cudaError_t compact_prologue(ps_ctx* h, int order, const double* rho, const double* phi,
+                                    double* b, int dt_r, void* r, cudaStream_t s) {
   const double n = (double)h->d0.ni() * h->d0.nj() * h->d0.nk();
   prof_begin(h, PC_RHS0, n * 16.0, n * (order == 6 ? 19.0 : 12.0), 1, s);
   cudaError_t e = (h->nlaunch += 1, launch_c27_rhs(h->d0, h->du, order, rho, 4.0 * M_PI * h->bc.G, b, s));
   prof_end(h, s);
   if (e != cudaSuccess) return e;
   prof_begin(h, PC_NORM0, n * (16.0 + (double)dt_size(dt_r)), n * 18.0, 1, s);
-  e = (h->nlaunch += 1, launch_c27_init(h->d0, A0, phi, b, dt_r, r, h->partials, s));
+  int nb = 0, nref = 0, kernels = 0;
+  e = launch_c27_init(h->d0, order, h->h0[0], phi, b, dt_r, r, h->partials, h->st, &nb, &nref, &kernels, s);
+  h->nlaunch += kernels;
   prof_end(h, s);
   if (e != cudaSuccess) return e;
-  if ((e = (h->nlaunch += 1, launch_finish_norm(h->partials + 2 * nb, nb, 1.0, 0, h->st, s))) != cudaSuccess) return e;
+  if ((e = (h->nlaunch += 1, launch_finish_norm(h->partials + 2 * nb, nref, 1.0, 0, h->st, s))) != cudaSuccess) return e;
   return (h->nlaunch += 1, launch_finish_norm(h->partials, nb, 1.0, 1, h->st, s));
 }
 
@@ -957,12 +959,12 @@ ps_status begin_mg_compact(ps_ctx* h, const double* rho, const ps_solve_opts* o,
   for (int l = 0; l < h->nlev; l++) hl.push_back(H->lv[l].h[0]);
   auto C = std::make_shared<CompactLevels>(make_compact_levels(order, hl));
   const int nb = c27_blocks(h->d0);
-  if ((r = ensure_partials(h, 2 * nb)) != PS_OK) return r;
+  if ((r = ensure_partials(h, 2 * nb + C27_SHELL_BLOCKS)) != PS_OK) return r;
   double* b = h->fs64;
   double* rr = (double*)H->lv[0].tmp;
   // b = R_h (4 pi G rho); initial residual and reference ||b - A u0|| (u0:
   // boundary data only) in one pass
-  TRY(compact_prologue(h, order, C->A[0], rho, phi, b, DT_F64, rr, nb, s));
+  TRY(compact_prologue(h, order, rho, phi, b, DT_F64, rr, s));
   const int nu1 = o->nu1, nu2 = o->nu2;
   h->act.body = [h, H, C, phi, b, rr, nb, nu1, nu2](unsigned long long cond, int chunk, cudaStream_t q) -> cudaError_t {
     cudaError_t e = vcycle_compact(h, H, *C, 0, nu1, nu2, q);
@@ -996,7 +998,7 @@ ps_status begin_ir_compact(ps_ctx* h, const double* rho, const ps_solve_opts* o,
   for (int l = 0; l < h->nlev; l++) hl.push_back(H->lv[l].h[0]);
   auto C = std::make_shared<CompactLevels>(make_compact_levels(order, hl));
   const int nb = c27_blocks(h->d0);
-  if ((r = ensure_partials(h, 2 * nb)) != PS_OK) return r;
+  if ((r = ensure_partials(h, 2 * nb + C27_SHELL_BLOCKS)) != PS_OK) return r;
   double* phi = h->phi0;
   double* b64 = h->fs64;
   Level& L0 = H->lv[0];
@@ -1007,10 +1009,10 @@ ps_status begin_ir_compact(ps_ctx* h, const double* rho, const ps_solve_opts* o,
     if (!L.phib) return fail(PS_ERR_CUDA, "compact refinement: level %d has no second array", l);
     TRY(cudaMemsetAsync(L.phib, 0, (size_t)L.d.size() * dt_size(L.dt), s));
   }
-  TRY(compact_prologue(h, order, C->A[0], rho, phi, b64, DT_F32, L0.fs, nb, s));
+  TRY(compact_prologue(h, order, rho, phi, b64, DT_F32, L0.fs, s));
   const int nu1 = o->nu1, nu2 = o->nu2, inner = std::max(1, o->inner_cycles);
   h->act.inner_per_iter = inner;
-  h->act.body = [h, H, C, phi, b64, nb, nu1, nu2, inner](unsigned long long cond, int chunk, cudaStream_t q) -> cudaError_t {
+  h->act.body = [h, H, C, phi, b64, order, nu1, nu2, inner](unsigned long long cond, int chunk, cudaStream_t q) -> cudaError_t {
     Level& L = H->lv[0];
     cudaError_t e = cudaMemsetAsync(L.phi, 0, (size_t)L.d.size() * sizeof(float), q);
     for (int c = 0; c < inner && e == cudaSuccess; c++) e = vcycle_compact(h, H, *C, 0, nu1, nu2, q);
@@ -1021,9 +1023,10 @@ ps_status begin_ir_compact(ps_ctx* h, const double* rho, const ps_solve_opts* o,
       e = (h->nlaunch += 1, launch_correct(h->d0, DT_F32, L.phi, 1.0, phi, h->st, q));
       prof_end(h, q);
     }
+    int nb = 0;
     if (e == cudaSuccess) {
       prof_begin(h, PC_NORM0, n * 20.0, n * 17.0, 1, q);
-      e = (h->nlaunch += 1, launch_c27_resid_dt(h->d0, C->A[0], phi, b64, DT_F32, L.fs, h->partials, h->st, q));
+      e = (h->nlaunch += 1, launch_c27_outer(h->d0, order, h->h0[0], phi, b64, (float*)L.fs, h->partials, h->st, &nb, q));
       prof_end(h, q);
     }
     if (e == cudaSuccess) e = (h->nlaunch += 1, launch_finish_norm(h->partials, nb, 1.0, 2, h->st, q, cond, chunk));
@@ -1745,7 +1748,7 @@ ps_status poisson_create(const ps_grid* grid, const double* const coords_host[3]
     if ((s = alloc_zero((void**)&h->phi0, (size_t)h->d0.size() * 8, &h->bytes)) != PS_OK) return bail(s);
     if ((s = ensure_partials(h, std::max({cart_partials_count(h->d0), delta_colours_partials(h->d0, stencil_order),
                                                   batch_norm_partials(h->d0, stencil_order),
-                                                  stencil_order == 2 ? 2 * c27_blocks(h->d0) : 0}))) != PS_OK)
+                                                  stencil_order == 2 ? 2 * c27_blocks(h->d0) + C27_SHELL_BLOCKS : 0}))) != PS_OK)
       return bail(s);
     if (b.outer == PS_BC_MULTIPOLE) {
       build_multipole_tables(l_max, &h->mpt);

@@ -118,6 +118,7 @@ __device__ __forceinline__ void finish_norm_block(const double* __restrict__ par
   }
   st->rr = rr;
   st->amax = m;
+  st->umax = 0u;   // the residual pass that used it has run
   const double rel = sqrt(rr) / st->ref;
   st->rel = rel;
   // IR: the scale of the next stored inner right-hand side (power of two)

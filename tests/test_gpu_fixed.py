@@ -1,0 +1,105 @@
+"""Residual passes whose neighbour sums run on the integer pipe: the relative
+residual of a given guess (max_iter = 0), 7- and 13-point and compact 27-point,
+against a plain FP64 evaluation, on a grid above the size from which these
+passes are taken and ragged against their 64 x 16 tile, and just below that
+size (the FP64 passes).  Guesses: smooth, random from node to node (second
+differences as large as the values), one spike 1e8 above the rest, zero
+inside non-zero boundary data, values near the lower end of the exponent
+range (the march's FP64 form), and one infinity (divergence).
+
+Tolerance, derived before the first run: a residual of r.m.s. r formed from
+values of size U with the stencil's weights W (sum of magnitudes) may be off by
+a few roundings of W U at every node, here 32 of them, 32 2^-53 W U / r
+relative; the norms themselves add 1e-12.  The refinement's norm is summed in
+FP32: 1e-5.
+"""
+import numpy as np
+import pytest
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+BIG, SMALL = (96, 112, 80), (80, 96, 64)
+
+
+def _residual(u, f, h, order, compact):
+    g = order // 2
+    def sh(a, dx, dy, dz):
+        nz, ny, nx = a.shape
+        return a[g + dz:nz - g + dz, g + dy:ny - g + dy, g + dx:nx - g + dx]
+    c = sh(u, 0, 0, 0)
+    if compact:
+        w = {2: (-6, 1, 0, 0), 4: (-4, 1 / 3, 1 / 6, 0), 6: (-128 / 30, 14 / 30, 3 / 30, 1 / 30)}[compact]
+        acc = 0.0
+        for dz in (-1, 0, 1):
+            for dy in (-1, 0, 1):
+                for dx in (-1, 0, 1):
+                    acc = acc + w[abs(dx) + abs(dy) + abs(dz)] * sh(u, dx, dy, dz)
+        return f - acc / h ** 2, sum(abs(w[k]) * n for k, n in enumerate((1, 6, 12, 8))) / h ** 2
+    acc = 0.0
+    for d in ((1, 0, 0), (0, 1, 0), (0, 0, 1)):
+        n1 = sh(u, *d) + sh(u, *(-v for v in d))
+        if order == 4:
+            n2 = sh(u, *(2 * v for v in d)) + sh(u, *(-2 * v for v in d))
+            acc = acc + (16 * n1 - n2 - 30 * c) / 12.0
+        else:
+            acc = acc + (n1 - 2 * c)
+    return f - acc / h ** 2, (16.0 if order == 4 else 12.0) / h ** 2
+
+
+def _guess(kind, shape, g):
+    rng = np.random.Generator(np.random.PCG64(4))
+    z, y, x = np.meshgrid(*(np.linspace(0, 1, s) for s in shape), indexing="ij")
+    u = np.exp(-((x - .4) ** 2 + (y - .5) ** 2 + (z - .6) ** 2) / .1) - 2.0
+    if kind == "rough":
+        u = rng.standard_normal(shape)
+    elif kind == "spike":
+        u[shape[0] // 2, shape[1] // 3, shape[2] // 4] = 1e8
+    elif kind == "boundary":
+        u[g:-g, g:-g, g:-g] = 0.0
+    elif kind == "tiny":
+        u = u * 1e-270
+    return u
+
+
+@pytest.mark.parametrize("kind", ["smooth", "rough", "spike", "boundary", "tiny"])
+@pytest.mark.parametrize("order,compact,prec", [(2, 0, "fp64"), (4, 0, "fp64"), (2, 0, "mixed_fp32"), (4, 0, "mixed_bf16"),
+                                                (2, 2, "fp64"), (2, 4, "mixed_fp32"), (2, 6, "fp64"), (2, 6, "mixed_fp32")])
+@pytest.mark.parametrize("n", [BIG, SMALL])
+def test_initial_residual(n, order, compact, prec, kind):
+    import paper_2605_03563_gb300 as P
+    g, h = order // 2, 1.0 / 64
+    hi = tuple(v * h for v in n)
+    shape = tuple(n[a] + 2 * g - 1 for a in (2, 1, 0))
+    u = _guess(kind, shape, g)
+    u0 = u.copy()
+    u0[g:-g, g:-g, g:-g] = 0.0
+    f = np.zeros(tuple(s - 2 * g for s in shape))   # rho = 0: the residual is the operator's value
+    r, W = _residual(u, f, h, order, compact)
+    r0, _ = _residual(u0, f, h, order, compact)
+    want = np.sqrt(np.sum((r / np.max(np.abs(r))) ** 2)) * np.max(np.abs(r)) / (
+        np.sqrt(np.sum((r0 / np.max(np.abs(r0))) ** 2)) * np.max(np.abs(r0)))
+    rms = np.sqrt(np.mean((r / np.max(np.abs(r))) ** 2)) * np.max(np.abs(r))
+    tol = 32 * 2.0 ** -53 * W * np.max(np.abs(u)) / rms + (1e-12 if prec == "fp64" or compact else 1e-5)
+    phi = torch.from_numpy(u).to("cuda:0")
+    with P.CartesianSolver(n, order, hi=hi) as s:
+        info = s.solve(torch.zeros_like(phi), phi, tol=0.0, max_iter=0, prec=prec, compact_order=compact)
+    if kind == "tiny":   # the squares of the norm underflow in any FP64 evaluation
+        assert info.status in (P.capi.PS_OK, P.capi.PS_NOT_CONVERGED, P.capi.PS_DIVERGED)
+        return
+    assert abs(info.rel_residual - want) <= tol * want, (info.rel_residual, want, tol)
+    assert np.array_equal(phi.cpu().numpy(), u)
+
+
+@pytest.mark.parametrize("order,compact", [(2, 0), (4, 0), (2, 6)])
+def test_infinite_guess_diverges(order, compact):
+    import paper_2605_03563_gb300 as P
+    g, h = order // 2, 1.0 / 64
+    shape = tuple(BIG[a] + 2 * g - 1 for a in (2, 1, 0))
+    u = _guess("smooth", shape, g)
+    u[40, 50, 60] = np.inf
+    phi = torch.from_numpy(u).to("cuda:0")
+    with P.CartesianSolver(BIG, order, hi=tuple(v * h for v in BIG)) as s:
+        for prec in ("fp64", "mixed_fp32"):
+            info = s.solve(torch.zeros_like(phi), phi, tol=1e-8, max_iter=3, prec=prec, compact_order=compact)
+            assert info.status == P.capi.PS_DIVERGED
