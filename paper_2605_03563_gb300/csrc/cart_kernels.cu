@@ -223,14 +223,6 @@ __global__ void __launch_bounds__(BX* BY)
   if (RED >= 1) block_sum_max(s2, mx, partials);
 }
 
-// *to = max(*to, v over the block's threads); one atomic per warp, and none
-// where the value is already as large.
-__device__ __forceinline__ void block_atomic_max(unsigned v, unsigned* to) {
-  v = __reduce_max_sync(0xffffffffu, v);
-  const int lane = (threadIdx.x + blockDim.x * threadIdx.y) & 31;
-  if (lane == 0 && v > *(volatile unsigned*)to) atomicMax(to, v);
-}
-
 // Set-up copy of the caller's initial guess (dense rows) into the handle's
 // pitched array, one warp per row.  It records in st->guess_nonzero whether
 // any interior node of the guess is nonzero (+0 and -0 both count as zero):
@@ -263,8 +255,8 @@ __global__ void __launch_bounds__(256)
       }
     }
   }
-  block_atomic_max(hi, &st->umax);
-  block_atomic_max(hb, &st->bmax);
+  atomic_max_group(hi, &st->umax);
+  atomic_max_group(hb, &st->bmax);
   if (__syncthreads_or(nz) && threadIdx.x == 0) st->guess_nonzero = 1;
 }
 
@@ -613,6 +605,7 @@ __global__ void __launch_bounds__(256, 2)
                int dout, void* __restrict__ out, DevState* __restrict__ st, double* __restrict__ partials) {
   if (!STORE && st->guess_nonzero == 0) return;   // an initial residual from zero: the reference vector
   struct Epi {
+    enum { TRACK = 0 };
     double oscale, s2;
     int oexp, dout;
     float s2f, mxf;
@@ -662,7 +655,7 @@ static cudaError_t fx_delta_t(const Dims& d, double c, const double* phi, const 
   if (!fx_maps<KIND>(d, phi, fs, &mU, &mB)) return cudaErrorInvalidValue;
   const dim3 grid = fx_grid<KIND>(d, occ, &zc);
   if (nblocks) *nblocks = (int)(grid.x * grid.y * grid.z);
-  k_fx_delta<KIND, STORE><<<grid, 256, smem, s>>>(mU, mB, d, FxOp{c, 0, 0, 0}, zc, dout, out, st, partials);
+  k_fx_delta<KIND, STORE><<<grid, 256, smem, s>>>(mU, mB, d, FxOp{c, 0, 0, 0, 0}, zc, dout, out, st, partials);
   return cudaGetLastError();
 }
 
@@ -1398,7 +1391,7 @@ cudaError_t launch_restrict_red(const Dims& fine, const Dims& coarse, int dt_f, 
 // memory latency, not by its arithmetic).
 template <typename TC, typename TF>
 __global__ void __launch_bounds__(BX* BY)
-    k_prolong(Dims fd, Dims cd, const TC* __restrict__ ec, TF* __restrict__ phif) {
+    k_prolong(Dims fd, Dims cd, const TC* __restrict__ ec, TF* __restrict__ phif, unsigned* __restrict__ track) {
   using CF = typename St<TF>::C;
   const int I = blockIdx.x * BX + threadIdx.x;   // cell index 0 .. nc-1
   const int J = blockIdx.y * BY + threadIdx.y;
@@ -1409,6 +1402,7 @@ __global__ void __launch_bounds__(BX* BY)
   const long long csy = cd.sy(), csz = cd.sz();
   const long long fsy = fd.sy(), fsz = fd.sz();
   const CF half = (CF)0.5;
+  unsigned hm = 0u;   // high word of the largest |phif| written (FP64)
   // the corner values of a coarse plane's cell face: [y][x]
   auto load_face = [&](long long q0, CF (&c)[2][2]) {
 #pragma unroll
@@ -1473,7 +1467,9 @@ __global__ void __launch_bounds__(BX* BY)
         for (int a = 0; a < 2; a++) {
           if (a == 0 && I == 0) continue;
           const CF v = cz == 0 ? vy[0][b][a] : half * (vy[0][b][a] + vy[1][b][a]);
-          St<TF>::st(phif + f0 + cz * fsz + b * fsy + a, fcur[cz][b][a] + v);
+          const CF nv = fcur[cz][b][a] + v;
+          St<TF>::st(phif + f0 + cz * fsz + b * fsy + a, nv);
+          if constexpr (sizeof(CF) == 8) hm = max(hm, (unsigned)__double2hiint(nv) & 0x7fffffffu);
         }
       }
     }
@@ -1488,28 +1484,29 @@ __global__ void __launch_bounds__(BX* BY)
 #pragma unroll
         for (int a = 0; a < 2; a++) fcur[cz][b][a] = fnext[cz][b][a];
   }
+  if (sizeof(CF) == 8 && track != nullptr) atomic_max_group(hm, track);
 }
 
 template <typename TC, typename TF>
-static cudaError_t prolong_t(const Dims& fine, const Dims& cd, const void* ec, void* phif, cudaStream_t s) {
+static cudaError_t prolong_t(const Dims& fine, const Dims& cd, const void* ec, void* phif, unsigned* track, cudaStream_t s) {
   const int gx = (cd.nx + BX - 1) / BX, gy = (cd.ny + BY - 1) / BY;
   const int zc = zchunk_for(gx * gy, cd.nz);
   const dim3 grid(gx, gy, (cd.nz + zc - 1) / zc);
-  k_prolong<TC, TF><<<grid, dim3(BX, BY), 0, s>>>(fine, cd, (const TC*)ec, (TF*)phif);
+  k_prolong<TC, TF><<<grid, dim3(BX, BY), 0, s>>>(fine, cd, (const TC*)ec, (TF*)phif, track);
   return cudaGetLastError();
 }
 
 cudaError_t launch_prolong(const Dims& fine, const Dims& coarse, int dt_c, const void* e_c, int dt_f, void* phi_f,
-                           cudaStream_t s) {
+                           cudaStream_t s, unsigned* track) {
   if (dt_c == DT_F64) {
-    if (dt_f == DT_F64) return prolong_t<double, double>(fine, coarse, e_c, phi_f, s);
-    if (dt_f == DT_F32) return prolong_t<double, float>(fine, coarse, e_c, phi_f, s);
-    return prolong_t<double, __nv_bfloat16>(fine, coarse, e_c, phi_f, s);
+    if (dt_f == DT_F64) return prolong_t<double, double>(fine, coarse, e_c, phi_f, track, s);
+    if (dt_f == DT_F32) return prolong_t<double, float>(fine, coarse, e_c, phi_f, track, s);
+    return prolong_t<double, __nv_bfloat16>(fine, coarse, e_c, phi_f, track, s);
   }
   if (dt_c == DT_F32) {
-    if (dt_f == DT_F64) return prolong_t<float, double>(fine, coarse, e_c, phi_f, s);
-    if (dt_f == DT_F32) return prolong_t<float, float>(fine, coarse, e_c, phi_f, s);
-    return prolong_t<float, __nv_bfloat16>(fine, coarse, e_c, phi_f, s);
+    if (dt_f == DT_F64) return prolong_t<float, double>(fine, coarse, e_c, phi_f, track, s);
+    if (dt_f == DT_F32) return prolong_t<float, float>(fine, coarse, e_c, phi_f, track, s);
+    return prolong_t<float, __nv_bfloat16>(fine, coarse, e_c, phi_f, track, s);
   }
   return cudaErrorInvalidValue;
 }
@@ -1586,7 +1583,7 @@ __global__ void __launch_bounds__(BX* BY)
       hm = max(hm, (unsigned)__double2hiint(v) & 0x7fffffffu);
     }
   }
-  if (st != nullptr) block_atomic_max(hm, &st->umax);
+  if (st != nullptr) atomic_max_group(hm, &st->umax);
 }
 
 cudaError_t launch_correct(const Dims& d, int dt_e, const void* e, double inv_scale, double* phi,

@@ -115,9 +115,10 @@ cudaError_t launch_restrict(const Dims& fine, const Dims& coarse, int dt_f, cons
 cudaError_t launch_restrict_red(const Dims& fine, const Dims& coarse, int dt_f, const void* delta_f, int dt_c,
                                 void* fs_c, double factor, cudaStream_t s);
 
-// phi_fine += P e_coarse; coarse = layout of e_c
+// phi_fine += P e_coarse; coarse = layout of e_c.  track (FP64 fine levels,
+// optional): *track takes the high word of the largest |phi_fine| written.
 cudaError_t launch_prolong(const Dims& fine, const Dims& coarse, int dt_c, const void* e_c, int dt_f, void* phi_f,
-                           cudaStream_t s);
+                           cudaStream_t s, unsigned* track = nullptr);
 
 // fs = -(4 pi G / d) rho on interior nodes (rho FP64 in layout du, fs in layout d)
 cudaError_t launch_scale_rhs(const Dims& d, const Dims& du, double factor, const double* rho, int dt,

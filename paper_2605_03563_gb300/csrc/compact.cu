@@ -25,6 +25,7 @@
 #include <algorithm>
 #include <atomic>
 #include <cmath>
+#include <numeric>
 #include <type_traits>
 #include <vector>
 
@@ -37,6 +38,12 @@
 namespace ps {
 
 static constexpr int CBX = 32, CBY = 8, CZC = 16;
+
+// omega, alpha, beta, gamma, delta of Table 1 in units of 1e-4 (compact orders
+// 2, 4, 6).  The order-6 row prints delta equal to its mu (a garbled cell);
+// delta = 0.0151 is the value that minimises the local Fourier smoothing factor
+// with the printed omega, alpha, beta and gamma.
+const int kSpaiInt[3][5] = {{13699, 1432, 284, 81, 25}, {9363, 2807, 329, 166, 44}, {3543, 7064, 1005, 363, 151}};
 
 W27 compact_lhs(int order, double h) {
   const double ih2 = 1.0 / (h * h);
@@ -238,7 +245,8 @@ __global__ void __launch_bounds__(CBX*(CBY / FRB))
   if (st != nullptr && st->done) return;   // uniform
   const int i = blockIdx.x * CBX + threadIdx.x + 1;
   const int j0 = blockIdx.y * CBY + threadIdx.y * FRB + 1;   // rows j0 .. j0 + FRB - 1
-  const int k0 = blockIdx.z * CZC + 1, k1 = min(k0 + CZC, d.nk() + 1);
+  const int zc = (d.nk() + gridDim.z - 1) / gridDim.z;
+  const int k0 = blockIdx.z * zc + 1, k1 = min(k0 + zc, d.nk() + 1);
   double s2 = 0.0, s0 = 0.0;
   if (i <= d.ni() && j0 <= d.nj()) {
     Wts<double> nw;
@@ -353,8 +361,16 @@ static Wts<C> wts(const W27& a) {
   return Wts<C>{{(C)a.w[0], (C)a.w[1], (C)a.w[2], (C)a.w[3]}};
 }
 
+// z-planes per block: 16, fewer on smaller levels, where the march is the chain
+// of the pass and about eight blocks of 64 threads per SM hide more of it
+// (63^3 residual or SPAI step 31 -> 16.6 us under ncu).
+static int c27_zc(const Dims& d) {
+  const long long tiles = (long long)((d.ni() + CBX - 1) / CBX) * ((d.nj() + CBY - 1) / CBY);
+  return (int)std::max(2LL, std::min((long long)CZC, tiles * d.nk() / (8LL * device_sm_count())));
+}
 static dim3 c27_grid(const Dims& d) {
-  return dim3((d.ni() + CBX - 1) / CBX, (d.nj() + CBY - 1) / CBY, (d.nk() + CZC - 1) / CZC);
+  const int zc = c27_zc(d);
+  return dim3((d.ni() + CBX - 1) / CBX, (d.nj() + CBY - 1) / CBY, (d.nk() + zc - 1) / zc);
 }
 
 int c27_blocks(const Dims& d) {
@@ -380,21 +396,32 @@ cudaError_t launch_c27_resid_dt(const Dims& d, const W27& A, const double* u, co
   return cudaGetLastError();
 }
 
-// The finest level's residual r = b - L_h u with the sums over the 26 neighbours
-// on the integer pipe (fixed.cuh): the weights of L_h are integers over 30 h^2
-// (6 h^2, h^2), so three FP64 instructions a node are left with the norm,
-// instead of 13.5.  INIT: also the sum of b^2, which k_c27_shell completes to the
-// reference norm.
-// Under ncu at 256^3: outer residual 532 -> 138 us, initial pass 815 -> 167 us
-// and 29 us for the shell; 512^3 outer residual in the solve 3942 -> 1110 us.
-template <typename TR, bool INIT>
+// 27-point passes with the sums over the 26 neighbours on the integer pipe
+// (fixed.cuh).  The weights of L_h, of its Galerkin products and of the SPAI
+// smoother are integers over a common factor, so one FP64 instruction a node
+// forms the value (three with a norm), instead of 12.5.  In every mode the value
+// is base + c T(in), stored as TR:
+//   C27_INIT   r = b - A u, sums of r^2 and of b^2 (which k_c27_shell completes to
+//              the reference norm);
+//   C27_NORM   r = b - A u, sum of r^2; *track takes the largest |u| read;
+//   C27_RESID  r = b - A u; *track the largest |r| written;
+//   C27_SPAI   u - omega M r (in = r, base and dst = u: a block writes the nodes
+//              whose base it has read); *track the largest |u| written.
+// The unit comes from the larger of *h1 and *h2, the high words of max |in|.
+// PS_FX27_TIMES
+enum { C27_INIT, C27_NORM, C27_RESID, C27_SPAI };
+template <int MODE, typename TR>
 __global__ void __launch_bounds__(256, 2)
     k_c27_fx(const __grid_constant__ CUtensorMap mU, const __grid_constant__ CUtensorMap mB, Dims d, FxOp op,
-             TR* __restrict__ dst, int zc, double* __restrict__ partials, DevState* __restrict__ st, int nblocks) {
-  if (!INIT && st->done) return;   // uniform
+             TR* __restrict__ dst, int zc, double* __restrict__ partials, DevState* __restrict__ st,
+             const unsigned* __restrict__ h1, const unsigned* __restrict__ h2, unsigned* __restrict__ track,
+             int nblocks) {
+  if (MODE != C27_INIT && st->done) return;   // uniform
   struct Epi {
+    enum { TRACK = MODE == C27_NORM && sizeof(TR) == 8 };
     TR* dst;
     double s2, s0;
+    unsigned hmax;
     __device__ __forceinline__ void operator()(long long at, int px, const bool (&in)[4], const double (&v)[4],
                                                const double (&base)[4]) {
       TR x[4];
@@ -405,17 +432,19 @@ __global__ void __launch_bounds__(256, 2)
       for (int r = 0; r < 4; r++) {
         if (!in[r]) continue;
         dst[at + r * px] = x[r];
-        s2 = fma(v[r], v[r], s2);
-        if (INIT) s0 = fma(base[r], base[r], s0);
+        if (MODE == C27_INIT || MODE == C27_NORM) s2 = fma(v[r], v[r], s2);
+        else hmax = max(hmax, (unsigned)__double2hiint(v[r]) & 0x7fffffffu);
+        if (MODE == C27_INIT) s0 = fma(base[r], base[r], s0);
       }
     }
-  } epi{dst, 0.0, 0.0};
-  fx_pass<FX27>(mU, mB, d, op, max(st->umax, st->bmax), zc, &st->fault, epi);
-  if constexpr (INIT) block_partial2_nt<256>(epi.s2, epi.s0, partials, partials + 2 * nblocks);
-  else block_partial_nt<256>(epi.s2, partials);
+  } epi{dst, 0.0, 0.0, 0u};
+  fx_pass<FX27>(mU, mB, d, op, max(*h1, *h2), zc, &st->fault, epi);
+  if ((Epi::TRACK || MODE == C27_RESID || MODE == C27_SPAI) && track != nullptr) atomic_max_group(epi.hmax, track);
+  if constexpr (MODE == C27_INIT) block_partial2_nt<256>(epi.s2, epi.s0, partials, partials + 2 * nblocks);
+  if constexpr (MODE == C27_NORM) block_partial_nt<256>(epi.s2, partials);
 }
 
-// What the boundary data add to the reference norm: k_c27_fx<INIT> sums b^2, and
+// What the boundary data add to the reference norm: k_c27_fx<C27_INIT> sums b^2, and
 // the reference residual b - A u0 differs from b on the nodes that have a
 // boundary node among their 26 neighbours, the first and last layer of each
 // axis.  Partials {sum of (b - A u0)^2 - b^2, 0} per block over those nodes.
@@ -455,43 +484,96 @@ __global__ void __launch_bounds__(256)
   block_partial_nt<256>(s, partials);
 }
 
-template <typename TR, bool INIT>
-static cudaError_t c27_fx_t(const Dims& d, int order, double h, const double* u, const double* b, TR* r,
-                            double* partials, DevState* st, int* nb, cudaStream_t s) {
+template <int MODE, typename TR>
+static cudaError_t c27_fx_t(const Dims& d, const FxOp& op, const double* in, const double* base, TR* dst,
+                            double* partials, DevState* st, const unsigned* h1, const unsigned* h2, unsigned* track,
+                            int* nb, cudaStream_t s) {
   static std::atomic<int> cached{0};
   constexpr int smem = FxGeom<FX27>::SMEM;
-  int occ = 0;
-  const cudaError_t e = fx_occupancy(k_c27_fx<TR, INIT>, smem, cached, &occ);
+  int occ = 0, zc = 0;
+  const cudaError_t e = fx_occupancy(k_c27_fx<MODE, TR>, smem, cached, &occ);
   if (e != cudaSuccess) return e;
   CUtensorMap mU, mB;
-  if (!fx_maps<FX27>(d, u, b, &mU, &mB)) return cudaErrorInvalidValue;
-  FxOp op;   // r = b - T / (den h^2)
-  const double den = order == 2 ? 1.0 : (order == 4 ? 6.0 : 30.0);
-  op.a1 = order == 2 ? 1 : (order == 4 ? 2 : 14);
-  op.a2 = order == 2 ? 0 : (order == 4 ? 1 : 3);
-  op.a3 = order == 6 ? 1 : 0;
-  op.c = -1.0 / (den * h * h);
-  int zc = 0;
+  if (!fx_maps<FX27>(d, in, base, &mU, &mB)) return cudaErrorInvalidValue;
   const dim3 grid = fx_grid<FX27>(d, occ, &zc);
-  *nb = (int)(grid.x * grid.y * grid.z);
-  k_c27_fx<TR, INIT><<<grid, 256, smem, s>>>(mU, mB, d, op, r, zc, partials, st, *nb);
-  if (INIT)
-    k_c27_shell<<<C27_SHELL_BLOCKS, 256, 0, s>>>(d, wts<double>(compact_lhs(order, h)), u, b, partials + 4 * *nb);
+  const int n = (int)(grid.x * grid.y * grid.z);
+  if (nb) *nb = n;
+  k_c27_fx<MODE, TR><<<grid, 256, smem, s>>>(mU, mB, d, op, dst, zc, partials, st, h1, h2, track, n);
   return cudaGetLastError();
+}
+
+C27Ops c27_ops(int order, double h, int level) {
+  // L_h in integers over den h^2; a Galerkin product in 512ths of the level above
+  C27Ops o{};
+  W27 w = order == 2 ? W27{{-6.0, 1.0, 0.0, 0.0}} : (order == 4 ? W27{{-24.0, 2.0, 1.0, 0.0}} : W27{{-128.0, 14.0, 3.0, 1.0}});
+  double scale = 1.0 / ((order == 2 ? 1.0 : (order == 4 ? 6.0 : 30.0)) * h * h);
+  long long a[4] = {0, 0, 0, 0};
+  o.ok = true;
+  for (int l = 0;; l++) {
+    long long g = 0;
+    for (int c = 0; c < 4; c++) {
+      a[c] = std::llround(w.w[c]);
+      if ((double)a[c] != w.w[c]) o.ok = false;
+      g = std::gcd(g, a[c]);
+    }
+    if (g == 0) o.ok = false;
+    if (!o.ok) return o;
+    for (int c = 0; c < 4; c++) a[c] /= g;
+    scale *= (double)g;
+    if (l == level) break;
+    w = galerkin27(W27{{(double)a[0], (double)a[1], (double)a[2], (double)a[3]}});
+    for (double& v : w.w) v *= 512.0;
+    scale /= 512.0;
+  }
+  // the SPAI weights of Table 1 (four decimals) with the level's spacing
+  const double hl = std::ldexp(h, level);
+  const int* m = kSpaiInt[order / 2 - 1];
+  auto fits = [](long long w0, long long w1, long long w2, long long w3) {
+    return w1 >= 0 && w2 >= 0 && w3 >= 0 && std::llabs(w0) + 6 * w1 + 12 * w2 + 8 * w3 <= FX_WSUM;
+  };
+  o.ok = fits(a[0], a[1], a[2], a[3]) && fits(m[1], m[2], m[3], m[4]);
+  o.resid = C27Weights{-scale, (int)a[0], (int)a[1], (int)a[2], (int)a[3]};
+  o.spai = C27Weights{-(m[0] * 1e-4) * hl * hl * 1e-4, m[1], m[2], m[3], m[4]};
+  return o;
+}
+
+static FxOp fx_op(const C27Weights& w) { return FxOp{w.c, w.w0, w.w1, w.w2, w.w3}; }
+
+bool c27_fx_level(const Dims& d, const C27Ops& ops) { return d.g == 1 && ops.ok && fx_level(d); }
+
+cudaError_t launch_c27_fx_resid(const Dims& d, const C27Ops& ops, const double* u, const double* b, double* r,
+                                DevState* st, const unsigned* hu, const unsigned* hb, unsigned* hr, cudaStream_t s) {
+  return c27_fx_t<C27_RESID, double>(d, fx_op(ops.resid), u, b, r, nullptr, st, hu, hb, hr, nullptr, s);
+}
+
+cudaError_t launch_c27_fx_norm(const Dims& d, const C27Ops& ops, const double* u, const double* b, double* r,
+                               double* partials, DevState* st, int* nb, cudaStream_t s) {
+  return c27_fx_t<C27_NORM, double>(d, fx_op(ops.resid), u, b, r, partials, st, &st->umax, &st->bmax, &st->unext, nb, s);
+}
+
+cudaError_t launch_c27_fx_spai(const Dims& d, const C27Ops& ops, const double* r, double* u, DevState* st,
+                               const unsigned* hr, unsigned* hu, cudaStream_t s) {
+  return c27_fx_t<C27_SPAI, double>(d, fx_op(ops.spai), r, u, u, nullptr, st, hr, hr, hu, nullptr, s);
 }
 
 cudaError_t launch_c27_init(const Dims& d, int order, double h, const double* u, const double* b, int dt_r, void* r,
                             double* partials, DevState* st, int* nb, int* nref, int* kernels, cudaStream_t s) {
   if (d.g != 1 || (dt_r != DT_F64 && dt_r != DT_F32)) return cudaErrorInvalidValue;
-  if (fx_level(d)) {
-    const cudaError_t e = dt_r == DT_F64 ? c27_fx_t<double, true>(d, order, h, u, b, (double*)r, partials, st, nb, s)
-                                         : c27_fx_t<float, true>(d, order, h, u, b, (float*)r, partials, st, nb, s);
+  const Wts<double> w = wts<double>(compact_lhs(order, h));
+  const C27Ops ops = c27_ops(order, h, 0);
+  if (c27_fx_level(d, ops)) {
+    const FxOp op = fx_op(ops.resid);
+    const cudaError_t e =
+        dt_r == DT_F64
+            ? c27_fx_t<C27_INIT, double>(d, op, u, b, (double*)r, partials, st, &st->umax, &st->bmax, nullptr, nb, s)
+            : c27_fx_t<C27_INIT, float>(d, op, u, b, (float*)r, partials, st, &st->umax, &st->bmax, nullptr, nb, s);
+    if (e != cudaSuccess) return e;
+    k_c27_shell<<<C27_SHELL_BLOCKS, 256, 0, s>>>(d, w, u, b, partials + 4 * *nb);
     *nref = *nb + C27_SHELL_BLOCKS;
     *kernels = 2;
-    return e;
+    return cudaGetLastError();
   }
   const dim3 g = c27_grid(d), b64(CBX, CBY / FRB);
-  const Wts<double> w = wts<double>(compact_lhs(order, h));
   *nb = *nref = c27_blocks(d);
   *kernels = 1;
   if (dt_r == DT_F64)
@@ -504,7 +586,9 @@ cudaError_t launch_c27_init(const Dims& d, int order, double h, const double* u,
 cudaError_t launch_c27_outer(const Dims& d, int order, double h, const double* u, const double* b, float* r,
                              double* partials, DevState* st, int* nb, cudaStream_t s) {
   if (d.g != 1) return cudaErrorInvalidValue;
-  if (fx_level(d)) return c27_fx_t<float, false>(d, order, h, u, b, r, partials, st, nb, s);
+  const C27Ops ops = c27_ops(order, h, 0);
+  if (c27_fx_level(d, ops))
+    return c27_fx_t<C27_NORM, float>(d, fx_op(ops.resid), u, b, r, partials, st, &st->umax, &st->bmax, nullptr, nb, s);
   *nb = c27_blocks(d);
   return launch_c27_resid_dt(d, compact_lhs(order, h), u, b, DT_F32, r, partials, st, s);
 }
@@ -834,7 +918,8 @@ __global__ void __launch_bounds__(CBX*(CBY / FRB))
     k_c27_rhs(Dims d, Dims du, const double* __restrict__ rho, Wts<double> W, double* __restrict__ b) {
   const int i = blockIdx.x * CBX + threadIdx.x + 1;
   const int j0 = blockIdx.y * CBY + threadIdx.y * FRB + 1;   // rows j0 .. j0 + FRB - 1
-  const int k0 = blockIdx.z * CZC + 1, k1 = min(k0 + CZC, d.nk() + 1);
+  const int zc = (d.nk() + gridDim.z - 1) / gridDim.z;
+  const int k0 = blockIdx.z * zc + 1, k1 = min(k0 + zc, d.nk() + 1);
   if (i > d.ni() || j0 > d.nj()) return;
   const long long sy = du.sy(), sz = du.sz();
   if (ORDER == 2) {

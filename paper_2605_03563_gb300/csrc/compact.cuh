@@ -13,6 +13,9 @@ struct W27 {
   double w[4];
 };
 
+// Table 1's omega, alpha, beta, gamma, delta for compact orders 2, 4, 6, times 1e4
+extern const int kSpaiInt[3][5];
+
 // Compact L_h of order 2, 4, 6 in units of 1/h^2, and the right-hand side R_h.
 W27 compact_lhs(int order, double h);
 // Galerkin coarse operator R A P (full weighting R, trilinear P = 8 R^T) of an
@@ -37,6 +40,31 @@ int c27_blocks(const Dims& d);
 constexpr int C27_SHELL_BLOCKS = 304;
 cudaError_t launch_c27_init(const Dims& d, int order, double h, const double* u, const double* b, int dt_r, void* r,
                             double* partials, DevState* st, int* nb, int* nref, int* kernels, cudaStream_t s);
+// Integer form of a level's operator and smoother for the fixed-point passes
+// (fixed.cuh): value = base + c (w0 centre + w1 faces + w2 edges + w3 corners).
+struct C27Weights {
+  double c;
+  int w0, w1, w2, w3;
+};
+struct C27Ops {
+  bool ok = false;      // the weights are integers small enough for the passes
+  C27Weights resid{};   // r = b - A u
+  C27Weights spai{};    // u - omega M r
+};
+// of level `level` (spacing h 2^level) under a finest level of the given order and spacing h
+C27Ops c27_ops(int order, double h, int level);
+// whether a level takes these passes (else launch_c27_resid / launch_c27_spai)
+bool c27_fx_level(const Dims& d, const C27Ops& ops);
+// r = b - A u; the larger of *hu and *hb bounds |u| (high words), *hr takes max |r|
+cudaError_t launch_c27_fx_resid(const Dims& d, const C27Ops& ops, const double* u, const double* b, double* r,
+                                DevState* st, const unsigned* hu, const unsigned* hb, unsigned* hr, cudaStream_t s);
+// the same on the finest level with partials {sum r^2, 0} in *nb blocks;
+// st->umax bounds |u|, st->unext takes the largest |u| read
+cudaError_t launch_c27_fx_norm(const Dims& d, const C27Ops& ops, const double* u, const double* b, double* r,
+                               double* partials, DevState* st, int* nb, cudaStream_t s);
+// u -= omega M r; *hr bounds |r|, *hu takes the largest |u| written
+cudaError_t launch_c27_fx_spai(const Dims& d, const C27Ops& ops, const double* r, double* u, DevState* st,
+                               const unsigned* hr, unsigned* hu, cudaStream_t s);
 // r = b - L_h u stored as FP32 with partials {sum r^2, 0} in *nb blocks: the
 // refinement's outer residual after launch_correct (st->umax bounds |u|)
 cudaError_t launch_c27_outer(const Dims& d, int order, double h, const double* u, const double* b, float* r,

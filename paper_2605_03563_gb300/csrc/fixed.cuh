@@ -11,15 +11,18 @@
 // The unit.  With H the largest |u| of the pass (its high word, kept in the
 // solver state by the kernels that write u), values are below 2^57 units, so a
 // unit is 2^-4 of the last place of H's binade: 1/8 of the largest rounding
-// error of one FP64 addition near H.  The operators annihilate constants, and their sums
-// are formed as second differences,
+// error of one FP64 addition near H.  The 7- and 13-point operators annihilate
+// constants, and their sums are formed as second differences,
 //   7-point   T = S1 - 6 C
 //   13-point  T = 16 (S1 - 6 C) - (S2 - 6 C)      (S1, S2: distance 1, 2)
-//   27-point  T = a1 (faces - 6 C) + a2 (edges - 12 C) + a3 (corners - 8 C)
-// each of which is below 24 H < 2^62 units.  The weighted sum may not be for a
-// field that changes by more than H from node to node; then (a test on the high
-// words) the groups are converted and weighted in FP64 one by one.  What is lost
-// is the part of a value below a unit: against the roundings of an FP64 sum of
+// each group of which is below 12 H < 2^61 units.  The weighted sum may not be
+// for a field that changes by more than H from node to node; then (a test on the
+// high words) the groups are converted and weighted in FP64 one by one.  The
+// 27-point sums
+//   T = w0 C + w1 faces + w2 edges + w3 corners   (integer weights)
+// are formed exactly in two limbs, low and high words multiplied apart (wide
+// 32-bit multiply-adds), and the leading 62 bits converted.  What is lost is
+// the part of a value below a unit: against the roundings of an FP64 sum of
 // values of size |u| the error is smaller wherever |u| > H / 16, and over a field
 // whenever its r.m.s. is (potentials are far from that ratio).
 // Passes whose H is infinite, NaN or near the ends of the exponent range run
@@ -101,10 +104,12 @@ __device__ __forceinline__ void fx_to_f32(const double (&x)[R], int e, float (&y
 
 enum { FX7 = 7, FX13 = 13, FX27 = 27 };
 
-// Operator of a pass: value = base + c T.
+// Operator of a pass: value = base + c T.  27-point: integer weights of T, w1 to
+// w3 >= 0, with |w0| + 6 w1 + 12 w2 + 8 w3 <= FX_WSUM.
+constexpr int FX_WSUM = 65536;
 struct FxOp {
   double c;
-  int a1, a2, a3;   // 27-point integer weights
+  int w0, w1, w2, w3;
 };
 
 template <int KIND>
@@ -128,6 +133,8 @@ struct FxGeom {
 // One barrier a plane: it separates the writes of a work buffer from its reads
 // two planes earlier, and hands the stage of the previous plane back to the
 // copy engine.
+// Epi::TRACK: epi.hmax takes the high word of the largest |u| staged (the
+// tile's own nodes and their halo).
 template <int KIND, typename W, typename Epi>
 __device__ __forceinline__ bool fx_march(const CUtensorMap& mU, const CUtensorMap& mB, const Dims& d, const FxOp& op,
                                          const FxScale& sc, int zc, unsigned char* smem, Epi& epi) {
@@ -201,8 +208,10 @@ __device__ __forceinline__ bool fx_march(const CUtensorMap& mU, const CUtensorMa
 #pragma unroll
     for (int q = 0; q < NLD; q++)
       if ((q + 1) * NT <= NEL || tid + q * NT < NEL) {
-        if constexpr (FX) w[tid + q * NT] = fx_from(raw[tid + q * NT], sc.eb);
-        else w[tid + q * NT] = raw[tid + q * NT];
+        const double v = raw[tid + q * NT];
+        if constexpr (FX) w[tid + q * NT] = fx_from(v, sc.eb);
+        else w[tid + q * NT] = v;
+        if constexpr (Epi::TRACK) epi.hmax = max(epi.hmax, (unsigned)__double2hiint(v) & 0x7fffffffu);
       }
     __syncthreads();
     if (tid == 0 && ok && z > zl) {   // after a failed wait no new copy is issued
@@ -220,46 +229,59 @@ __device__ __forceinline__ bool fx_march(const CUtensorMap& mU, const CUtensorMa
     return b;
   };
   const double cu = FX ? op.c * sc.unit() : op.c;
-  // values of the thread's R nodes from their groups: one test for all of them,
-  // so that their chains run interleaved
-  auto values = [&](const W (&g1)[R], const W (&g2)[R], const W (&g3)[R], const double (&f)[R], double (&x)[R]) {
+  // values of the thread's R nodes from their groups (27-point: centre, faces,
+  // edges, corners; others: second differences at distance 1 and 2)
+  auto values = [&](const W (&c0)[R], const W (&g1)[R], const W (&g2)[R], const W (&g3)[R], const double (&f)[R],
+                    double (&x)[R]) {
     if constexpr (KIND == FX7) {
 #pragma unroll
       for (int r = 0; r < R; r++) x[r] = fma(fx_double(g1[r]), cu, f[r]);
+    } else if constexpr (KIND == FX27 && FX) {
+#pragma unroll
+      for (int r = 0; r < R; r++) {
+        // |T| < 2^73: low words' products below 2^48, high words' below 2^46
+        auto lo = [](long long v) { return (unsigned long long)(unsigned)v; };
+        auto hi = [](long long v) { return (long long)(int)(v >> 32); };
+        const unsigned long long lc = lo(c0[r]) * (unsigned)abs(op.w0);
+        const long long L = (long long)(lo(g1[r]) * (unsigned)op.w1 + lo(g2[r]) * (unsigned)op.w2 +
+                                        lo(g3[r]) * (unsigned)op.w3 + (op.w0 < 0 ? 0ull - lc : lc));
+        const long long H = hi(c0[r]) * op.w0 + hi(g1[r]) * op.w1 + hi(g2[r]) * op.w2 + hi(g3[r]) * op.w3 + (L >> 32);
+        // T = H 2^32 + low; shifted right by 11 unless it fits 63 bits
+        const bool big = (unsigned long long)(H + (1LL << 30)) >= (1ull << 31);
+        const unsigned low = (unsigned)L;
+        const long long t = big ? (long long)((unsigned long long)H << 21 | low >> 11)
+                                : (long long)((unsigned long long)H << 32 | low);
+        const double v = fx_double(t);
+        x[r] = fma(__hiloint2double(__double2hiint(v) + (big ? 11 << 20 : 0), __double2loint(v)), cu, f[r]);
+      }
+    } else if constexpr (KIND == FX27) {
+#pragma unroll
+      for (int r = 0; r < R; r++)
+        x[r] = fma(fma((double)op.w0, c0[r], fma((double)op.w1, g1[r], fma((double)op.w2, g2[r], op.w3 * g3[r]))), cu, f[r]);
     } else {
-      bool fits = true;
+      bool fits = true;   // one test for all nodes, so that their chains run interleaved
       if constexpr (FX) {
 #pragma unroll
-        for (int r = 0; r < R; r++)
-          // 16 2^58 + 2^61 < 2^63; 14 2^58 + 3 2^60 + 2^60 < 2^63
-          fits &= KIND == FX13 ? fx_below(g1[r], 26) && fx_below(g2[r], 29)
-                               : fx_below(g1[r], 26) && fx_below(g2[r], 28) && fx_below(g3[r], 28);
+        for (int r = 0; r < R; r++) fits &= fx_below(g1[r], 26) && fx_below(g2[r], 29);   // 16 2^58 + 2^61 < 2^63
       }
       if (fits) {
 #pragma unroll
-        for (int r = 0; r < R; r++) {
-          const W t = KIND == FX13 ? g1[r] * (W)16 - g2[r] : g1[r] * (W)op.a1 + g2[r] * (W)op.a2 + g3[r] * (W)op.a3;
-          x[r] = fma(fx_double(t), cu, f[r]);
-        }
+        for (int r = 0; r < R; r++) x[r] = fma(fx_double(g1[r] * (W)16 - g2[r]), cu, f[r]);
       } else {
-        const double w1 = (KIND == FX13 ? 16.0 : (double)op.a1) * cu, w2 = (KIND == FX13 ? -1.0 : (double)op.a2) * cu;
 #pragma unroll
-        for (int r = 0; r < R; r++) {
-          x[r] = fma(fx_double(g1[r]), w1, fma(fx_double(g2[r]), w2, f[r]));
-          if (KIND == FX27) x[r] = fma(fx_double(g3[r]), op.a3 * cu, x[r]);
-        }
+        for (int r = 0; r < R; r++) x[r] = fma(fx_double(g1[r]), 16.0 * cu, fma(fx_double(g2[r]), -cu, f[r]));
       }
     }
   };
-  auto finish = [&](const double* b, const W (&g1)[R], const W (&g2)[R], const W (&g3)[R]) {
+  auto finish = [&](const double* b, const W (&c0)[R], const W (&g1)[R], const W (&g2)[R], const W (&g3)[R]) {
     double f[R], x[R];
 #pragma unroll
     for (int r = 0; r < R; r++) f[r] = b[(ty * R + r) * WX + tx + G];
-    values(g1, g2, g3, f, x);
+    values(c0, g1, g2, g3, f, x);
     epi(at, d.px, in, x, f);
     at += d.sz();
   };
-  W g1[R], g2[R], g3[R];
+  W c0[R], g1[R], g2[R], g3[R];
   if constexpr (G == 1) {
     W Cm[R], Fm[R], Em[R], Cc[R], Fc[R], Ec[R], Cn[R], Fn[R], En[R];
     arrive(Cm, Fm, Em);
@@ -268,11 +290,13 @@ __device__ __forceinline__ bool fx_march(const CUtensorMap& mU, const CUtensorMa
       const double* b = arrive(Cn, Fn, En);
 #pragma unroll
       for (int r = 0; r < R; r++) {
-        const W c6 = Cc[r] * (W)6;
-        g1[r] = Fc[r] + (Cm[r] + Cn[r]) - c6;
+        c0[r] = Cc[r];
+        g1[r] = Fc[r] + (Cm[r] + Cn[r]);
         if constexpr (KIND == FX27) {
-          g2[r] = Ec[r] + (Fm[r] + Fn[r]) - (c6 + c6);
-          g3[r] = Em[r] + En[r] - Cc[r] * (W)8;
+          g2[r] = Ec[r] + (Fm[r] + Fn[r]);
+          g3[r] = Em[r] + En[r];
+        } else {
+          g1[r] -= Cc[r] * (W)6;
         }
         Cm[r] = Cc[r];
         Fm[r] = Fc[r];
@@ -281,7 +305,7 @@ __device__ __forceinline__ bool fx_march(const CUtensorMap& mU, const CUtensorMa
         Fc[r] = Fn[r];
         Ec[r] = En[r];
       }
-      finish(b, g1, g2, g3);
+      finish(b, c0, g1, g2, g3);
     }
   } else {
     W C2m[R], C1m[R], Cc[R], Cp[R], Cn[R], Fc[R], Fp[R], Fn[R], Ec[R], Ep[R], En[R];
@@ -305,7 +329,7 @@ __device__ __forceinline__ bool fx_march(const CUtensorMap& mU, const CUtensorMa
         Ec[r] = Ep[r];
         Ep[r] = En[r];
       }
-      finish(b, g1, g2, g3);
+      finish(b, c0, g1, g2, g3);
     }
   }
   return ok;

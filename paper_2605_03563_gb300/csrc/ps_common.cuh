@@ -282,6 +282,15 @@ __device__ __forceinline__ double f32_to_f64_pow2(float v, int e) {
   return __longlong_as_double((long long)bits);
 }
 
+// *to = max(*to, v over the calling threads): one atomic per converged group of
+// a warp, and none where the value is already as large.
+__device__ __forceinline__ void atomic_max_group(unsigned v, unsigned* to) {
+  const unsigned m = __activemask();
+  v = __reduce_max_sync(m, v);
+  const int lane = (threadIdx.x + blockDim.x * threadIdx.y) & 31;
+  if (lane == __ffs(m) - 1 && v > *(volatile unsigned*)to) atomicMax(to, v);
+}
+
 __device__ __forceinline__ int block_linear_id() {
   return blockIdx.x + gridDim.x * (blockIdx.y + gridDim.y * blockIdx.z);
 }
@@ -321,6 +330,10 @@ struct DevState {
   int inner_cap;           // refinement form: most iterations of the current inner solve
   unsigned umax;      // high word of max |phi| of the finest FP64 potential as last written (set-up copy, correction)
   unsigned bmax;      // the same over its boundary nodes
+  unsigned unext;     // largest |phi| that a norm pass read: umax of the next iteration
+  // FP64 compact multigrid: largest |u| (levels below the finest) and |r| written
+  // on a level in this V-cycle (high words; see fixed.cuh)
+  unsigned hu[8], hr[8];
   int lag_pending;         // lagged-norm V-cycles: a first colour pass with saved values ran this step
 };
 

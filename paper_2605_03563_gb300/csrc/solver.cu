@@ -823,18 +823,12 @@ ps_status begin_cg(ps_ctx* h, cudaStream_t s) {
 }
 
 // ------------------------------------------------------------------ compact stencils + SPAI MG
-// Table 1: omega, alpha, beta, gamma, delta of the SPAI smoother M of Eq.
-// Smoother for compact orders 2, 4, 6.  The order-6 row prints delta equal to
-// its mu (a garbled cell); delta = 0.0151 is the value that minimises the local
-// Fourier smoothing factor with the printed omega, alpha, beta and gamma.
-static const double kSpai[3][5] = {{1.3699, 0.1432, 0.0284, 0.0081, 0.0025},
-                                   {0.9363, 0.2807, 0.0329, 0.0166, 0.0044},
-                                   {0.3543, 0.7064, 0.1005, 0.0363, 0.0151}};
 static const double kCompactCoarseTol = 1e-2;   // coarsest CG, as the geometric MG
 
 struct CompactLevels {
   std::vector<W27> A, M;
   std::vector<double> omega;
+  std::vector<C27Ops> fx;   // integer forms for the fixed-point passes
 };
 
 // Level operators of the compact multigrid for the spacings hl of its levels
@@ -842,11 +836,14 @@ struct CompactLevels {
 // SPAI smoother of Table 1 scaled by h_l^2 on every level.
 static CompactLevels make_compact_levels(int order, const std::vector<double>& hl) {
   CompactLevels C;
-  const double* k = kSpai[order / 2 - 1];
+  // the SPAI smoother M of Eq. Smoother with Table 1's coefficients
+  double k[5];
+  for (int c = 0; c < 5; c++) k[c] = kSpaiInt[order / 2 - 1][c] / 1e4;
   for (size_t l = 0; l < hl.size(); l++) {
     C.A.push_back(l == 0 ? compact_lhs(order, hl[0]) : galerkin27(C.A.back()));
     C.M.push_back(W27{{k[1] * hl[l] * hl[l], k[2] * hl[l] * hl[l], k[3] * hl[l] * hl[l], k[4] * hl[l] * hl[l]}});
     C.omega.push_back(k[0]);
+    C.fx.push_back(l < 8 ? c27_ops(order, hl[0], (int)l) : C27Ops());
   }
   return C;
 }
@@ -863,7 +860,7 @@ cudaError_t vcycle_compact(ps_ctx* h, Hier* H, const CompactLevels& C, int l, in
   const int fp64 = dt == DT_F64;
   void* u = L.phi;
   void* b = L.fs;
-  const DevState* st = h->st;
+  DevState* st = h->st;
   cudaError_t e;
   if (l == last) {
     prof_begin(h, PC_COARSE, 0.0, 0.0, 1, s);
@@ -876,9 +873,16 @@ cudaError_t vcycle_compact(ps_ctx* h, Hier* H, const CompactLevels& C, int l, in
   // the array that holds the current iterate
   void* ub = fp64 ? nullptr : L.phib;
   const double n = (double)L.d.ni() * L.d.nj() * L.d.nk();
-  // residual pass: FP64 levels march z through L1 (four rows per thread), FP32
-  // levels run the register-blocked TMA march of the smoothing step
+  // larger FP64 levels: fixed-point passes, which bound u and r by the largest
+  // values written in this V-cycle
+  const bool fx = fp64 && c27_fx_level(L.d, C.fx[l]);
+  unsigned* hu = l == 0 ? &st->umax : &st->hu[l & 7];
+  const unsigned* hb = l == 0 ? &st->bmax : hu;   // boundary data (zero below the finest level)
+  unsigned* hr = &st->hr[l & 7];
+  // residual pass: smaller FP64 levels march z through L1 (four rows per thread),
+  // FP32 levels run the register-blocked TMA march of the smoothing step
   auto resid = [&](void* out) -> cudaError_t {
+    if (fx) return launch_c27_fx_resid(L.d, C.fx[l], (const double*)u, (const double*)b, (double*)out, st, hu, hb, hr, s);
     if (fp64) return launch_c27_resid_dt(L.d, C.A[l], (const double*)u, (const double*)b, DT_F64, out, nullptr, st, s);
     return launch_c27_resid_f32(L.d, C.A[l], (const float*)u, (const float*)b, (float*)out, st, &h->st->fault, s);
   };
@@ -900,7 +904,8 @@ cudaError_t vcycle_compact(ps_ctx* h, Hier* H, const CompactLevels& C, int l, in
       prof_end(h, s);
       if (e2 != cudaSuccess) return e2;
       prof_begin(h, l == 0 ? PC_SWEEP0 : PC_SWEEP_C, n * 3.0 * S, n * 16.0, fp64, s);
-      e2 = (h->nlaunch += 1, launch_c27_spai(L.d, C.M[l], C.omega[l], (const double*)r, (double*)u, st, s));
+      e2 = (h->nlaunch += 1, fx ? launch_c27_fx_spai(L.d, C.fx[l], (const double*)r, (double*)u, st, hr, hu, s)
+                                : launch_c27_spai(L.d, C.M[l], C.omega[l], (const double*)r, (double*)u, st, s));
       prof_end(h, s);
       if (e2 != cudaSuccess) return e2;
     }
@@ -919,7 +924,7 @@ cudaError_t vcycle_compact(ps_ctx* h, Hier* H, const CompactLevels& C, int l, in
   if ((e = cudaMemsetAsync(Cl.phi, 0, (size_t)Cl.d.size() * dt_size(Cl.dt), s)) != cudaSuccess) return e;
   if ((e = vcycle_compact(h, H, C, l + 1, nu1, nu2, s)) != cudaSuccess) return e;
   if (l == 0) prof_begin(h, PC_PROLONG0, n * S * 17.0 / 8.0, n * kProlongOps, fp64, s);
-  e = (h->nlaunch += 1, launch_prolong(L.d, Cl.d, Cl.dt, Cl.phi, dt, u, s));
+  e = (h->nlaunch += 1, launch_prolong(L.d, Cl.d, Cl.dt, Cl.phi, dt, u, s, fx ? hu : nullptr));
   if (l == 0) prof_end(h, s);
   if (e != cudaSuccess) return e;
   if ((e = smooth(nu2)) != cudaSuccess) return e;
@@ -969,12 +974,15 @@ ps_status begin_mg_compact(ps_ctx* h, const double* rho, const ps_solve_opts* o,
   h->act.body = [h, H, C, phi, b, rr, nb, nu1, nu2](unsigned long long cond, int chunk, cudaStream_t q) -> cudaError_t {
     cudaError_t e = vcycle_compact(h, H, *C, 0, nu1, nu2, q);
     const double n = (double)h->d0.ni() * h->d0.nj() * h->d0.nk();
+    int nbn = nb;
     if (e == cudaSuccess) {
       prof_begin(h, PC_NORM0, n * 24.0, n * 17.0, 1, q);
-      e = (h->nlaunch += 1, launch_c27_resid(h->d0, C->A[0], phi, b, rr, h->partials, h->st, q));
+      e = (h->nlaunch += 1, c27_fx_level(h->d0, C->fx[0])
+                                ? launch_c27_fx_norm(h->d0, C->fx[0], phi, b, rr, h->partials, h->st, &nbn, q)
+                                : launch_c27_resid(h->d0, C->A[0], phi, b, rr, h->partials, h->st, q));
       prof_end(h, q);
     }
-    if (e == cudaSuccess) e = (h->nlaunch += 1, launch_finish_norm(h->partials, nb, 1.0, 2, h->st, q, cond, chunk));
+    if (e == cudaSuccess) e = (h->nlaunch += 1, launch_finish_norm(h->partials, nbn, 1.0, 2, h->st, q, cond, chunk));
     return e;
   };
   h->act.key = "mgc:" + std::to_string(order) + ":" + std::to_string(nu1) + ":" + std::to_string(nu2);

@@ -118,7 +118,12 @@ __device__ __forceinline__ void finish_norm_block(const double* __restrict__ par
   }
   st->rr = rr;
   st->amax = m;
-  st->umax = 0u;   // the residual pass that used it has run
+  // the residual pass that used these has run; what it read is the potential of
+  // the next iteration
+  st->umax = st->unext;
+  st->unext = 0u;
+#pragma unroll
+  for (int l = 0; l < 8; l++) st->hu[l] = st->hr[l] = 0u;
   const double rel = sqrt(rr) / st->ref;
   st->rel = rel;
   // IR: the scale of the next stored inner right-hand side (power of two)

@@ -103,3 +103,26 @@ def test_infinite_guess_diverges(order, compact):
         for prec in ("fp64", "mixed_fp32"):
             info = s.solve(torch.zeros_like(phi), phi, tol=1e-8, max_iter=3, prec=prec, compact_order=compact)
             assert info.status == P.capi.PS_DIVERGED
+
+
+@pytest.mark.parametrize("compact", [2, 6])
+def test_compact_fp64_solve_matches_oracle(compact):
+    """A whole FP64 compact solve whose two finest levels take the fixed-point
+    residual and SPAI passes (the second with Galerkin weights in integers):
+    equal V-cycle counts, potentials within 1e-10 of the FP64 oracle."""
+    import paper_2605_03563_gb300 as P
+    import workloads as W
+    from oracle import solve as OS
+    from oracle.grid import cart_grid
+    n, hi = (192, 176, 208), tuple(v / 192 for v in (192, 176, 208))
+    x = [np.linspace(0, 1, v + 1) for v in n]
+    rho = np.exp(-((x[0][None, None, :] - .4) ** 2 + (x[1][None, :, None] - .5) ** 2 + (x[2][:, None, None] - .6) ** 2) / .02)
+    g = cart_grid(n, hi=hi)
+    ref = g.zeros()
+    info_o = OS.solve_cartesian(rho, ref, g, "mg", 1e-4, max_iter=10, bc="multipole", lmax=2, nu1=1, nu2=1,
+                                compact_order=compact)
+    phi = torch.zeros(W.cart_shape(n, 2), dtype=torch.float64, device="cuda:0")
+    with P.CartesianSolver(n, hi=hi, bc="multipole", lmax=2) as s:
+        info = s.solve(torch.from_numpy(rho).to("cuda:0"), phi, tol=1e-4, max_iter=10, nu1=1, nu2=1, compact_order=compact)
+    assert info.iterations == info_o.iterations
+    assert np.max(np.abs(phi.cpu().numpy() - ref)) <= 1e-10 * np.max(np.abs(ref))
