@@ -44,6 +44,14 @@ cudaError_t launch_sweep_colour(const Dims& d, int order, const double h[3], int
                                 const void* fs, int colour, double omega, const DevState* st,
                                 cudaStream_t s, const double* wtab = nullptr, int wlen = 0);
 
+// 7-point SOR steps up to the budget st->chunk_end in one cooperative launch
+// (state as after launch_set_budget), for grids of at most SOR_STEPS_MAX nodes;
+// alt: scratch array of phi's layout; partials holds npart doubles or more.
+constexpr long long SOR_STEPS_MAX = 1000000;
+bool sor_steps_fit(const Dims& d);
+cudaError_t launch_sor_steps(const Dims& d, const double h[3], double* phi, double* alt, const double* fs, double omega,
+                             const double* wtab, int wlen, DevState* st, double* partials, int npart, cudaStream_t s);
+
 // fs = factor * f on interior nodes, both of storage dt
 cudaError_t launch_scale_rhs_any(const Dims& d, double factor, int dt, const void* f, void* fs,
                                  cudaStream_t s);

@@ -334,6 +334,7 @@ struct DevState {
   // FP64 compact multigrid: largest |u| (levels below the finest) and |r| written
   // on a level in this V-cycle (high words; see fixed.cuh)
   unsigned hu[8], hr[8];
+  unsigned gbar;      // grid barrier of the one-launch iterations (zeroed before each launch)
   int lag_pending;         // lagged-norm V-cycles: a first colour pass with saved values ran this step
 };
 

@@ -117,6 +117,8 @@ struct Active {
   int restrict_tile = 0;              // tile variant of the fused FP32/BF16 residual + restriction
   long long body_kernels = 0;
   int inner_per_iter = 0;
+  // the iterations of a step in one launch (instead of the loop graph), where set
+  std::function<cudaError_t(cudaStream_t)> steps;
   // enqueued by every step before the iterations / after them (may be empty)
   std::function<cudaError_t(cudaStream_t)> prologue, epilogue;
 };
@@ -186,6 +188,7 @@ struct ps_ctx {
   int has_tun[3] = {0, 0, 0};
   // Cartesian SOR: weights of the Chebyshev sequence, one per colour pass
   double* sor_wtab = nullptr;
+  double* sor_alt = nullptr;   // second red array of the one-launch steps
   int sor_wlen = 0;
   cudaEvent_t ev[3] = {nullptr, nullptr, nullptr};
   size_t bytes = 0;
@@ -783,6 +786,15 @@ ps_status begin_sor(ps_ctx* h, const ps_solve_opts* o, cudaStream_t s) {
     if (e != cudaSuccess) return e;
     return norm_pass(h, phi, 2, DT_F64, nullptr, q, cond, chunk);
   };
+  if (sor_steps_fit(h->d0)) {
+    if (!h->sor_alt) {
+      ps_status r = alloc_zero((void**)&h->sor_alt, (size_t)h->d0.size() * sizeof(double), &h->bytes);
+      if (r != PS_OK) return r;
+    }
+    h->act.steps = [h, phi, omega, wtab, wlen](cudaStream_t q) -> cudaError_t {
+      return launch_sor_steps(h->d0, h->h0, phi, h->sor_alt, h->fs64, omega, wtab, wlen, h->st, h->partials, 2 * h->npart, q);
+    };
+  }
   char key[64];
   if (wtab) snprintf(key, sizeof(key), "sor:chebyshev");
   else snprintf(key, sizeof(key), "sor:%.17g", omega);
@@ -1352,6 +1364,12 @@ ps_status step_active(ps_ctx* h, int k) {
     h->act.plain_steps = true;
     return PS_OK;
   }
+  if (h->act.steps) {
+    h->act.body_kernels = 0;
+    TRY((h->nlaunch += 1, launch_set_budget(h->st, k, s)));
+    TRY((h->nlaunch += 1, h->act.steps(s)));
+    return PS_OK;
+  }
   LoopGraph& g = h->graphs[h->act.key];
   if (!g.exec && (r = build_loop_graph(h, &g)) != PS_OK) return r;
   h->act.body_kernels = g.body_kernels;
@@ -1804,6 +1822,7 @@ void poisson_destroy(ps_handle h) {
   cudaFree(h->sph_w);
   cudaFree(h->sph_g);
   cudaFree(h->sor_wtab);
+  cudaFree(h->sor_alt);
   cart_multipole_free(&h->mp);
   sph_tables_free(&h->stab);
   for (auto& p : h->sv) cudaFree(p);

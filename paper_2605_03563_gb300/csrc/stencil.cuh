@@ -153,6 +153,40 @@ __device__ __forceinline__ double recip(double x) {
   return fma(y, fma(-x, y, 1.0), y);
 }
 
+// ------------------------------------------------------------------ grid barrier
+// Barrier over the blocks of a cooperative launch (all resident at once):
+// *bar counts arrivals, target = blocks times the barriers passed so far.  What
+// any block wrote before it is visible after it (to loads that go to L2: the L1
+// caches are not coherent, so data that other blocks write are read with
+// __ldcg).  The wait is bounded (2 s): past it ok turns false in thread 0's
+// block, which then stops, and so do the others in turn.
+__device__ __forceinline__ void grid_barrier(unsigned* bar, unsigned target, bool& ok) {
+  __shared__ int alive;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(bar) : "memory");
+    unsigned v, spins = 0;
+    unsigned long long t0 = 0;
+    int good = 1;
+    for (;;) {
+      asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
+      if (v >= target) break;
+      if ((++spins & 255u) == 0) {
+        unsigned long long t;
+        asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+        if (t0 == 0) t0 = t;
+        if (t - t0 > 2000000000ull) {
+          good = 0;
+          break;
+        }
+      }
+    }
+    alive = good;
+  }
+  __syncthreads();
+  ok = ok && alive != 0;
+}
+
 // ------------------------------------------------------------------ thread-block cluster
 __device__ __forceinline__ unsigned cluster_rank() {
   unsigned r;
