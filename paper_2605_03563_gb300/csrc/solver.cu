@@ -182,6 +182,7 @@ struct ps_ctx {
   void* sv[8] = {nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr};
   int sv_dt = -1;
   double* sz = nullptr;   // BiCGSTAB group-wise increments of the iterate (FP64)
+  double* sph_part = nullptr;   // one-launch BiCGSTAB: the warps' partial sums
   double* sph_w = nullptr;   // spherical SOR weights, two buffers of Ntheta * Nr
   double* sph_g = nullptr;   // spherical SOR: scaled right-hand side -f / a_c (field layout)
   ps_tuning tun[3] = {};     // tuned multigrid settings per precision (poisson_set_tuning)
@@ -640,6 +641,7 @@ ps_status cart_prepare(ps_ctx* h, const double* rho, double* phi, double tol, in
 }
 
 static const int MG_CHUNK = 32, KRYLOV_GRAPH_CHUNK = 64;
+static const int STEPS_CHUNK = 1024;   // iterations per cooperative launch of a whole solve
 
 // Each begin_* enqueues the initial residual pass and installs the iteration
 // body (one V-cycle / refinement step / SOR step / Krylov iteration) that the
@@ -1141,6 +1143,15 @@ ps_status bicg_start(ps_ctx* h, int dt, const double* rho, double fscale, double
   }
   TRY(cudaMemsetAsync(h->sz, 0, (size_t)h->sd.size() * sizeof(double), s));
   double* z = h->sz;
+  if (bicg_steps_fit(h->sd)) {
+    if (!h->sph_part) {
+      ps_status r = alloc_zero((void**)&h->sph_part, bicg_steps_doubles(h->sd) * sizeof(double), &h->bytes);
+      if (r != PS_OK) return r;
+    }
+    h->act.steps = [h, dt, rho, fscale, x, z, v, st](cudaStream_t q) -> cudaError_t {
+      return launch_bicg_steps(h->sd, h->stab, dt, rho, fscale, x, z, v, h->sph_part, st, q);
+    };
+  }
   *body = [h, dt, rho, fscale, x, z, v, st](unsigned long long cond, int chunk, cudaStream_t q) -> cudaError_t {
     const double n = (double)h->sd.nr * h->sd.nt * h->sd.np;
     const double S = dt == DT_F64 ? 8.0 : 4.0;
@@ -1819,6 +1830,7 @@ void poisson_destroy(ps_handle h) {
   cudaFree(h->cg_p);
   cudaFree(h->cg_q);
   cudaFree(h->cg_z);
+  cudaFree(h->sph_part);
   cudaFree(h->sph_w);
   cudaFree(h->sph_g);
   cudaFree(h->sor_wtab);
@@ -1978,7 +1990,7 @@ ps_status poisson_solve(ps_handle h, const double* rho_dev, double* phi_dev, dou
   int done = 0;
   if ((r = poll_active(h, &done)) != PS_OK) { h->act.on = false; return r; }
   while (!done) {
-    if ((r = step_active(h, h->act.chunk)) != PS_OK || (r = poll_active(h, &done)) != PS_OK) {
+    if ((r = step_active(h, h->act.steps ? STEPS_CHUNK : h->act.chunk)) != PS_OK || (r = poll_active(h, &done)) != PS_OK) {
       h->act.on = false;
       return r;
     }

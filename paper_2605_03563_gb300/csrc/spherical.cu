@@ -19,6 +19,7 @@
 
 #include "cart_kernels.cuh"
 #include "spherical.cuh"
+#include "stencil.cuh"
 
 namespace ps {
 
@@ -581,18 +582,10 @@ __device__ __forceinline__ void sum_partials2(const double* __restrict__ partial
   block_sum<2>(v, sh);
 }
 
+// Scalar steps of an iteration on the state st (one thread) from the sums v.
 // which: 0 alpha; 2 omega; 3 recurrence residual (direction update, or a
-// replacement request that k_bicg_replace_finish completes).
-__global__ void k_bicg_scalar(const double* __restrict__ partials, int nblk, int which,
-                              DevState* __restrict__ st, unsigned long long cond, int chunk) {
-  __shared__ double sh[64];
-  if (st->done) {
-    if (which == 3 && threadIdx.x == 0) bicg_set_loop(st, cond, chunk);
-    return;
-  }
-  double v[2];
-  sum_partials2(partials, nblk, sh, v);
-  if (threadIdx.x != 0) return;
+// replacement request that bicg_replace_logic completes).
+__device__ __forceinline__ void bicg_scalar_logic(DevState* st, int which, const double (&v)[2]) {
   if (which == 0) {
     st->restart = 0;
     const double al = st->rho / v[0];
@@ -628,26 +621,33 @@ __global__ void k_bicg_scalar(const double* __restrict__ partials, int nblk, int
     const bool claims = !st->restart_on_replace && rn / st->ref <= st->tol;
     if (!isfinite(rn) || st->broke || rn <= st->replace_drop * st->rmax || claims ||
         st->iter >= st->max_iter || inner_end) {
-      st->replace = 1;   // k_bicg_replace_finish decides and sets the loop
+      st->replace = 1;   // the replacement's finish decides
       return;
     }
     st->rmax = fmax(st->rmax, rn);
     st->rr = v[0];
     st->rel = rn / st->ref;
     bicg_direction(st, v[0], v[1]);
-    bicg_set_loop(st, cond, chunk);
   }
+}
+
+__global__ void k_bicg_scalar(const double* __restrict__ partials, int nblk, int which,
+                              DevState* __restrict__ st, unsigned long long cond, int chunk) {
+  __shared__ double sh[64];
+  if (st->done) {
+    if (which == 3 && threadIdx.x == 0) bicg_set_loop(st, cond, chunk);
+    return;
+  }
+  double v[2];
+  sum_partials2(partials, nblk, sh, v);
+  if (threadIdx.x != 0) return;
+  bicg_scalar_logic(st, which, v);
+  if (which == 3 && !st->replace) bicg_set_loop(st, cond, chunk);   // k_bicg_replace_finish sets it otherwise
 }
 
 // After a residual replacement: stop on the true residual, else continue the
 // search direction from it.
-__global__ void k_bicg_replace_finish(const double* __restrict__ partials, int nblk,
-                                      DevState* __restrict__ st, unsigned long long cond, int chunk) {
-  __shared__ double sh[64];
-  if (st->done || !st->replace) return;   // the loop condition is already set
-  double v[2];
-  sum_partials2(partials, nblk, sh, v);
-  if (threadIdx.x != 0) return;
+__device__ __forceinline__ void bicg_replace_logic(DevState* st, const double (&v)[2]) {
   st->replace = 0;
   st->inner_cycles += 1;
   if (st->restart_on_replace)
@@ -671,6 +671,16 @@ __global__ void k_bicg_replace_finish(const double* __restrict__ partials, int n
       bicg_direction(st, v[0], v[1]);
     }
   }
+}
+
+__global__ void k_bicg_replace_finish(const double* __restrict__ partials, int nblk,
+                                      DevState* __restrict__ st, unsigned long long cond, int chunk) {
+  __shared__ double sh[64];
+  if (st->done || !st->replace) return;   // the loop condition is already set
+  double v[2];
+  sum_partials2(partials, nblk, sh, v);
+  if (threadIdx.x != 0) return;
+  bicg_replace_logic(st, v);
   bicg_set_loop(st, cond, chunk);
 }
 
@@ -758,6 +768,342 @@ cudaError_t launch_bicg_iter(const SphDims& d, const SphTables& t, int dt, const
   if (dt == DT_F64)
     return iter_t<double>(d, t, rho, fscale, x, z, r, rhat, p, phat, v, sv, shat, tv, partials, st, s, cond, chunk);
   return iter_t<float>(d, t, rho, fscale, x, z, r, rhat, p, phat, v, sv, shat, tv, partials, st, s, cond, chunk);
+}
+
+// ------------------------------------------------------------------ BiCGSTAB in one launch
+// Iterations up to the step's budget in one cooperative launch, for grids whose
+// iterations are made of launches and latency (11 kernels, 62 us at 96 x 48 x 32).
+// A warp of a vector kernel (32 r, one theta row of the 8, BKC phi planes) is the
+// unit of work here, four to a block and one per SM sub-partition, because a
+// warp-wide FP64 instruction holds its sub-partition for 76 cycles: the same
+// warps spread over all SMs instead of eight to a block on half of them.  The
+// warps' partial sums are added exactly as the kernels' blocks and the scalar
+// kernels add them (eight warps of a block, then 32 blocks, then those sums), by
+// every block for itself, so that alpha, omega, beta, the iterates and the
+// iteration count equal the kernels' bit for bit; each block keeps the solver
+// state in shared memory and takes the same decisions on it.
+// 96 x 48 x 32 to 1e-8 (316 iterations): 20.6 -> 12.3 ms (17.0 before a chunk's
+// operands were loaded ahead of its stores); 64 x 24 x 16: 9.8 -> 4.8 ms.
+constexpr int BS_WARPS = 4;
+
+// {sum, sum} over nblk virtual blocks of 8 warps each from W[block][warp][2]
+__device__ __forceinline__ void bicg_reduce(const double* __restrict__ W, int nblk, double (*bs)[1024],
+                                            double (*gs)[32], double (&v)[2]) {
+  const int tid = threadIdx.x, nthr = BS_WARPS * 32, lane = tid & 31, warp = tid >> 5;
+  const int nt = min((nblk + 31) / 32 * 32, 1024);
+  for (int e = tid; e < 2 * nt; e += nthr) {
+    const int c = e & 1, t = e >> 1;
+    double a = 0.0;
+    for (int b = t; b < nblk; b += 1024) {
+      const double* w = W + (long long)b * 16 + c;
+      const double w0 = __ldcg(w), w1 = __ldcg(w + 2), w2 = __ldcg(w + 4), w3 = __ldcg(w + 6), w4 = __ldcg(w + 8),
+                   w5 = __ldcg(w + 10), w6 = __ldcg(w + 12), w7 = __ldcg(w + 14);
+      a += ((w0 + w4) + (w2 + w6)) + ((w1 + w5) + (w3 + w7));
+    }
+    bs[c][t] = a;
+  }
+  if (tid < 64) gs[tid >> 5][tid & 31] = 0.0;
+  __syncthreads();
+  for (int e = warp; e < nt / 16; e += BS_WARPS) {   // (group of 32, component)
+    const int c = e & 1, g = e >> 1;
+    const double x = warp_sum(bs[c][g * 32 + lane]);
+    if (lane == 0) gs[c][g] = x;
+  }
+  __syncthreads();
+  v[0] = warp_sum(gs[0][lane]);
+  v[1] = warp_sum(gs[1][lane]);
+}
+
+template <typename T>
+__global__ void __launch_bounds__(BS_WARPS * 32)
+    k_bicg_steps(SphDims d, Tab<typename St<T>::C> tb, Tab<double> tb64, const double* __restrict__ vol,
+                 const double* __restrict__ rho, double fscale, double* __restrict__ x, double* __restrict__ z,
+                 T* __restrict__ r, T* __restrict__ rhat, T* __restrict__ p, T* __restrict__ phat,
+                 T* __restrict__ vv, T* __restrict__ sv, T* __restrict__ shat, T* __restrict__ tv,
+                 double* __restrict__ W, long long wset, DevState* __restrict__ st) {
+  using C = typename St<T>::C;
+  __shared__ DevState S;
+  __shared__ double bs[2][1024], gs[2][32];
+  const int tid = threadIdx.x, lane = tid & 31;
+  if (tid == 0) S = *st;
+  __syncthreads();
+  if (S.done) return;   // uniform over the grid
+  const int gx = (d.nr + SBX - 1) / SBX, gy = (d.nt + SBY - 1) / SBY, gz = (d.np + BKC - 1) / BKC;
+  const int nblk = gx * gy * gz, nblk1 = gx * gy * d.np;
+  const int w0 = blockIdx.x * BS_WARPS + (tid >> 5), nw = gridDim.x * BS_WARPS;
+  const long long sy = d.sy(), sz = d.sz(), wrap = (long long)(d.np - 1) * sz;
+  unsigned target = 0;
+  bool ok = true;
+  auto ld = [](const auto* a) { return __ldcg(a); };   // other SMs write the vectors
+  auto barrier = [&]() { grid_barrier(&st->gbar, target += gridDim.x, ok); };
+  // f(virtual warp, i, j, k0, k1, inside) over the warps of the vector kernels
+  auto each = [&](auto f) {
+    for (int q = w0; q < nblk * SBY; q += nw) {
+      const int b = q / SBY, by = b / gx % gy, bz = b / (gx * gy);
+      const int i = (b % gx) * SBX + lane, j = by * SBY + q % SBY;
+      f(q, i, j, bz * BKC, min(bz * BKC + BKC, d.np), i < d.nr && j < d.nt);
+    }
+  };
+  auto put = [&](int set, int q, double a, double b) {
+    a = warp_sum(a);
+    b = warp_sum(b);
+    if (lane == 0) {
+      __stcg(W + set * wset + 2 * q, a);
+      __stcg(W + set * wset + 2 * q + 1, b);
+    }
+  };
+  // the sums of a set after a barrier, and the scalar step they feed
+  auto scalar = [&](int set, int n, int which) {
+    double v[2];
+    bicg_reduce(W + set * wset, n, bs, gs, v);
+    if (tid == 0) {
+      if (which == 4) bicg_replace_logic(&S, v);
+      else bicg_scalar_logic(&S, which, v);
+    }
+    __syncthreads();
+  };
+  // dst = L src with {dst.w1, dst.dst}: k_bicg_apply's arithmetic
+  auto apply = [&](const T* src, T* dst, const T* w1, bool with_tt, int set) {
+    each([&](int q, int i, int j, int k0, int k1, bool in) {
+      double s0 = 0.0, s1 = 0.0;
+      if (in) {
+        const C rp = tb.rad_p[i], rm = tb.rad_m[i], ir2 = tb.inv_r2[i];
+        const C tp = tb.th_p[j], tm = tb.th_m[j], phc = tb.ph[j];
+        C vs = (C)1;
+        if constexpr (sizeof(C) == 4) vs = tb.vol[j * d.nr + i];
+        // every operand of the chunk is loaded before the first store (the arrays
+        // might overlap as far as the compiler knows, and an L2 round trip per
+        // plane would be the chain); planes past the chunk repeat its last
+        const long long c0 = d.at(i, j, k0);
+        const int n = k1 - k0;
+        T col[BKC + 2], im[BKC], ip[BKC], jm[BKC], jp[BKC], wv[BKC];
+        col[0] = k0 == 0 ? ld(src + c0 + wrap) : ld(src + c0 - sz);
+#pragma unroll
+        for (int m = 0; m < BKC; m++) {
+          const long long c = c0 + min(m, n - 1) * sz;
+          col[m + 1] = ld(src + c);
+          im[m] = i == 0 && !d.inner_ghost ? ld(src + c + 1) : ld(src + c - 1);
+          ip[m] = ld(src + c + 1);
+          jm[m] = j == 0 ? col[m + 1] : ld(src + c - sy);
+          jp[m] = j == d.nt - 1 ? col[m + 1] : ld(src + c + sy);
+          wv[m] = ld(w1 + c);
+        }
+        const T last = k1 == d.np ? ld(src + c0 + (n - 1) * sz - wrap) : ld(src + c0 + n * sz);
+#pragma unroll
+        for (int m = 0; m < BKC; m++) {
+          if (m >= n) break;
+          const C pc = (C)col[m + 1], pkm = (C)col[m], pkp = (C)(m == n - 1 ? last : col[min(m + 2, BKC)]);
+          const C pim = (C)im[m], pip = (C)ip[m], pjm = (C)jm[m], pjp = (C)jp[m];
+          C kk;
+          if constexpr (sizeof(C) == 4) kk = (pkp - pc) + (pkm - pc);
+          else kk = (pkp + pkm) - (C)2 * pc;
+          const C ang = fma(tp, pjp - pc, fma(-tm, pc - pjm, phc * kk));
+          C v = fma(rp, pip - pc, fma(-rm, pc - pim, ir2 * ang));
+          if constexpr (sizeof(C) == 4) v *= vs;
+          dst[c0 + m * sz] = (T)v;
+          const double vd = (double)v;
+          s0 = fma(vd, (double)wv[m], s0);
+          if (with_tt) s1 = fma(vd, vd, s1);
+        }
+      }
+      put(set, q, s0, s1);
+    });
+  };
+  while (ok && S.done == DONE_NO && S.iter < S.chunk_end) {
+    apply(phat, vv, rhat, false, 0);
+    barrier();
+    if (!ok) break;
+    scalar(0, nblk, 0);
+    {
+      const C alpha = (C)S.alpha;
+      each([&](int, int i, int j, int k0, int k1, bool in) {
+        if (!in) return;
+        const C idg = tb.inv_diag[j * d.nr + i];
+        const long long c0 = d.at(i, j, k0);
+        const int n = k1 - k0;
+        T a[BKC], b[BKC];
+#pragma unroll
+        for (int m = 0; m < BKC; m++) {
+          const long long c = c0 + min(m, n - 1) * sz;
+          a[m] = ld(vv + c);
+          b[m] = ld(r + c);
+        }
+#pragma unroll
+        for (int m = 0; m < BKC; m++) {
+          if (m >= n) break;
+          const C s = fma(-alpha, (C)a[m], (C)b[m]);
+          sv[c0 + m * sz] = (T)s;
+          shat[c0 + m * sz] = (T)(s * idg);
+        }
+      });
+    }
+    barrier();
+    if (!ok) break;
+    apply(shat, tv, sv, true, 1);
+    barrier();
+    if (!ok) break;
+    scalar(1, nblk, 2);
+    {
+      const double alpha = S.alpha, omega = S.omega;
+      each([&](int q, int i, int j, int k0, int k1, bool in) {
+        double s0 = 0.0, s1 = 0.0;
+        if (in) {
+          const long long c0 = d.at(i, j, k0);
+          const int n = k1 - k0;
+          double za[BKC];
+          T sh[BKC], ph[BKC], ta[BKC], sa[BKC], rh[BKC];
+#pragma unroll
+          for (int m = 0; m < BKC; m++) {
+            const long long c = c0 + min(m, n - 1) * sz;
+            za[m] = ld(z + c);
+            sh[m] = ld(shat + c);
+            ph[m] = ld(phat + c);
+            ta[m] = ld(tv + c);
+            sa[m] = ld(sv + c);
+            rh[m] = ld(rhat + c);
+          }
+#pragma unroll
+          for (int m = 0; m < BKC; m++) {
+            if (m >= n) break;
+            z[c0 + m * sz] = za[m] + fma(omega, (double)sh[m], alpha * (double)ph[m]);
+            const C rv = fma(-(C)omega, (C)ta[m], (C)sa[m]);
+            r[c0 + m * sz] = (T)rv;
+            const double rd = (double)rv;
+            s0 = fma(rd, rd, s0);
+            s1 = fma(rd, (double)rh[m], s1);
+          }
+        }
+        put(2, q, s0, s1);
+      });
+    }
+    barrier();
+    if (!ok) break;
+    scalar(2, nblk, 3);
+    if (S.replace) {
+      // x += z, z = 0, then the true residual (k_bicg_fold, k_bicg_resid mode 2)
+      const bool discard = S.discard != 0;
+      each([&](int, int i, int j, int k0, int k1, bool in) {
+        if (!in) return;
+        long long c = d.at(i, j, k0);
+        for (int k = k0; k < k1; k++, c += sz) {
+          if (!discard) x[c] = ld(x + c) + ld(z + c);
+          z[c] = 0.0;
+        }
+      });
+      barrier();
+      if (!ok) break;
+      for (int q = w0; q < nblk1 * SBY; q += nw) {
+        const int b = q / SBY, by = b / gx % gy, k = b / (gx * gy);
+        const int i = (b % gx) * SBX + lane, j = by * SBY + q % SBY;
+        double s0 = 0.0, s1 = 0.0;
+        if (i < d.nr && j < d.nt) {
+          const long long c = d.at(i, j, k);
+          const double pc = ld(x + c);
+          const double pim = i == 0 && !d.inner_ghost ? ld(x + c + 1) : ld(x + c - 1), pip = ld(x + c + 1);
+          const double pjm = j == 0 ? pc : ld(x + c - sy), pjp = j == d.nt - 1 ? pc : ld(x + c + sy);
+          const double pkm = k == 0 ? ld(x + c + wrap) : ld(x + c - sz);
+          const double pkp = k == d.np - 1 ? ld(x + c - wrap) : ld(x + c + sz);
+          const double kk = (pkp + pkm) - 2.0 * pc;
+          const double ang = fma(tb64.th_p[j], pjp - pc, fma(-tb64.th_m[j], pc - pjm, tb64.ph[j] * kk));
+          const double Lx = fma(tb64.rad_p[i], pip - pc, fma(-tb64.rad_m[i], pc - pim, tb64.inv_r2[i] * ang));
+          const double rv = __dsub_rn(__dmul_rn(fscale, rho[c]), Lx);
+          s0 = rv * rv;
+          if constexpr (sizeof(T) == 4) {
+            const double rsv = rv * vol[j * d.nr + i];
+            s1 = rsv * rsv;
+            r[c] = (T)rsv;
+          } else {
+            const T rs = (T)rv;
+            r[c] = rs;
+            s1 = (double)rs * (double)ld(rhat + c);
+          }
+        }
+        put(3, q, s0, s1);
+      }
+      barrier();
+      if (!ok) break;
+      scalar(3, nblk1, 4);
+    }
+    if (S.done == DONE_NO) {
+      const C beta = (C)S.beta, omega = (C)S.omega;
+      const int restart = S.restart;
+      each([&](int, int i, int j, int k0, int k1, bool in) {
+        if (!in) return;
+        const C idg = tb.inv_diag[j * d.nr + i];
+        const long long c0 = d.at(i, j, k0);
+        const int n = k1 - k0;
+        T ra[BKC], va[BKC], pa[BKC];
+#pragma unroll
+        for (int m = 0; m < BKC; m++) {
+          const long long c = c0 + min(m, n - 1) * sz;
+          ra[m] = ld(r + c);
+          va[m] = ld(vv + c);
+          pa[m] = ld(p + c);
+        }
+#pragma unroll
+        for (int m = 0; m < BKC; m++) {
+          if (m >= n) break;
+          const long long c = c0 + m * sz;
+          if (restart) {
+            rhat[c] = ra[m];
+            p[c] = ra[m];
+            phat[c] = (T)((C)ra[m] * idg);
+          } else {
+            const C pv = fma(beta, fma(-omega, (C)va[m], (C)pa[m]), (C)ra[m]);
+            p[c] = (T)pv;
+            phat[c] = (T)(pv * idg);
+          }
+        }
+      });
+    }
+    barrier();
+  }
+  if (blockIdx.x == 0 && tid == 0) {
+    if (!ok) {
+      S.done = DONE_FAULT;
+      S.fault = 1;
+    }
+    S.gbar = 0u;
+    *st = S;
+  }
+}
+
+static long long bicg_wset(const SphDims& d) {
+  const long long tiles = (long long)((d.nr + SBX - 1) / SBX) * ((d.nt + SBY - 1) / SBY);
+  return tiles * d.np * SBY * 2;   // of the residual's planes, the largest set
+}
+
+// Grids that take the one-launch form: with more warps of work than about two
+// per SM sub-partition the kernels' larger blocks use the memory system better.
+bool bicg_steps_fit(const SphDims& d) {
+  const long long warps = bicg_wset(d) / 2 / d.np * ((d.np + BKC - 1) / BKC);
+  return warps <= 2LL * BS_WARPS * device_sm_count();
+}
+
+size_t bicg_steps_doubles(const SphDims& d) { return (size_t)(4 * bicg_wset(d)); }
+
+template <typename T>
+static cudaError_t bicg_steps_t(const SphDims& d, const SphTables& t, const double* rho, double fscale, double* x,
+                                double* z, void* const* v, double* W, DevState* st, cudaStream_t s) {
+  using C = typename St<T>::C;
+  const long long wset = bicg_wset(d), warps = wset / 2 / d.np * ((d.np + BKC - 1) / BKC);
+  const int blocks = (int)std::min<long long>(device_sm_count(), (warps + BS_WARPS - 1) / BS_WARPS);
+  SphDims dd = d;
+  Tab<C> tb = tab_of<C>(t);
+  Tab<double> tb64 = tab_of<double>(t);
+  const double* vol = t.vol;
+  T* q[8];
+  for (int i = 0; i < 8; i++) q[i] = (T*)v[i];
+  long long ws = wset;
+  void* args[] = {&dd, &tb, &tb64, (void*)&vol, (void*)&rho, &fscale, &x, &z, &q[0], &q[1], &q[2], &q[3],
+                  &q[4], &q[5], &q[6], &q[7], &W, &ws, &st};
+  return cudaLaunchCooperativeKernel((const void*)k_bicg_steps<T>, dim3(blocks), dim3(BS_WARPS * 32), args, 0, s);
+}
+
+cudaError_t launch_bicg_steps(const SphDims& d, const SphTables& t, int dt, const double* rho, double fscale, double* x,
+                              double* z, void* const* v, double* W, DevState* st, cudaStream_t s) {
+  return dt == DT_F64 ? bicg_steps_t<double>(d, t, rho, fscale, x, z, v, W, st, s)
+                      : bicg_steps_t<float>(d, t, rho, fscale, x, z, v, W, st, s);
 }
 
 int bicg_iter_kernels(int) { return 11; }

@@ -90,6 +90,14 @@ cudaError_t launch_bicg_iter(const SphDims& d, const SphTables& t, int dt, const
                              DevState* st, cudaStream_t s, unsigned long long cond = 0,
                              int chunk = 0);
 int bicg_iter_kernels(int dt);
+// The same iterations, bit for bit, up to the budget st->chunk_end in one
+// cooperative launch (state as after launch_set_budget), on grids that
+// bicg_steps_fit; v: the eight vectors in launch_bicg_iter's order (r, rhat, p,
+// phat, v, s, shat, t), W: scratch of bicg_steps_doubles doubles.
+bool bicg_steps_fit(const SphDims& d);
+size_t bicg_steps_doubles(const SphDims& d);
+cudaError_t launch_bicg_steps(const SphDims& d, const SphTables& t, int dt, const double* rho, double fscale, double* x,
+                              double* z, void* const* v, double* W, DevState* st, cudaStream_t s);
 // scalar finisher for the reference / initial residual (mode 0/1)
 cudaError_t launch_bicg_start(const double* partials, int nblk, int mode, DevState* st,
                               cudaStream_t s, double replace_drop = 0.01, int restart_on_replace = 0);
