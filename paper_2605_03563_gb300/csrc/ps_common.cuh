@@ -326,6 +326,7 @@ struct DevState {
   double replace_drop;     // BiCGSTAB: replace when ||r|| <= replace_drop * rmax
   int restart_on_replace;  // BiCGSTAB: restart rhat = p = r at every replacement
   int iter_repl;           // BiCGSTAB: iteration of the last replacement
+  const double* rhs;       // BiCGSTAB: the density of this solve (captured loops outlive a solve's buffers)
   int discard;             // refinement form: the inner solve failed, drop its increments
   int inner_cap;           // refinement form: most iterations of the current inner solve
   unsigned umax;      // high word of max |phi| of the finest FP64 potential as last written (set-up copy, correction)

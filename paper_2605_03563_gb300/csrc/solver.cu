@@ -1136,7 +1136,7 @@ ps_status bicg_start(ps_ctx* h, int dt, const double* rho, double fscale, double
   TRY((h->nlaunch += 1, launch_bicg_resid(h->sd, h->stab, dt, 0, rho, fscale, x, nullptr, nullptr, nullptr, nullptr, h->partials, &nb, s)));
   TRY((h->nlaunch += 1, launch_bicg_start(h->partials, nb, 0, st, s)));
   TRY((h->nlaunch += 1, launch_bicg_resid(h->sd, h->stab, dt, 1, rho, fscale, x, v[0], v[1], v[2], v[3], h->partials, &nb, s)));
-  TRY((h->nlaunch += 1, launch_bicg_start(h->partials, nb, 1, st, s, drop, restart_on_replace)));
+  TRY((h->nlaunch += 1, launch_bicg_start(h->partials, nb, 1, st, s, drop, restart_on_replace, rho)));
   if (!h->sz) {
     ps_status r = alloc_zero((void**)&h->sz, (size_t)h->sd.size() * sizeof(double), &h->bytes);
     if (r != PS_OK) return r;
@@ -1152,7 +1152,7 @@ ps_status bicg_start(ps_ctx* h, int dt, const double* rho, double fscale, double
       return launch_bicg_steps(h->sd, h->stab, dt, rho, fscale, x, z, v, h->sph_part, st, q);
     };
   }
-  *body = [h, dt, rho, fscale, x, z, v, st](unsigned long long cond, int chunk, cudaStream_t q) -> cudaError_t {
+  *body = [h, dt, fscale, x, z, v, st](unsigned long long cond, int chunk, cudaStream_t q) -> cudaError_t {
     const double n = (double)h->sd.nr * h->sd.nt * h->sd.np;
     const double S = dt == DT_F64 ? 8.0 : 4.0;
     // 21 vector streams of the storage type (apply 3, s 4, apply 3, x/r 6,
@@ -1161,7 +1161,7 @@ ps_status bicg_start(ps_ctx* h, int dt, const double* rho, double fscale, double
     const double bytes = n * (S * 21.0 + 16.0);
     prof_begin(h, PC_KRYLOV, bytes, n * 60.0, dt == DT_F64, q);
     h->nlaunch += bicg_iter_kernels(dt);
-    cudaError_t e = launch_bicg_iter(h->sd, h->stab, dt, rho, fscale, x, z, v[0], v[1], v[2], v[3], v[4], v[5], v[6], v[7], h->partials, st, q, cond, chunk);
+    cudaError_t e = launch_bicg_iter(h->sd, h->stab, dt, fscale, x, z, v[0], v[1], v[2], v[3], v[4], v[5], v[6], v[7], h->partials, st, q, cond, chunk);
     prof_end(h, q);
     return e;
   };

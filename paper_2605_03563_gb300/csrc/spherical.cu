@@ -347,11 +347,14 @@ cudaError_t launch_sph_rednorm(const SphDims& d, const SphTables& t, const doubl
 template <typename T>
 __global__ void __launch_bounds__(SBX* SBY)
     k_bicg_resid(SphDims d, Tab<double> tb, const double* __restrict__ vol, int mode,
-                 const double* __restrict__ rho, double fscale,
+                 const double* rho, double fscale,
                  const double* __restrict__ x, T* __restrict__ r, T* __restrict__ rhat,
                  T* __restrict__ p, T* __restrict__ phat, double* __restrict__ partials,
                  const DevState* __restrict__ st) {
-  if (mode == 2 && (st->done || !st->replace)) return;
+  if (mode == 2) {
+    if (st->done || !st->replace) return;
+    rho = st->rhs;   // not an argument: the loop graph is captured once per handle
+  }
   const int i = blockIdx.x * SBX + threadIdx.x, j = blockIdx.y * SBY + threadIdx.y, k = blockIdx.z;
   double s0 = 0.0, s1 = 0.0;
   if (i < d.nr && j < d.nt) {
@@ -685,7 +688,8 @@ __global__ void k_bicg_replace_finish(const double* __restrict__ partials, int n
 }
 
 __global__ void k_bicg_start(const double* __restrict__ partials, int nblk, int mode,
-                             DevState* __restrict__ st, double replace_drop, int restart_on_replace) {
+                             DevState* __restrict__ st, double replace_drop, int restart_on_replace,
+                             const double* rho) {
   __shared__ double sh[64];
   double v[2];
   sum_partials2(partials, nblk, sh, v);
@@ -699,6 +703,7 @@ __global__ void k_bicg_start(const double* __restrict__ partials, int nblk, int 
   st->rr = v[0];
   st->rho = v[1];
   st->rmax = restart_on_replace ? sqrt(v[1]) : sqrt(v[0]);
+  st->rhs = rho;
   st->replace_drop = replace_drop;
   st->restart_on_replace = restart_on_replace;
   st->iter_repl = 0;
@@ -731,13 +736,13 @@ cudaError_t launch_bicg_resid(const SphDims& d, const SphTables& t, int dt, int 
 }
 
 cudaError_t launch_bicg_start(const double* partials, int nblk, int mode, DevState* st,
-                              cudaStream_t s, double replace_drop, int restart_on_replace) {
-  k_bicg_start<<<1, 256, 0, s>>>(partials, nblk, mode, st, replace_drop, restart_on_replace);
+                              cudaStream_t s, double replace_drop, int restart_on_replace, const double* rho) {
+  k_bicg_start<<<1, 256, 0, s>>>(partials, nblk, mode, st, replace_drop, restart_on_replace, rho);
   return cudaGetLastError();
 }
 
 template <typename T>
-static cudaError_t iter_t(const SphDims& d, const SphTables& t, const double* rho, double fscale,
+static cudaError_t iter_t(const SphDims& d, const SphTables& t, double fscale,
                           double* x, double* z, void* r, void* rhat, void* p, void* phat, void* v,
                           void* sv, void* shat, void* tv, double* partials, DevState* st,
                           cudaStream_t s, unsigned long long cond, int chunk) {
@@ -754,20 +759,20 @@ static cudaError_t iter_t(const SphDims& d, const SphTables& t, const double* rh
                                 (const T*)shat, (const T*)tv, partials, st);
   k_bicg_scalar<<<1, 1024, 0, s>>>(partials, nblk_k, 3, st, cond, chunk);
   k_bicg_fold<<<g, b, 0, s>>>(d, x, z, st);
-  k_bicg_resid<T><<<g, b, 0, s>>>(d, tab_of<double>(t), t.vol, 2, rho, fscale, x, (T*)r, (T*)rhat,
+  k_bicg_resid<T><<<g, b, 0, s>>>(d, tab_of<double>(t), t.vol, 2, nullptr, fscale, x, (T*)r, (T*)rhat,
                                   nullptr, nullptr, partials, st);
   k_bicg_replace_finish<<<1, 1024, 0, s>>>(partials, nblk, st, cond, chunk);
   k_bicg_p<T><<<gk, b, 0, s>>>(d, tb, (const T*)r, (T*)rhat, (T*)p, (const T*)v, (T*)phat, st);
   return cudaGetLastError();
 }
 
-cudaError_t launch_bicg_iter(const SphDims& d, const SphTables& t, int dt, const double* rho,
+cudaError_t launch_bicg_iter(const SphDims& d, const SphTables& t, int dt,
                              double fscale, double* x, double* z, void* r, void* rhat, void* p,
                              void* phat, void* v, void* sv, void* shat, void* tv, double* partials,
                              DevState* st, cudaStream_t s, unsigned long long cond, int chunk) {
   if (dt == DT_F64)
-    return iter_t<double>(d, t, rho, fscale, x, z, r, rhat, p, phat, v, sv, shat, tv, partials, st, s, cond, chunk);
-  return iter_t<float>(d, t, rho, fscale, x, z, r, rhat, p, phat, v, sv, shat, tv, partials, st, s, cond, chunk);
+    return iter_t<double>(d, t, fscale, x, z, r, rhat, p, phat, v, sv, shat, tv, partials, st, s, cond, chunk);
+  return iter_t<float>(d, t, fscale, x, z, r, rhat, p, phat, v, sv, shat, tv, partials, st, s, cond, chunk);
 }
 
 // ------------------------------------------------------------------ BiCGSTAB in one launch

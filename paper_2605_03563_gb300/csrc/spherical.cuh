@@ -84,7 +84,7 @@ cudaError_t launch_bicg_resid(const SphDims& d, const SphTables& t, int dt, int 
 // kernel sets.
 // x is the FP64 iterate, z (FP64, zero at the start) accumulates its
 // increments between replacements (group-wise update).
-cudaError_t launch_bicg_iter(const SphDims& d, const SphTables& t, int dt, const double* rho,
+cudaError_t launch_bicg_iter(const SphDims& d, const SphTables& t, int dt,
                              double fscale, double* x, double* z, void* r, void* rhat, void* p,
                              void* phat, void* v, void* sv, void* shat, void* tv, double* partials,
                              DevState* st, cudaStream_t s, unsigned long long cond = 0,
@@ -98,9 +98,11 @@ bool bicg_steps_fit(const SphDims& d);
 size_t bicg_steps_doubles(const SphDims& d);
 cudaError_t launch_bicg_steps(const SphDims& d, const SphTables& t, int dt, const double* rho, double fscale, double* x,
                               double* z, void* const* v, double* W, DevState* st, cudaStream_t s);
-// scalar finisher for the reference / initial residual (mode 0/1)
+// scalar finisher for the reference / initial residual (mode 0/1); mode 1
+// records rho as the density of the solve's replacements
 cudaError_t launch_bicg_start(const double* partials, int nblk, int mode, DevState* st,
-                              cudaStream_t s, double replace_drop = 0.01, int restart_on_replace = 0);
+                              cudaStream_t s, double replace_drop = 0.01, int restart_on_replace = 0,
+                              const double* rho = nullptr);
 
 // ---- red-black SOR (Sec. 2.1.1) on the spherical grid, FP64.
 // One colour pass: nodes with (i + j + k) mod 2 == colour take

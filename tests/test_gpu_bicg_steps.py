@@ -40,3 +40,21 @@ def test_steps_equal_kernels(nr, nt, npp, inner, prec):
     assert (cut.iterations, cut.status) == (refc.iterations, refc.status)
     assert stepped.iterations == refs.iterations
     assert torch.equal(phi, phr) and torch.equal(phc, phrc) and torch.equal(phs, phrs)
+
+
+@pytest.mark.parametrize("prec", ["fp64", "mixed_fp32"])
+def test_handle_reused_with_another_density(prec):
+    """A loop graph captured for one density buffer serves a solve of another."""
+    import paper_2605_03563_gb300 as P
+    r, th, ph = W.spherical_coords(160, 56, 40, r_in=0.1)   # above the one-launch size
+    a = torch.from_numpy(W.spherical_density(r, th, ph)).to("cuda:0")
+    b = torch.flip(a, (1,)).contiguous() * 3.0 + 1.0
+    def solve(s, rho):
+        phi = torch.zeros_like(rho)
+        return s.solve(rho, phi, tol=1e-8, prec=prec, max_iter=3000), phi
+    with P.SphericalSolver(r, th, ph, lmax=2) as s, P.SphericalSolver(r, th, ph, lmax=2) as fresh:
+        solve(s, a)
+        again, phi = solve(s, b)
+        want, ref = solve(fresh, b)
+    assert (again.iterations, again.status, again.rel_residual) == (want.iterations, want.status, want.rel_residual)
+    assert torch.equal(phi, ref)
