@@ -303,7 +303,8 @@ __device__ __forceinline__ double add_ghost_terms(double v, const double* __rest
 template <int G>
 __global__ void __launch_bounds__(BX* BY)
     k_scale_rhs_ref(Dims d, Dims du, double factor, Coef<double> cf, const double* __restrict__ rho,
-                    const double* __restrict__ phi, double* __restrict__ fs, double* __restrict__ partials) {
+                    const double* __restrict__ phi, double* __restrict__ fs, double* __restrict__ partials,
+                    DevState* __restrict__ st) {
   const int i = blockIdx.x * BX + threadIdx.x + G;
   const int j = blockIdx.y * BY + threadIdx.y + G;
   const int zc = zchunk(d.nk());
@@ -316,12 +317,14 @@ __global__ void __launch_bounds__(BX* BY)
   const bool yb = j < 2 * G || j >= nj;
   double s2 = 0.0;
   AbsMax mx;
+  unsigned hf = 0u;   // high word of the largest |fs|
   if (act) {
     const long long syu = du.sy(), szu = du.sz();
     for (int k = k0; k < k1; k++) {
       const long long pu = du.at(i, j, k);
       const double f = factor * rho[pu];
       fs[d.at(i, j, k)] = f;
+      hf = max(hf, (unsigned)__double2hiint(f) & 0x7fffffffu);
       double v = f;
       if (wx) v = add_ghost_terms<G>(v, phi, pu, 1, i, ni, cf, 0);
       if (yb) v = add_ghost_terms<G>(v, phi, pu, syu, j, nj, cf, 1);
@@ -330,17 +333,18 @@ __global__ void __launch_bounds__(BX* BY)
       mx.take(v);
     }
   }
+  atomic_max_group(hf, &st->fmax);
   block_sum_max(s2, mx.value(), partials);
 }
 
 cudaError_t launch_scale_rhs_ref(const Dims& d, const Dims& du, int order, const double h[3], double factor,
                                  const double* rho, const double* phi, double* fs, double* partials,
-                                 cudaStream_t s) {
+                                 DevState* st, cudaStream_t s) {
   if (du.ex != d.ex || du.ey != d.ey || du.ez != d.ez || du.g != d.g || d.g != order / 2)
     return cudaErrorInvalidValue;
   const Coef<double> cf = make_coef<double>(d, h, order);
-  if (order == 2) k_scale_rhs_ref<1><<<point_grid(d), dim3(BX, BY), 0, s>>>(d, du, factor, cf, rho, phi, fs, partials);
-  else k_scale_rhs_ref<2><<<point_grid(d), dim3(BX, BY), 0, s>>>(d, du, factor, cf, rho, phi, fs, partials);
+  if (order == 2) k_scale_rhs_ref<1><<<point_grid(d), dim3(BX, BY), 0, s>>>(d, du, factor, cf, rho, phi, fs, partials, st);
+  else k_scale_rhs_ref<2><<<point_grid(d), dim3(BX, BY), 0, s>>>(d, du, factor, cf, rho, phi, fs, partials, st);
   return cudaGetLastError();
 }
 
@@ -1268,7 +1272,8 @@ cudaError_t launch_sweep_colour(const Dims& d, int order, const double h[3], int
 // scaled right-hand side because d_coarse = d_fine / 4).
 template <typename TF, typename TC>
 __global__ void __launch_bounds__(BX* BY)
-    k_restrict(Dims fd, Dims cd, const TF* __restrict__ df, TC* __restrict__ fsc, double factor) {
+    k_restrict(Dims fd, Dims cd, const TF* __restrict__ df, TC* __restrict__ fsc, double factor,
+               unsigned* __restrict__ track) {
   using CF = typename St<TF>::C;
   using CC = typename St<TC>::C;
   const int I = blockIdx.x * BX + threadIdx.x + 1;
@@ -1291,35 +1296,39 @@ __global__ void __launch_bounds__(BX* BY)
     }
     return (rows[0] + rows[2]) + (CF)2 * rows[1];
   };
+  unsigned hm = 0u;   // high word of the largest value written (FP64)
   CF below = plane_sum(fd.at(2 * I + g - 1, 2 * J + g - 1, 2 * K0 + g - 2));
   for (int K = K0; K < K1; K++) {
     const long long c = fd.at(2 * I + g - 1, 2 * J + g - 1, 2 * K + g - 1);
     const CF mid = plane_sum(c), above = plane_sum(c + sz);
     CF acc = (below + above) + (CF)2 * mid;
-    St<TC>::st(fsc + cd.at(I + g - 1, J + g - 1, K + g - 1), (CC)(acc * sc));
+    const CC v = (CC)(acc * sc);
+    St<TC>::st(fsc + cd.at(I + g - 1, J + g - 1, K + g - 1), v);
+    if constexpr (sizeof(CC) == 8) hm = max(hm, (unsigned)__double2hiint(v) & 0x7fffffffu);
     below = above;
   }
+  if (sizeof(CC) == 8 && track != nullptr) atomic_max_group(hm, track);
 }
 
 template <typename TF, typename TC>
 static cudaError_t restrict_t(const Dims& fine, const Dims& cd, const void* df, void* fsc, double factor,
-                              cudaStream_t s) {
+                              unsigned* track, cudaStream_t s) {
   dim3 grid = point_grid(cd);
-  k_restrict<TF, TC><<<grid, dim3(BX, BY), 0, s>>>(fine, cd, (const TF*)df, (TC*)fsc, factor);
+  k_restrict<TF, TC><<<grid, dim3(BX, BY), 0, s>>>(fine, cd, (const TF*)df, (TC*)fsc, factor, track);
   return cudaGetLastError();
 }
 
 cudaError_t launch_restrict(const Dims& fine, const Dims& coarse, int dt_f, const void* delta_f, int dt_c, void* fs_c,
-                            double factor, cudaStream_t s) {
+                            double factor, cudaStream_t s, unsigned* track) {
   if (dt_c == DT_F64) {
-    if (dt_f == DT_F64) return restrict_t<double, double>(fine, coarse, delta_f, fs_c, factor, s);
-    if (dt_f == DT_F32) return restrict_t<float, double>(fine, coarse, delta_f, fs_c, factor, s);
-    return restrict_t<__nv_bfloat16, double>(fine, coarse, delta_f, fs_c, factor, s);
+    if (dt_f == DT_F64) return restrict_t<double, double>(fine, coarse, delta_f, fs_c, factor, track, s);
+    if (dt_f == DT_F32) return restrict_t<float, double>(fine, coarse, delta_f, fs_c, factor, track, s);
+    return restrict_t<__nv_bfloat16, double>(fine, coarse, delta_f, fs_c, factor, track, s);
   }
   if (dt_c == DT_F32) {
-    if (dt_f == DT_F64) return restrict_t<double, float>(fine, coarse, delta_f, fs_c, factor, s);
-    if (dt_f == DT_F32) return restrict_t<float, float>(fine, coarse, delta_f, fs_c, factor, s);
-    return restrict_t<__nv_bfloat16, float>(fine, coarse, delta_f, fs_c, factor, s);
+    if (dt_f == DT_F64) return restrict_t<double, float>(fine, coarse, delta_f, fs_c, factor, track, s);
+    if (dt_f == DT_F32) return restrict_t<float, float>(fine, coarse, delta_f, fs_c, factor, track, s);
+    return restrict_t<__nv_bfloat16, float>(fine, coarse, delta_f, fs_c, factor, track, s);
   }
   return cudaErrorInvalidValue;
 }
@@ -1334,7 +1343,8 @@ cudaError_t launch_restrict(const Dims& fine, const Dims& coarse, int dt_f, cons
 // (a + b) + 4 c.  The result equals k_restrict's up to the sign of zeros.
 template <typename TF, typename TC>
 __global__ void __launch_bounds__(BX* BY)
-    k_restrict_red(Dims fd, Dims cd, const TF* __restrict__ df, TC* __restrict__ fsc, double factor) {
+    k_restrict_red(Dims fd, Dims cd, const TF* __restrict__ df, TC* __restrict__ fsc, double factor,
+                   unsigned* __restrict__ track) {
   using CF = typename St<TF>::C;
   using CC = typename St<TC>::C;
   const int I = blockIdx.x * BX + threadIdx.x + 1;
@@ -1349,6 +1359,7 @@ __global__ void __launch_bounds__(BX* BY)
   auto odd_half = [&](long long q) -> CF {
     return (St<TF>::ld(df + q - sy) + St<TF>::ld(df + q + sy)) + (St<TF>::ld(df + q - 1) + St<TF>::ld(df + q + 1));
   };
+  unsigned hm = 0u;   // high word of the largest value written (FP64)
   CF below = odd_half(fd.at(2 * I + g - 1, 2 * J + g - 1, 2 * K0 + g - 2));
   for (int K = K0; K < K1; K++) {
     const long long c = fd.at(2 * I + g - 1, 2 * J + g - 1, 2 * K + g - 1);
@@ -1356,22 +1367,25 @@ __global__ void __launch_bounds__(BX* BY)
     const CF b = St<TF>::ld(df + c + sy - 1) + St<TF>::ld(df + c + sy + 1);
     const CF even = fma((CF)4, St<TF>::ld(df + c), a + b);
     const CF above = odd_half(c + sz);
-    St<TC>::st(fsc + cd.at(I + g - 1, J + g - 1, K + g - 1), (CC)(((below + above) + even) * sc2));
+    const CC v = (CC)(((below + above) + even) * sc2);
+    St<TC>::st(fsc + cd.at(I + g - 1, J + g - 1, K + g - 1), v);
+    if constexpr (sizeof(CC) == 8) hm = max(hm, (unsigned)__double2hiint(v) & 0x7fffffffu);
     below = above;
   }
+  if (sizeof(CC) == 8 && track != nullptr) atomic_max_group(hm, track);
 }
 
 cudaError_t launch_restrict_red(const Dims& fine, const Dims& coarse, int dt_f, const void* delta_f, int dt_c,
-                                void* fs_c, double factor, cudaStream_t s) {
+                                void* fs_c, double factor, cudaStream_t s, unsigned* track) {
   const dim3 grid = point_grid(coarse), blk(BX, BY);
   if (dt_f == DT_F64 && dt_c == DT_F64)
-    k_restrict_red<double, double><<<grid, blk, 0, s>>>(fine, coarse, (const double*)delta_f, (double*)fs_c, factor);
+    k_restrict_red<double, double><<<grid, blk, 0, s>>>(fine, coarse, (const double*)delta_f, (double*)fs_c, factor, track);
   else if (dt_f == DT_F32 && dt_c == DT_F32)
-    k_restrict_red<float, float><<<grid, blk, 0, s>>>(fine, coarse, (const float*)delta_f, (float*)fs_c, factor);
+    k_restrict_red<float, float><<<grid, blk, 0, s>>>(fine, coarse, (const float*)delta_f, (float*)fs_c, factor, track);
   else if (dt_f == DT_F32 && dt_c == DT_F64)
-    k_restrict_red<float, double><<<grid, blk, 0, s>>>(fine, coarse, (const float*)delta_f, (double*)fs_c, factor);
+    k_restrict_red<float, double><<<grid, blk, 0, s>>>(fine, coarse, (const float*)delta_f, (double*)fs_c, factor, track);
   else if (dt_f == DT_F64 && dt_c == DT_F32)
-    k_restrict_red<double, float><<<grid, blk, 0, s>>>(fine, coarse, (const double*)delta_f, (float*)fs_c, factor);
+    k_restrict_red<double, float><<<grid, blk, 0, s>>>(fine, coarse, (const double*)delta_f, (float*)fs_c, factor, track);
   else
     return cudaErrorInvalidValue;
   return cudaGetLastError();

@@ -94,9 +94,10 @@ cudaError_t launch_copy_guess(const Dims& dd, const Dims& sd, const double* src,
 // zero (only the boundary data enter), per block of point_grid(d)
 // (cart_partials_count blocks); the values equal launch_delta's with
 // zero_interior up to the order in which the boundary terms are added.
+// st->fmax takes the high word of the largest |fs|.
 cudaError_t launch_scale_rhs_ref(const Dims& d, const Dims& du, int order, const double h[3], double factor,
                                  const double* rho, const double* phi, double* fs, double* partials,
-                                 cudaStream_t s);
+                                 DevState* st, cudaStream_t s);
 
 // FP64 residual pass of the 7-point stencil on equal spacings along (j, k)
 // diagonals (every delta equal to launch_delta's / launch_delta_st's bit for
@@ -111,9 +112,10 @@ cudaError_t launch_delta_diag(const Dims& d, const double h[3], const double* ph
                               void* out, DevState* st, bool initial, double* partials, int* nblocks,
                               cudaStream_t s);
 
-// fs_coarse = factor * R(delta_fine)  (scaled coarse right-hand side); coarse = layout of fs_c
+// fs_coarse = factor * R(delta_fine)  (scaled coarse right-hand side); coarse = layout of fs_c.
+// track (FP64 coarse levels, optional): *track takes the high word of the largest value written.
 cudaError_t launch_restrict(const Dims& fine, const Dims& coarse, int dt_f, const void* delta_f, int dt_c,
-                            void* fs_c, double factor, cudaStream_t s);
+                            void* fs_c, double factor, cudaStream_t s, unsigned* track = nullptr);
 
 // The same for a 7-point residual that is exactly zero on the black nodes
 // ((i+j+k) odd), as launch_delta_after_sweep leaves it for order 2: the zero
@@ -121,7 +123,7 @@ cudaError_t launch_restrict(const Dims& fine, const Dims& coarse, int dt_f, cons
 // equal to launch_restrict bit for bit up to the sign of zero sums.  dt_f is
 // FP64 or FP32.
 cudaError_t launch_restrict_red(const Dims& fine, const Dims& coarse, int dt_f, const void* delta_f, int dt_c,
-                                void* fs_c, double factor, cudaStream_t s);
+                                void* fs_c, double factor, cudaStream_t s, unsigned* track = nullptr);
 
 // phi_fine += P e_coarse; coarse = layout of e_c.  track (FP64 fine levels,
 // optional): *track takes the high word of the largest |phi_fine| written.

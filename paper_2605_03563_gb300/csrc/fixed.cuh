@@ -376,20 +376,22 @@ inline cudaError_t fx_occupancy(K kern, int smem, std::atomic<int>& cached, int*
 }
 
 // Launch geometry: as many z-chunks as fill the resident blocks of whole waves
-// (blocks_per_sm of the kernel), of 8 to 96 planes each (a chunk stages 2 G
+// (blocks_per_sm of the kernel), of `least` to 96 planes each (a chunk stages 2 G
 // planes that it does not write).
-template <int KIND>
-inline dim3 fx_grid(const Dims& d, int blocks_per_sm, int* zc) {
-  using Gm = FxGeom<KIND>;
-  const int gx = (d.ni() + Gm::TX - 1) / Gm::TX, gy = (d.nj() + Gm::TY - 1) / Gm::TY, nk = d.nk();
+inline dim3 fx_chunks(int gx, int gy, int nk, int blocks_per_sm, int least, int* zc) {
   const long long slots = (long long)device_sm_count() * blocks_per_sm, tiles = (long long)gx * gy;
   long long n = slots / tiles;                             // one wave
   if (n < (nk + 95) / 96) n = ((nk + 95) / 96 * tiles + slots - 1) / slots * slots / tiles;
   n = n < 1 ? 1 : n;
-  const int most = nk < 8 ? 1 : nk / 8;
+  const int most = nk < least ? 1 : nk / least;
   if (n > most) n = most;
   *zc = (int)((nk + n - 1) / n);
   return dim3(gx, gy, (nk + *zc - 1) / *zc);
+}
+template <int KIND>
+inline dim3 fx_grid(const Dims& d, int blocks_per_sm, int* zc) {
+  using Gm = FxGeom<KIND>;
+  return fx_chunks((d.ni() + Gm::TX - 1) / Gm::TX, (d.nj() + Gm::TY - 1) / Gm::TY, d.nk(), blocks_per_sm, 8, zc);
 }
 
 }  // namespace ps

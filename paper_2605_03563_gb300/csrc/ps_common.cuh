@@ -332,8 +332,13 @@ struct DevState {
   unsigned umax;      // high word of max |phi| of the finest FP64 potential as last written (set-up copy, correction)
   unsigned bmax;      // the same over its boundary nodes
   unsigned unext;     // largest |phi| that a norm pass read: umax of the next iteration
-  // FP64 compact multigrid: largest |u| (levels below the finest) and |r| written
-  // on a level in this V-cycle (high words; see fixed.cuh)
+  // FP64 multigrid (fixed_sweeps.cu), high words: the largest |fs| of the finest
+  // level, the largest |phi| at the start of this V-cycle and as read by the pass
+  // that ends it, and the bound the last lagged pass used
+  unsigned fmax, vmax, vnext, lmax;
+  // FP64 multigrid: largest |u| written on a level by the prolongation (compact:
+  // and by the smoother) and largest |r| (right-hand side; compact: residual)
+  // written on it in this V-cycle (high words; see fixed.cuh)
   unsigned hu[8], hr[8];
   unsigned gbar;      // grid barrier of the one-launch iterations (zeroed before each launch)
   int lag_pending;         // lagged-norm V-cycles: a first colour pass with saved values ran this step

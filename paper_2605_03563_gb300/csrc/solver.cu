@@ -25,6 +25,7 @@
 #include <vector>
 
 #include "cart_kernels.cuh"
+#include "fixed_sweeps.cuh"
 #include "tiled_kernels.cuh"
 #include "batch.cuh"
 #include "multipole.cuh"
@@ -119,6 +120,7 @@ struct Active {
   int inner_per_iter = 0;
   // the iterations of a step in one launch (instead of the loop graph), where set
   std::function<cudaError_t(cudaStream_t)> steps;
+  bool fc = false;                    // V-cycle passes of the larger levels on the integer pipe (fixed_sweeps.cu)
   // enqueued by every step before the iterations / after them (may be empty)
   std::function<cudaError_t(cudaStream_t)> prologue, epilogue;
 };
@@ -391,20 +393,37 @@ Work work_of(const Level& L, int order) {
   return w;
 }
 
+// Level l of the FP64 hierarchy takes the fixed-point passes; their bounds
+// before (post = false) and after the coarse-level correction.
+bool use_fc(const ps_ctx* h, const Level& L) {
+  return h->act.fc && L.dt == DT_F64 && L.dt_tmp == DT_F64 && fc_level(L.d, h->order, L.h);
+}
+FcBounds fc_bounds(const ps_ctx* h, int l, bool post) {
+  DevState* st = h->st;
+  if (l == 0) return {post ? &st->hu[0] : &st->vmax, &st->bmax, &st->fmax, nullptr};
+  return {post ? &st->hu[l & 7] : &st->hr[l & 7], &st->hr[l & 7], &st->hr[l & 7], nullptr};
+}
+
 cudaError_t sweep_level(ps_ctx* h, Level& L, int l, double omega, const DevState* st, cudaStream_t s,
-                        const double* wtab = nullptr, int wlen = 0, int first_colour = 0) {
+                        const double* wtab = nullptr, int wlen = 0, int first_colour = 0, bool post = false) {
   const int ncol = h->order == 2 ? 2 : 3;
   const Work w = work_of(L, h->order);
   cudaError_t e;
   // FP64 passes on equal spacings walk (j, k) diagonals: 5 FP64 instructions
   // per update instead of 6 (13-point: 10 instead of 12)
   const bool diag = L.dt == DT_F64 && L.h[0] == L.h[1] && L.h[1] == L.h[2];
-  const double per_update = diag ? 5.0 * w.G : 6.0 * w.G;
+  // (fixed point: one FMA, unequal spacings three)
+  const bool fc = use_fc(h, L) && omega == 1.0 && wtab == nullptr;
+  const double per_update = fc ? (diag ? 1.0 : 3.0) : diag ? 5.0 * w.G : 6.0 * w.G;
   for (int c = first_colour; c < ncol; c++) {
     // one colour pass reads phi everywhere, fs and phi on its colour, writes phi on its colour
     prof_begin(h, l == 0 ? PC_SWEEP0 : PC_SWEEP_C, w.n * w.S * (1.0 + 2.0 / ncol),
                w.n / ncol * (per_update + (omega != 1.0 || wtab ? 2.0 : 0.0)), w.fp64, s);
-    e = (h->nlaunch += 1, launch_sweep_colour(L.d, h->order, L.h, L.dt, L.phi, L.fs, c, omega, st, s, wtab, wlen));
+    if (fc)
+      e = (h->nlaunch += 1, launch_fc_pass(L.d, h->order, L.h, FC_SWEEP, c, (double*)L.phi, (const double*)L.fs, nullptr,
+                                           h->st, fc_bounds(h, l, post), nullptr, nullptr, s));
+    else
+      e = (h->nlaunch += 1, launch_sweep_colour(L.d, h->order, L.h, L.dt, L.phi, L.fs, c, omega, st, s, wtab, wlen));
     prof_end(h, s);
     if (e != cudaSuccess) return e;
   }
@@ -429,12 +448,13 @@ bool use_tiles(const ps_ctx* h, const Level& L, int l) {
 // count GS sweeps (omega = 1) on level l, starting and ending in L.phi: pairs of
 // out-of-place fused sweeps phi -> phib -> phi on tiled 7-point levels, colour
 // passes otherwise (and for an odd last sweep).  skip_first: the first colour
-// pass of the first sweep has already run (colour-pass levels only).
-cudaError_t smooth(ps_ctx* h, Level& L, int l, int count, cudaStream_t s, bool skip_first = false) {
+// pass of the first sweep has already run (colour-pass levels only).  post: after
+// the coarse-level correction.
+cudaError_t smooth(ps_ctx* h, Level& L, int l, int count, cudaStream_t s, bool post, bool skip_first = false) {
   cudaError_t e = cudaSuccess;
   int done = 0;
   if (skip_first && count >= 1) {
-    if ((e = sweep_level(h, L, l, 1.0, nullptr, s, nullptr, 0, 1)) != cudaSuccess) return e;
+    if ((e = sweep_level(h, L, l, 1.0, nullptr, s, nullptr, 0, 1, post)) != cudaSuccess) return e;
     done = 1;
   }
   if (!skip_first && L.phib && h->order == 2 && use_tiles(h, L, l)) {
@@ -452,7 +472,7 @@ cudaError_t smooth(ps_ctx* h, Level& L, int l, int count, cudaStream_t s, bool s
     }
   }
   for (; done < count; done++)
-    if ((e = sweep_level(h, L, l, 1.0, nullptr, s)) != cudaSuccess) return e;
+    if ((e = sweep_level(h, L, l, 1.0, nullptr, s, nullptr, 0, 0, post)) != cudaSuccess) return e;
   return cudaSuccess;
 }
 
@@ -469,8 +489,11 @@ cudaError_t vcycle(ps_ctx* h, Hier& H, int l, int nu1, int nu2, cudaStream_t s, 
     return e;
   }
   const Work w = work_of(L, h->order);
-  if ((e = smooth(h, L, l, nu1, s, skip_first)) != cudaSuccess) return e;
+  if ((e = smooth(h, L, l, nu1, s, false, skip_first)) != cudaSuccess) return e;
   Level& Cl = H.lv[l + 1];
+  const bool fc = use_fc(h, L);
+  // where the coarse level takes the fixed-point passes, its right-hand side is tracked
+  unsigned* track_c = l + 1 < h->nlev - 1 && use_fc(h, Cl) ? &h->st->hr[l + 1 & 7] : nullptr;
   if (use_tiles(h, L, l)) {
     const int rtile = h->order == 2 ? (h->act.restrict_tile != 0 ? h->act.restrict_tile : rr_default_tile(L.dt)) : 0;
     if (l == 0) prof_begin(h, PC_RESTRICT_FUSED0, w.n * 2.0 * w.S + w.n / 8.0 * dt_size(Cl.dt), w.n * (6.0 * w.G + 3.0), w.fp64, s, rtile);
@@ -483,8 +506,11 @@ cudaError_t vcycle(ps_ctx* h, Hier& H, int l, int nu1, int nu2, cudaStream_t s, 
     // storage, where it is the rounding error of the stored value)
     const double frac = h->order == 2 ? 0.5 : 2.0 / 3.0;
     const bool diag = L.dt == DT_F64 && L.h[0] == L.h[1] && L.h[1] == L.h[2];
-    if (l == 0) prof_begin(h, PC_DELTA0, w.n * (w.S * (1.0 + frac) + w.St), w.n * frac * ((diag ? 5.0 * w.G : 6.0 * w.G) + 1.0), w.fp64, s);
-    e = (h->nlaunch += 1, launch_delta_after_sweep(L.d, h->order, L.h, L.dt, L.phi, L.fs, L.dt_tmp, L.tmp, s));
+    if (l == 0) prof_begin(h, PC_DELTA0, w.n * (w.S * (1.0 + frac) + w.St), w.n * frac * (fc ? (diag ? 1.0 : 3.0) : (diag ? 5.0 * w.G : 6.0 * w.G) + 1.0), w.fp64, s);
+    e = (h->nlaunch += 1,
+         fc ? launch_fc_pass(L.d, h->order, L.h, FC_RESID, 0, (double*)L.phi, (const double*)L.fs, (double*)L.tmp, h->st,
+                             fc_bounds(h, l, false), nullptr, nullptr, s)
+            : launch_delta_after_sweep(L.d, h->order, L.h, L.dt, L.phi, L.fs, L.dt_tmp, L.tmp, s));
     if (l == 0) prof_end(h, s);
     if (e != cudaSuccess) return e;
     // 7-point: the residual is zero on the black nodes, which the restriction skips
@@ -492,8 +518,8 @@ cudaError_t vcycle(ps_ctx* h, Hier& H, int l, int nu1, int nu2, cudaStream_t s, 
     if (l == 0)
       prof_begin(h, PC_RESTRICT0, w.n * w.St + w.n / 8.0 * dt_size(Cl.dt), w.n * (red ? kRestrictRedOps : kRestrictOps),
                  w.St == 8.0, s);
-    e = (h->nlaunch += 1, red ? launch_restrict_red(L.d, Cl.d, L.dt_tmp, L.tmp, Cl.dt, Cl.fs, 4.0, s)
-                              : launch_restrict(L.d, Cl.d, L.dt_tmp, L.tmp, Cl.dt, Cl.fs, 4.0, s));
+    e = (h->nlaunch += 1, red ? launch_restrict_red(L.d, Cl.d, L.dt_tmp, L.tmp, Cl.dt, Cl.fs, 4.0, s, track_c)
+                              : launch_restrict(L.d, Cl.d, L.dt_tmp, L.tmp, Cl.dt, Cl.fs, 4.0, s, track_c));
     if (l == 0) prof_end(h, s);
     if (e != cudaSuccess) return e;
   } else {
@@ -509,10 +535,10 @@ cudaError_t vcycle(ps_ctx* h, Hier& H, int l, int nu1, int nu2, cudaStream_t s, 
   if ((e = cudaMemsetAsync(Cl.phi, 0, (size_t)Cl.d.size() * dt_size(Cl.dt), s)) != cudaSuccess) return e;
   if ((e = vcycle(h, H, l + 1, nu1, nu2, s)) != cudaSuccess) return e;
   if (l == 0) prof_begin(h, PC_PROLONG0, w.n * 2.0 * w.S + w.n / 8.0 * dt_size(Cl.dt), w.n * kProlongOps, w.fp64, s);
-  e = (h->nlaunch += 1, launch_prolong(L.d, Cl.d, Cl.dt, Cl.phi, L.dt, L.phi, s));
+  e = (h->nlaunch += 1, launch_prolong(L.d, Cl.d, Cl.dt, Cl.phi, L.dt, L.phi, s, fc ? &h->st->hu[l & 7] : nullptr));
   if (l == 0) prof_end(h, s);
   if (e != cudaSuccess) return e;
-  return smooth(h, L, l, nu2, s);
+  return smooth(h, L, l, nu2, s, true);
 }
 
 // Convergence pass on the finest FP64 level (optionally storing the IR inner RHS).
@@ -533,9 +559,16 @@ cudaError_t norm_pass(ps_ctx* h, double* phi, int mode, int dout, void* out, cud
   if (after_sweep && out == nullptr) {
     const double frac = h->order == 2 ? 0.5 : 2.0 / 3.0;   // colours evaluated
     const bool diag = h->h0[0] == h->h0[1] && h->h0[1] == h->h0[2];   // diagonal walks
-    prof_begin(h, PC_NORM0, n * 8.0 * (1.0 + frac), n * frac * ((diag ? 5.0 * G : 6.0 * G) + 2.0), 1, s);
+    const bool fc = h->act.fc && fc_level(h->d0, h->order, h->h0);
+    prof_begin(h, PC_NORM0, n * 8.0 * (1.0 + frac), n * frac * (fc ? (diag ? 2.0 : 4.0) : (diag ? 5.0 * G : 6.0 * G) + 2.0), 1, s);
     int nb = 0;
-    cudaError_t e = (h->nlaunch += 1, launch_delta_colours(h->d0, h->order, h->h0, phi, h->fs64, h->partials, &nb, s));
+    FcBounds fb = fc_bounds(h, 0, true);
+    fb.track = &h->st->vnext;
+    cudaError_t e =
+        (h->nlaunch += 1,
+         fc
+             ? launch_fc_pass(h->d0, h->order, h->h0, FC_NORM, 0, phi, h->fs64, nullptr, h->st, fb, h->partials, &nb, s)
+             : launch_delta_colours(h->d0, h->order, h->h0, phi, h->fs64, h->partials, &nb, s));
     prof_end(h, s);
     if (e != cudaSuccess) return e;
     return (h->nlaunch += 1, launch_finish_norm(h->partials, nb, dd, mode, h->st, s, cond, chunk));
@@ -543,15 +576,16 @@ cudaError_t norm_pass(ps_ctx* h, double* phi, int mode, int dout, void* out, cud
   if (h->h0[0] == h->h0[1] && h->h0[1] == h->h0[2]) {
     // (j, k) diagonal walks: 5 + 1 FP64 instructions per node (13-point: 10 + 1),
     // + 1 for the FP64 sum of squares
-    const double per = h->order == 2 ? 6.0 : 11.0;
+    // (fixed-point passes: one FMA)
     const bool gate = initial && mode == 1 && out == nullptr;
     // 7-point initial pass with a store: from a zero guess its deltas come from
     // fs and the ghost values alone
     const bool zg = initial && mode == 1 && h->order == 2;
+    DevState* st = out != nullptr || gate ? h->st : nullptr;
+    const double per = st != nullptr && fc_level(h->d0, h->order, h->h0) ? 1.0 : h->order == 2 ? 6.0 : 11.0;
     // (the initial passes are not timed: from a zero guess they do little or no work)
     if (!initial) prof_begin(h, PC_NORM0, n * (16.0 + (out ? (double)dt_size(dout) : 0.0)), n * (out ? per : per + 1.0), 1, s);
     int nb = 0;
-    DevState* st = out != nullptr || gate ? h->st : nullptr;
     cudaError_t e = (h->nlaunch += 1,
                      h->order == 2 ? launch_delta_diag(h->d0, h->h0, phi, h->fs64, dout, out, st, zg, h->partials, &nb, s)
                                    : launch_delta_diag13(h->d0, h->h0, out ? 3 : 2, phi, h->fs64, dout, out, st,
@@ -627,12 +661,12 @@ ps_status cart_prepare(ps_ctx* h, const double* rho, double* phi, double tol, in
   TRY(cudaEventRecord(h->ev[1], s));
   Coef<double> cf = make_coef<double>(h->d0, h->h0, h->order);
   const double fscale = -4.0 * M_PI * h->bc.G * cf.inv_d;
+  TRY((h->nlaunch += 1, launch_init_state(h->st, tol, max_iter, s)));
   // fs and the partials of the reference norm ||f - A phi0||, phi0 = boundary
   // data only (the compact schemes form R_h f and their reference norm themselves)
   if (!own_rhs)
     TRY((h->nlaunch += 1, launch_scale_rhs_ref(h->d0, h->du, h->order, h->h0, fscale, rho, phi, h->fs64,
-                                               h->partials, s)));
-  TRY((h->nlaunch += 1, launch_init_state(h->st, tol, max_iter, s)));
+                                               h->partials, h->st, s)));
   // iterate on the handle's own (pitched) copy of phi: captured loop graphs reference it
   TRY((h->nlaunch += 1, launch_copy_guess(h->d0, h->du, phi, h->phi0, h->st, s)));
   if (own_rhs) return PS_OK;
@@ -654,6 +688,8 @@ ps_status begin_mg64(ps_ctx* h, const ps_solve_opts* o, cudaStream_t s) {
   H->lv[0].phi = phi;
   TRY(norm_pass(h, phi, 1, DT_F64, nullptr, s, 0, 0, false, true));
   const int nu1 = o->nu1, nu2 = o->nu2;
+  h->act.fc = fx_sweeps_fit(h->order, nu1) && fx_sweeps_fit(h->order, nu2);
+  const bool fc0 = h->nlev >= 2 && use_fc(h, H->lv[0]);
   // 7-point on equal spacings with nu1, nu2 >= 1: the convergence check of
   // V-cycle n lags into the first colour pass of V-cycle n + 1 (that pass's
   // x_GS - x_old on colour 0 is V-cycle n's whole residual, colour 1's being
@@ -670,19 +706,28 @@ ps_status begin_mg64(ps_ctx* h, const ps_solve_opts* o, cudaStream_t s) {
   if (lag) {
     double* save = (double*)L0.tmp;
     const double dd = make_coef<double>(h->d0, h->h0, 2).d;
-    h->act.body = [h, H, phi, save, nu1, nu2, dd](unsigned long long cond, int chunk, cudaStream_t q) -> cudaError_t {
+    h->act.body = [h, H, phi, save, nu1, nu2, dd, fc0](unsigned long long cond, int chunk, cudaStream_t q) -> cudaError_t {
       cudaError_t e = vcycle(h, *H, 0, nu1, nu2, q, true);
       if (e != cudaSuccess) return e;
       const double n = (double)h->d0.ni() * h->d0.nj() * h->d0.nk();
       int nb = 0;
-      prof_begin(h, PC_NORM0, n * 8.0 * 2.0, n * 0.5 * 7.0, 1, q);
-      e = (h->nlaunch += 1, launch_sweep_lag(h->d0, h->h0, phi, h->fs64, save, true, h->st, h->partials, &nb, q));
+      prof_begin(h, PC_NORM0, n * 8.0 * 2.0, n * 0.5 * (fc0 ? 3.0 : 7.0), 1, q);
+      FcBounds fb = fc_bounds(h, 0, true);
+      fb.track = &h->st->vnext;
+      e = (h->nlaunch += 1,
+           fc0 ? launch_fc_pass(h->d0, 2, h->h0, FC_LAG, 0, phi, h->fs64, save, h->st, fb, h->partials, &nb, q)
+               : launch_sweep_lag(h->d0, h->h0, phi, h->fs64, save, true, h->st, h->partials, &nb, q));
       prof_end(h, q);
       if (e != cudaSuccess) return e;
       return (h->nlaunch += 1, launch_finish_norm(h->partials, nb, dd, 2, h->st, q, cond, chunk));
     };
-    h->act.prologue = [h, phi, save](cudaStream_t q) -> cudaError_t {
-      return (h->nlaunch += 1, launch_sweep_lag(h->d0, h->h0, phi, h->fs64, save, false, h->st, nullptr, nullptr, q));
+    h->act.prologue = [h, phi, save, fc0](cudaStream_t q) -> cudaError_t {
+      // fixed-point: with the unit of the lagged pass whose values it forms again
+      const unsigned* lm = &h->st->lmax;
+      return (h->nlaunch += 1,
+              fc0 ? launch_fc_pass(h->d0, 2, h->h0, FC_OPEN, 0, phi, h->fs64, nullptr, h->st, {lm, lm, lm, nullptr},
+                                   nullptr, nullptr, q)
+                  : launch_sweep_lag(h->d0, h->h0, phi, h->fs64, save, false, h->st, nullptr, nullptr, q));
     };
     h->act.epilogue = [h, phi, save](cudaStream_t q) -> cudaError_t {
       return (h->nlaunch += 1, launch_restore_colour0(h->d0, phi, save, h->st, q));
@@ -1784,7 +1829,7 @@ ps_status poisson_create(const ps_grid* grid, const double* const coords_host[3]
     if ((s = alloc_zero((void**)&h->fs64, (size_t)h->d0.size() * 8, &h->bytes)) != PS_OK) return bail(s);
     if ((s = alloc_zero((void**)&h->phi0, (size_t)h->d0.size() * 8, &h->bytes)) != PS_OK) return bail(s);
     if ((s = ensure_partials(h, std::max({cart_partials_count(h->d0), delta_colours_partials(h->d0, stencil_order),
-                                                  batch_norm_partials(h->d0, stencil_order),
+                                                  batch_norm_partials(h->d0, stencil_order), fc_partials(h->d0),
                                                   stencil_order == 2 ? 2 * c27_blocks(h->d0) + C27_SHELL_BLOCKS : 0}))) != PS_OK)
       return bail(s);
     if (b.outer == PS_BC_MULTIPOLE) {

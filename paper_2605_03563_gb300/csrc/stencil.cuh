@@ -120,6 +120,10 @@ __device__ __forceinline__ void finish_norm_block(const double* __restrict__ par
   st->amax = m;
   // the residual pass that used these has run; what it read is the potential of
   // the next iteration
+  const unsigned vb = max(st->bmax, st->fmax);
+  st->vmax = mode == 1 ? max(st->umax, st->bmax) : st->vnext;
+  st->lmax = max(mode == 1 ? st->umax : st->hu[0], vb);
+  st->vnext = 0u;
   st->umax = st->unext;
   st->unext = 0u;
 #pragma unroll

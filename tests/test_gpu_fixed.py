@@ -126,3 +126,42 @@ def test_compact_fp64_solve_matches_oracle(compact):
         info = s.solve(torch.from_numpy(rho).to("cuda:0"), phi, tol=1e-4, max_iter=10, nu1=1, nu2=1, compact_order=compact)
     assert info.iterations == info_o.iterations
     assert np.max(np.abs(phi.cpu().numpy() - ref)) <= 1e-10 * np.max(np.abs(ref))
+
+
+@pytest.mark.parametrize("n,h,order,nu1,nu2", [
+    ((96, 112, 80), (1, 1, 1), 2, 1, 1),          # 8-row tiles, lagged check
+    ((176, 144, 144), (1, 1, 1), 2, 3, 2),        # 16-row tiles (above 3 10^6 nodes)
+    ((176, 144, 144), (1, 1.25, 0.75), 2, 1, 2),  # unequal spacings, norm of colour 0
+    ((112, 80, 96), (1, 0.75, 1.25), 2, 2, 3),
+    ((192, 176, 208), (1, 1, 1), 2, 2, 1),        # the second level too
+    ((96, 112, 80), (1, 1, 1), 4, 2, 2),          # 13-point
+    ((144, 112, 112), (1, 1, 1), 4, 1, 2),
+])
+def test_fp64_solve_matches_oracle(n, h, order, nu1, nu2):
+    """FP64 multigrid solves whose colour passes run on the integer pipe: equal
+    V-cycle counts and potentials within 1e-10 of the FP64 oracle (the bound of
+    solves that differ in rounding alone, as above), one V-cycle a step the
+    same bits as the whole solve."""
+    import paper_2605_03563_gb300 as P
+    import workloads as W
+    from oracle import solve as OS
+    from oracle.grid import cart_grid
+    hi = tuple(v * w / 128 for v, w in zip(n, h))
+    g = order // 2
+    x = [np.arange(1 - g, v + g) / v for v in n]
+    rho = np.exp(-((x[0][None, None, :] - .4) ** 2 + (x[1][None, :, None] - .5) ** 2 + (x[2][:, None, None] - .6) ** 2) / .02)
+    rho += 0.1 * np.random.Generator(np.random.PCG64(6)).standard_normal(rho.shape)
+    ref = cart_grid(n, order, hi=hi).zeros()
+    info_o = OS.solve_cartesian(rho, ref, cart_grid(n, order, hi=hi), "mg", 1e-4, max_iter=12, bc="multipole", lmax=2, nu1=nu1, nu2=nu2)
+    rd = torch.from_numpy(rho).to("cuda:0")
+    phi = torch.zeros(W.cart_shape(n, order), dtype=torch.float64, device="cuda:0")
+    again = phi.clone()
+    with P.CartesianSolver(n, order, hi=hi, bc="multipole", lmax=2) as s:
+        info = s.solve(rd, phi, tol=1e-4, max_iter=12, nu1=nu1, nu2=nu2)
+        s.begin(rd, again, tol=1e-4, max_iter=12, nu1=nu1, nu2=nu2)
+        for _ in range(20):
+            s.step(1)
+        s.end()
+    assert info.iterations == info_o.iterations
+    assert torch.equal(phi, again)
+    assert np.max(np.abs(phi.cpu().numpy() - ref)) <= 1e-10 * np.max(np.abs(ref))
