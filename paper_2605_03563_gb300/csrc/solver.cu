@@ -26,6 +26,7 @@
 
 #include "cart_kernels.cuh"
 #include "fixed_sweeps.cuh"
+#include "staged_sweeps.cuh"
 #include "tiled_kernels.cuh"
 #include "batch.cuh"
 #include "multipole.cuh"
@@ -422,6 +423,8 @@ cudaError_t sweep_level(ps_ctx* h, Level& L, int l, double omega, const DevState
     if (fc)
       e = (h->nlaunch += 1, launch_fc_pass(L.d, h->order, L.h, FC_SWEEP, c, (double*)L.phi, (const double*)L.fs, nullptr,
                                            h->st, fc_bounds(h, l, post), nullptr, nullptr, s));
+    else if (omega == 1.0 && wtab == nullptr && st == nullptr && colour_staged_level(L.d, h->order, L.dt))
+      e = (h->nlaunch += 1, launch_colour_staged(L.d, h->order, L.h, L.dt, c, L.phi, L.fs, &h->st->fault, s));
     else
       e = (h->nlaunch += 1, launch_sweep_colour(L.d, h->order, L.h, L.dt, L.phi, L.fs, c, omega, st, s, wtab, wlen));
     prof_end(h, s);
@@ -2387,12 +2390,20 @@ ps_status ps_op_sweep(const ps_grid* grid, int order, int dtype, void* phi, cons
   cudaStream_t st = (cudaStream_t)stream;
   Coef<double> cf = make_coef<double>(d, h, order);
   void* fs = nullptr;
-  TRY(cudaMalloc(&fs, (size_t)d.size() * dt_size(dtype)));
+  const size_t fb = ((size_t)d.size() * dt_size(dtype) + 15) / 16 * 16;
+  TRY(cudaMalloc(&fs, fb + 16));
+  int* fault = (int*)((char*)fs + fb);
+  int faulted = 0;
   cudaError_t e = launch_scale_rhs_any(d, -cf.inv_d, dtype, f, fs, st);
+  if (e == cudaSuccess) e = cudaMemsetAsync(fault, 0, sizeof(int), st);
   const int ncol = order == 2 ? 2 : 3;
+  const bool vec = omega == 1.0 && ((uintptr_t)phi & 15) == 0 && colour_staged_level(d, order, dtype);
   for (int c = 0; c < ncol && e == cudaSuccess; c++)
-    e = launch_sweep_colour(d, order, h, dtype, phi, fs, c, omega, nullptr, st);
+    e = vec ? launch_colour_staged(d, order, h, dtype, c, phi, fs, fault, st)
+            : launch_sweep_colour(d, order, h, dtype, phi, fs, c, omega, nullptr, st);
+  if (e == cudaSuccess && vec) e = cudaMemcpyAsync(&faulted, fault, sizeof(int), cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+  if (e == cudaSuccess && faulted) e = cudaErrorLaunchTimeout;
   cudaFree(fs);
   if (e != cudaSuccess) return fail(PS_ERR_CUDA, "ps_op_sweep: %s", cudaGetErrorString(e));
   return PS_OK;
