@@ -1001,8 +1001,11 @@ cudaError_t vcycle_compact(ps_ctx* h, Hier* H, const CompactLevels& C, int l, in
 static cudaError_t compact_prologue(ps_ctx* h, int order, const double* rho, const double* phi,
                                     double* b, int dt_r, void* r, cudaStream_t s) {
   const double n = (double)h->d0.ni() * h->d0.nj() * h->d0.nk();
-  prof_begin(h, PC_RHS0, n * 16.0, n * (order == 6 ? 19.0 : 12.0), 1, s);
-  cudaError_t e = (h->nlaunch += 1, launch_c27_rhs(h->d0, h->du, order, rho, 4.0 * M_PI * h->bc.G, b, s));
+  const bool fx = order != 2 && c27_fx_rhs_level(h->d0);   // on the integer pipe: two FP64 instructions a node
+  prof_begin(h, PC_RHS0, n * 16.0, n * (fx ? 2.0 : order == 6 ? 19.0 : 12.0), 1, s);
+  int nrhs = 0;
+  cudaError_t e = launch_c27_rhs(h->d0, h->du, order, rho, 4.0 * M_PI * h->bc.G, b, h->st, &nrhs, s);
+  h->nlaunch += nrhs;
   prof_end(h, s);
   if (e != cudaSuccess) return e;
   prof_begin(h, PC_NORM0, n * (16.0 + (double)dt_size(dt_r)), n * 18.0, 1, s);

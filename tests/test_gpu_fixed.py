@@ -165,3 +165,56 @@ def test_fp64_solve_matches_oracle(n, h, order, nu1, nu2):
     assert info.iterations == info_o.iterations
     assert torch.equal(phi, again)
     assert np.max(np.abs(phi.cpu().numpy() - ref)) <= 1e-10 * np.max(np.abs(ref))
+
+
+@pytest.mark.parametrize("order", [4, 6])
+@pytest.mark.parametrize("kind", ["smooth", "rough", "spike", "steps"])
+@pytest.mark.parametrize("n", [(96, 112, 80), (160, 64, 96)])
+def test_compact_right_hand_side(n, kind, order):
+    """R_h on the integer pipe: the initial residual b - L_h phi of a solve from
+    phi = 0 inside boundary data that make the reference norm known, against
+    R_h rho evaluated in FP64 with the cubic extrapolation; the residual that
+    is compared is ||b|| / ||b + boundary terms||, all of b.
+
+    Tolerance, derived before the first run: b is formed from values truncated
+    by less than 2^-56 of the largest (binade) with weights summing to 1.05, and
+    the FP64 evaluation has 20 roundings: 32 2^-53 max|rho| / rms(b) relative."""
+    import paper_2605_03563_gb300 as P
+    h = 1.0 / 64
+    shape = tuple(v + 1 for v in n[::-1])
+    rho = _guess("smooth", shape, 1)
+    rng = np.random.Generator(np.random.PCG64(9))
+    if kind == "rough":
+        rho = rng.standard_normal(shape)
+    elif kind == "spike":
+        rho[shape[0] // 2, shape[1] // 3, 0] = 1e7
+    elif kind == "steps":
+        rho = np.where(rng.random(shape) < 0.5, 1.0, -1e-3)
+    f = np.pad(rho, 1)
+    for ax in range(3):
+        g = np.moveaxis(f, ax, 0)
+        g[0] = 4 * g[1] - 6 * g[2] + 4 * g[3] - g[4]
+        g[-1] = 4 * g[-2] - 6 * g[-3] + 4 * g[-4] - g[-5]
+    def sh(dz, dy, dx):
+        return f[2 + dz:f.shape[0] - 2 + dz, 2 + dy:f.shape[1] - 2 + dy, 2 + dx:f.shape[2] - 2 + dx]
+    fa = ed = ax2 = 0.0
+    for p in (-1, 1):
+        fa = fa + sh(p, 0, 0) + sh(0, p, 0) + sh(0, 0, p)
+        ax2 = ax2 + sh(2 * p, 0, 0) + sh(0, 2 * p, 0) + sh(0, 0, 2 * p)
+        for q in (-1, 1):
+            ed = ed + sh(p, q, 0) + sh(p, 0, q) + sh(0, p, q)
+    b = sh(0, 0, 0) / 2 + fa / 12 if order == 4 else 67 / 120 * sh(0, 0, 0) + fa / 18 + ed / 90 - ax2 / 240
+    b = 4 * np.pi * b
+    # a guess v whose residual is compared: r = b - L_h v, the reference that of v's boundary alone (0 here: b)
+    v = 1e-3 * _guess("smooth", shape, 1)
+    v[0] = v[-1] = 0.0
+    v[:, 0] = v[:, -1] = 0.0
+    v[:, :, 0] = v[:, :, -1] = 0.0
+    v *= np.max(np.abs(rho)) * h * h
+    lv, W = _residual(v, np.zeros(tuple(s - 2 for s in shape)), h, 2, order)   # -L_h v
+    want = np.linalg.norm(b + lv) / np.linalg.norm(b)
+    tol = 32 * 2.0 ** -53 * (4 * np.pi * np.max(np.abs(rho)) + W * np.max(np.abs(v))) / np.sqrt(np.mean(b * b)) + 1e-12
+    phi = torch.from_numpy(v).to("cuda:0")
+    with P.CartesianSolver(n, hi=tuple(a * h for a in n)) as s:
+        info = s.solve(torch.from_numpy(rho).to("cuda:0"), phi, tol=0.0, max_iter=0, compact_order=order)
+    assert abs(info.rel_residual - want) <= tol * max(want, 1.0), (info.rel_residual, want, tol)
