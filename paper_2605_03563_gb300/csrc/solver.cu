@@ -231,14 +231,13 @@ ps_status fail(ps_status s, const char* fmt, ...) {
 // Full weighting: per coarse node two carried plane sums of 8 (three row sums of
 // an add and an FMA, then an add and an FMA), the z-triple (add, FMA) and the
 // scale: 19 per 8 fine nodes.  Trilinear prolongation: per coarse cell one face
-// (4 midpoints of an add and a multiply), 4 z-midpoints and 8 accumulations:
-// 24 per 8 fine nodes.
+// (4 sums), 4 z-sums and 8 accumulations: 16 per 8 fine nodes.
 constexpr double kRestrictOps = 19.0 / 8.0;
 // Full weighting of a residual that is zero on the black nodes: a carried half
 // sum of the odd-offset plane (3 adds), the even-offset plane (2 adds, 1 FMA),
 // the z-triple (2 adds) and the scale: 9 per 8 fine nodes.
 constexpr double kRestrictRedOps = 9.0 / 8.0;
-constexpr double kProlongOps = 3.0;
+constexpr double kProlongOps = 2.0;
 
 // Profiler: begin/end pair around one launch on stream s.
 void prof_begin(ps_ctx* h, int cls, double bytes, double ops, int fp64, cudaStream_t s, int variant = 0) {
