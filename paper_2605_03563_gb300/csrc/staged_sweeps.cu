@@ -13,8 +13,8 @@
 // during the pass, so what a neighbour tile stages meanwhile is not ambiguous
 // where it is used.  Measured (us a pass, per-node pass before): 256^3 FP32
 // 42.6 -> 29.4 (200 MB, 30 at the copy rate), 128^3 FP32 9.8 -> 8.3; 512^3 BF16
-// 181.7 -> 177.7 (800 MB, 118 at the copy rate; bound by shared-memory wavefronts,
-// 84 % of their peak).  64^3 FP32 is slower (5.5 against 3.6: a few tiles, a
+// 181.7 -> 177.7 (800 MB, 118 at the copy rate; bound by issue and the L1 data
+// path: 2.4 instructions a cycle, L1 at 84 % of its peak).  64^3 FP32 is slower (5.5 against 3.6: a few tiles, a
 // chain from plane to plane), hence SS_MIN_NODES.  Two rows a lane: with one, 196
 // on 512^3 (more halo to stage).
 #include <algorithm>
