@@ -95,7 +95,11 @@ typedef struct {
  * residual and run in FP64. */
 typedef enum { PS_SOR = 0, PS_CG = 1, PS_MG = 2, PS_BICGSTAB = 3, PS_PCG = 4 } ps_method;
 
-/* PS_FP64: every kernel computes and stores in FP64.
+/* PS_FP64: every field is stored in FP64.  Arithmetic is FP64, except that on
+ *   levels of 7 x 10^5 unknowns and more the passes of multigrid add neighbours
+ *   as 64-bit fixed-point numbers of one unit per pass (1/16 of the last place
+ *   of the largest value's binade; 13-point colour passes 1/8), exactly, and
+ *   round once to FP64; their error is no larger than that of the FP64 sums.
  * PS_MIXED_FP32: Cartesian: FP64 iterative refinement (outer residual,
  *   correction, norms, multipole moments and coarsest solve in FP64) around
  *   FP32 inner V-cycles.  Spherical: FP64 iterative refinement around inner
@@ -212,7 +216,8 @@ ps_status poisson_solve(ps_handle h, const double* rho_dev, double* phi_dev, dou
  *   begin  validates, enqueues the multipole boundary, right-hand side,
  *          reference and initial residual (no host synchronisation)
  *   step   enqueues up to max_iterations more iterations (one CUDA-graph
- *          launch whose device-side while loop stops at convergence)
+ *          launch whose device-side while loop stops at convergence; SOR and
+ *          BiCGSTAB on small grids: one cooperative launch)
  *   poll   waits for the handle's stream and reports *done (converged, not
  *          converged or diverged); info (may be NULL) gets the progress
  *   end    copies the iterate to phi_dev, waits, fills info and returns the

@@ -418,7 +418,7 @@ cudaError_t sweep_level(ps_ctx* h, Level& L, int l, double omega, const DevState
   for (int c = first_colour; c < ncol; c++) {
     // one colour pass reads phi everywhere, fs and phi on its colour, writes phi on its colour
     prof_begin(h, l == 0 ? PC_SWEEP0 : PC_SWEEP_C, w.n * w.S * (1.0 + 2.0 / ncol),
-               w.n / ncol * (per_update + (omega != 1.0 || wtab ? 2.0 : 0.0)), w.fp64, s);
+               w.n / ncol * (per_update + (omega != 1.0 || wtab ? 2.0 : 0.0)), w.fp64 && !fc, s);
     if (fc)
       e = (h->nlaunch += 1, launch_fc_pass(L.d, h->order, L.h, FC_SWEEP, c, (double*)L.phi, (const double*)L.fs, nullptr,
                                            h->st, fc_bounds(h, l, post), nullptr, nullptr, s));
@@ -508,7 +508,7 @@ cudaError_t vcycle(ps_ctx* h, Hier& H, int l, int nu1, int nu2, cudaStream_t s, 
     // storage, where it is the rounding error of the stored value)
     const double frac = h->order == 2 ? 0.5 : 2.0 / 3.0;
     const bool diag = L.dt == DT_F64 && L.h[0] == L.h[1] && L.h[1] == L.h[2];
-    if (l == 0) prof_begin(h, PC_DELTA0, w.n * (w.S * (1.0 + frac) + w.St), w.n * frac * (fc ? (diag ? 1.0 : 3.0) : (diag ? 5.0 * w.G : 6.0 * w.G) + 1.0), w.fp64, s);
+    if (l == 0) prof_begin(h, PC_DELTA0, w.n * (w.S * (1.0 + frac) + w.St), w.n * frac * (fc ? (diag ? 1.0 : 3.0) : (diag ? 5.0 * w.G : 6.0 * w.G) + 1.0), w.fp64 && !fc, s);
     e = (h->nlaunch += 1,
          fc ? launch_fc_pass(L.d, h->order, L.h, FC_RESID, 0, (double*)L.phi, (const double*)L.fs, (double*)L.tmp, h->st,
                              fc_bounds(h, l, false), nullptr, nullptr, s)
@@ -562,7 +562,7 @@ cudaError_t norm_pass(ps_ctx* h, double* phi, int mode, int dout, void* out, cud
     const double frac = h->order == 2 ? 0.5 : 2.0 / 3.0;   // colours evaluated
     const bool diag = h->h0[0] == h->h0[1] && h->h0[1] == h->h0[2];   // diagonal walks
     const bool fc = h->act.fc && fc_level(h->d0, h->order, h->h0);
-    prof_begin(h, PC_NORM0, n * 8.0 * (1.0 + frac), n * frac * (fc ? (diag ? 2.0 : 4.0) : (diag ? 5.0 * G : 6.0 * G) + 2.0), 1, s);
+    prof_begin(h, PC_NORM0, n * 8.0 * (1.0 + frac), n * frac * (fc ? (diag ? 2.0 : 4.0) : (diag ? 5.0 * G : 6.0 * G) + 2.0), fc ? 0 : 1, s);
     int nb = 0;
     FcBounds fb = fc_bounds(h, 0, true);
     fb.track = &h->st->vnext;
@@ -586,7 +586,7 @@ cudaError_t norm_pass(ps_ctx* h, double* phi, int mode, int dout, void* out, cud
     DevState* st = out != nullptr || gate ? h->st : nullptr;
     const double per = st != nullptr && fc_level(h->d0, h->order, h->h0) ? 1.0 : h->order == 2 ? 6.0 : 11.0;
     // (the initial passes are not timed: from a zero guess they do little or no work)
-    if (!initial) prof_begin(h, PC_NORM0, n * (16.0 + (out ? (double)dt_size(dout) : 0.0)), n * (out ? per : per + 1.0), 1, s);
+    if (!initial) prof_begin(h, PC_NORM0, n * (16.0 + (out ? (double)dt_size(dout) : 0.0)), n * (out ? per : per + 1.0), per == 1.0 ? 0 : 1, s);
     int nb = 0;
     cudaError_t e = (h->nlaunch += 1,
                      h->order == 2 ? launch_delta_diag(h->d0, h->h0, phi, h->fs64, dout, out, st, zg, h->partials, &nb, s)
@@ -713,7 +713,7 @@ ps_status begin_mg64(ps_ctx* h, const ps_solve_opts* o, cudaStream_t s) {
       if (e != cudaSuccess) return e;
       const double n = (double)h->d0.ni() * h->d0.nj() * h->d0.nk();
       int nb = 0;
-      prof_begin(h, PC_NORM0, n * 8.0 * 2.0, n * 0.5 * (fc0 ? 3.0 : 7.0), 1, q);
+      prof_begin(h, PC_NORM0, n * 8.0 * 2.0, n * 0.5 * (fc0 ? 3.0 : 7.0), fc0 ? 0 : 1, q);
       FcBounds fb = fc_bounds(h, 0, true);
       fb.track = &h->st->vnext;
       e = (h->nlaunch += 1,
@@ -836,13 +836,14 @@ ps_status begin_sor(ps_ctx* h, const ps_solve_opts* o, cudaStream_t s) {
     return norm_pass(h, phi, 2, DT_F64, nullptr, q, cond, chunk);
   };
   if (sor_steps_fit(h->d0)) {
-    if (!h->sor_alt) {
-      ps_status r = alloc_zero((void**)&h->sor_alt, (size_t)h->d0.size() * sizeof(double), &h->bytes);
-      if (r != PS_OK) return r;
+    if (!h->sor_alt && alloc_zero((void**)&h->sor_alt, (size_t)h->d0.size() * sizeof(double), &h->bytes) != PS_OK) {
+      (void)cudaGetLastError();   // no room: the separate passes, which need none
+      h->sor_alt = nullptr;
     }
-    h->act.steps = [h, phi, omega, wtab, wlen](cudaStream_t q) -> cudaError_t {
-      return launch_sor_steps(h->d0, h->h0, phi, h->sor_alt, h->fs64, omega, wtab, wlen, h->st, h->partials, 2 * h->npart, q);
-    };
+    if (h->sor_alt)
+      h->act.steps = [h, phi, omega, wtab, wlen](cudaStream_t q) -> cudaError_t {
+        return launch_sor_steps(h->d0, h->h0, phi, h->sor_alt, h->fs64, omega, wtab, wlen, h->st, h->partials, 2 * h->npart, q);
+      };
   }
   char key[64];
   if (wtab) snprintf(key, sizeof(key), "sor:chebyshev");
@@ -1001,7 +1002,7 @@ static cudaError_t compact_prologue(ps_ctx* h, int order, const double* rho, con
                                     double* b, int dt_r, void* r, cudaStream_t s) {
   const double n = (double)h->d0.ni() * h->d0.nj() * h->d0.nk();
   const bool fx = order != 2 && c27_fx_rhs_level(h->d0);   // on the integer pipe: two FP64 instructions a node
-  prof_begin(h, PC_RHS0, n * 16.0, n * (fx ? 2.0 : order == 6 ? 19.0 : 12.0), 1, s);
+  prof_begin(h, PC_RHS0, n * 16.0, n * (fx ? 2.0 : order == 6 ? 19.0 : 12.0), fx ? 0 : 1, s);
   int nrhs = 0;
   cudaError_t e = launch_c27_rhs(h->d0, h->du, order, rho, 4.0 * M_PI * h->bc.G, b, h->st, &nrhs, s);
   h->nlaunch += nrhs;
@@ -1194,13 +1195,14 @@ ps_status bicg_start(ps_ctx* h, int dt, const double* rho, double fscale, double
   TRY(cudaMemsetAsync(h->sz, 0, (size_t)h->sd.size() * sizeof(double), s));
   double* z = h->sz;
   if (bicg_steps_fit(h->sd)) {
-    if (!h->sph_part) {
-      ps_status r = alloc_zero((void**)&h->sph_part, bicg_steps_doubles(h->sd) * sizeof(double), &h->bytes);
-      if (r != PS_OK) return r;
+    if (!h->sph_part && alloc_zero((void**)&h->sph_part, bicg_steps_doubles(h->sd) * sizeof(double), &h->bytes) != PS_OK) {
+      (void)cudaGetLastError();   // no room: the separate kernels, which need none
+      h->sph_part = nullptr;
     }
-    h->act.steps = [h, dt, rho, fscale, x, z, v, st](cudaStream_t q) -> cudaError_t {
-      return launch_bicg_steps(h->sd, h->stab, dt, rho, fscale, x, z, v, h->sph_part, st, q);
-    };
+    if (h->sph_part)
+      h->act.steps = [h, dt, rho, fscale, x, z, v, st](cudaStream_t q) -> cudaError_t {
+        return launch_bicg_steps(h->sd, h->stab, dt, rho, fscale, x, z, v, h->sph_part, st, q);
+      };
   }
   *body = [h, dt, fscale, x, z, v, st](unsigned long long cond, int chunk, cudaStream_t q) -> cudaError_t {
     const double n = (double)h->sd.nr * h->sd.nt * h->sd.np;
@@ -1743,8 +1745,14 @@ size_t poisson_workspace_bytes(const ps_grid* grid, int stencil_order, int l_max
     const size_t n = (size_t)(grid->n[0] + 2) * (grid->n[1] + 2) * (grid->n[2] + 2);
     const size_t vec = prec == PS_FP64 ? 8 : 4;
     // 8 Krylov vectors, the FP64 iterate and its increments, and the
-    // (r, theta) tables (diagonal, rJ, the SOR form)
-    return n * (8 * vec + 16) + (size_t)grid->n[0] * grid->n[1] * 80;
+    // (r, theta) tables (diagonal, rJ, the SOR form); the one-launch
+    // iterations' partial sums where the grid takes them
+    SphDims sd{};
+    sd.nr = grid->n[0];
+    sd.nt = grid->n[1];
+    sd.np = grid->n[2];
+    const size_t part = sd.nr > 0 && sd.nt > 0 && sd.np > 0 && bicg_steps_fit(sd) ? bicg_steps_doubles(sd) * 8 : 0;
+    return n * (8 * vec + 16) + (size_t)grid->n[0] * grid->n[1] * 80 + part;
   }
   return 0;
 }
