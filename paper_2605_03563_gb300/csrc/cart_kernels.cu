@@ -1273,7 +1273,7 @@ cudaError_t launch_sweep_colour(const Dims& d, int order, const double h[3], int
 template <typename TF, typename TC>
 __global__ void __launch_bounds__(BX* BY)
     k_restrict(Dims fd, Dims cd, const TF* __restrict__ df, TC* __restrict__ fsc, double factor,
-               unsigned* __restrict__ track) {
+               unsigned* __restrict__ track, TC* __restrict__ zero) {
   using CF = typename St<TF>::C;
   using CC = typename St<TC>::C;
   const int I = blockIdx.x * BX + threadIdx.x + 1;
@@ -1303,7 +1303,9 @@ __global__ void __launch_bounds__(BX* BY)
     const CF mid = plane_sum(c), above = plane_sum(c + sz);
     CF acc = (below + above) + (CF)2 * mid;
     const CC v = (CC)(acc * sc);
-    St<TC>::st(fsc + cd.at(I + g - 1, J + g - 1, K + g - 1), v);
+    const long long p = cd.at(I + g - 1, J + g - 1, K + g - 1);
+    St<TC>::st(fsc + p, v);
+    if (zero != nullptr) St<TC>::st(zero + p, (CC)0);
     if constexpr (sizeof(CC) == 8) hm = max(hm, (unsigned)__double2hiint(v) & 0x7fffffffu);
     below = above;
   }
@@ -1312,23 +1314,23 @@ __global__ void __launch_bounds__(BX* BY)
 
 template <typename TF, typename TC>
 static cudaError_t restrict_t(const Dims& fine, const Dims& cd, const void* df, void* fsc, double factor,
-                              unsigned* track, cudaStream_t s) {
+                              unsigned* track, void* zero, cudaStream_t s) {
   dim3 grid = point_grid(cd);
-  k_restrict<TF, TC><<<grid, dim3(BX, BY), 0, s>>>(fine, cd, (const TF*)df, (TC*)fsc, factor, track);
+  k_restrict<TF, TC><<<grid, dim3(BX, BY), 0, s>>>(fine, cd, (const TF*)df, (TC*)fsc, factor, track, (TC*)zero);
   return cudaGetLastError();
 }
 
 cudaError_t launch_restrict(const Dims& fine, const Dims& coarse, int dt_f, const void* delta_f, int dt_c, void* fs_c,
-                            double factor, cudaStream_t s, unsigned* track) {
+                            double factor, cudaStream_t s, unsigned* track, void* zero) {
   if (dt_c == DT_F64) {
-    if (dt_f == DT_F64) return restrict_t<double, double>(fine, coarse, delta_f, fs_c, factor, track, s);
-    if (dt_f == DT_F32) return restrict_t<float, double>(fine, coarse, delta_f, fs_c, factor, track, s);
-    return restrict_t<__nv_bfloat16, double>(fine, coarse, delta_f, fs_c, factor, track, s);
+    if (dt_f == DT_F64) return restrict_t<double, double>(fine, coarse, delta_f, fs_c, factor, track, zero, s);
+    if (dt_f == DT_F32) return restrict_t<float, double>(fine, coarse, delta_f, fs_c, factor, track, zero, s);
+    return restrict_t<__nv_bfloat16, double>(fine, coarse, delta_f, fs_c, factor, track, zero, s);
   }
   if (dt_c == DT_F32) {
-    if (dt_f == DT_F64) return restrict_t<double, float>(fine, coarse, delta_f, fs_c, factor, track, s);
-    if (dt_f == DT_F32) return restrict_t<float, float>(fine, coarse, delta_f, fs_c, factor, track, s);
-    return restrict_t<__nv_bfloat16, float>(fine, coarse, delta_f, fs_c, factor, track, s);
+    if (dt_f == DT_F64) return restrict_t<double, float>(fine, coarse, delta_f, fs_c, factor, track, zero, s);
+    if (dt_f == DT_F32) return restrict_t<float, float>(fine, coarse, delta_f, fs_c, factor, track, zero, s);
+    return restrict_t<__nv_bfloat16, float>(fine, coarse, delta_f, fs_c, factor, track, zero, s);
   }
   return cudaErrorInvalidValue;
 }
@@ -1344,7 +1346,7 @@ cudaError_t launch_restrict(const Dims& fine, const Dims& coarse, int dt_f, cons
 template <typename TF, typename TC>
 __global__ void __launch_bounds__(BX* BY)
     k_restrict_red(Dims fd, Dims cd, const TF* __restrict__ df, TC* __restrict__ fsc, double factor,
-                   unsigned* __restrict__ track) {
+                   unsigned* __restrict__ track, TC* __restrict__ zero) {
   using CF = typename St<TF>::C;
   using CC = typename St<TC>::C;
   const int I = blockIdx.x * BX + threadIdx.x + 1;
@@ -1368,7 +1370,9 @@ __global__ void __launch_bounds__(BX* BY)
     const CF even = fma((CF)4, St<TF>::ld(df + c), a + b);
     const CF above = odd_half(c + sz);
     const CC v = (CC)(((below + above) + even) * sc2);
-    St<TC>::st(fsc + cd.at(I + g - 1, J + g - 1, K + g - 1), v);
+    const long long p = cd.at(I + g - 1, J + g - 1, K + g - 1);
+    St<TC>::st(fsc + p, v);
+    if (zero != nullptr) St<TC>::st(zero + p, (CC)0);
     if constexpr (sizeof(CC) == 8) hm = max(hm, (unsigned)__double2hiint(v) & 0x7fffffffu);
     below = above;
   }
@@ -1376,16 +1380,16 @@ __global__ void __launch_bounds__(BX* BY)
 }
 
 cudaError_t launch_restrict_red(const Dims& fine, const Dims& coarse, int dt_f, const void* delta_f, int dt_c,
-                                void* fs_c, double factor, cudaStream_t s, unsigned* track) {
+                                void* fs_c, double factor, cudaStream_t s, unsigned* track, void* zero) {
   const dim3 grid = point_grid(coarse), blk(BX, BY);
   if (dt_f == DT_F64 && dt_c == DT_F64)
-    k_restrict_red<double, double><<<grid, blk, 0, s>>>(fine, coarse, (const double*)delta_f, (double*)fs_c, factor, track);
+    k_restrict_red<double, double><<<grid, blk, 0, s>>>(fine, coarse, (const double*)delta_f, (double*)fs_c, factor, track, (double*)zero);
   else if (dt_f == DT_F32 && dt_c == DT_F32)
-    k_restrict_red<float, float><<<grid, blk, 0, s>>>(fine, coarse, (const float*)delta_f, (float*)fs_c, factor, track);
+    k_restrict_red<float, float><<<grid, blk, 0, s>>>(fine, coarse, (const float*)delta_f, (float*)fs_c, factor, track, (float*)zero);
   else if (dt_f == DT_F32 && dt_c == DT_F64)
-    k_restrict_red<float, double><<<grid, blk, 0, s>>>(fine, coarse, (const float*)delta_f, (double*)fs_c, factor, track);
+    k_restrict_red<float, double><<<grid, blk, 0, s>>>(fine, coarse, (const float*)delta_f, (double*)fs_c, factor, track, (double*)zero);
   else if (dt_f == DT_F64 && dt_c == DT_F32)
-    k_restrict_red<double, float><<<grid, blk, 0, s>>>(fine, coarse, (const double*)delta_f, (float*)fs_c, factor, track);
+    k_restrict_red<double, float><<<grid, blk, 0, s>>>(fine, coarse, (const double*)delta_f, (float*)fs_c, factor, track, (float*)zero);
   else
     return cudaErrorInvalidValue;
   return cudaGetLastError();

@@ -113,9 +113,11 @@ cudaError_t launch_delta_diag(const Dims& d, const double h[3], const double* ph
                               cudaStream_t s);
 
 // fs_coarse = factor * R(delta_fine)  (scaled coarse right-hand side); coarse = layout of fs_c.
-// track (FP64 coarse levels, optional): *track takes the high word of the largest value written.
+// track (FP64 coarse levels, optional): *track takes the high word of the largest value written;
+// zero (optional): an array like fs_c whose interior is set to zero.
 cudaError_t launch_restrict(const Dims& fine, const Dims& coarse, int dt_f, const void* delta_f, int dt_c,
-                            void* fs_c, double factor, cudaStream_t s, unsigned* track = nullptr);
+                            void* fs_c, double factor, cudaStream_t s, unsigned* track = nullptr,
+                            void* zero = nullptr);
 
 // The same for a 7-point residual that is exactly zero on the black nodes
 // ((i+j+k) odd), as launch_delta_after_sweep leaves it for order 2: the zero
@@ -123,7 +125,8 @@ cudaError_t launch_restrict(const Dims& fine, const Dims& coarse, int dt_f, cons
 // equal to launch_restrict bit for bit up to the sign of zero sums.  dt_f is
 // FP64 or FP32.
 cudaError_t launch_restrict_red(const Dims& fine, const Dims& coarse, int dt_f, const void* delta_f, int dt_c,
-                                void* fs_c, double factor, cudaStream_t s, unsigned* track = nullptr);
+                                void* fs_c, double factor, cudaStream_t s, unsigned* track = nullptr,
+                            void* zero = nullptr);
 
 // phi_fine += P e_coarse; coarse = layout of e_c.  track (FP64 fine levels,
 // optional): *track takes the high word of the largest |phi_fine| written.

@@ -490,6 +490,8 @@ cudaError_t vcycle(ps_ctx* h, Hier& H, int l, int nu1, int nu2, cudaStream_t s, 
     prof_end(h, s);
     return e;
   }
+  // (each restriction also zeroes the coarse guess: the boundary of those arrays is
+  // zero from their allocation on, and only interiors are written; a memset node is 2 us)
   const Work w = work_of(L, h->order);
   if ((e = smooth(h, L, l, nu1, s, false, skip_first)) != cudaSuccess) return e;
   Level& Cl = H.lv[l + 1];
@@ -499,7 +501,7 @@ cudaError_t vcycle(ps_ctx* h, Hier& H, int l, int nu1, int nu2, cudaStream_t s, 
   if (use_tiles(h, L, l)) {
     const int rtile = h->order == 2 ? (h->act.restrict_tile != 0 ? h->act.restrict_tile : rr_default_tile(L.dt)) : 0;
     if (l == 0) prof_begin(h, PC_RESTRICT_FUSED0, w.n * 2.0 * w.S + w.n / 8.0 * dt_size(Cl.dt), w.n * (6.0 * w.G + 3.0), w.fp64, s, rtile);
-    e = (h->nlaunch += 1, launch_resid_restrict(L.d, Cl.d, h->order, L.h, L.dt, L.phi, L.fs, Cl.dt, Cl.fs, 4.0, &h->st->fault, s, rtile));
+    e = (h->nlaunch += 1, launch_resid_restrict(L.d, Cl.d, h->order, L.h, L.dt, L.phi, L.fs, Cl.dt, Cl.fs, 4.0, &h->st->fault, s, rtile, Cl.phi));
     if (l == 0) prof_end(h, s);
     if (e != cudaSuccess) return e;
   } else if (nu1 >= 1 && L.dt != DT_BF16) {
@@ -520,8 +522,8 @@ cudaError_t vcycle(ps_ctx* h, Hier& H, int l, int nu1, int nu2, cudaStream_t s, 
     if (l == 0)
       prof_begin(h, PC_RESTRICT0, w.n * w.St + w.n / 8.0 * dt_size(Cl.dt), w.n * (red ? kRestrictRedOps : kRestrictOps),
                  w.St == 8.0, s);
-    e = (h->nlaunch += 1, red ? launch_restrict_red(L.d, Cl.d, L.dt_tmp, L.tmp, Cl.dt, Cl.fs, 4.0, s, track_c)
-                              : launch_restrict(L.d, Cl.d, L.dt_tmp, L.tmp, Cl.dt, Cl.fs, 4.0, s, track_c));
+    e = (h->nlaunch += 1, red ? launch_restrict_red(L.d, Cl.d, L.dt_tmp, L.tmp, Cl.dt, Cl.fs, 4.0, s, track_c, Cl.phi)
+                              : launch_restrict(L.d, Cl.d, L.dt_tmp, L.tmp, Cl.dt, Cl.fs, 4.0, s, track_c, Cl.phi));
     if (l == 0) prof_end(h, s);
     if (e != cudaSuccess) return e;
   } else {
@@ -530,11 +532,10 @@ cudaError_t vcycle(ps_ctx* h, Hier& H, int l, int nu1, int nu2, cudaStream_t s, 
     if (l == 0) prof_end(h, s);
     if (e != cudaSuccess) return e;
     if (l == 0) prof_begin(h, PC_RESTRICT0, w.n * w.St + w.n / 8.0 * dt_size(Cl.dt), w.n * kRestrictOps, w.St == 8.0, s);
-    e = (h->nlaunch += 1, launch_restrict(L.d, Cl.d, L.dt_tmp, L.tmp, Cl.dt, Cl.fs, 4.0, s));
+    e = (h->nlaunch += 1, launch_restrict(L.d, Cl.d, L.dt_tmp, L.tmp, Cl.dt, Cl.fs, 4.0, s, nullptr, Cl.phi));
     if (l == 0) prof_end(h, s);
     if (e != cudaSuccess) return e;
   }
-  if ((e = cudaMemsetAsync(Cl.phi, 0, (size_t)Cl.d.size() * dt_size(Cl.dt), s)) != cudaSuccess) return e;
   if ((e = vcycle(h, H, l + 1, nu1, nu2, s)) != cudaSuccess) return e;
   if (l == 0) prof_begin(h, PC_PROLONG0, w.n * 2.0 * w.S + w.n / 8.0 * dt_size(Cl.dt), w.n * kProlongOps, w.fp64, s);
   e = (h->nlaunch += 1, launch_prolong(L.d, Cl.d, Cl.dt, Cl.phi, L.dt, L.phi, s, fc ? &h->st->hu[l & 7] : nullptr));
@@ -980,10 +981,9 @@ cudaError_t vcycle_compact(ps_ctx* h, Hier* H, const CompactLevels& C, int l, in
   if (e != cudaSuccess) return e;
   Level& Cl = H->lv[l + 1];
   if (l == 0) prof_begin(h, PC_RESTRICT0, n * S * 9.0 / 8.0, n * kRestrictOps, fp64, s);
-  e = (h->nlaunch += 1, launch_restrict(L.d, Cl.d, dt, r, Cl.dt, Cl.fs, 1.0, s));
+  e = (h->nlaunch += 1, launch_restrict(L.d, Cl.d, dt, r, Cl.dt, Cl.fs, 1.0, s, nullptr, Cl.phi));
   if (l == 0) prof_end(h, s);
   if (e != cudaSuccess) return e;
-  if ((e = cudaMemsetAsync(Cl.phi, 0, (size_t)Cl.d.size() * dt_size(Cl.dt), s)) != cudaSuccess) return e;
   if ((e = vcycle_compact(h, H, C, l + 1, nu1, nu2, s)) != cudaSuccess) return e;
   if (l == 0) prof_begin(h, PC_PROLONG0, n * S * 17.0 / 8.0, n * kProlongOps, fp64, s);
   e = (h->nlaunch += 1, launch_prolong(L.d, Cl.d, Cl.dt, Cl.phi, dt, u, s, fx ? hu : nullptr));

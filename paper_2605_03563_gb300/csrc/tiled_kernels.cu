@@ -446,7 +446,7 @@ struct RRGeom {
 template <typename TF, typename TC, int G, bool ISO, int TXC, int TYC>
 __global__ void __launch_bounds__(NT)
     k_resid_restrict(const __grid_constant__ CUtensorMap mP, const __grid_constant__ CUtensorMap mF,
-                     Dims fd, Dims cd, Coef<typename St<TF>::C> cf, TC* __restrict__ fsc,
+                     Dims fd, Dims cd, Coef<typename St<TF>::C> cf, TC* __restrict__ fsc, TC* __restrict__ zero,
                      typename St<TF>::C sc, int kc, int* __restrict__ fault) {
   using C = typename St<TF>::C;
   using S = St<TF>;
@@ -596,7 +596,9 @@ __global__ void __launch_bounds__(NT)
         const int I = I0 + li, J = J0 + lj;
         if (K >= K0 && I >= 1 && I < cd.nx && J >= 1 && J < cd.ny) {
           const C acc = (pm[e] + plane) + (C)2 * p0[e];
-          St<TC>::st(fsc + cd.at(I + G - 1, J + G - 1, K + G - 1), (typename St<TC>::C)(acc * sc));
+          const long long p = cd.at(I + G - 1, J + G - 1, K + G - 1);
+          St<TC>::st(fsc + p, (typename St<TC>::C)(acc * sc));
+          if (zero != nullptr) St<TC>::st(zero + p, (typename St<TC>::C)0);
         }
         pm[e] = plane;
       }
@@ -663,6 +665,7 @@ struct RrbMarch {
   bool hin;          // lane l < ND: the halo node (2 I0 - 1, row l + 1) is interior in x and y
   unsigned jok;      // bit j: coarse row Jw + j is interior; 0 if coarse column I is not
   float* o;          // coarse node (I, Jw, 0)
+  float* zo;         // the same node of the array to zero, or null
   long long cpy, cpz;
   bool ok;
   int wq, qm, q0, q1;
@@ -724,7 +727,10 @@ struct RrbMarch {
 #pragma unroll
       for (int j = 0; j < RC; j++) {
         const float pl = (rs[2 * j] + rs[2 * j + 2]) + 2.f * rs[2 * j + 1];
-        if (K >= K0 && K < K1 && ((jok >> j) & 1u)) o[j * cpy + K * cpz] = ((pm[j] + pl) + 2.f * p0[j]) * sc;
+        if (K >= K0 && K < K1 && ((jok >> j) & 1u)) {
+          o[j * cpy + K * cpz] = ((pm[j] + pl) + 2.f * p0[j]) * sc;
+          if (zo != nullptr) zo[j * cpy + K * cpz] = 0.f;
+        }
         pm[j] = pl;
       }
     }
@@ -737,7 +743,7 @@ struct RrbMarch {
 template <typename T, bool ISO, int RC, int NWC, int NS>
 __global__ void __launch_bounds__(32 * NWC, 2)
     k_resid_restrict_rb(const __grid_constant__ CUtensorMap mP, const __grid_constant__ CUtensorMap mF, Dims fd,
-                        Dims cd, Coef<float> cf, float* __restrict__ fsc, float sc, int kc,
+                        Dims cd, Coef<float> cf, float* __restrict__ fsc, float* __restrict__ zero, float sc, int kc,
                         int* __restrict__ fault) {
   using Gm = RrbGeom<T, RC, NWC, NS>;
   using M = RrbMarch<T, ISO, RC, NWC, NS>;
@@ -808,6 +814,7 @@ __global__ void __launch_bounds__(32 * NWC, 2)
   }
   m.jok = jok;
   m.o = fsc + cd.at(min(I, cd.ex - 1), min(Jw, cd.ey - 1), 0);
+  m.zo = zero == nullptr ? nullptr : zero + (m.o - fsc);
   m.cpy = cd.sy();
   m.cpz = cd.sz();
   m.ok = true;
@@ -855,7 +862,7 @@ __global__ void __launch_bounds__(32 * NWC, 2)
 
 template <typename T, bool ISO, int RC, int NWC, int NS>
 static cudaError_t rr_rb_t(const Dims& fd, const Dims& cd, const double h[3], const void* phi, const void* fs,
-                           void* fsc, double factor, int* fault, cudaStream_t s) {
+                           void* fsc, void* zero, double factor, int* fault, cudaStream_t s) {
   using Gm = RrbGeom<T, RC, NWC, NS>;
   auto kern = k_resid_restrict_rb<T, ISO, RC, NWC, NS>;
   static int blocks_per_sm = 0;
@@ -877,13 +884,13 @@ static cudaError_t rr_rb_t(const Dims& fd, const Dims& cd, const double h[3], co
   const int kc = (nk + nchunk - 1) / nchunk;
   const dim3 grid(gx, gy, (nk + kc - 1) / kc);
   const Coef<float> cf = make_coef<float>(fd, h, 2);
-  kern<<<grid, Gm::NTH, Gm::SMEM, s>>>(mP, mF, fd, cd, cf, (float*)fsc, (float)(factor / 64.0), kc, fault);
+  kern<<<grid, Gm::NTH, Gm::SMEM, s>>>(mP, mF, fd, cd, cf, (float*)fsc, (float*)zero, (float)(factor / 64.0), kc, fault);
   return cudaGetLastError();
 }
 
 template <typename TF, typename TC, int G, bool ISO>
 static cudaError_t rr_t(const Dims& fd, const Dims& cd, const double h[3], int order, const void* phi,
-                        const void* fs, void* fsc, double factor, int* fault, cudaStream_t s) {
+                        const void* fs, void* fsc, void* zero, double factor, int* fault, cudaStream_t s) {
   using C = typename St<TF>::C;
   constexpr int TXC = 32, TYC = sizeof(TF) == 8 ? 4 : 8;
   using Gm = RRGeom<TF, G, TXC, TYC>;
@@ -909,7 +916,7 @@ static cudaError_t rr_t(const Dims& fd, const Dims& cd, const double h[3], int o
   const int kc = (nk + nchunk - 1) / nchunk;
   const dim3 grid(gx, gy, (nk + kc - 1) / kc);
   Coef<C> cf = make_coef<C>(fd, h, order);
-  kern<<<grid, NT, smem, s>>>(mP, mF, fd, cd, cf, (TC*)fsc, (C)(factor / 64.0), kc, fault);
+  kern<<<grid, NT, smem, s>>>(mP, mF, fd, cd, cf, (TC*)fsc, (TC*)zero, (C)(factor / 64.0), kc, fault);
   return cudaGetLastError();
 }
 
@@ -921,40 +928,40 @@ int rr_default_tile(int) { return 3; }
 
 template <typename T, bool ISO>
 static cudaError_t rr_rb_tile(const Dims& fd, const Dims& cd, const double h[3], const void* phi, const void* fs,
-                              void* fsc, double factor, int* fault, int tile, cudaStream_t s) {
+                              void* fsc, void* zero, double factor, int* fault, int tile, cudaStream_t s) {
   switch (tile) {
-    case 1: return rr_rb_t<T, ISO, 4, 4, 5>(fd, cd, h, phi, fs, fsc, factor, fault, s);
-    case 2: return rr_rb_t<T, ISO, 2, 4, 5>(fd, cd, h, phi, fs, fsc, factor, fault, s);
-    case 3: return rr_rb_t<T, ISO, 3, 4, 5>(fd, cd, h, phi, fs, fsc, factor, fault, s);
+    case 1: return rr_rb_t<T, ISO, 4, 4, 5>(fd, cd, h, phi, fs, fsc, zero, factor, fault, s);
+    case 2: return rr_rb_t<T, ISO, 2, 4, 5>(fd, cd, h, phi, fs, fsc, zero, factor, fault, s);
+    case 3: return rr_rb_t<T, ISO, 3, 4, 5>(fd, cd, h, phi, fs, fsc, zero, factor, fault, s);
     default: return cudaErrorInvalidValue;
   }
 }
 
 template <typename TF, typename TC>
 static cudaError_t rr_dispatch(const Dims& fd, const Dims& cd, int order, const double h[3], const void* phi,
-                               const void* fs, void* fsc, double factor, int* fault, int tile, cudaStream_t s) {
+                               const void* fs, void* fsc, void* zero, double factor, int* fault, int tile, cudaStream_t s) {
   const bool iso = h[0] == h[1] && h[1] == h[2];
   if constexpr (!std::is_same<TF, double>::value && std::is_same<TC, float>::value) {
     if (order == 2) {
       if (tile == 0) tile = rr_default_tile(sizeof(TF) == 4 ? DT_F32 : DT_BF16);
-      return iso ? rr_rb_tile<TF, true>(fd, cd, h, phi, fs, fsc, factor, fault, tile, s)
-                 : rr_rb_tile<TF, false>(fd, cd, h, phi, fs, fsc, factor, fault, tile, s);
+      return iso ? rr_rb_tile<TF, true>(fd, cd, h, phi, fs, fsc, zero, factor, fault, tile, s)
+                 : rr_rb_tile<TF, false>(fd, cd, h, phi, fs, fsc, zero, factor, fault, tile, s);
     }
   }
   if (order == 2)
-    return iso ? rr_t<TF, TC, 1, true>(fd, cd, h, order, phi, fs, fsc, factor, fault, s)
-               : rr_t<TF, TC, 1, false>(fd, cd, h, order, phi, fs, fsc, factor, fault, s);
-  return iso ? rr_t<TF, TC, 2, true>(fd, cd, h, order, phi, fs, fsc, factor, fault, s)
-             : rr_t<TF, TC, 2, false>(fd, cd, h, order, phi, fs, fsc, factor, fault, s);
+    return iso ? rr_t<TF, TC, 1, true>(fd, cd, h, order, phi, fs, fsc, zero, factor, fault, s)
+               : rr_t<TF, TC, 1, false>(fd, cd, h, order, phi, fs, fsc, zero, factor, fault, s);
+  return iso ? rr_t<TF, TC, 2, true>(fd, cd, h, order, phi, fs, fsc, zero, factor, fault, s)
+             : rr_t<TF, TC, 2, false>(fd, cd, h, order, phi, fs, fsc, zero, factor, fault, s);
 }
 
 cudaError_t launch_resid_restrict(const Dims& fine, const Dims& coarse, int order, const double h[3], int dt_f,
                                   const void* phi, const void* fs, int dt_c, void* fs_c,
-                                  double factor, int* fault, cudaStream_t s, int tile) {
+                                  double factor, int* fault, cudaStream_t s, int tile, void* zero) {
   if (tile < 0 || tile > kRrTiles) return cudaErrorInvalidValue;
-  if (dt_f == DT_F64 && dt_c == DT_F64) return rr_dispatch<double, double>(fine, coarse, order, h, phi, fs, fs_c, factor, fault, tile, s);
-  if (dt_f == DT_F32 && dt_c == DT_F32) return rr_dispatch<float, float>(fine, coarse, order, h, phi, fs, fs_c, factor, fault, tile, s);
-  if (dt_f == DT_BF16 && dt_c == DT_F32) return rr_dispatch<__nv_bfloat16, float>(fine, coarse, order, h, phi, fs, fs_c, factor, fault, tile, s);
+  if (dt_f == DT_F64 && dt_c == DT_F64) return rr_dispatch<double, double>(fine, coarse, order, h, phi, fs, fs_c, zero, factor, fault, tile, s);
+  if (dt_f == DT_F32 && dt_c == DT_F32) return rr_dispatch<float, float>(fine, coarse, order, h, phi, fs, fs_c, zero, factor, fault, tile, s);
+  if (dt_f == DT_BF16 && dt_c == DT_F32) return rr_dispatch<__nv_bfloat16, float>(fine, coarse, order, h, phi, fs, fs_c, zero, factor, fault, tile, s);
   return cudaErrorNotSupported;
 }
 
