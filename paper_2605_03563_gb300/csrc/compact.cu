@@ -402,8 +402,8 @@ cudaError_t launch_c27_resid_dt(const Dims& d, const W27& A, const double* u, co
 // forms the value (three with a norm), instead of 12.5.  In every mode the value
 // is base + c T(in), stored as TR:
 //   C27_INIT   r = b - A u, sums of r^2 and of b^2 (which k_c27_shell completes to
-//              the reference norm);
-//   C27_NORM   r = b - A u, sum of r^2; *track takes the largest |u| read;
+//              the reference norm); *track takes the largest |u| read;
+//   C27_NORM   r = b - A u, sum of r^2; *track the same;
 //   C27_RESID  r = b - A u; *track the largest |r| written;
 //   C27_SPAI   u - omega M r (in = r, base and dst = u: a block writes the nodes
 //              whose base it has read); *track the largest |u| written.
@@ -420,7 +420,7 @@ __global__ void __launch_bounds__(256, 2)
              int nblocks) {
   if (MODE != C27_INIT && st->done) return;   // uniform
   struct Epi {
-    enum { TRACK = MODE == C27_NORM && sizeof(TR) == 8 };
+    enum { TRACK = (MODE == C27_INIT || MODE == C27_NORM) && sizeof(TR) == 8 };
     TR* dst;
     double s2, s0;
     unsigned hmax;
@@ -567,7 +567,8 @@ cudaError_t launch_c27_init(const Dims& d, int order, double h, const double* u,
     const FxOp op = fx_op(ops.resid);
     const cudaError_t e =
         dt_r == DT_F64
-            ? c27_fx_t<C27_INIT, double>(d, op, u, b, (double*)r, partials, st, &st->umax, &st->bmax, nullptr, nb, s)
+            // (the bound of the first V-cycle's passes; the refinement's comes from its first correction)
+            ? c27_fx_t<C27_INIT, double>(d, op, u, b, (double*)r, partials, st, &st->umax, &st->bmax, &st->unext, nb, s)
             : c27_fx_t<C27_INIT, float>(d, op, u, b, (float*)r, partials, st, &st->umax, &st->bmax, nullptr, nb, s);
     if (e != cudaSuccess) return e;
     k_c27_shell<<<C27_SHELL_BLOCKS, 256, 0, s>>>(d, w, u, b, partials + 4 * *nb);
