@@ -676,6 +676,31 @@ __device__ __forceinline__ void bicg_replace_logic(DevState* st, const double (&
   }
 }
 
+// What the scalar steps change, from a block's copy S into the state.  The rest
+// stays as it is, above all the counter of the grid barrier: other blocks may
+// still poll it when the first one leaves its last barrier (the next launch's
+// k_set_budget zeroes it).
+__device__ __forceinline__ void bicg_store(DevState* __restrict__ st, const DevState& S) {
+  st->alpha = S.alpha;
+  st->beta = S.beta;
+  st->omega = S.omega;
+  st->rho = S.rho;
+  st->ts = S.ts;
+  st->tt = S.tt;
+  st->rr = S.rr;
+  st->rel = S.rel;
+  st->rmax = S.rmax;
+  st->iter = S.iter;
+  st->iter_repl = S.iter_repl;
+  st->inner_cycles = S.inner_cycles;
+  st->inner_cap = S.inner_cap;
+  st->broke = S.broke;
+  st->restart = S.restart;
+  st->replace = S.replace;
+  st->discard = S.discard;
+  st->done = S.done;
+}
+
 __global__ void k_bicg_replace_finish(const double* __restrict__ partials, int nblk,
                                       DevState* __restrict__ st, unsigned long long cond, int chunk) {
   __shared__ double sh[64];
@@ -1066,10 +1091,9 @@ __global__ void __launch_bounds__(BS_WARPS * 32)
   if (blockIdx.x == 0 && tid == 0) {
     if (!ok) {
       S.done = DONE_FAULT;
-      S.fault = 1;
+      st->fault = 1;
     }
-    S.gbar = 0u;
-    *st = S;
+    bicg_store(st, S);
   }
 }
 
