@@ -494,6 +494,18 @@ ps_status ps_probe_fp64(int kind, int blocks, int iters, double* out_dev, double
  * for a NULL out_dev, PS_ERR_CUDA if the launch or copy fails. */
 ps_status ps_probe_bounded_wait(int first_wait, long long* out_dev, double* waited_ms_host, void* stream);
 
+/* The same check of the grid barrier of the one-launch iterations: `blocks`
+ * blocks pass `rounds` barriers over an arrival counter that starts at `start`,
+ * each looking behind every barrier whether all others have arrived.  missing
+ * != 0: one more arrival is waited for than comes, so the first wait runs out
+ * after its 2 s in every block.  Synchronises `stream`; *waited_ms_host (may be
+ * NULL) = the longest wait.  out_dev: caller-owned device scratch of
+ * 5 + blocks int32.  Returns PS_OK, PS_ERR_TIMEOUT when a wait ran out and
+ * was reported, PS_ERR_INVALID_ARG for blocks outside 1..SMs of the device,
+ * rounds outside 1..1000 or a NULL out_dev, else PS_ERR_CUDA. */
+ps_status ps_probe_grid_barrier(int blocks, int rounds, unsigned start, int missing, int* out_dev,
+                                double* waited_ms_host, void* stream);
+
 #ifdef __cplusplus
 }
 #endif

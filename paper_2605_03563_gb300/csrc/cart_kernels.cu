@@ -1870,7 +1870,7 @@ __global__ void __launch_bounds__(NT)
   bool ok = true;
   // the boundary's red nodes of the second red array
   for (long long u = t0; u < d.size(); u += nthr) __stcg(alt + u, phi[u]);
-  grid_barrier(&st->gbar, target += gridDim.x, ok);
+  grid_barrier(&st->gbar, target += gridDim.x, &st->fault, ok);
   // x_GS of node p from the other colour's array (L2 loads: other blocks write it)
   auto gs = [&](const double* nb, long long p, double f) -> double {
     auto ld = [&](long long q) { return __ldcg(nb + q); };
@@ -1908,7 +1908,7 @@ __global__ void __launch_bounds__(NT)
       s2 = block_sum_warp0(s2, threadIdx.x, NT, sh);
       if (threadIdx.x == 0) __stcg(partials + blockIdx.x, s2);
     }
-    grid_barrier(&st->gbar, target += gridDim.x, ok);
+    grid_barrier(&st->gbar, target += gridDim.x, &st->fault, ok);
     if (!ok) break;
     if (!first) {
       double a = 0.0;
@@ -1941,7 +1941,7 @@ __global__ void __launch_bounds__(NT)
     double* c = cur;
     cur = nxt;
     nxt = c;
-    grid_barrier(&st->gbar, target += gridDim.x, ok);   // also keeps the partials until all blocks have read them
+    grid_barrier(&st->gbar, target += gridDim.x, &st->fault, ok);   // also keeps the partials until all blocks have read them
   }
   if (ok && cur != phi)   // red values of the state into phi
     for (int t = t0; t < npair; t += nthr) {
@@ -1954,7 +1954,6 @@ __global__ void __launch_bounds__(NT)
     st->rr = rr;
     st->rel = sqrt(rr) / st->ref;
     st->done = ok ? done : DONE_FAULT;
-    if (!ok) st->fault = 1;
   }
 }
 

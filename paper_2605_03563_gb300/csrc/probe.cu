@@ -10,6 +10,7 @@
 // warps per SM to hide the pipe's latency, and writes one value per block so
 // that no chain can be removed.
 #include "ps_common.cuh"
+#include "stencil.cuh"
 #include "tma.cuh"
 
 namespace ps {
@@ -71,10 +72,61 @@ __global__ void k_probe_bounded_wait(int first_wait, long long* out) {
   }
 }
 
+// `rounds` grid barriers of the one-launch iterations over a counter that starts
+// at `start`.  Before each a block publishes its round, after it thread b looks at
+// block b's: out[2] counts those behind.  missing != 0: the targets count one
+// arrival too many, the first wait runs out and every block leaves.
+// out: counter, fault flag, blocks seen behind, blocks whose wait ran out,
+// longest wait in microseconds, then a round per block.
+__global__ void __launch_bounds__(kThreads) k_probe_grid_barrier(int rounds, unsigned start, int missing, int* out) {
+  bool ok = true;
+  unsigned target = start + (missing ? 1u : 0u);
+  for (int r = 1; r <= rounds && ok; r++) {
+    if (threadIdx.x == 0) __stcg(out + 5 + blockIdx.x, r);
+    const unsigned long long t0 = global_ns();
+    grid_barrier((unsigned*)out, target += gridDim.x, out + 1, ok);
+    if (threadIdx.x == 0) atomicMax(out + 4, (int)((global_ns() - t0) / 1000));
+    for (int b = threadIdx.x; ok && b < (int)gridDim.x; b += kThreads)
+      if (__ldcg(out + 5 + b) < r) atomicAdd(out + 2, 1);
+  }
+  if (!ok && threadIdx.x == 0) atomicAdd(out + 3, 1);
+}
+
 }  // namespace
 }  // namespace ps
 
 using namespace ps;
+
+extern "C" ps_status ps_probe_grid_barrier(int blocks, int rounds, unsigned start, int missing, int* out_dev,
+                                           double* waited_ms_host, void* stream) {
+  if (out_dev == nullptr || blocks < 1 || blocks > device_sm_count() || rounds < 1 || rounds > 1000) {
+    set_error("ps_probe_grid_barrier: out_dev must be non-NULL, blocks 1 to the device's SMs, rounds 1 to 1000");
+    return PS_ERR_INVALID_ARG;
+  }
+  cudaStream_t s = static_cast<cudaStream_t>(stream);
+  int h[5] = {(int)start, 0, 0, 0, 0};
+  cudaError_t e = cudaMemsetAsync(out_dev, 0, (5 + (size_t)blocks) * sizeof(int), s);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(out_dev, h, sizeof(int), cudaMemcpyHostToDevice, s);
+  void* args[] = {&rounds, &start, &missing, &out_dev};
+  if (e == cudaSuccess)
+    e = cudaLaunchCooperativeKernel((const void*)k_probe_grid_barrier, dim3(blocks), dim3(kThreads), args, 0, s);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(h, out_dev, sizeof(h), cudaMemcpyDeviceToHost, s);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+  if (e != cudaSuccess) {
+    set_error("ps_probe_grid_barrier: %s", cudaGetErrorString(e));
+    return PS_ERR_CUDA;
+  }
+  if (waited_ms_host) *waited_ms_host = h[4] * 1e-3;
+  if (h[3] > 0 && h[1] != 0) {
+    set_error("ps_probe_grid_barrier: the barrier's wait ran out in %d of %d blocks", h[3], blocks);
+    return PS_ERR_TIMEOUT;
+  }
+  if (h[1] != 0 || h[2] != 0 || h[3] != 0) {
+    set_error("ps_probe_grid_barrier: fault %d, %d blocks seen behind, %d waits ran out", h[1], h[2], h[3]);
+    return PS_ERR_CUDA;
+  }
+  return PS_OK;
+}
 
 extern "C" ps_status ps_probe_bounded_wait(int first_wait, long long* out_dev, double* waited_ms_host,
                                            void* stream) {

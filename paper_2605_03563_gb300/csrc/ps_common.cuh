@@ -322,7 +322,7 @@ struct DevState {
   int broke;          // alpha or omega broke down in this iteration
   int restart;        // the next direction update restarts rhat = p = r
   int replace;        // the true residual replaces the recurrence one this iteration
-  int fault;          // a tile kernel's TMA copy did not complete in time
+  int fault;          // a kernel's bounded wait (TMA copy, grid barrier) ran out: the result is invalid
   double replace_drop;     // BiCGSTAB: replace when ||r|| <= replace_drop * rmax
   int restart_on_replace;  // BiCGSTAB: restart rhat = p = r at every replacement
   int iter_repl;           // BiCGSTAB: iteration of the last replacement

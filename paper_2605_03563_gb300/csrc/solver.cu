@@ -1451,6 +1451,8 @@ ps_status poll_active(ps_ctx* h, int* done) {
   if (!h->act.plain_steps && h->hst->iter > it0)
     h->nlaunch += h->act.body_kernels * (h->hst->iter - it0);
   h->act.plain_steps = false;
+  // also where the kernel that reports the end went on without the faulty block
+  if (h->hst->fault) h->hst->done = DONE_FAULT;
   *done = h->hst->done != DONE_NO;
   return PS_OK;
 }
@@ -2034,7 +2036,7 @@ ps_status poisson_solve_end(ps_handle h, ps_info* info) {
   ps_status out = PS_OK;
   if (h->hst->done == DONE_MAXITER || h->hst->done == DONE_NO) out = PS_NOT_CONVERGED;
   else if (h->hst->done == DONE_DIVERGED) out = PS_DIVERGED;
-  else if (h->hst->done == DONE_FAULT) return fail(PS_ERR_TIMEOUT, "a tile kernel's TMA copy did not complete; the result is invalid");
+  else if (h->hst->done == DONE_FAULT) return fail(PS_ERR_TIMEOUT, "a kernel's bounded wait ran out (a TMA copy or a grid barrier did not complete); the result is invalid");
   if (out == PS_NOT_CONVERGED) fail(out, "not converged: relative residual %.3e after %d iterations", h->hst->rel, h->hst->iter);
   if (out == PS_DIVERGED) fail(out, "diverged: relative residual %.3e after %d iterations", h->hst->rel, h->hst->iter);
   fill_info(h, info, out, true);

@@ -865,7 +865,7 @@ __global__ void __launch_bounds__(BS_WARPS * 32)
   unsigned target = 0;
   bool ok = true;
   auto ld = [](const auto* a) { return __ldcg(a); };   // other SMs write the vectors
-  auto barrier = [&]() { grid_barrier(&st->gbar, target += gridDim.x, ok); };
+  auto barrier = [&]() { grid_barrier(&st->gbar, target += gridDim.x, &st->fault, ok); };
   // f(virtual warp, i, j, k0, k1, inside) over the warps of the vector kernels
   auto each = [&](auto f) {
     for (int q = w0; q < nblk * SBY; q += nw) {
@@ -1089,10 +1089,7 @@ __global__ void __launch_bounds__(BS_WARPS * 32)
     barrier();
   }
   if (blockIdx.x == 0 && tid == 0) {
-    if (!ok) {
-      S.done = DONE_FAULT;
-      st->fault = 1;
-    }
+    if (!ok) S.done = DONE_FAULT;
     bicg_store(st, S);
   }
 }

@@ -162,9 +162,10 @@ __device__ __forceinline__ double recip(double x) {
 // *bar counts arrivals, target = blocks times the barriers passed so far.  What
 // any block wrote before it is visible after it (to loads that go to L2: the L1
 // caches are not coherent, so data that other blocks write are read with
-// __ldcg).  The wait is bounded (2 s): past it ok turns false in thread 0's
-// block, which then stops, and so do the others in turn.
-__device__ __forceinline__ void grid_barrier(unsigned* bar, unsigned target, bool& ok) {
+// __ldcg).  The wait is bounded (2 s): past it ok turns false in the block, which
+// sets *fault (the result is invalid even if the other blocks went on) and then
+// stops, and so do the others in turn.
+__device__ __forceinline__ void grid_barrier(unsigned* bar, unsigned target, int* fault, bool& ok) {
   __shared__ int alive;
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -181,6 +182,7 @@ __device__ __forceinline__ void grid_barrier(unsigned* bar, unsigned target, boo
         if (t0 == 0) t0 = t;
         if (t - t0 > 2000000000ull) {
           good = 0;
+          atomicExch(fault, 1);
           break;
         }
       }

@@ -143,3 +143,17 @@ def probe_bounded_wait(first_wait, out, stream=None):
     ms = C.c_double()
     st = lib().ps_probe_bounded_wait(1 if first_wait else 0, _p(out), C.byref(ms), _s(stream))
     return st, ms.value
+
+
+def probe_grid_barrier(blocks, rounds, out, start=0, missing=False, stream=None):
+    """Pass `rounds` grid barriers of the one-launch iterations with `blocks`
+    blocks over a counter that starts at `start` (missing: one arrival short,
+    the wait runs out).  out: int32 CUDA tensor of at least 5 + blocks
+    elements.  Returns (status, longest wait in ms)."""
+    import torch
+    if out.dtype != torch.int32 or out.numel() < 5 + blocks:
+        raise ValueError("out must be int32 with at least 5 + blocks elements")
+    ms = C.c_double()
+    st = lib().ps_probe_grid_barrier(int(blocks), int(rounds), int(start), 1 if missing else 0, _p(out), C.byref(ms),
+                                     _s(stream))
+    return st, ms.value

@@ -52,3 +52,11 @@ def test_the_end_of_a_launch_stores_what_the_scalar_steps_change():
         changed |= set(re.findall(r"st->(\w+)\s*[-+*]?=(?!=)", _body(code, f)))
     stored = set(re.findall(r"st->(\w+)\s*=(?!=)", _body(code, "bicg_store")))
     assert changed and stored == changed, stored ^ changed
+
+
+def test_a_wait_that_ran_out_is_reported():
+    """Any block whose wait runs out sets the solve's fault flag, and the host
+    honours the flag whatever the kernel's first block reports."""
+    code = _code()
+    assert re.search(r"atomicExch\(\s*fault\s*,\s*1\s*\)", _body(code["stencil.cuh"], "grid_barrier"))
+    assert re.search(r"->fault\s*\)\s*\w[\w>.-]*done\s*=\s*DONE_FAULT", _body(code["solver.cu"], "poll_active"))
