@@ -162,9 +162,10 @@ __device__ __forceinline__ double recip(double x) {
 // *bar counts arrivals, target = blocks times the barriers passed so far.  What
 // any block wrote before it is visible after it (to loads that go to L2: the L1
 // caches are not coherent, so data that other blocks write are read with
-// __ldcg).  The wait is bounded (2 s): past it ok turns false in the block, which
-// sets *fault (the result is invalid even if the other blocks went on) and then
-// stops, and so do the others in turn.
+// __ldcg).  The count may pass 2^32 (very long launches): it is compared by its
+// distance from the target.  The wait is bounded (2 s): past it ok turns false
+// in the block, which sets *fault (the result is invalid even if the other
+// blocks went on) and then stops, and so do the others in turn.
 __device__ __forceinline__ void grid_barrier(unsigned* bar, unsigned target, int* fault, bool& ok) {
   __shared__ int alive;
   __syncthreads();
@@ -175,7 +176,7 @@ __device__ __forceinline__ void grid_barrier(unsigned* bar, unsigned target, int
     int good = 1;
     for (;;) {
       asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(bar) : "memory");
-      if (v >= target) break;
+      if ((int)(v - target) >= 0) break;
       if ((++spins & 255u) == 0) {
         unsigned long long t;
         asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));

@@ -1,13 +1,14 @@
 """The grid barrier of the one-launch iterations: every block sees all others'
-writes behind it; a barrier that an arrival is missing from is given up after its
-limit by every block, sets the fault flag and leaves the context usable."""
+writes behind it, also where the arrival counter passes 2^32; a barrier that
+an arrival is missing from is given up after its limit by every block, sets the
+fault flag and leaves the context usable."""
 import pytest
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("start", [0, 12345])
+@pytest.mark.parametrize("start", [0, 2 ** 32 - 1000, 2 ** 31 - 50])
 @pytest.mark.parametrize("blocks", [1, 7, 0])
 def test_blocks_stay_in_step(blocks, start):
     from paper_2605_03563_gb300 import capi, ops
