@@ -229,17 +229,23 @@ __global__ void __launch_bounds__(BX* BY)
 // from a zero guess the initial residual f - A phi0 is the reference vector,
 // and the initial residual pass takes the reference norm instead.  The largest
 // |phi| of the interior and of the boundary nodes (high words) go to st->umax
-// and st->bmax, which set the unit of the fixed-point residual passes.
+// and st->bmax, which set the unit of the fixed-point residual passes.  A
+// boundary node counts if the operator reads it, that is if at most `reach` of its
+// coordinates lie outside the interior (1: a cross, 2: edges of the 27-point box
+// too, 3: its corners): what a program leaves on the others must not coarsen
+// the unit.  Infinities and NaN count anywhere, so that a 27-point pass forms its
+// products with zero weights in FP64.
 __global__ void __launch_bounds__(256)
     k_copy_guess(Dims dd, Dims sd, const double* __restrict__ src, double* __restrict__ dst,
-                 DevState* __restrict__ st) {
+                 DevState* __restrict__ st, int reach) {
   const long long rows = (long long)sd.ey * sd.ez;
   const long long row = blockIdx.x * 8LL + (threadIdx.x >> 5);
   int nz = 0;
   unsigned hi = 0u, hb = 0u;
   if (row < rows) {
     const int j = (int)(row % sd.ey), k = (int)(row / sd.ey), g = sd.g;
-    const bool inrow = j >= g && j < sd.ey - g && k >= g && k < sd.ez - g;
+    const bool inj = j >= g && j < sd.ey - g, ink = k >= g && k < sd.ez - g, inrow = inj && ink;
+    const int out = (inj ? 0 : 1) + (ink ? 0 : 1);
     const double* a = src + row * sd.px;
     double* b = dst + row * dd.px;
 #pragma unroll 4
@@ -247,10 +253,11 @@ __global__ void __launch_bounds__(256)
       const double v = a[i];
       b[i] = v;
       const unsigned h = (unsigned)__double2hiint(v) & 0x7fffffffu;
-      if (inrow && i >= g && i < sd.ex - g) {
+      const bool ini = i >= g && i < sd.ex - g;
+      if (inrow && ini) {
         if (((unsigned long long)__double_as_longlong(v) << 1) != 0ull) nz = 1;
         hi = max(hi, h);
-      } else {
+      } else if (out + (ini ? 0 : 1) <= reach || h >= 0x7ff00000u) {
         hb = max(hb, h);
       }
     }
@@ -260,12 +267,12 @@ __global__ void __launch_bounds__(256)
   if (__syncthreads_or(nz) && threadIdx.x == 0) st->guess_nonzero = 1;
 }
 
-cudaError_t launch_copy_guess(const Dims& dd, const Dims& sd, const double* src, double* dst, DevState* st,
+cudaError_t launch_copy_guess(const Dims& dd, const Dims& sd, const double* src, double* dst, DevState* st, int reach,
                               cudaStream_t s) {
   if (dd.ex != sd.ex || dd.ey != sd.ey || dd.ez != sd.ez || dd.g != sd.g || dd.px < sd.px)
     return cudaErrorInvalidValue;
   const long long rows = (long long)sd.ey * sd.ez;
-  k_copy_guess<<<(unsigned)((rows + 7) / 8), 256, 0, s>>>(dd, sd, src, dst, st);
+  k_copy_guess<<<(unsigned)((rows + 7) / 8), 256, 0, s>>>(dd, sd, src, dst, st, reach);
   return cudaGetLastError();
 }
 

@@ -84,8 +84,10 @@ cudaError_t launch_restore_colour0(const Dims& d, double* phi, const double* sav
                                    cudaStream_t s);
 
 // Set-up copy of the initial guess (same logical extents, dst pitch >= src
-// pitch) that sets st->guess_nonzero when an interior node is nonzero.
-cudaError_t launch_copy_guess(const Dims& dd, const Dims& sd, const double* src, double* dst, DevState* st,
+// pitch) that sets st->guess_nonzero when an interior node is nonzero, and
+// st->umax, st->bmax; reach: most coordinates outside the interior of a node that
+// the operator reads.
+cudaError_t launch_copy_guess(const Dims& dd, const Dims& sd, const double* src, double* dst, DevState* st, int reach,
                               cudaStream_t s);
 
 // FP64 set-up pass: fs = factor * rho on interior nodes (rho in the layout du,

@@ -133,8 +133,9 @@ struct FxGeom {
 // One barrier a plane: it separates the writes of a work buffer from its reads
 // two planes earlier, and hands the stage of the previous plane back to the
 // copy engine.
-// Epi::TRACK: epi.hmax takes the high word of the largest |u| staged (the
-// tile's own nodes and their halo).
+// Epi::TRACK: epi.hmax takes the high word of the largest |u| of the interior nodes
+// staged (the tile's own and their neighbours; not the boundary's, some of which
+// no stencil reads).
 template <int KIND, typename W, typename Epi>
 __device__ __forceinline__ bool fx_march(const CUtensorMap& mU, const CUtensorMap& mB, const Dims& d, const FxOp& op,
                                          const FxScale& sc, int zc, unsigned char* smem, Epi& epi) {
@@ -172,6 +173,14 @@ __device__ __forceinline__ bool fx_march(const CUtensorMap& mU, const CUtensorMa
 #pragma unroll
   for (int r = 0; r < R; r++) in[r] = i0 + tx < G + d.ni() && jr + r < G + d.nj();
   long long at = d.at(i0 + tx, jr, k0);
+  unsigned inner = 0u;   // bit q: the thread's q-th staged node is interior in x and y
+  if constexpr (Epi::TRACK) {
+#pragma unroll
+    for (int q = 0; q < NLD; q++) {
+      const int el = tid + q * NT, x = i0 + el % WX, y = j0 + el / WX;   // + G
+      inner |= (unsigned)(x >= 2 * G && x < 2 * G + d.ni() && y >= 2 * G && y < 2 * G + d.nj()) << q;
+    }
+  }
   // in-plane groups of a staged plane: C centre; F the four faces; E the four
   // diagonals (27-point) or the four nodes at distance 2 (13-point)
   auto sums = [&](const W* b, W (&C)[R], W (&F)[R], W (&E)[R]) {
@@ -211,7 +220,8 @@ __device__ __forceinline__ bool fx_march(const CUtensorMap& mU, const CUtensorMa
         const double v = raw[tid + q * NT];
         if constexpr (FX) w[tid + q * NT] = fx_from(v, sc.eb);
         else w[tid + q * NT] = v;
-        if constexpr (Epi::TRACK) epi.hmax = max(epi.hmax, (unsigned)__double2hiint(v) & 0x7fffffffu);
+        if constexpr (Epi::TRACK)
+          if ((inner >> q & 1u) && z >= G && z < G + d.nk()) epi.hmax = max(epi.hmax, (unsigned)__double2hiint(v) & 0x7fffffffu);
       }
     __syncthreads();
     if (tid == 0 && ok && z > zl) {   // after a failed wait no new copy is issued

@@ -118,14 +118,17 @@ __device__ __forceinline__ bool fc_march(const CUtensorMap& mU, const CUtensorMa
   int wq = 0, cw = ND - 1;   // stage and work plane of the plane that arrived last
   unsigned wph = 0;
   const int jr = j0 + warp * R;   // array row of the warp's first row
-  // bit q: the thread's q-th staged node has colour 1 in the planes of even z (the
-  // colour-0 nodes may be written meanwhile; they are tracked as they are written)
-  unsigned black = 0u;
-  if constexpr (MODE == FC_LAG) {
+  // bit q: the thread's q-th staged node is interior in x and y (boundary nodes are
+  // bounded by themselves, and some are read by no stencil) / has colour 1 in the
+  // planes of even z (the colour-0 nodes may be written meanwhile; they are tracked
+  // as they are written)
+  unsigned inner = 0u, black = 0u;
+  if constexpr (MODE == FC_LAG || MODE == FC_NORM) {
 #pragma unroll
     for (int q = 0; q < NLD; q++) {
-      const int el = tid + q * NT;
-      black |= (unsigned)((i0 - G + el % WX + j0 - G + el / WX) & 1) << q;
+      const int el = tid + q * NT, x = i0 - G + el % WX, y = j0 - G + el / WX;
+      inner |= (unsigned)(x >= G && x < G + d.ni() && y >= G && y < G + d.nj()) << q;
+      black |= (unsigned)((x + y) & 1) << q;
     }
   }
   for (int z = zl; z <= zh; z++) {
@@ -152,7 +155,7 @@ __device__ __forceinline__ bool fc_march(const CUtensorMap& mU, const CUtensorMa
           const double v = raw[tid + q * NT];
           if constexpr (FX) w[tid + q * NT] = fx_from_wide<Gm::XC>(v, sc.eb);
           else w[tid + q * NT] = v;
-          if (MODE == FC_NORM || (MODE == FC_LAG && ((black >> q ^ z) & 1)))
+          if ((MODE == FC_NORM || (MODE == FC_LAG && ((black >> q ^ z) & 1))) && (inner >> q & 1u) && z >= G && z < G + d.nk())
             hmax = max(hmax, (unsigned)__double2hiint(v) & 0x7fffffffu);
         }
     }

@@ -7,7 +7,7 @@ namespace ps {
 enum { FC_SWEEP = 0, FC_LAG = 1, FC_RESID = 2, FC_NORM = 3, FC_OPEN = 4 };
 
 // High words of the largest |phi| as last tracked, of the boundary data and of
-// the largest |fs| (device); track (FC_LAG, FC_NORM; optional) takes the largest
+// the largest |fs| (device); track (FC_LAG, FC_NORM; optional) takes the largest interior
 // |phi| read.
 struct FcBounds {
   const unsigned *phi, *boundary, *fs;

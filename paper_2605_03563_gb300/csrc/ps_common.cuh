@@ -330,7 +330,7 @@ struct DevState {
   int discard;             // refinement form: the inner solve failed, drop its increments
   int inner_cap;           // refinement form: most iterations of the current inner solve
   unsigned umax;      // high word of max |phi| of the finest FP64 potential as last written (set-up copy, correction)
-  unsigned bmax;      // the same over its boundary nodes
+  unsigned bmax;      // the same over those of its boundary nodes that the operator reads
   unsigned unext;     // largest |phi| that an FP64 compact residual (initial or norm) read: umax of the next iteration
   // FP64 multigrid (fixed_sweeps.cu), high words: the largest |fs| of the finest
   // level, the largest |phi| at the start of this V-cycle and as read by the pass

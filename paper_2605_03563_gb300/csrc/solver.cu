@@ -642,9 +642,11 @@ ps_status ensure_partials(ps_ctx* h, int nblk) {
 
 // ------------------------------------------------------------------ Cartesian solves
 // Multipole boundary (t_mp), scaled right-hand side, state reset and reference
-// norm, all enqueued on s without a host round trip.
+// norm, all enqueued on s without a host round trip.  compact: order of the compact
+// scheme, 0 for the 7- and 13-point operators.
 ps_status cart_prepare(ps_ctx* h, const double* rho, double* phi, double tol, int max_iter,
-                       bool own_rhs, cudaStream_t s) {
+                       int compact, cudaStream_t s) {
+  const bool own_rhs = compact != 0;
   TRY(cudaEventRecord(h->ev[0], s));
   if (h->bc.outer == PS_BC_MULTIPOLE) {
     const double n = (double)h->d0.ni() * h->d0.nj() * h->d0.nk();
@@ -671,7 +673,7 @@ ps_status cart_prepare(ps_ctx* h, const double* rho, double* phi, double tol, in
     TRY((h->nlaunch += 1, launch_scale_rhs_ref(h->d0, h->du, h->order, h->h0, fscale, rho, phi, h->fs64,
                                                h->partials, h->st, s)));
   // iterate on the handle's own (pitched) copy of phi: captured loop graphs reference it
-  TRY((h->nlaunch += 1, launch_copy_guess(h->d0, h->du, phi, h->phi0, h->st, s)));
+  TRY((h->nlaunch += 1, launch_copy_guess(h->d0, h->du, phi, h->phi0, h->st, compact ? compact / 2 : 1, s)));
   if (own_rhs) return PS_OK;
   TRY((h->nlaunch += 1, launch_finish_norm(h->partials, cart_partials_count(h->d0), cf.d, 0, h->st, s)));
   return PS_OK;
@@ -1988,7 +1990,7 @@ ps_status poisson_solve_begin(ps_handle h, const double* rho_dev, double* phi_de
   if (h->sph) {
     r = begin_sph(h, rho_dev, phi_dev, tol, &o, s);
   } else {
-    const bool compact = o.method == PS_MG && o.compact_order != 0;
+    const int compact = o.method == PS_MG ? o.compact_order : 0;
     if ((r = cart_prepare(h, rho_dev, phi_dev, tol, o.max_iter, compact, s)) != PS_OK) return r;
     if (o.method == PS_MG && o.compact_order != 0)
       r = o.prec == PS_FP64 ? begin_mg_compact(h, rho_dev, &o, s) : begin_ir_compact(h, rho_dev, &o, s);
@@ -2190,7 +2192,7 @@ ps_status poisson_batch_add(ps_batch b, ps_handle h, const double* rho_dev, doub
   TRY(cudaStreamWaitEvent(s, h->ev_in, 0));
   h->nlaunch = 0;
   ps_status r;
-  if ((r = cart_prepare(h, rho_dev, phi_dev, tol, max_iter, false, s)) != PS_OK) return r;
+  if ((r = cart_prepare(h, rho_dev, phi_dev, tol, max_iter, 0, s)) != PS_OK) return r;
   Hier* H = b->prec == PS_FP64 ? &h->h64 : &h->hmx[0];
   if ((r = build_hier(h, b->prec == PS_FP64 ? 0 : 1, H)) != PS_OK) return r;
   if (b->prec == PS_FP64) {
