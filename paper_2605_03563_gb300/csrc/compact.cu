@@ -1040,17 +1040,23 @@ constexpr int RH_TX = 64, RH_R = 4, RH_TY = 16, RH_NT = 256, RH_WX = RH_TX + 4, 
 constexpr int RH_NEL = RH_WX * RH_WY, RH_NLD = (RH_NEL + RH_NT - 1) / RH_NT, RH_NS = 3;
 constexpr int RH_SMEM = (RH_NS + 2) * RH_NEL * 8;
 
-__global__ void __launch_bounds__(256) k_rho_max(const double* __restrict__ rho, long long n, DevState* __restrict__ st) {
-  const long long step = (long long)gridDim.x * 256;
+// The largest |rho| of the nodes that R_h reads, those with at most `reach` coordinates
+// on the boundary (fourth order 1, sixth order 2): what a program leaves on
+// the others must not coarsen the unit.  A warp per row.
+__global__ void __launch_bounds__(256)
+    k_rho_max(Dims du, const double* __restrict__ rho, int reach, DevState* __restrict__ st) {
+  const long long rows = (long long)du.ey * du.ez;
+  const int lane = threadIdx.x & 31;
   unsigned hm = 0u;
-  long long p = (long long)blockIdx.x * 256 + threadIdx.x;
-  for (; p + 3 * step < n; p += 4 * step) {
-    unsigned h[4];
-#pragma unroll
-    for (int q = 0; q < 4; q++) h[q] = (unsigned)__double2hiint(rho[p + q * step]) & 0x7fffffffu;
-    hm = max(hm, max(max(h[0], h[1]), max(h[2], h[3])));
+  for (long long row = blockIdx.x * 8LL + (threadIdx.x >> 5); row < rows; row += 8LL * gridDim.x) {
+    const int j = (int)(row % du.ey), k = (int)(row / du.ey);
+    const int out = (j == 0 || j == du.ey - 1 ? 1 : 0) + (k == 0 || k == du.ez - 1 ? 1 : 0);
+    const double* a = rho + row * du.px;
+    // the row's ends lie on one face more
+    const int i0 = out < reach ? 0 : 1, i1 = out > reach ? 0 : (out < reach ? du.ex : du.ex - 1);
+#pragma unroll 4
+    for (int i = i0 + lane; i < i1; i += 32) hm = max(hm, (unsigned)__double2hiint(a[i]) & 0x7fffffffu);
   }
-  for (; p < n; p += step) hm = max(hm, (unsigned)__double2hiint(rho[p]) & 0x7fffffffu);
   atomic_max_group(hm, &st->fmax);
 }
 
@@ -1244,7 +1250,7 @@ static cudaError_t rhs_fx_t(const Dims& d, const Dims& du, const double* rho, do
   int occ = 0, zc = 0;
   cudaError_t e = fx_occupancy(k_c27_rhs_fx<ORDER>, RH_SMEM, cached, &occ);
   if (e != cudaSuccess) return e;
-  k_rho_max<<<8 * device_sm_count(), 256, 0, s>>>(rho, du.size(), st);
+  k_rho_max<<<8 * device_sm_count(), 256, 0, s>>>(du, rho, ORDER == 6 ? 2 : 1, st);
   const dim3 grid = fx_chunks((d.ni() + RH_TX - 1) / RH_TX, (d.nj() + RH_TY - 1) / RH_TY, d.nk(), occ, 8, &zc);
   // fscale over the denominator, and what its rounding leaves (a rounded factor
   // alone would scale all of b)

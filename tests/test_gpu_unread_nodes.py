@@ -61,3 +61,27 @@ def test_guess(order, compact, prec, nu1, nu2, box):
         info, got = solve(a)
         assert info.iterations == ref.iterations
         assert np.max(np.abs(got - want)) <= (1e-10 if prec == "fp64" else 1e-8) * np.max(np.abs(want))
+
+
+@pytest.mark.parametrize("order,prec", [(4, "fp64"), (6, "fp64"), (6, "mixed_fp32")])
+def test_density(order, prec):
+    """The same for the density of a compact solve: R_h of fourth order reads the
+    centre and the faces, of sixth order the edges and the nodes at distance 2."""
+    import paper_2605_03563_gb300 as P
+    shape = tuple(n + 1 for n in N[::-1])
+    rng = np.random.Generator(np.random.PCG64(5))
+    rho = np.where(rng.random(shape) < 0.3, 1.0, 0.25)   # values that every unit in question holds exactly
+    unread = _outside(shape, 1) > (1 if order == 4 else 2)
+    rho[unread] = 0.0
+
+    def solve(a):
+        phi = torch.zeros(shape, dtype=torch.float64, device="cuda:0")
+        with P.CartesianSolver(N, hi=HI) as s:
+            info = s.solve(torch.from_numpy(a).to("cuda:0"), phi, tol=1e-8, max_iter=30, prec=prec, compact_order=order)
+        return info, phi.cpu().numpy()
+    ref, want = solve(rho)
+    assert ref.converged
+    a = rho.copy()
+    a[unread] = -1e30
+    info, got = solve(a)
+    assert info.iterations == ref.iterations and np.array_equal(got, want)
