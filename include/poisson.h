@@ -410,6 +410,13 @@ ps_status ps_op_residual_noalloc(const ps_grid* grid, int stencil_order, const d
                                  const double* f_dev, double* r_dev, double* norm2_host,
                                  void* stream);
 
+/* b = R_h (scale rho) on the interior nodes (Sec. 2.1.3): the right-hand side of
+ * the compact scheme of order 2, 4 or 6 on equal spacings, as its solves form
+ * it.  rho and b: FP64, node arrays with the boundary layer (stencil_order 2's
+ * layout); b's boundary is left alone. */
+ps_status ps_op_compact_rhs(const ps_grid* grid, int compact_order, double scale, const double* rho_dev,
+                            double* b_dev, void* stream);
+
 /* One multicolour SOR step in place (Sec. 2.1.1): colours (i+j+k) mod 2 for
  * order 2, mod 3 for order 4, ascending; phi += omega (phi_GS - phi). */
 ps_status ps_op_sweep(const ps_grid* grid, int stencil_order, int dtype, void* phi_dev,

@@ -1023,257 +1023,10 @@ __global__ void __launch_bounds__(CBX*(CBY / FRB))
   }
 }
 
-// R_h of the larger levels on the integer pipe (fixed.cuh).  R_h's weights are
-// integers over one denominator, (402, 40, 8, -3) / 720 of sixth and (6, 1) / 12 of
-// fourth order, so a node is an exact integer sum, converted once: two FP64
-// instructions instead of 19 (12).  Planes of rho, whose caller's rows have any
-// alignment, come through a ring of 8-byte asynchronous copies; each thread turns
-// the values that it copied into units in one of two work planes, forms the
-// in-plane groups of its R rows there, and adds them to the groups of the planes
-// around, kept in registers.  The nodes next to the boundary, whose +-2 offsets
-// leave the node array, are left to k_c27_rhs_shell.  The unit comes from a pass
-// over |rho| (k_rho_max).  Sixth order on 512^3: 4869 -> 2015 us
-// (2.1 GB, 315 at the copy rate), on 256^3 676 -> 334 (271 here, the rest the
-// maximum and the shell); bound by the issue and latency of 64-bit integer
-// instructions at two blocks an SM (the groups of two planes take 72 registers).
-constexpr int RH_TX = 64, RH_R = 4, RH_TY = 16, RH_NT = 256, RH_WX = RH_TX + 4, RH_WY = RH_TY + 4;
-constexpr int RH_NEL = RH_WX * RH_WY, RH_NLD = (RH_NEL + RH_NT - 1) / RH_NT, RH_NS = 3;
-constexpr int RH_SMEM = (RH_NS + 2) * RH_NEL * 8;
-
-// The largest |rho| of the nodes that R_h reads, those with at most `reach` coordinates
-// on the boundary (fourth order 1, sixth order 2): what a program leaves on
-// the others must not coarsen the unit.  A warp per row.
-__global__ void __launch_bounds__(256)
-    k_rho_max(Dims du, const double* __restrict__ rho, int reach, DevState* __restrict__ st) {
-  const long long rows = (long long)du.ey * du.ez;
-  const int lane = threadIdx.x & 31;
-  unsigned hm = 0u;
-  for (long long row = blockIdx.x * 8LL + (threadIdx.x >> 5); row < rows; row += 8LL * gridDim.x) {
-    const int j = (int)(row % du.ey), k = (int)(row / du.ey);
-    const int out = (j == 0 || j == du.ey - 1 ? 1 : 0) + (k == 0 || k == du.ez - 1 ? 1 : 0);
-    const double* a = rho + row * du.px;
-    // the row's ends lie on one face more
-    const int i0 = out < reach ? 0 : 1, i1 = out > reach ? 0 : (out < reach ? du.ex : du.ex - 1);
-#pragma unroll 4
-    for (int i = i0 + lane; i < i1; i += 32) hm = max(hm, (unsigned)__double2hiint(a[i]) & 0x7fffffffu);
-  }
-  atomic_max_group(hm, &st->fmax);
-}
-
-// v in quarter units of fixed.cuh, so below 2^59 (sums of 12 are the largest
-// formed), rounded to nearest: R_h does not annihilate constants, so its rounding
-// counts against b itself.
-__device__ __forceinline__ long long rh_from(double v, int eb) {
-  const int hi = __double2hiint(v);
-  const int e = (hi >> 20) & 0x7ff;
-  const unsigned long long m =
-      ((unsigned long long)((hi & 0xfffff) | 0x100000) << 32 | (unsigned)__double2loint(v)) << 7;
-  long long r;
-  asm("shr.u64 %0, %1, %2;" : "=l"(r) : "l"(m), "r"(eb - e));   // shifts past 63 give 0
-  const long long s = (long long)(hi >> 31);
-  return (((r + 1) >> 1) ^ s) - s;
-}
-
-// w0 S0 + w1 S1 + w2 S2 - w3 S3 as a double: exact in two limbs, its leading 62 bits converted
-__device__ __forceinline__ double rh_sum(const int4& w, long long s0, long long s1, long long s2, long long s3) {
-  auto lo = [](int w, long long s) { return (long long)((unsigned long long)(unsigned)w * (unsigned)s); };
-  auto hi = [](int w, long long s) { return (long long)w * (int)(s >> 32); };
-  const long long L = (lo(w.x, s0) + lo(w.y, s1)) + (lo(w.z, s2) - lo(w.w, s3));
-  const long long H = ((hi(w.x, s0) + hi(w.y, s1)) + (hi(w.z, s2) - hi(w.w, s3))) + (L >> 32);
-  const bool big = (unsigned long long)(H + (1LL << 30)) >= (1ull << 31);
-  const unsigned low = (unsigned)L;
-  const long long t = big ? (long long)((unsigned long long)H << 21 | low >> 11) : (long long)((unsigned long long)H << 32 | low);
-  const double v = fx_double(t);
-  return __hiloint2double(__double2hiint(v) + (big ? 11 << 20 : 0), __double2loint(v));
-}
-__device__ __forceinline__ double rh_sum(const int4& w, double s0, double s1, double s2, double s3) {
-  return fma((double)w.x, s0, fma((double)w.y, s1, fma((double)w.z, s2, -(double)w.w * s3)));
-}
-
-template <int ORDER, typename W>
-__device__ __forceinline__ void rh_march(const Dims& d, const Dims& du, const double* __restrict__ rho, const int4& w,
-                                         double c, double cl, const FxScale& sc, int zc, double* __restrict__ b, double* smem) {
-  constexpr bool FX = !std::is_same<W, double>::value;
-  constexpr int R = RH_R, WX = RH_WX;
-  W* const work = reinterpret_cast<W*>(smem + RH_NS * RH_NEL);
-  const int tid = threadIdx.x, tx = tid & (RH_TX - 1), ty = tid / RH_TX;
-  const int i0 = blockIdx.x * RH_TX + 1, j0 = blockIdx.y * RH_TY + 1;
-  const int k0 = blockIdx.z * zc + 1, k1 = min(k0 + zc, d.nk() + 1);
-  if (FX) {
-    c *= 0.25 * sc.unit();
-    cl *= 0.25 * sc.unit();
-  }
-  // the thread's staged nodes: offset in the plane of rho, and whether they are in the node array
-  int off[RH_NLD];   // within 20 rows of up to 8193 nodes
-  unsigned in = 0u;
-#pragma unroll
-  for (int q = 0; q < RH_NLD; q++) {
-    const int el = tid + q * RH_NT, x = i0 - 2 + el % WX, y = j0 - 2 + el / WX;
-    off[q] = (el / WX) * (int)du.sy() + el % WX;
-    in |= (unsigned)(el < RH_NEL && x >= 0 && x <= du.nx && y >= 0 && y <= du.ny) << q;
-  }
-  const int zl = k0 - 2, zh = k1 + 1;
-  auto issue = [&](int z, int slot) {
-    const bool zin = z >= 0 && z <= du.nz && z <= zh;
-    const double* p = rho + du.at(i0 - 2, j0 - 2, zin ? z : 0);
-#pragma unroll
-    for (int q = 0; q < RH_NLD; q++)
-      if ((q + 1) * RH_NT <= RH_NEL || tid + q * RH_NT < RH_NEL) {
-        const bool v = zin && (in >> q & 1u);
-        asm volatile("cp.async.ca.shared.global [%0], [%1], 8, %2;" ::"r"(smem_u32(smem + slot * RH_NEL + tid + q * RH_NT)),
-                     "l"(v ? p + off[q] : rho), "r"(v ? 8 : 0)
-                     : "memory");
-      }
-    asm volatile("cp.async.commit_group;" ::: "memory");
-  };
-  issue(zl, 0);
-  issue(zl + 1, 1);
-  // plane z - 1 and z - 2: centre, and the groups of weights 1, 2, 3 so far
-  W p1[4][R], p2[4][R], F1[R];
-#pragma unroll
-  for (int r = 0; r < R; r++) {
-    F1[r] = 0;
-#pragma unroll
-    for (int g = 0; g < 4; g++) p1[g][r] = p2[g][r] = 0;
-  }
-  const int i = i0 + tx, jr = j0 + ty * R;
-  const bool own = i <= d.ni() && (ORDER == 4 || (i > 1 && i < d.ni()));
-  int slot = 0, wb = 0;
-  for (int z = zl; z <= zh; z++) {
-    issue(z + 2, slot == 0 ? 2 : slot - 1);
-    asm volatile("cp.async.wait_group 2;" ::: "memory");
-    {
-      const double* raw = smem + slot * RH_NEL;
-      W* wp = work + wb * RH_NEL;
-#pragma unroll
-      for (int q = 0; q < RH_NLD; q++)
-        if ((q + 1) * RH_NT <= RH_NEL || tid + q * RH_NT < RH_NEL) {
-          const double v = raw[tid + q * RH_NT];   // copied by this thread
-          if constexpr (FX) wp[tid + q * RH_NT] = rh_from(v, sc.eb);
-          else wp[tid + q * RH_NT] = v;
-        }
-    }
-    __syncthreads();
-    const W* s = work + wb * RH_NEL + (ty * R) * WX + tx + 2;   // row jr - 2, the thread's column
-    W m[R + 4], a[R + 4];
-#pragma unroll
-    for (int q = 0; q < R + 4; q++) m[q] = s[q * WX];
-#pragma unroll
-    for (int q = 1; q < R + 3; q++) a[q] = s[q * WX - 1] + s[q * WX + 1];
-    const int k = z - 2;
-    double* o = b + d.at(i, jr, k);
-#pragma unroll
-    for (int r = 0; r < R; r++) {
-      const W C = m[r + 2], F = a[r + 2] + (m[r + 1] + m[r + 3]);
-      if (k >= k0) {   // complete: the plane z holds its centres at +2
-        const int j = jr + r;
-        const double t = rh_sum(w, p2[0][r], p2[1][r], p2[2][r], p2[3][r] + C), v = fma(t, c, t * cl);
-        if (own && (ORDER == 4 ? j <= d.nj() : j > 1 && j < d.nj() && k > 1 && k < d.nk())) o[r * d.sy()] = v;
-      }
-      W S2 = 0, S3 = 0;
-      if (ORDER == 6) {
-        S2 = (a[r + 1] + a[r + 3]) + F1[r];
-        S3 = ((s[(r + 2) * WX - 2] + s[(r + 2) * WX + 2]) + (m[r] + m[r + 4])) + p2[0][r];
-      }
-      const W S1 = F + p1[0][r];
-      p2[0][r] = p1[0][r];
-      p2[1][r] = p1[1][r] + C;
-      p2[2][r] = ORDER == 6 ? p1[2][r] + F : (W)0;
-      p2[3][r] = ORDER == 6 ? p1[3][r] : (W)0;
-      p1[0][r] = C;
-      p1[1][r] = S1;
-      p1[2][r] = S2;
-      p1[3][r] = S3;
-      F1[r] = F;
-    }
-    slot = slot == RH_NS - 1 ? 0 : slot + 1;
-    wb ^= 1;
-  }
-  asm volatile("cp.async.wait_all;" ::: "memory");
-}
-
-template <int ORDER>
-__global__ void __launch_bounds__(RH_NT, 2)
-    k_c27_rhs_fx(Dims d, Dims du, const double* __restrict__ rho, int4 w, double c, double cl, int zc, double* __restrict__ b,
-                 const DevState* __restrict__ st) {
-  extern __shared__ __align__(16) double rh_smem[];
-  const FxScale sc(st->fmax);
-  if (sc.fx) rh_march<ORDER, long long>(d, du, rho, w, c, cl, sc, zc, b, rh_smem);
-  else rh_march<ORDER, double>(d, du, rho, w, c, cl, sc, zc, b, rh_smem);
-}
-
-// The nodes next to the boundary (sixth order): both sides of each axis in turn;
-// nodes on two sides are formed twice, alike.
-__global__ void __launch_bounds__(256)
-    k_c27_rhs_shell(Dims d, Dims du, const double* __restrict__ rho, Wts<double> W, double* __restrict__ b) {
-  const long long ni = d.ni(), nj = d.nj(), nk = d.nk();
-  const long long cz = ni * nj, cy = ni * nk, cx = nj * nk;
-  long long t = (long long)blockIdx.x * 256 + threadIdx.x;
-  if (t >= 2 * (cz + cy + cx)) return;
-  int i, j, k;
-  if (t < 2 * cz) {
-    k = t < cz ? 1 : (int)nk;
-    t %= cz;
-    i = (int)(t % ni) + 1;
-    j = (int)(t / ni) + 1;
-  } else if ((t -= 2 * cz) < 2 * cy) {
-    j = t < cy ? 1 : (int)nj;
-    t %= cy;
-    i = (int)(t % ni) + 1;
-    k = (int)(t / ni) + 1;
-  } else {
-    t -= 2 * cy;
-    i = t < cx ? 1 : (int)ni;
-    t %= cx;
-    j = (int)(t % nj) + 1;
-    k = (int)(t / nj) + 1;
-  }
-  auto at = [&](int x, int y, int z) { return rho[du.at(i + x, j + y, k + z)]; };
-  const double fa = ((at(-1, 0, 0) + at(1, 0, 0)) + (at(0, -1, 0) + at(0, 1, 0))) + (at(0, 0, -1) + at(0, 0, 1));
-  double ed = 0.0;
-#pragma unroll
-  for (int p = -1; p <= 1; p += 2)
-#pragma unroll
-    for (int q = -1; q <= 1; q += 2) ed += (at(p, q, 0) + at(p, 0, q)) + at(0, p, q);
-  const double ax = ((f_ext(du, rho, i - 2, j, k) + f_ext(du, rho, i + 2, j, k)) +
-                     (f_ext(du, rho, i, j - 2, k) + f_ext(du, rho, i, j + 2, k))) +
-                    (f_ext(du, rho, i, j, k - 2) + f_ext(du, rho, i, j, k + 2));
-  b[d.at(i, j, k)] = fma(W.w[0], at(0, 0, 0), fma(W.w[1], fa, fma(W.w[2], ed, W.w[3] * ax)));
-}
-
-bool c27_fx_rhs_level(const Dims& d) { return (long long)d.ni() * d.nj() * d.nk() >= FX_MIN_NODES; }
-
-template <int ORDER>
-static cudaError_t rhs_fx_t(const Dims& d, const Dims& du, const double* rho, double fscale, double* b, DevState* st,
-                            int* kernels, cudaStream_t s) {
-  static std::atomic<int> cached{0};
-  int occ = 0, zc = 0;
-  cudaError_t e = fx_occupancy(k_c27_rhs_fx<ORDER>, RH_SMEM, cached, &occ);
-  if (e != cudaSuccess) return e;
-  k_rho_max<<<8 * device_sm_count(), 256, 0, s>>>(du, rho, ORDER == 6 ? 2 : 1, st);
-  const dim3 grid = fx_chunks((d.ni() + RH_TX - 1) / RH_TX, (d.nj() + RH_TY - 1) / RH_TY, d.nk(), occ, 8, &zc);
-  // fscale over the denominator, and what its rounding leaves (a rounded factor
-  // alone would scale all of b)
-  const double den = ORDER == 6 ? 720.0 : 12.0, c = fscale / den, cl = -std::fma(c, den, -fscale) / den;
-  const int4 w = ORDER == 6 ? make_int4(402, 40, 8, 3) : make_int4(6, 1, 0, 0);
-  k_c27_rhs_fx<ORDER><<<grid, RH_NT, RH_SMEM, s>>>(d, du, rho, w, c, cl, zc, b, st);
-  *kernels = 2;
-  if (ORDER == 6) {
-    const long long n = 2LL * ((long long)d.ni() * d.nj() + (long long)d.ni() * d.nk() + (long long)d.nj() * d.nk());
-    k_c27_rhs_shell<<<(unsigned)((n + 255) / 256), 256, 0, s>>>(
-        d, du, rho, Wts<double>{{fscale * (67.0 / 120.0), fscale / 18.0, fscale / 90.0, -fscale / 240.0}}, b);
-    *kernels = 3;
-  }
-  return cudaGetLastError();
-}
-
 cudaError_t launch_c27_rhs(const Dims& d, const Dims& du, int order, const double* rho, double fscale,
-                           double* b, DevState* st, int* kernels, cudaStream_t s) {
+                           double* b, cudaStream_t s) {
   if (d.g != 1 || du.g != 1) return cudaErrorInvalidValue;
   if (order == 6 && (d.nx < 4 || d.ny < 4 || d.nz < 4)) return cudaErrorInvalidValue;
-  *kernels = 1;
-  if (order != 2 && c27_fx_rhs_level(d))
-    return order == 4 ? rhs_fx_t<4>(d, du, rho, fscale, b, st, kernels, s) : rhs_fx_t<6>(d, du, rho, fscale, b, st, kernels, s);
   const dim3 g = c27_grid(d), blk(CBX, CBY / FRB);
   // R_h weights per class (centre, faces, edges, +-2 offsets) times the source scale
   if (order == 2) {

@@ -72,12 +72,9 @@ cudaError_t launch_c27_outer(const Dims& d, int order, double h, const double* u
 // u -= omega M r on the interior (Eq. richardson for A = -L_h with M of Eq. Smoother)
 cudaError_t launch_c27_spai(const Dims& d, const W27& M, double omega, const double* r, double* u,
                             const DevState* st, cudaStream_t s);
-// Levels whose R_h (order 4, 6) runs on the integer pipe.
-bool c27_fx_rhs_level(const Dims& d);
 // b = R_h (fscale rho) on the interior; rho in the caller's dense layout du
-// (st: initialised, st->fmax takes the high word of the largest |rho|; *kernels: launches)
 cudaError_t launch_c27_rhs(const Dims& d, const Dims& du, int order, const double* rho, double fscale,
-                           double* b, DevState* st, int* kernels, cudaStream_t s);
+                           double* b, cudaStream_t s);
 // coarsest level: CG on -A u = -b from u = 0 in one CTA, to ||r|| <= tol ||b||
 // or as many iterations as unknowns; u receives the result
 cudaError_t launch_c27_coarse_cg(const Dims& d, const W27& A, const double* b, double* u, double tol,

@@ -1003,11 +1003,8 @@ cudaError_t vcycle_compact(ps_ctx* h, Hier* H, const CompactLevels& C, int l, in
 static cudaError_t compact_prologue(ps_ctx* h, int order, const double* rho, const double* phi,
                                     double* b, int dt_r, void* r, cudaStream_t s) {
   const double n = (double)h->d0.ni() * h->d0.nj() * h->d0.nk();
-  const bool fx = order != 2 && c27_fx_rhs_level(h->d0);   // on the integer pipe: two FP64 instructions a node
-  prof_begin(h, PC_RHS0, n * 16.0, n * (fx ? 2.0 : order == 6 ? 19.0 : 12.0), fx ? 0 : 1, s);
-  int nrhs = 0;
-  cudaError_t e = launch_c27_rhs(h->d0, h->du, order, rho, 4.0 * M_PI * h->bc.G, b, h->st, &nrhs, s);
-  h->nlaunch += nrhs;
+  prof_begin(h, PC_RHS0, n * 16.0, n * (order == 6 ? 19.0 : 12.0), 1, s);
+  cudaError_t e = (h->nlaunch += 1, launch_c27_rhs(h->d0, h->du, order, rho, 4.0 * M_PI * h->bc.G, b, s));
   prof_end(h, s);
   if (e != cudaSuccess) return e;
   prof_begin(h, PC_NORM0, n * (16.0 + (double)dt_size(dt_r)), n * 18.0, 1, s);
@@ -2390,6 +2387,25 @@ ps_status ps_op_residual(const ps_grid* grid, int order, int dtype, const void* 
   cudaFree(fs);
   cudaFree(part);
   if (e != cudaSuccess) return fail(PS_ERR_CUDA, "ps_op_residual: %s", cudaGetErrorString(e));
+  return PS_OK;
+}
+
+ps_status ps_op_compact_rhs(const ps_grid* grid, int compact_order, double scale, const double* rho, double* b,
+                            void* stream) {
+  Dims d;
+  double h[3];
+  ps_status s = op_dims(grid, 2, DT_F64, &d, h);
+  if (s != PS_OK) return s;
+  if (!rho || !b) return fail(PS_ERR_INVALID_ARG, "NULL buffer");
+  if (compact_order != 2 && compact_order != 4 && compact_order != 6)
+    return fail(PS_ERR_INVALID_ARG, "compact_order must be 2, 4 or 6 (got %d)", compact_order);
+  if (!(h[0] == h[1] && h[1] == h[2])) return fail(PS_ERR_INVALID_ARG, "the compact schemes need equal spacings");
+  if (compact_order == 6 && (d.nx < 4 || d.ny < 4 || d.nz < 4))
+    return fail(PS_ERR_INVALID_ARG, "the sixth-order right-hand side needs at least 4 intervals per axis");
+  cudaStream_t st = (cudaStream_t)stream;
+  cudaError_t e = launch_c27_rhs(d, d, compact_order, rho, scale, b, st);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(st);
+  if (e != cudaSuccess) return fail(PS_ERR_CUDA, "ps_op_compact_rhs: %s", cudaGetErrorString(e));
   return PS_OK;
 }
 

@@ -48,6 +48,16 @@ def sweep(n, order, phi, f, omega=1.0, lo=(0, 0, 0), hi=(1, 1, 1), stream=None):
           "ps_op_sweep")
 
 
+def compact_rhs(n, compact_order, rho, b, scale=1.0, lo=(0, 0, 0), hi=(1, 1, 1), stream=None):
+    """b = R_h (scale rho) of the compact scheme on the interior nodes (ps_op_compact_rhs)."""
+    import torch
+    if rho.dtype != torch.float64 or b.dtype != torch.float64 or rho.shape != b.shape:
+        raise ValueError("rho and b must be FP64 tensors of one shape")
+    g = capi.make_grid(n, lo, hi)
+    check(lib().ps_op_compact_rhs(C.byref(g), int(compact_order), float(scale), _p(rho), _p(b), _s(stream)),
+          "ps_op_compact_rhs")
+
+
 def restrict(n, order, r_fine, f_coarse, lo=(0, 0, 0), hi=(1, 1, 1), stream=None):
     g = capi.make_grid(n, lo, hi)
     check(lib().ps_op_restrict(C.byref(g), order, _dt(r_fine), _p(r_fine), _p(f_coarse), _s(stream)),

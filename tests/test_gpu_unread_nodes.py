@@ -70,7 +70,7 @@ def test_density(order, prec):
     import paper_2605_03563_gb300 as P
     shape = tuple(n + 1 for n in N[::-1])
     rng = np.random.Generator(np.random.PCG64(5))
-    rho = np.where(rng.random(shape) < 0.3, 1.0, 0.25)   # values that every unit in question holds exactly
+    rho = np.where(rng.random(shape) < 0.3, 1.0, 0.25)   # (exact in fixed point as well)
     unread = _outside(shape, 1) > (1 if order == 4 else 2)
     rho[unread] = 0.0
 
