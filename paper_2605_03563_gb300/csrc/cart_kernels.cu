@@ -649,7 +649,7 @@ __global__ void __launch_bounds__(256, 2)
   epi.dout = dout;
   epi.s2f = epi.mxf = 0.0f;
   epi.out = out;
-  fx_pass<KIND>(mU, mB, d, op, max(st->umax, st->bmax), zc, &st->fault, epi);
+  fx_pass<KIND>(mU, mB, d, op, max(st->umax, st->bmax), zc, st, epi);
   if (STORE) block_sum_max_scaled(epi.s2f, epi.mxf, epi.oscale, partials);
   else block_sum_max(epi.s2, 0.0, partials);
 }
@@ -1770,7 +1770,7 @@ __global__ void k_set_budget(DevState* st, int k) {
   st->gbar = 0u;
 }
 
-__global__ void k_init_state(DevState* st, double tol, int max_iter) {
+__global__ void k_init_state(DevState* st, double tol, int max_iter, double fx_noise) {
   DevState z;
   memset(&z, 0, sizeof(z));
   z.tol = tol;
@@ -1778,11 +1778,12 @@ __global__ void k_init_state(DevState* st, double tol, int max_iter) {
   z.scale_cur = 1.0;
   z.scale_next = 1.0;
   z.ref = 1.0;
+  z.fx_noise = fx_noise;
   *st = z;
 }
 
-cudaError_t launch_init_state(DevState* st, double tol, int max_iter, cudaStream_t s) {
-  k_init_state<<<1, 1, 0, s>>>(st, tol, max_iter);
+cudaError_t launch_init_state(DevState* st, double tol, int max_iter, cudaStream_t s, double fx_noise) {
+  k_init_state<<<1, 1, 0, s>>>(st, tol, max_iter, fx_noise);
   return cudaGetLastError();
 }
 

@@ -201,7 +201,8 @@ cudaError_t launch_set_budget(DevState* st, int k, cudaStream_t s);
 cudaError_t launch_add_pow2_f32(const float* e, long long n, int p, double* phi, cudaStream_t s);
 cudaError_t launch_pow2_to_f32(const double* x, long long n, int e, float* out, cudaStream_t s);
 // reset a solve's state on the device (no host round trip)
-cudaError_t launch_init_state(DevState* st, double tol, int max_iter, cudaStream_t s);
+// fx_noise: see DevState (0: none of the solve's passes are fixed-point)
+cudaError_t launch_init_state(DevState* st, double tol, int max_iter, cudaStream_t s, double fx_noise = 0.0);
 // first node of a loop graph: sets the while condition from the state
 cudaError_t launch_loop_gate(const DevState* st, unsigned long long cond, cudaStream_t s);
 

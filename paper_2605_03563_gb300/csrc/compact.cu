@@ -440,7 +440,7 @@ __global__ void __launch_bounds__(256, 2)
       }
     }
   } epi{dst, 0.0, 0.0, 0u};
-  fx_pass<FX27>(mU, mB, d, op, max(*h1, *h2), zc, &st->fault, epi);
+  fx_pass<FX27>(mU, mB, d, op, max(*h1, *h2), zc, st, epi);
   if ((Epi::TRACK || MODE == C27_RESID || MODE == C27_SPAI) && track != nullptr) atomic_max_group(epi.hmax, track);
   if constexpr (MODE == C27_INIT) block_partial2_nt<256>(epi.s2, epi.s0, partials, partials + 2 * nblocks);
   if constexpr (MODE == C27_NORM) block_partial_nt<256>(epi.s2, partials);

@@ -24,9 +24,16 @@
 // 32-bit multiply-adds), and the leading 62 bits converted.  What is lost is
 // the part of a value below a unit: against the roundings of an FP64 sum of
 // values of size |u| the error is smaller wherever |u| > H / 16, and over a field
-// whenever its r.m.s. is (potentials are far from that ratio).
-// Passes whose H is infinite, NaN or near the ends of the exponent range run
-// the same march in FP64.
+// whenever its r.m.s. is (potentials of extended sources are; a source of a few
+// nodes has its peak 100 r.m.s. high, and its faint parts keep that many fewer bits).
+//
+// The floor.  What the units leave in a residual bounds how far a solve can
+// converge, at 1e-14 relative for a point source on 256^3, where FP64 sums reach
+// 6e-16.  So the norm finisher compares each residual norm with the units' share
+// (fx_noise of the operator, times H) and, from FX_FLOOR times that share on, the passes
+// run the same march in FP64 (st->exact): no convergence factor is lost on the
+// way, and the accuracy that can be reached is that of the FP64 sums.  Passes whose H
+// is infinite, NaN or near the ends of the exponent range do so as well.
 #pragma once
 #include <atomic>
 #include <type_traits>
@@ -40,9 +47,9 @@ namespace ps {
 struct FxScale {
   int eb;
   bool fx;
-  __device__ __forceinline__ explicit FxScale(unsigned hmax) {
+  __device__ __forceinline__ explicit FxScale(unsigned hmax, int exact) {
     eb = (int)(hmax >> 20);
-    fx = hmax == 0u || (eb >= 200 && eb <= 0x7f0);
+    fx = !exact && (hmax == 0u || (eb >= 200 && eb <= 0x7f0));
     if (hmax == 0u) eb = 1023;   // every value is zero
   }
   // one unit as a binary64: 2^(eb - 1079)
@@ -75,7 +82,6 @@ __device__ __forceinline__ double fx_double(long long v) {
   const unsigned hi = (unsigned)(m >> 32) + ((unsigned)(1085 - lz) << 20);
   return a == 0 ? 0.0 : __hiloint2double((int)(hi | ((unsigned)s & 0x80000000u)), (int)(unsigned)m);
 }
-__device__ __forceinline__ double fx_double(double v) { return v; }
 
 // |x| < 2^(32 + b), from the high word
 __device__ __forceinline__ bool fx_below(long long x, int b) {
@@ -240,10 +246,13 @@ __device__ __forceinline__ bool fx_march(const CUtensorMap& mU, const CUtensorMa
   };
   const double cu = FX ? op.c * sc.unit() : op.c;
   // values of the thread's R nodes from their groups (27-point: centre, faces,
-  // edges, corners; others: second differences at distance 1 and 2)
+  // edges, corners; others: second differences at distance 1 and 2, in FP64 the sums)
   auto values = [&](const W (&c0)[R], const W (&g1)[R], const W (&g2)[R], const W (&g3)[R], const double (&f)[R],
                     double (&x)[R]) {
-    if constexpr (KIND == FX7) {
+    if constexpr (!FX && KIND != FX27) {   // x_GS - x, with x_GS as the FP64 sweeps form it
+#pragma unroll
+      for (int r = 0; r < R; r++) x[r] = fma(KIND == FX7 ? g1[r] : fma(16.0, g1[r], -g2[r]), cu, f[r]) - c0[r];
+    } else if constexpr (KIND == FX7) {
 #pragma unroll
       for (int r = 0; r < R; r++) x[r] = fma(fx_double(g1[r]), cu, f[r]);
     } else if constexpr (KIND == FX27 && FX) {
@@ -270,13 +279,11 @@ __device__ __forceinline__ bool fx_march(const CUtensorMap& mU, const CUtensorMa
         x[r] = fma(fma((double)op.w0, c0[r], fma((double)op.w1, g1[r], fma((double)op.w2, g2[r], op.w3 * g3[r]))), cu, f[r]);
     } else {
       bool fits = true;   // one test for all nodes, so that their chains run interleaved
-      if constexpr (FX) {
 #pragma unroll
-        for (int r = 0; r < R; r++) fits &= fx_below(g1[r], 26) && fx_below(g2[r], 29);   // 16 2^58 + 2^61 < 2^63
-      }
+      for (int r = 0; r < R; r++) fits &= fx_below(g1[r], 26) && fx_below(g2[r], 29);   // 16 2^58 + 2^61 < 2^63
       if (fits) {
 #pragma unroll
-        for (int r = 0; r < R; r++) x[r] = fma(fx_double(g1[r] * (W)16 - g2[r]), cu, f[r]);
+        for (int r = 0; r < R; r++) x[r] = fma(fx_double(g1[r] * 16 - g2[r]), cu, f[r]);
       } else {
 #pragma unroll
         for (int r = 0; r < R; r++) x[r] = fma(fx_double(g1[r]), 16.0 * cu, fma(fx_double(g2[r]), -cu, f[r]));
@@ -305,8 +312,8 @@ __device__ __forceinline__ bool fx_march(const CUtensorMap& mU, const CUtensorMa
         if constexpr (KIND == FX27) {
           g2[r] = Ec[r] + (Fm[r] + Fn[r]);
           g3[r] = Em[r] + En[r];
-        } else {
-          g1[r] -= Cc[r] * (W)6;
+        } else if constexpr (FX) {
+          g1[r] -= Cc[r] * 6;
         }
         Cm[r] = Cc[r];
         Fm[r] = Fc[r];
@@ -327,7 +334,8 @@ __device__ __forceinline__ bool fx_march(const CUtensorMap& mU, const CUtensorMa
       const double* b = arrive(Cn, Fn, En);
 #pragma unroll
       for (int r = 0; r < R; r++) {
-        const W c6 = Cc[r] * (W)6;
+        const W c6 = FX ? Cc[r] * (W)6 : (W)0;
+        c0[r] = Cc[r];
         g1[r] = Fc[r] + (C1m[r] + Cp[r]) - c6;
         g2[r] = Ec[r] + (C2m[r] + Cn[r]) - c6;
         C2m[r] = C1m[r];
@@ -345,15 +353,15 @@ __device__ __forceinline__ bool fx_march(const CUtensorMap& mU, const CUtensorMa
   return ok;
 }
 
-// The pass in the arithmetic that its scale allows.
+// The pass in the arithmetic that its scale (and the residual reached) allows.
 template <int KIND, typename Epi>
 __device__ __forceinline__ void fx_pass(const CUtensorMap& mU, const CUtensorMap& mB, const Dims& d, const FxOp& op,
-                                        unsigned hmax, int zc, int* fault, Epi& epi) {
+                                        unsigned hmax, int zc, DevState* __restrict__ st, Epi& epi) {
   extern __shared__ __align__(128) unsigned char fx_smem[];
-  const FxScale sc(hmax);
+  const FxScale sc(hmax, st->exact);
   const bool ok = sc.fx ? fx_march<KIND, long long>(mU, mB, d, op, sc, zc, fx_smem, epi)
                         : fx_march<KIND, double>(mU, mB, d, op, sc, zc, fx_smem, epi);
-  if (!ok) atomicExch(fault, 1);
+  if (!ok) atomicExch(&st->fault, 1);
 }
 
 // Levels a pass runs on: rows at 16-byte multiples (TMA), and tiles enough to

@@ -76,7 +76,6 @@ __device__ __forceinline__ double fx_sum13(long long a, long long b) {
   const double v = fx_double(t);
   return __hiloint2double(__double2hiint(v) + (big ? 11 << 20 : 0), __double2loint(v));
 }
-__device__ __forceinline__ double fx_sum13(double a, double b) { return fma(16.0, a, -b); }
 
 template <int KIND, bool ISO, int MODE, typename W, typename Gm>
 __device__ __forceinline__ bool fc_march(const CUtensorMap& mU, const CUtensorMap& mB, const Dims& d, double cx, double cy,
@@ -192,15 +191,26 @@ __device__ __forceinline__ bool fc_march(const CUtensorMap& mU, const CUtensorMa
         const double f = fb[(j - j0) * WX + G + NCOL * lane + m];
         const W C = P[a];
         const W ew = P[a + 1] + P[a - 1], ns = P[a + WX] + P[a - WX], ud = A1[a] + B1[a];
-        if constexpr (KIND == FX13) {
+        if constexpr (!FX) {   // residuals as x_GS - x: zero where a sweep would change nothing
+          const W S = (ew + ns) + ud;
+          if constexpr (KIND == FX13) {
+            const W S2 = ((P[a + 2] + P[a - 2]) + (P[a + 2 * WX] + P[a - 2 * WX])) + (A2[a] + B2[a]);
+            x[r][q] = fma(fma(16.0, S, -S2), cx, f);
+          } else if constexpr (ISO) {
+            x[r][q] = fma(S, cx, f);
+          } else {
+            x[r][q] = fma(ew, cx, fma(ns, cy, fma(ud, cz, f)));
+          }
+          dl[r][q] = x[r][q] - C;
+        } else if constexpr (KIND == FX13) {
           const W S1 = (ew + ns) + ud;
           const W S2 = ((P[a + 2] + P[a - 2]) + (P[a + 2 * WX] + P[a - 2 * WX])) + (A2[a] + B2[a]);
           if (MODE == FC_SWEEP || MODE == FC_OPEN || MODE == FC_LAG) x[r][q] = fma(fx_sum13(S1, S2), cx, f);
-          if (MODE != FC_SWEEP && MODE != FC_OPEN) dl[r][q] = fma(fx_sum13(S1 - C * (W)6, S2 - C * (W)6), cx, f);
+          if (MODE != FC_SWEEP && MODE != FC_OPEN) dl[r][q] = fma(fx_sum13(S1 - C * 6, S2 - C * 6), cx, f);
         } else if constexpr (ISO) {
           const W S = (ew + ns) + ud;
           if (MODE == FC_SWEEP || MODE == FC_OPEN || MODE == FC_LAG) x[r][q] = fma(fx_double(S), cx, f);
-          if (MODE != FC_SWEEP && MODE != FC_OPEN) dl[r][q] = fma(fx_double(S - C * (W)6), cx, f);
+          if (MODE != FC_SWEEP && MODE != FC_OPEN) dl[r][q] = fma(fx_double(S - C * 6), cx, f);
         } else {
           if (MODE == FC_SWEEP || MODE == FC_OPEN || MODE == FC_LAG)
             x[r][q] = fma(fx_double(ew), cx, fma(fx_double(ns), cy, fma(fx_double(ud), cz, f)));
@@ -245,7 +255,8 @@ __global__ void __launch_bounds__(256, 227 * 1024 / (Gm::SMEM + 1024) > 4 ? 4 : 
   extern __shared__ __align__(128) unsigned char fc_smem[];
   if ((MODE == FC_LAG || MODE == FC_OPEN) && st->done) return;   // uniform over the grid
   if (MODE == FC_OPEN && block_linear_id() == 0 && threadIdx.x == 0) st->lag_pending = 1;
-  const FxScale sc(max(*h1, max(*h2, *h3)));
+  // the pass that opens a step forms the values of the lagged pass again, in its arithmetic
+  const FxScale sc(max(*h1, max(*h2, *h3)), MODE == FC_OPEN ? st->lexact : st->exact);
   double s2 = 0.0;
   unsigned hmax = 0u;
   const bool ok =

@@ -336,6 +336,11 @@ struct DevState {
   // level, the largest |phi| at the start of this V-cycle and as read by the pass
   // that ends it, and the bound the last lagged pass used
   unsigned fmax, vmax, vnext, lmax;
+  // fixed-point passes: residual norm that one unit per value leaves when the
+  // largest value is 1; the residual is near that share, so the passes run in FP64;
+  // the same as the last lagged pass had it
+  double fx_noise;
+  int exact, lexact;
   // FP64 multigrid: largest |u| written on a level by the prolongation (compact:
   // and by the smoother) and largest |r| (right-hand side; compact: residual)
   // written on it in this V-cycle (high words; see fixed.cuh)

@@ -640,6 +640,27 @@ ps_status ensure_partials(ps_ctx* h, int nblk) {
   return PS_OK;
 }
 
+// Residual norm left by the units of the fixed-point passes when the largest value
+// is 1 (DevState::fx_noise): each value is off by a uniform error of one unit,
+// 2^-56 (13-point sweeps 2^-55), with standard deviation 1 / sqrt(12) units, and a
+// node adds its neighbours' and its own with the operator's weights.
+double fx_noise(const ps_ctx* h, int compact) {
+  const double n = (double)h->d0.ni() * h->d0.nj() * h->d0.nk();
+  double w2 = 0.0, c = 0.0, unit = std::ldexp(1.0, -56);
+  if (compact) {
+    const W27 a = compact_lhs(compact, h->h0[0]);
+    w2 = a.w[0] * a.w[0] + 6.0 * a.w[1] * a.w[1] + 12.0 * a.w[2] * a.w[2] + 8.0 * a.w[3] * a.w[3];
+  } else {
+    for (int a = 0; a < 3; a++) {
+      const double q = 1.0 / (h->h0[a] * h->h0[a]);
+      w2 += h->order == 2 ? 2.0 * q * q : 2.0 * (256.0 + 1.0) / 144.0 * q * q;
+      c += (h->order == 2 ? 2.0 : 30.0 / 12.0) * q;
+    }
+    if (h->order == 4) unit *= 2.0;
+  }
+  return unit * std::sqrt((w2 + c * c) * n / 12.0);
+}
+
 // ------------------------------------------------------------------ Cartesian solves
 // Multipole boundary (t_mp), scaled right-hand side, state reset and reference
 // norm, all enqueued on s without a host round trip.  compact: order of the compact
@@ -666,7 +687,7 @@ ps_status cart_prepare(ps_ctx* h, const double* rho, double* phi, double tol, in
   TRY(cudaEventRecord(h->ev[1], s));
   Coef<double> cf = make_coef<double>(h->d0, h->h0, h->order);
   const double fscale = -4.0 * M_PI * h->bc.G * cf.inv_d;
-  TRY((h->nlaunch += 1, launch_init_state(h->st, tol, max_iter, s)));
+  TRY((h->nlaunch += 1, launch_init_state(h->st, tol, max_iter, s, fx_noise(h, compact))));
   // fs and the partials of the reference norm ||f - A phi0||, phi0 = boundary
   // data only (the compact schemes form R_h f and their reference norm themselves)
   if (!own_rhs)

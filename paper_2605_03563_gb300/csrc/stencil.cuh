@@ -77,6 +77,9 @@ __device__ __forceinline__ void set_loop(const DevState* st, unsigned long long 
 // the integer pipe (10.8 us under ncu with 1024 threads, FP64 maxima, log2 and
 // exp2, most of it in the SM's FP64 pipe).
 constexpr int FINISH_THREADS = 256;
+// Residual norms below this many times the share of the fixed-point units turn the
+// passes to FP64: a V-cycle's factor (refinement step's: 100) above the share.
+constexpr double FX_FLOOR = 64.0;
 __device__ __forceinline__ void finish_norm_block(const double* __restrict__ partials, int nblocks,
                                                   double dscale, int mode, DevState* __restrict__ st,
                                                   unsigned long long cond, int chunk) {
@@ -123,6 +126,11 @@ __device__ __forceinline__ void finish_norm_block(const double* __restrict__ par
   const unsigned vb = max(st->bmax, st->fmax);
   st->vmax = mode == 1 ? max(st->umax, st->bmax) : st->vnext;
   st->lmax = max(mode == 1 ? st->umax : st->hu[0], vb);
+  // what the units of this residual's passes may leave of it (fixed.cuh)
+  const unsigned eb = max(max(max(st->umax, st->unext), st->vmax), vb) >> 20;
+  st->lexact = st->exact;
+  st->exact = eb < 0x7ffu && sqrt(rr) <= FX_FLOOR * st->fx_noise * __longlong_as_double((long long)eb << 52);
+  if (mode == 1) st->lexact = st->exact;
   st->vnext = 0u;
   st->umax = st->unext;
   st->unext = 0u;
