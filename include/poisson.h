@@ -488,6 +488,12 @@ ps_status ps_op_spherical_apply(ps_handle h, const double* phi_dev, double* out_
 ps_status ps_probe_fp64(int kind, int blocks, int iters, double* out_dev, double* instructions_host,
                         void* stream);
 
+/* y = 1 / x of n FP64 values (device arrays) by the reciprocal that the coarsest
+ * CG uses for its scalars, for a check of its error: x and 1 / x normal numbers.
+ * Does not synchronise.  Errors: PS_ERR_INVALID_ARG for n < 0 or NULL arrays,
+ * PS_ERR_CUDA if the launch fails. */
+ps_status ps_probe_recip(const double* x_dev, double* y_dev, long long n, void* stream);
+
 /* Failure-detection check of the bounded device waits (no paper counterpart).
  * The TMA tile kernels wait on mbarriers with a time limit read from the
  * global timer: 2 s for a kernel's first failing wait, 1 ms for every wait

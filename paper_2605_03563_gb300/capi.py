@@ -104,6 +104,7 @@ SIGNATURES = {
     "ps_probe_fp64": (C.c_int, [C.c_int, C.c_int, C.c_int, C.c_void_p, C.POINTER(C.c_double),
                                 C.c_void_p]),
     "ps_probe_bounded_wait": (C.c_int, [C.c_int, C.c_void_p, C.POINTER(C.c_double), C.c_void_p]),
+    "ps_probe_recip": (C.c_int, [C.c_void_p, C.c_void_p, C.c_int64, C.c_void_p]),
     "ps_probe_grid_barrier": (C.c_int, [C.c_int, C.c_int, C.c_uint, C.c_int, C.c_void_p, C.POINTER(C.c_double),
                                         C.c_void_p]),
     "poisson_batch_create": (C.c_int, [C.c_int, C.c_int, C.c_int, C.c_int, C.c_int, C.c_int, C.c_int,

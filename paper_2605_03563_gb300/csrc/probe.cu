@@ -72,6 +72,10 @@ __global__ void k_probe_bounded_wait(int first_wait, long long* out) {
   }
 }
 
+__global__ void k_probe_recip(const double* __restrict__ x, double* __restrict__ y, long long n) {
+  for (long long i = blockIdx.x * (long long)kThreads + threadIdx.x; i < n; i += (long long)gridDim.x * kThreads) y[i] = recip(x[i]);
+}
+
 // `rounds` grid barriers of the one-launch iterations over a counter that starts
 // at `start`.  Before each a block publishes its round, after it thread b looks at
 // block b's: out[2] counts those behind.  missing != 0: the targets count one
@@ -96,6 +100,22 @@ __global__ void __launch_bounds__(kThreads) k_probe_grid_barrier(int rounds, uns
 }  // namespace ps
 
 using namespace ps;
+
+extern "C" ps_status ps_probe_recip(const double* x_dev, double* y_dev, long long n, void* stream) {
+  if (n < 0 || (n > 0 && (x_dev == nullptr || y_dev == nullptr))) {
+    set_error("ps_probe_recip: n must be >= 0 and the arrays non-NULL");
+    return PS_ERR_INVALID_ARG;
+  }
+  if (n == 0) return PS_OK;
+  const long long blocks = (n + kThreads - 1) / kThreads;
+  k_probe_recip<<<(unsigned)(blocks < 1024 ? blocks : 1024), kThreads, 0, static_cast<cudaStream_t>(stream)>>>(x_dev, y_dev, n);
+  const cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) {
+    set_error("ps_probe_recip: %s", cudaGetErrorString(e));
+    return PS_ERR_CUDA;
+  }
+  return PS_OK;
+}
 
 extern "C" ps_status ps_probe_grid_barrier(int blocks, int rounds, unsigned start, int missing, int* out_dev,
                                            double* waited_ms_host, void* stream) {

@@ -155,9 +155,11 @@ __device__ __forceinline__ void finish_norm_block(const double* __restrict__ par
   set_loop(st, cond, chunk);
 }
 
-// 1 / x for normal x well inside the exponent range: the approximate reciprocal
-// instruction, then two Newton steps y += y (1 - x y), each doubling the correct
-// bits (4 FP64 instructions; a division takes about 10, 76 cycles each per warp).
+// 1 / x for normal x with 1 / x normal: PTX's approximate reciprocal, then two steps
+// of Newton's iteration y += y (1 - x y) for the root of 1 / y - x, each of which
+// squares the relative error, and fused, so that the last rounding alone is left
+// (4 FP64 instructions; a division takes about 10, 76 cycles each per warp).  Within
+// one unit in the last place (ps_probe_recip).
 __device__ __forceinline__ double recip(double x) {
   double y;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
@@ -404,7 +406,10 @@ __device__ __forceinline__ void coarse_cg_cluster(const Dims& d, const Coef<doub
     }
     const double beta = g * igamma;   // 0 in the first step
     den = fma(-beta * beta, den, dl);
-    // alpha = g / den and 1 / g (for the next beta) from one reciprocal
+    // alpha = g / den and 1 / g (for the next beta) from one reciprocal, within a few
+    // units in the last place: x and r move by the same alpha, so their agreement,
+    // and with it the accuracy reached, does not depend on these (divisions: 32^3
+    // solve 694 -> 721 us)
     const double gd = g * den;
     double alpha;
     if (fabs(gd) > 1e-280 && fabs(gd) < 1e280) {

@@ -155,6 +155,14 @@ def probe_bounded_wait(first_wait, out, stream=None):
     return st, ms.value
 
 
+def probe_recip(x, y, stream=None):
+    """y = 1 / x by the coarsest CG's reciprocal (FP64 CUDA tensors of one size)."""
+    import torch
+    if x.dtype != torch.float64 or y.dtype != torch.float64 or x.numel() != y.numel():
+        raise ValueError("x and y must be FP64 tensors of one size")
+    check(lib().ps_probe_recip(_p(x), _p(y), x.numel(), _s(stream)), "ps_probe_recip")
+
+
 def probe_grid_barrier(blocks, rounds, out, start=0, missing=False, stream=None):
     """Pass `rounds` grid barriers of the one-launch iterations with `blocks`
     blocks over a counter that starts at `start` (missing: one arrival short,
