@@ -16,7 +16,6 @@
 // launch still fills every SM instead of serialising memory latency along z.
 // Kernels recover the chunk from gridDim.z.
 #include <algorithm>
-#include <atomic>
 #include <cstdio>
 
 #include "cart_kernels.cuh"
@@ -657,10 +656,10 @@ __global__ void __launch_bounds__(256, 2)
 template <int KIND, bool STORE>
 static cudaError_t fx_delta_t(const Dims& d, double c, const double* phi, const double* fs, int dout, void* out,
                               DevState* st, double* partials, int* nblocks, cudaStream_t s) {
-  static std::atomic<int> cached{0};
+  static PerDevice cached;
   constexpr int smem = FxGeom<KIND>::SMEM;
   int occ = 0, zc = 0;
-  const cudaError_t e = fx_occupancy(k_fx_delta<KIND, STORE>, smem, cached, &occ);
+  const cudaError_t e = resident_blocks(k_fx_delta<KIND, STORE>, 256, smem, cached, &occ);
   if (e != cudaSuccess) return e;
   CUtensorMap mU, mB;
   if (!fx_maps<KIND>(d, phi, fs, &mU, &mB)) return cudaErrorInvalidValue;
@@ -1672,25 +1671,28 @@ size_t coarse_cg_smem_bytes(const Dims& d) { return (size_t)d.size() * sizeof(do
 // CTAs per cluster of the coarsest CG: 16 (the opt-in size) where the device
 // can place such a cluster, else the portable 8.
 int coarse_cg_cluster_ctas() {
-  static std::atomic<int> cached{0};
-  int nc = cached.load(std::memory_order_relaxed);
-  if (nc) return nc;
-  auto kern = k_coarse_cg<1, true, double, double, 1>;
-  nc = 8;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(CG_MAXNC);
-  cfg.blockDim = dim3(CG_MAXT);
-  cudaLaunchAttribute at[1];
-  at[0].id = cudaLaunchAttributeClusterDimension;
-  at[0].val.clusterDim = {CG_MAXNC, 1, 1};
-  cfg.attrs = at;
-  cfg.numAttrs = 1;
-  int n = 0;
-  if (cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
-      cudaOccupancyMaxActiveClusters(&n, kern, &cfg) == cudaSuccess && n > 0)
-    nc = CG_MAXNC;
-  (void)cudaGetLastError();
-  cached.store(nc, std::memory_order_relaxed);
+  static PerDevice cached;
+  int nc = 8;
+  (void)cached.get(
+      [](int* best) {
+        auto kern = k_coarse_cg<1, true, double, double, 1>;
+        *best = 8;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(CG_MAXNC);
+        cfg.blockDim = dim3(CG_MAXT);
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim = {CG_MAXNC, 1, 1};
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        int n = 0;
+        if (cudaFuncSetAttribute(kern, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) == cudaSuccess &&
+            cudaOccupancyMaxActiveClusters(&n, kern, &cfg) == cudaSuccess && n > 0)
+          *best = CG_MAXNC;
+        (void)cudaGetLastError();
+        return cudaSuccess;
+      },
+      &nc);
   return nc;
 }
 

@@ -23,7 +23,6 @@
 // serve the rows above and below as well (12.5 FP64 operations per node for
 // a residual instead of 27 multiply-adds).
 #include <algorithm>
-#include <atomic>
 #include <cmath>
 #include <numeric>
 #include <type_traits>
@@ -490,10 +489,10 @@ template <int MODE, typename TR>
 static cudaError_t c27_fx_t(const Dims& d, const FxOp& op, const double* in, const double* base, TR* dst,
                             double* partials, DevState* st, const unsigned* h1, const unsigned* h2, unsigned* track,
                             int* nb, cudaStream_t s) {
-  static std::atomic<int> cached{0};
+  static PerDevice cached;
   constexpr int smem = FxGeom<FX27>::SMEM;
   int occ = 0, zc = 0;
-  const cudaError_t e = fx_occupancy(k_c27_fx<MODE, TR>, smem, cached, &occ);
+  const cudaError_t e = resident_blocks(k_c27_fx<MODE, TR>, 256, smem, cached, &occ);
   if (e != cudaSuccess) return e;
   CUtensorMap mU, mB;
   if (!fx_maps<FX27>(d, in, base, &mU, &mB)) return cudaErrorInvalidValue;
@@ -845,14 +844,10 @@ static cudaError_t launch_march_t(const Dims& d, const W27& A, const W27& M, dou
   if (!encode_level_map(&mu, DT_F32, u, d, GBW, T::GUH)) return cudaErrorInvalidValue;
   if (!encode_level_map(&mb, DT_F32, b, d, GBW, T::GBH)) return cudaErrorInvalidValue;
   auto kern = k_c27_smooth<RESID, GW, GR>;
-  static int blocks_per_sm = 0;
-  if (blocks_per_sm == 0) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, T::SMEM);
-    if (e != cudaSuccess) return e;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks_per_sm, kern, 32 * GW, T::SMEM);
-    if (e != cudaSuccess) return e;
-    blocks_per_sm = std::max(1, blocks_per_sm);
-  }
+  static PerDevice cached;
+  int blocks_per_sm = 0;
+  const cudaError_t eo = resident_blocks(kern, 32 * GW, T::SMEM, cached, &blocks_per_sm);
+  if (eo != cudaSuccess) return eo;
   const int sms = device_sm_count();
   const int gx = (d.ni() + GTX - 1) / GTX, gy = (d.nj() + T::GTY - 1) / T::GTY, nk = d.nk();
   // z-chunks of at least 16 planes (4 extra staged planes each)
@@ -1139,12 +1134,11 @@ static cudaError_t coarse_cg_t(const Dims& d, const W27& A, const T* b, T* u, do
                                cudaStream_t s) {
   const size_t smem = c27_coarse_smem(d);
   if (smem > 200 * 1024) return cudaErrorInvalidValue;
-  static size_t opted = 0;
-  if (smem > 48 * 1024 && smem > opted) {
-    cudaError_t e = cudaFuncSetAttribute(k_c27_coarse_cg<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    opted = smem;
-  }
+  // (the largest size that is accepted, once per device)
+  static PerDevice cached;
+  int resident = 0;
+  const cudaError_t e = resident_blocks(k_c27_coarse_cg<T>, CCG_THREADS, 200 * 1024, cached, &resident);
+  if (e != cudaSuccess) return e;
   k_c27_coarse_cg<T><<<1, CCG_THREADS, smem, s>>>(d, A, b, u, tol, st);
   return cudaGetLastError();
 }

@@ -35,9 +35,9 @@
 // way, and the accuracy that can be reached is that of the FP64 sums.  Passes whose H
 // is infinite, NaN or near the ends of the exponent range do so as well.
 #pragma once
-#include <atomic>
 #include <type_traits>
 
+#include "per_device.cuh"
 #include "tma.cuh"
 
 namespace ps {
@@ -376,21 +376,6 @@ template <int KIND>
 inline bool fx_maps(const Dims& d, const double* u, const double* base, CUtensorMap* mU, CUtensorMap* mB) {
   return encode_level_map(mU, 0, u, d, FxGeom<KIND>::WX, FxGeom<KIND>::WY) &&
          encode_level_map(mB, 0, base, d, FxGeom<KIND>::WX, FxGeom<KIND>::TY);
-}
-
-// Resident blocks of a pass kernel per SM (its shared memory is set at the first call).
-template <typename K>
-inline cudaError_t fx_occupancy(K kern, int smem, std::atomic<int>& cached, int* out) {
-  int occ = cached.load(std::memory_order_relaxed);
-  if (occ == 0) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e != cudaSuccess) return e;
-    if ((e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kern, 256, smem)) != cudaSuccess) return e;
-    occ = occ < 1 ? 1 : occ;
-    cached.store(occ, std::memory_order_relaxed);
-  }
-  *out = occ;
-  return cudaSuccess;
 }
 
 // Launch geometry: as many z-chunks as fill the resident blocks of whole waves

@@ -278,9 +278,9 @@ __global__ void __launch_bounds__(256, 227 * 1024 / (Gm::SMEM + 1024) > 4 ? 4 : 
 template <int KIND, bool ISO, int MODE, typename Gm>
 static cudaError_t fc_v(const Dims& d, const Coef<double>& cf, int colour, double* phi, const double* fs, double* out,
                         DevState* st, const FcBounds& b, double* partials, int* nblocks, cudaStream_t s) {
-  static std::atomic<int> cached{0};
+  static PerDevice cached;
   int occ = 0, zc = 0;
-  const cudaError_t e = fx_occupancy(k_fc_pass<KIND, ISO, MODE, Gm>, Gm::SMEM, cached, &occ);
+  const cudaError_t e = resident_blocks(k_fc_pass<KIND, ISO, MODE, Gm>, 256, Gm::SMEM, cached, &occ);
   if (e != cudaSuccess) return e;
   CUtensorMap mU, mB;
   if (!encode_level_map(&mU, DT_F64, phi, d, Gm::WX, Gm::WY) || !encode_level_map(&mB, DT_F64, fs, d, Gm::WX, Gm::TY))

@@ -11,7 +11,6 @@
 // Convergence is decided on the device; the host reads the small state once per
 // V-cycle / refinement step, or once per chunk of Krylov/SOR iterations (the
 // kernels of an iteration body skip their work once the state says done).
-#include <atomic>
 #include <algorithm>
 #include <array>
 #include <cmath>
@@ -32,6 +31,7 @@
 #include "multipole.cuh"
 #include "spherical.cuh"
 #include "compact.cuh"
+#include "per_device.cuh"
 
 namespace ps {
 
@@ -47,15 +47,16 @@ void set_error(const char* fmt, ...) {
 }
 
 int device_sm_count() {
-  static std::atomic<int> cache[64];
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) return 152;
-  int n = cache[dev].load(std::memory_order_relaxed);
-  if (n <= 0) {
-    if (cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n <= 0) return 152;
-    cache[dev].store(n, std::memory_order_relaxed);
-  }
-  return n;
+  static PerDevice cached;
+  int n = 0;
+  const cudaError_t e = cached.get(
+      [](int* v) {
+        int dev = 0;
+        const cudaError_t q = cudaGetDevice(&dev);
+        return q != cudaSuccess ? q : cudaDeviceGetAttribute(v, cudaDevAttrMultiProcessorCount, dev);
+      },
+      &n);
+  return e == cudaSuccess ? n : 152;
 }
 
 static size_t dt_size(int dt) { return dt == DT_F64 ? 8 : dt == DT_F32 ? 4 : 2; }

@@ -151,10 +151,10 @@ __global__ void __launch_bounds__(256, 227 * 1024 / (SsGeom<T, G, R>::SMEM + 102
 template <typename T, int G, bool ISO, int R>
 cudaError_t ss_t(const Dims& d, const double h[3], int dt, int colour, void* phi, const void* fs, int* fault, cudaStream_t s) {
   using Gm = SsGeom<T, G, R>;
-  static std::atomic<int> cached{0};
+  static PerDevice cached;
   int occ = 0, zc = 0;
   auto kern = k_colour_staged<T, G, ISO, R>;
-  const cudaError_t e = fx_occupancy(kern, Gm::SMEM, cached, &occ);
+  const cudaError_t e = resident_blocks(kern, 256, Gm::SMEM, cached, &occ);
   if (e != cudaSuccess) return e;
   CUtensorMap mP, mF;
   if (!encode_level_map(&mP, dt, phi, d, Gm::WX, Gm::WY) || !encode_level_map(&mF, dt, fs, d, Gm::WX, Gm::TY))

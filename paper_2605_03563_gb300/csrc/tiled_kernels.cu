@@ -25,6 +25,7 @@
 #include <type_traits>
 
 #include "tiled_kernels.cuh"
+#include "per_device.cuh"
 #include "tma.cuh"
 
 namespace ps {
@@ -363,14 +364,10 @@ static cudaError_t rb_sweep_t(const Dims& d, const double h[3], const void* pin,
   constexpr int NS = 5;
   using Gm = SweepGeom<T, R, NWC, NS>;
   auto kern = k_rb_sweep<T, ISO, R, NWC, NS>;
-  static int blocks_per_sm = 0;
-  if (blocks_per_sm == 0) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Gm::SMEM);
-    if (e != cudaSuccess) return e;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks_per_sm, kern, Gm::NTH, Gm::SMEM);
-    if (e != cudaSuccess) return e;
-    blocks_per_sm = std::max(1, blocks_per_sm);
-  }
+  static PerDevice cached;
+  int blocks_per_sm = 0;
+  const cudaError_t eo = resident_blocks(kern, Gm::NTH, Gm::SMEM, cached, &blocks_per_sm);
+  if (eo != cudaSuccess) return eo;
   const int dt = sizeof(T) == 4 ? DT_F32 : DT_BF16;
   CUtensorMap mP, mF;
   if (!encode_level_map(&mP, dt, pin, d, Gm::WP, Gm::HP) || !encode_level_map(&mF, dt, fs, d, Gm::WP, Gm::HF))
@@ -865,14 +862,10 @@ static cudaError_t rr_rb_t(const Dims& fd, const Dims& cd, const double h[3], co
                            void* fsc, void* zero, double factor, int* fault, cudaStream_t s) {
   using Gm = RrbGeom<T, RC, NWC, NS>;
   auto kern = k_resid_restrict_rb<T, ISO, RC, NWC, NS>;
-  static int blocks_per_sm = 0;
-  if (blocks_per_sm == 0) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Gm::SMEM);
-    if (e != cudaSuccess) return e;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks_per_sm, kern, Gm::NTH, Gm::SMEM);
-    if (e != cudaSuccess) return e;
-    blocks_per_sm = std::max(1, blocks_per_sm);
-  }
+  static PerDevice cached;
+  int blocks_per_sm = 0;
+  const cudaError_t eo = resident_blocks(kern, Gm::NTH, Gm::SMEM, cached, &blocks_per_sm);
+  if (eo != cudaSuccess) return eo;
   const int dt = sizeof(T) == 4 ? DT_F32 : DT_BF16;
   CUtensorMap mP, mF;
   if (!encode_level_map(&mP, dt, phi, fd, Gm::WP, Gm::HP) || !encode_level_map(&mF, dt, fs, fd, Gm::WP, Gm::HF))
@@ -896,14 +889,10 @@ static cudaError_t rr_t(const Dims& fd, const Dims& cd, const double h[3], int o
   using Gm = RRGeom<TF, G, TXC, TYC>;
   const int smem = Gm::NS * (Gm::PB + Gm::FB) + 2 * align_up(Gm::DW * Gm::DH * (int)sizeof(C), 128) + Gm::NS * 8;
   auto kern = k_resid_restrict<TF, TC, G, ISO, TXC, TYC>;
-  static int blocks_per_sm = 0;
-  if (blocks_per_sm == 0) {
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
-    if (e != cudaSuccess) return e;
-    e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&blocks_per_sm, kern, NT, smem);
-    if (e != cudaSuccess) return e;
-    blocks_per_sm = std::max(1, blocks_per_sm);
-  }
+  static PerDevice cached;
+  int blocks_per_sm = 0;
+  const cudaError_t eo = resident_blocks(kern, NT, smem, cached, &blocks_per_sm);
+  if (eo != cudaSuccess) return eo;
   const int dt = sizeof(TF) == 8 ? DT_F64 : sizeof(TF) == 4 ? DT_F32 : DT_BF16;
   CUtensorMap mP, mF;
   if (!encode_level_map(&mP, dt, phi, fd, Gm::WP, Gm::HP) || !encode_level_map(&mF, dt, fs, fd, Gm::WP, Gm::HF))
