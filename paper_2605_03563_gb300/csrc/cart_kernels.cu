@@ -1858,11 +1858,13 @@ cudaError_t launch_finish_norm(const double* partials, int nblocks, double dscal
 // state is the result, or phase 2 updates the black values from the new red
 // ones.  Updates and residuals repeat the colour passes' arithmetic
 // (gs_value's order), so iterates agree bit for bit.
+// 32 registers a thread let as many solves stay resident beside each other as the
+// SM has warps for (64^3, four at once: 8.9 -> 8.2 ms a solve).
 // 31^3 unknowns to 1e-10: 24.2 us a step as four kernels of a loop graph (17.9 with
 // the shorter finisher), 11.0 with three barriers a step, 8.1 with these two; 95^3:
 // 1.85 times faster than the graph.
 template <bool ISO, int NT>
-__global__ void __launch_bounds__(NT)
+__global__ void __launch_bounds__(NT, 2048 / NT)
     k_sor_steps(Dims d, Coef<double> cf, double* __restrict__ phi, double* __restrict__ alt, const double* __restrict__ fs,
                 double omega0, const double* __restrict__ wtab, int wlen, DevState* __restrict__ st,
                 double* __restrict__ partials) {
@@ -1967,38 +1969,57 @@ __global__ void __launch_bounds__(NT)
   }
 }
 
-template <bool ISO, int NT>
-static cudaError_t sor_steps_t(const Dims& d, const Coef<double>& cf, double* phi, double* alt, const double* fs,
-                               double omega, const double* wtab, int wlen, DevState* st, double* partials, int npart,
-                               cudaStream_t s) {
-  // one block per SM, and at least an x pair per thread
-  const long long want = ((long long)(d.ni() + 1) / 2 * d.nj() * d.nk() + NT - 1) / NT;
-  const int blocks = (int)std::max(1LL, std::min<long long>({want, (long long)device_sm_count(), (long long)npart}));
-  Dims dd = d;
-  Coef<double> c = cf;
-  void* args[] = {&dd, &c, &phi, &alt, (void*)&fs, &omega, (void*)&wtab, &wlen, &st, &partials};
-  return cudaLaunchCooperativeKernel((const void*)k_sor_steps<ISO, NT>, dim3(blocks), dim3(NT), args, 0, s);
+// f(isotropic, threads) with the variant of a grid.  While one warp per SM
+// sub-partition covers the grid in two rounds, more warps would only queue at its
+// FP64 unit (76 cycles an instruction); larger grids take 8 and 16 warps per SM
+// to hide the L2 loads.
+template <typename F>
+static auto sor_variant(const Dims& d, const double h[3], F f) {
+  const long long n = (long long)d.ni() * d.nj() * d.nk(), round = 2 * 128LL * device_sm_count();
+  auto with = [&](auto nt) { return is_iso(h) ? f(std::true_type(), nt) : f(std::false_type(), nt); };
+  if (n <= 2 * round) return with(std::integral_constant<int, 128>());
+  if (n <= 4 * round) return with(std::integral_constant<int, 256>());
+  return with(std::integral_constant<int, 512>());
+}
+
+// one block per SM, and at least an x pair per thread
+static int sor_blocks(const Dims& d, int threads, int npart) {
+  const long long want = ((long long)(d.ni() + 1) / 2 * d.nj() * d.nk() + threads - 1) / threads;
+  return (int)std::max(1LL, std::min<long long>({want, (long long)device_sm_count(), (long long)npart}));
 }
 
 bool sor_steps_fit(const Dims& d) {
   return d.g == 1 && (long long)d.ni() * d.nj() * d.nk() <= SOR_STEPS_MAX;
 }
 
+// Several solves in flight (ms a solve, eight at once; loop graphs): 32^3 0.31 (0.71),
+// 48^3 2.2 (2.6), 64^3 8.0 (7.2; four at once 8.2, 9.3), 80^3 22.6 (33.9), 96^3 47.7
+// (71.2): below 350000 unknowns a launch that would wait for room beside the others
+// leaves the work to the loop graph, above the graph is never the faster one.
+int sor_steps_share(const Dims& d, const double h[3], int npart) {
+  if ((long long)d.ni() * d.nj() * d.nk() > 350000) return 0;
+  return sor_variant(d, h, [&](auto iso, auto nt) -> int {
+    constexpr int NT = decltype(nt)::value;
+    static PerDevice cached;
+    int occ = 1;
+    (void)cached.get(
+        [](int* n) { return cudaOccupancyMaxActiveBlocksPerMultiprocessor(n, k_sor_steps<decltype(iso)::value, NT>, NT, 0); },
+        &occ);
+    return steps_share(sor_blocks(d, NT, npart), occ);
+  });
+}
+
 cudaError_t launch_sor_steps(const Dims& d, const double h[3], double* phi, double* alt, const double* fs, double omega,
                              const double* wtab, int wlen, DevState* st, double* partials, int npart, cudaStream_t s) {
   if (!sor_steps_fit(d) || npart < 1) return cudaErrorInvalidValue;
-  const Coef<double> cf = make_coef<double>(d, h, 2);
-  // While one warp per SM sub-partition covers the grid in two rounds, more
-  // warps would only queue at its FP64 unit (76 cycles an instruction); larger
-  // grids take 8 and 16 warps per SM to hide the L2 loads.
-  const long long n = (long long)d.ni() * d.nj() * d.nk(), round = 2 * 128LL * device_sm_count();
-#define PS_SOR_STEPS(NT)                                                                                        \
-  return is_iso(h) ? sor_steps_t<true, NT>(d, cf, phi, alt, fs, omega, wtab, wlen, st, partials, npart, s)      \
-                   : sor_steps_t<false, NT>(d, cf, phi, alt, fs, omega, wtab, wlen, st, partials, npart, s)
-  if (n <= 2 * round) PS_SOR_STEPS(128);
-  if (n <= 4 * round) PS_SOR_STEPS(256);
-  PS_SOR_STEPS(512);
-#undef PS_SOR_STEPS
+  Coef<double> c = make_coef<double>(d, h, 2);
+  Dims dd = d;
+  void* args[] = {&dd, &c, &phi, &alt, (void*)&fs, &omega, (void*)&wtab, &wlen, &st, &partials};
+  return sor_variant(d, h, [&](auto iso, auto nt) -> cudaError_t {
+    constexpr int NT = decltype(nt)::value;
+    return cudaLaunchCooperativeKernel((const void*)k_sor_steps<decltype(iso)::value, NT>, dim3(sor_blocks(d, NT, npart)),
+                                       dim3(NT), args, 0, s);
+  });
 }
 
 // ------------------------------------------------------------------ CG kernels (FP64)

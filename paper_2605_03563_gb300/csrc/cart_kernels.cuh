@@ -49,6 +49,8 @@ cudaError_t launch_sweep_colour(const Dims& d, int order, const double h[3], int
 // alt: scratch array of phi's layout; partials holds npart doubles or more.
 constexpr long long SOR_STEPS_MAX = 1000000;
 bool sor_steps_fit(const Dims& d);
+// 1024ths of the device that a launch keeps resident (0: takes none into account)
+int sor_steps_share(const Dims& d, const double h[3], int npart);
 cudaError_t launch_sor_steps(const Dims& d, const double h[3], double* phi, double* alt, const double* fs, double omega,
                              const double* wtab, int wlen, DevState* st, double* partials, int npart, cudaStream_t s);
 

@@ -368,4 +368,6 @@ void set_error(const char* fmt, ...);
 // Streaming multiprocessors of the current device (queried once per device and
 // cached); launch geometries scale with it.
 int device_sm_count();
+// 1024ths of the device's room for `per_sm` blocks of a kernel per SM that `blocks` of them take
+inline int steps_share(int blocks, int per_sm) { return (int)((1024LL * blocks + (long long)per_sm * device_sm_count() - 1) / ((long long)per_sm * device_sm_count())); }
 }

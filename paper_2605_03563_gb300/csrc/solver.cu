@@ -13,6 +13,7 @@
 // kernels of an iteration body skip their work once the state says done).
 #include <algorithm>
 #include <array>
+#include <atomic>
 #include <cmath>
 #include <cstdarg>
 #include <cstdio>
@@ -103,6 +104,27 @@ static const char* kProfNames[PC_COUNT] = {
 // being captured into a loop graph.
 using Body = std::function<cudaError_t(unsigned long long, int, cudaStream_t)>;
 
+// The room that the one-launch iterations of the solves in flight keep on each
+// device, in 1024ths.  Such a launch runs only with all its blocks resident; where
+// the solves in flight, of any thread, want more than the device has, launches would
+// queue one behind the other, and each step takes its loop graph instead (the same
+// bits).  A solve holds its share from begin to end.
+class StepsShare {
+ public:
+  explicit StepsShare(int share) : share_(share) {
+    if (cudaGetDevice(&dev_) != cudaSuccess || dev_ < 0 || dev_ >= 64) dev_ = 0;
+    held_[dev_] += share_;
+  }
+  ~StepsShare() { held_[dev_] -= share_; }
+  StepsShare(const StepsShare&) = delete;
+  StepsShare& operator=(const StepsShare&) = delete;
+  bool fits() const { return share_ == 0 || held_[dev_].load() <= 1024; }
+
+ private:
+  int dev_ = 0, share_ = 0;
+  static inline std::atomic<int> held_[64] = {};
+};
+
 // The solve in flight on a handle (begin .. end).
 struct Active {
   bool on = false;
@@ -122,6 +144,8 @@ struct Active {
   int inner_per_iter = 0;
   // the iterations of a step in one launch (instead of the loop graph), where set
   std::function<cudaError_t(cudaStream_t)> steps;
+  std::shared_ptr<StepsShare> share;
+  bool steps_now() const { return steps && share->fits(); }
   bool fc = false;                    // V-cycle passes of the larger levels on the integer pipe (fixed_sweeps.cu)
   // enqueued by every step before the iterations / after them (may be empty)
   std::function<cudaError_t(cudaStream_t)> prologue, epilogue;
@@ -865,10 +889,12 @@ ps_status begin_sor(ps_ctx* h, const ps_solve_opts* o, cudaStream_t s) {
       (void)cudaGetLastError();   // no room: the separate passes, which need none
       h->sor_alt = nullptr;
     }
-    if (h->sor_alt)
+    if (h->sor_alt) {
+      h->act.share = std::make_shared<StepsShare>(sor_steps_share(h->d0, h->h0, 2 * h->npart));
       h->act.steps = [h, phi, omega, wtab, wlen](cudaStream_t q) -> cudaError_t {
         return launch_sor_steps(h->d0, h->h0, phi, h->sor_alt, h->fs64, omega, wtab, wlen, h->st, h->partials, 2 * h->npart, q);
       };
+    }
   }
   char key[64];
   if (wtab) snprintf(key, sizeof(key), "sor:chebyshev");
@@ -1220,10 +1246,12 @@ ps_status bicg_start(ps_ctx* h, int dt, const double* rho, double fscale, double
       (void)cudaGetLastError();   // no room: the separate kernels, which need none
       h->sph_part = nullptr;
     }
-    if (h->sph_part)
+    if (h->sph_part) {
+      h->act.share = std::make_shared<StepsShare>(bicg_steps_share(h->sd, dt));
       h->act.steps = [h, dt, rho, fscale, x, z, v, st](cudaStream_t q) -> cudaError_t {
         return launch_bicg_steps(h->sd, h->stab, dt, rho, fscale, x, z, v, h->sph_part, st, q);
       };
+    }
   }
   *body = [h, dt, fscale, x, z, v, st](unsigned long long cond, int chunk, cudaStream_t q) -> cudaError_t {
     const double n = (double)h->sd.nr * h->sd.nt * h->sd.np;
@@ -1386,6 +1414,12 @@ ps_status build_loop_graph(ps_ctx* h, LoopGraph* g) {
   return PS_OK;
 }
 
+// The solve is no longer in flight.
+void end_active(ps_ctx* h) {
+  h->act.on = false;
+  h->act.share.reset();
+}
+
 // Enqueue up to k more iterations of the active solve on the handle's stream.
 ps_status step_active(ps_ctx* h, int k) {
   cudaStream_t s = h->stream;
@@ -1448,7 +1482,7 @@ ps_status step_active(ps_ctx* h, int k) {
     h->act.plain_steps = true;
     return PS_OK;
   }
-  if (h->act.steps) {
+  if (h->act.steps_now()) {
     h->act.body_kernels = 0;
     TRY((h->nlaunch += 1, launch_set_budget(h->st, k, s)));
     TRY((h->nlaunch += 1, h->act.steps(s)));
@@ -2018,7 +2052,10 @@ ps_status poisson_solve_begin(ps_handle h, const double* rho_dev, double* phi_de
     else if (o.method == PS_PCG) r = begin_pcg(h, s);
     else r = begin_cg(h, s);
   }
-  if (r != PS_OK) return r;
+  if (r != PS_OK) {
+    end_active(h);
+    return r;
+  }
   h->hst->iter = 0;
   h->hst->done = DONE_NO;
   a.on = true;
@@ -2043,7 +2080,7 @@ ps_status poisson_solve_end(ps_handle h, ps_info* info) {
   if (!h || !h->act.on) return fail(PS_ERR_INVALID_ARG, "no solve in flight");
   Active& a = h->act;
   cudaStream_t s = h->stream;
-  a.on = false;
+  end_active(h);
   TRY(cudaEventRecord(h->ev[2], s));
   if (h->sph) TRY(cudaMemcpyAsync(a.phi_user, h->phi0, (size_t)h->sd.size() * sizeof(double), cudaMemcpyDeviceToDevice, s));
   else TRY(copy_rows(a.phi_user, h->du, h->phi0, h->d0, s));
@@ -2069,10 +2106,10 @@ ps_status poisson_solve(ps_handle h, const double* rho_dev, double* phi_dev, dou
   ps_status r = poisson_solve_begin(h, rho_dev, phi_dev, tol, opts);
   if (r != PS_OK) return r;
   int done = 0;
-  if ((r = poll_active(h, &done)) != PS_OK) { h->act.on = false; return r; }
+  if ((r = poll_active(h, &done)) != PS_OK) { end_active(h); return r; }
   while (!done) {
-    if ((r = step_active(h, h->act.steps ? STEPS_CHUNK : h->act.chunk)) != PS_OK || (r = poll_active(h, &done)) != PS_OK) {
-      h->act.on = false;
+    if ((r = step_active(h, h->act.steps_now() ? STEPS_CHUNK : h->act.chunk)) != PS_OK || (r = poll_active(h, &done)) != PS_OK) {
+      end_active(h);
       return r;
     }
   }
@@ -2094,7 +2131,7 @@ ps_status poisson_solve_batch(ps_handle* hs, const double* const* rho, double* c
   std::vector<int> done(n, 0);
   for (int i = 0; i < n; i++)
     if ((r = poisson_solve_begin(hs[i], rho[i], phi[i], tol[i], opts)) != PS_OK) {
-      for (int j = 0; j < i; j++) hs[j]->act.on = false;
+      for (int j = 0; j < i; j++) end_active(hs[j]);
       return r;
     }
   int left = n;

@@ -18,6 +18,7 @@
 #include <vector>
 
 #include "cart_kernels.cuh"
+#include "per_device.cuh"
 #include "spherical.cuh"
 #include "stencil.cuh"
 
@@ -814,6 +815,10 @@ cudaError_t launch_bicg_iter(const SphDims& d, const SphTables& t, int dt,
 // state in shared memory and takes the same decisions on it.
 // 96 x 48 x 32 to 1e-8 (316 iterations): 20.6 -> 12.3 ms (17.0 before a chunk's
 // operands were loaded ahead of its stores); 64 x 24 x 16: 9.8 -> 4.8 ms.
+// 128 registers a thread (a few spilled) let four launches stay resident beside
+// each other: four solves of 96 x 48 x 32 at once 8.7 -> 5.8 ms a solve (loop graphs
+// 6.5; eight at once 7.3 -> 6.1, 4.8: a launch that would wait for room beside the
+// others leaves the work to the loop graph), one alone 12.2 either way.
 constexpr int BS_WARPS = 4;
 
 // {sum, sum} over nblk virtual blocks of 8 warps each from W[block][warp][2]
@@ -845,7 +850,7 @@ __device__ __forceinline__ void bicg_reduce(const double* __restrict__ W, int nb
 }
 
 template <typename T>
-__global__ void __launch_bounds__(BS_WARPS * 32)
+__global__ void __launch_bounds__(BS_WARPS * 32, 4)
     k_bicg_steps(SphDims d, Tab<typename St<T>::C> tb, Tab<double> tb64, const double* __restrict__ vol,
                  const double* __restrict__ rho, double fscale, double* __restrict__ x, double* __restrict__ z,
                  T* __restrict__ r, T* __restrict__ rhat, T* __restrict__ p, T* __restrict__ phat,
@@ -1108,22 +1113,37 @@ bool bicg_steps_fit(const SphDims& d) {
 
 size_t bicg_steps_doubles(const SphDims& d) { return (size_t)(4 * bicg_wset(d)); }
 
+static int bicg_blocks(const SphDims& d) {
+  const long long warps = bicg_wset(d) / 2 / d.np * ((d.np + BKC - 1) / BKC);
+  return (int)std::min<long long>(device_sm_count(), (warps + BS_WARPS - 1) / BS_WARPS);
+}
+
+int bicg_steps_share(const SphDims& d, int dt) {
+  static PerDevice cached[2];
+  int occ = 1;
+  (void)cached[dt == DT_F64].get(
+      [&](int* n) {
+        return dt == DT_F64 ? cudaOccupancyMaxActiveBlocksPerMultiprocessor(n, k_bicg_steps<double>, BS_WARPS * 32, 0)
+                            : cudaOccupancyMaxActiveBlocksPerMultiprocessor(n, k_bicg_steps<float>, BS_WARPS * 32, 0);
+      },
+      &occ);
+  return steps_share(bicg_blocks(d), occ);
+}
+
 template <typename T>
 static cudaError_t bicg_steps_t(const SphDims& d, const SphTables& t, const double* rho, double fscale, double* x,
                                 double* z, void* const* v, double* W, DevState* st, cudaStream_t s) {
   using C = typename St<T>::C;
-  const long long wset = bicg_wset(d), warps = wset / 2 / d.np * ((d.np + BKC - 1) / BKC);
-  const int blocks = (int)std::min<long long>(device_sm_count(), (warps + BS_WARPS - 1) / BS_WARPS);
   SphDims dd = d;
   Tab<C> tb = tab_of<C>(t);
   Tab<double> tb64 = tab_of<double>(t);
   const double* vol = t.vol;
   T* q[8];
   for (int i = 0; i < 8; i++) q[i] = (T*)v[i];
-  long long ws = wset;
+  long long ws = bicg_wset(d);
   void* args[] = {&dd, &tb, &tb64, (void*)&vol, (void*)&rho, &fscale, &x, &z, &q[0], &q[1], &q[2], &q[3],
                   &q[4], &q[5], &q[6], &q[7], &W, &ws, &st};
-  return cudaLaunchCooperativeKernel((const void*)k_bicg_steps<T>, dim3(blocks), dim3(BS_WARPS * 32), args, 0, s);
+  return cudaLaunchCooperativeKernel((const void*)k_bicg_steps<T>, dim3(bicg_blocks(d)), dim3(BS_WARPS * 32), args, 0, s);
 }
 
 cudaError_t launch_bicg_steps(const SphDims& d, const SphTables& t, int dt, const double* rho, double fscale, double* x,

@@ -96,6 +96,7 @@ int bicg_iter_kernels(int dt);
 // phat, v, s, shat, t), W: scratch of bicg_steps_doubles doubles.
 bool bicg_steps_fit(const SphDims& d);
 size_t bicg_steps_doubles(const SphDims& d);
+int bicg_steps_share(const SphDims& d, int dt);   // 1024ths of the device that a launch keeps resident
 cudaError_t launch_bicg_steps(const SphDims& d, const SphTables& t, int dt, const double* rho, double fscale, double* x,
                               double* z, void* const* v, double* W, DevState* st, cudaStream_t s);
 // scalar finisher for the reference / initial residual (mode 0/1); mode 1
