@@ -26,10 +26,18 @@
 // slots busy), on the smallest by the chain of TMA wait, barrier and update from
 // plane to plane.
 //
-// Bounds.  With H the largest of |phi| (as last tracked) and |fs|, a pass adds at
-// most |fs| to the largest value (13-point: and a factor 102/90), so over the
-// sweeps between two trackings (up to 2 or 3, see fx_sweeps_fit) values stay
-// below 10.6 H, sums of six below 2^63 units.
+// Bounds.  H: the largest of |phi| as last tracked, the boundary data and |fs|,
+// below 2^57 units (13-point 2^56).  A 7-point update is a mean of its neighbours
+// plus fs, so a pass adds at most H to the largest value: 7 H after the three sweeps
+// that fx_sweeps_fit allows between two trackings, sums of six below 42 H < 2^63.
+// The 13-point weights' magnitudes add up to 102 / 90: after two sweeps (six passes)
+// values are below 10.6 H, sums of six and S1 - 6 C below 127.2 H < 2^63.
+// The 7-point S - 6 C has a closer bound, because residuals are formed after a sweep
+// at least: C = S' / 6 + fs with S' the neighbours' sum of the time, so S - 6 C =
+// (S - S') - 6 fs.  In its first pass after the tracking a node changes by at most
+// 3 H (first colour) or 4 H (second), in a later one by the mean of its
+// neighbours' last changes, 4 H again: |S - S'| <= 24 H, |S - 6 C| <= 30 H < 2^62.  Unequal
+// spacings form u(-1) + u(1) - 2 C per axis, below 28 H.
 #include "fixed.cuh"
 
 #include "cart_kernels.cuh"
@@ -50,19 +58,38 @@ struct FcGeom {
   static constexpr int SMEM = NS * (UB + BB) + ND * UB + NS * 8;
 };
 
-// v as fx_from gives it, in units of 2^(eb - 1079 + C) and for values up to 2^C
-// times 16 H; the negative of a value is its negation, so that values from H / 16
-// on are exact and a smooth field gets no drift from one-sided truncation.
+// v in units of 2^(eb - 1079 + C), for values up to 2^C times 16 H, rounded to
+// nearest, ties away from zero: an update keeps the sum of its neighbours, so a
+// one-sided rounding of the values below H / 16 (those above are exact) is a source
+// all over the faint part of a field, which the coarse levels sum up.
+// R.m.s. error of one V-cycle from a peak of 10^4 over values of 1 (96 x 112 x 80,
+// 7- / 13-point): 2.6e-11 / 4.8e-11 truncated, 4.6e-13 / 7.1e-13 as here, 1.3e-12 /
+// 2.6e-12 of the FP64 passes.
 template <int C>
 __device__ __forceinline__ long long fx_from_wide(double v, int eb) {
   const int hi = __double2hiint(v);
   const int e = (hi >> 20) & 0x7ff;
   const unsigned long long m =
-      ((unsigned long long)((hi & 0xfffff) | 0x100000) << 32 | (unsigned)__double2loint(v)) << 8;
+      ((unsigned long long)((hi & 0xfffff) | 0x100000) << 32 | (unsigned)__double2loint(v)) << 9;
   unsigned long long r;
   asm("shr.u64 %0, %1, %2;" : "=l"(r) : "l"(m), "r"(eb + 4 + C - e));   // shifts past 63 give 0
   const long long s = (long long)(hi >> 31);
-  return ((long long)r ^ s) - s;
+  return ((long long)((r + 1) >> 1) ^ s) - s;
+}
+
+// The same from three bits below the unit, where three to five eighths go to the even
+// neighbour: as often up as down for values in general and for exact ties.  Where
+// fs is zero a 7-point mean on equal spacings is a whole number of sixths of a unit,
+// every sixth a tie.
+__device__ __forceinline__ long long fx_from_even(double v, int eb) {
+  const int hi = __double2hiint(v);
+  const int e = (hi >> 20) & 0x7ff;
+  const unsigned long long m =
+      ((unsigned long long)((hi & 0xfffff) | 0x100000) << 32 | (unsigned)__double2loint(v)) << 11;
+  unsigned long long r;
+  asm("shr.u64 %0, %1, %2;" : "=l"(r) : "l"(m), "r"(eb + 4 - e));
+  const long long s = (long long)(hi >> 31);
+  return ((long long)((r + 3u + ((unsigned)r >> 2 & 2u)) >> 3) ^ s) - s;
 }
 
 // 16 a - b as a double, exact up to its 62 leading bits (the sum may exceed 64 bits)
@@ -152,7 +179,8 @@ __device__ __forceinline__ bool fc_march(const CUtensorMap& mU, const CUtensorMa
       for (int q = 0; q < NLD; q++)
         if ((q + 1) * NT <= NEL || tid + q * NT < NEL) {
           const double v = raw[tid + q * NT];
-          if constexpr (FX) w[tid + q * NT] = fx_from_wide<Gm::XC>(v, sc.eb);
+          if constexpr (FX && KIND == FX7 && ISO) w[tid + q * NT] = fx_from_even(v, sc.eb);
+          else if constexpr (FX) w[tid + q * NT] = fx_from_wide<Gm::XC>(v, sc.eb);
           else w[tid + q * NT] = v;
           if ((MODE == FC_NORM || (MODE == FC_LAG && ((black >> q ^ z) & 1))) && (inner >> q & 1u) && z >= G && z < G + d.nk())
             hmax = max(hmax, (unsigned)__double2hiint(v) & 0x7fffffffu);
