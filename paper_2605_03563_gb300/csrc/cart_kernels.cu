@@ -615,7 +615,7 @@ __global__ void __launch_bounds__(256, 2)
                int dout, void* __restrict__ out, DevState* __restrict__ st, double* __restrict__ partials) {
   if (!STORE && st->guess_nonzero == 0) return;   // an initial residual from zero: the reference vector
   struct Epi {
-    enum { TRACK = 0 };
+    enum { TRACK = 0, LAYERS = 0 };
     double oscale, s2;
     int oexp, dout;
     float s2f, mxf;

@@ -400,8 +400,8 @@ cudaError_t launch_c27_resid_dt(const Dims& d, const W27& A, const double* u, co
 // smoother are integers over a common factor, so one FP64 instruction a node
 // forms the value (three with a norm), instead of 12.5.  In every mode the value
 // is base + c T(in), stored as TR:
-//   C27_INIT   r = b - A u, sums of r^2 and of b^2 (which k_c27_shell completes to
-//              the reference norm); *track takes the largest |u| read;
+//   C27_INIT   r = b - A u, sums of r^2 and, inside the first and last layers, of b^2
+//              (which k_c27_shell completes to the reference norm); *track takes the largest |u| read;
 //   C27_NORM   r = b - A u, sum of r^2; *track the same;
 //   C27_RESID  r = b - A u; *track the largest |r| written;
 //   C27_SPAI   u - omega M r (in = r, base and dst = u: a block writes the nodes
@@ -419,10 +419,11 @@ __global__ void __launch_bounds__(256, 2)
              int nblocks) {
   if (MODE != C27_INIT && st->done) return;   // uniform
   struct Epi {
-    enum { TRACK = (MODE == C27_INIT || MODE == C27_NORM) && sizeof(TR) == 8 };
+    enum { TRACK = (MODE == C27_INIT || MODE == C27_NORM) && sizeof(TR) == 8, LAYERS = MODE == C27_INIT };
     TR* dst;
     double s2, s0;
     unsigned hmax;
+    bool layer[4];
     __device__ __forceinline__ void operator()(long long at, int px, const bool (&in)[4], const double (&v)[4],
                                                const double (&base)[4]) {
       TR x[4];
@@ -435,7 +436,7 @@ __global__ void __launch_bounds__(256, 2)
         dst[at + r * px] = x[r];
         if (MODE == C27_INIT || MODE == C27_NORM) s2 = fma(v[r], v[r], s2);
         else hmax = max(hmax, (unsigned)__double2hiint(v[r]) & 0x7fffffffu);
-        if (MODE == C27_INIT) s0 = fma(base[r], base[r], s0);
+        if (MODE == C27_INIT && !layer[r]) s0 = fma(base[r], base[r], s0);
       }
     }
   } epi{dst, 0.0, 0.0, 0u};
@@ -445,10 +446,9 @@ __global__ void __launch_bounds__(256, 2)
   if constexpr (MODE == C27_NORM) block_partial_nt<256>(epi.s2, partials);
 }
 
-// What the boundary data add to the reference norm: k_c27_fx<C27_INIT> sums b^2, and
-// the reference residual b - A u0 differs from b on the nodes that have a
-// boundary node among their 26 neighbours, the first and last layer of each
-// axis.  Partials {sum of (b - A u0)^2 - b^2, 0} per block over those nodes.
+// The reference residual b - A u0 on the nodes that have a boundary node among their
+// 26 neighbours, the first and last layer of each axis; elsewhere it is b, which
+// k_c27_fx<C27_INIT> sums.  Partials {sum of (b - A u0)^2, 0} per block.
 __global__ void __launch_bounds__(256)
     k_c27_shell(Dims d, Wts<double> W, const double* __restrict__ u, const double* __restrict__ b,
                 double* __restrict__ partials) {
@@ -480,7 +480,7 @@ __global__ void __launch_bounds__(256)
     const double r0 = plane_p_plus(nw, plane_of(plane_load<true>(d, u, i, j, k)), f,
                                    plane_q(nw, plane_of(plane_load<true>(d, u, i, j, k - 1))),
                                    plane_q(nw, plane_of(plane_load<true>(d, u, i, j, k + 1))));
-    s += fma(r0, r0, -(f * f));
+    s = fma(r0, r0, s);
   }
   block_partial_nt<256>(s, partials);
 }

@@ -139,6 +139,7 @@ struct FxGeom {
 // One barrier a plane: it separates the writes of a work buffer from its reads
 // two planes earlier, and hands the stage of the previous plane back to the
 // copy engine.
+// Epi::LAYERS: epi.layer[r] says whether node r lies on the first or last layer of an axis.
 // Epi::TRACK: epi.hmax takes the high word of the largest |u| of the interior nodes
 // staged (the tile's own and their neighbours; not the boundary's, some of which
 // no stencil reads).
@@ -295,6 +296,12 @@ __device__ __forceinline__ bool fx_march(const CUtensorMap& mU, const CUtensorMa
 #pragma unroll
     for (int r = 0; r < R; r++) f[r] = b[(ty * R + r) * WX + tx + G];
     values(c0, g1, g2, g3, f, x);
+    if constexpr (Epi::LAYERS) {
+      const int k = z - 1 - G, i = i0 + tx;   // the plane that arrived last is z - 1
+      const bool l = i == G || i == G + d.ni() - 1 || k == G || k == G + d.nk() - 1;
+#pragma unroll
+      for (int r = 0; r < R; r++) epi.layer[r] = l || jr + r == G || jr + r == G + d.nj() - 1;
+    }
     epi(at, d.px, in, x, f);
     at += d.sz();
   };
