@@ -83,6 +83,18 @@ __device__ __forceinline__ double fx_double(long long v) {
   return a == 0 ? 0.0 : __hiloint2double((int)(hi | ((unsigned)s & 0x80000000u)), (int)(unsigned)m);
 }
 
+// H 2^32 + L, up to 2^93 in size, as a double: exact up to its 62 leading bits.
+__device__ __forceinline__ double fx_two_limbs(long long H, long long L) {
+  H += L >> 32;
+  // shifted right by 11 unless it fits 63 bits
+  const bool big = (unsigned long long)(H + (1LL << 30)) >= (1ull << 31);
+  const unsigned low = (unsigned)L;
+  const long long t = big ? (long long)((unsigned long long)H << 21 | low >> 11)
+                          : (long long)((unsigned long long)H << 32 | low);
+  const double v = fx_double(t);
+  return __hiloint2double(__double2hiint(v) + (big ? 11 << 20 : 0), __double2loint(v));
+}
+
 // |x| < 2^(32 + b), from the high word
 __device__ __forceinline__ bool fx_below(long long x, int b) {
   return (unsigned)((int)(x >> 32) + (1 << b)) < (2u << b);
@@ -265,14 +277,8 @@ __device__ __forceinline__ bool fx_march(const CUtensorMap& mU, const CUtensorMa
         const unsigned long long lc = lo(c0[r]) * (unsigned)abs(op.w0);
         const long long L = (long long)(lo(g1[r]) * (unsigned)op.w1 + lo(g2[r]) * (unsigned)op.w2 +
                                         lo(g3[r]) * (unsigned)op.w3 + (op.w0 < 0 ? 0ull - lc : lc));
-        const long long H = hi(c0[r]) * op.w0 + hi(g1[r]) * op.w1 + hi(g2[r]) * op.w2 + hi(g3[r]) * op.w3 + (L >> 32);
-        // T = H 2^32 + low; shifted right by 11 unless it fits 63 bits
-        const bool big = (unsigned long long)(H + (1LL << 30)) >= (1ull << 31);
-        const unsigned low = (unsigned)L;
-        const long long t = big ? (long long)((unsigned long long)H << 21 | low >> 11)
-                                : (long long)((unsigned long long)H << 32 | low);
-        const double v = fx_double(t);
-        x[r] = fma(__hiloint2double(__double2hiint(v) + (big ? 11 << 20 : 0), __double2loint(v)), cu, f[r]);
+        const long long H = hi(c0[r]) * op.w0 + hi(g1[r]) * op.w1 + hi(g2[r]) * op.w2 + hi(g3[r]) * op.w3;
+        x[r] = fma(fx_two_limbs(H, L), cu, f[r]);
       }
     } else if constexpr (KIND == FX27) {
 #pragma unroll

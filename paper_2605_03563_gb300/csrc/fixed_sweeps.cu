@@ -92,16 +92,9 @@ __device__ __forceinline__ long long fx_from_even(double v, int eb) {
   return ((long long)((r + 3u + ((unsigned)r >> 2 & 2u)) >> 3) ^ s) - s;
 }
 
-// 16 a - b as a double, exact up to its 62 leading bits (the sum may exceed 64 bits)
+// 16 a - b as a double (the sum may exceed 64 bits)
 __device__ __forceinline__ double fx_sum13(long long a, long long b) {
-  const long long L = ((long long)(unsigned)a << 4) - (long long)(unsigned)b;
-  const long long H = ((a >> 32) << 4) - (b >> 32) + (L >> 32);
-  const bool big = (unsigned long long)(H + (1LL << 30)) >= (1ull << 31);
-  const unsigned low = (unsigned)L;
-  const long long t = big ? (long long)((unsigned long long)H << 21 | low >> 11)
-                          : (long long)((unsigned long long)H << 32 | low);
-  const double v = fx_double(t);
-  return __hiloint2double(__double2hiint(v) + (big ? 11 << 20 : 0), __double2loint(v));
+  return fx_two_limbs(((a >> 32) << 4) - (b >> 32), ((long long)(unsigned)a << 4) - (long long)(unsigned)b);
 }
 
 template <int KIND, bool ISO, int MODE, typename W, typename Gm>
