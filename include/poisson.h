@@ -96,10 +96,18 @@ typedef struct {
 typedef enum { PS_SOR = 0, PS_CG = 1, PS_MG = 2, PS_BICGSTAB = 3, PS_PCG = 4 } ps_method;
 
 /* PS_FP64: every field is stored in FP64.  Arithmetic is FP64, except that on
- *   levels of 7 x 10^5 unknowns and more the passes of multigrid add neighbours
- *   as 64-bit fixed-point numbers of one unit per pass (1/16 of the last place
- *   of the largest value's binade; 13-point colour passes 1/8), exactly, and
- *   round once to FP64; their error is no larger than that of the FP64 sums.
+ *   levels of 7 x 10^5 unknowns and more the passes of multigrid (and of the
+ *   initial residual of SOR, CG and PCG) add neighbours as 64-bit fixed-point
+ *   numbers of one unit per pass (1/16 of the last place of the largest
+ *   value's binade; 13-point colour passes 1/8), exactly, and round once to FP64.
+ *   What a value has below that unit is rounded off (to nearest where the sum
+ *   is kept, down where only differences are): an absolute error of at most one
+ *   unit per value, below the rounding of FP64 sums where values are above 1/16
+ *   of the largest one, above it where they are smaller.  Values that no stencil
+ *   reads (box edges and corners) do not enter the largest one, and once a
+ *   residual is within 64 times of what the units can leave in it the passes run
+ *   in FP64, so the accuracy that a solve can reach is that of FP64 sums.  The right-hand side,
+ *   also the compact schemes', is formed in FP64.
  * PS_MIXED_FP32: Cartesian: FP64 iterative refinement (outer residual,
  *   correction, norms, multipole moments and coarsest solve in FP64) around
  *   FP32 inner V-cycles.  Spherical: FP64 iterative refinement around inner

@@ -408,7 +408,7 @@ cudaError_t launch_c27_resid_dt(const Dims& d, const W27& A, const double* u, co
 //              whose base it has read); *track the largest |u| written.
 // The unit comes from the larger of *h1 and *h2, the high words of max |in|.
 // Under ncu at 256^3: FP64 residual 453 -> 125 us and SPAI step 445 -> 126 us
-// (DRAM 39%, integer pipe 46% busy), initial pass 815 -> 170 us and 29 us for the
+// (DRAM 39%, integer pipe 46% busy), initial pass 815 -> 178 us and 29 us for the
 // shell; 512^3 outer residual in the solve 3942 -> 1000 us.
 enum { C27_INIT, C27_NORM, C27_RESID, C27_SPAI };
 template <int MODE, typename TR>

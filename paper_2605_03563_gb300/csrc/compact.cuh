@@ -62,7 +62,10 @@ cudaError_t launch_c27_fx_resid(const Dims& d, const C27Ops& ops, const double* 
 // st->umax bounds |u|, st->unext takes the largest |u| read
 cudaError_t launch_c27_fx_norm(const Dims& d, const C27Ops& ops, const double* u, const double* b, double* r,
                                double* partials, DevState* st, int* nb, cudaStream_t s);
-// u -= omega M r; *hr bounds |r|, *hu takes the largest |u| written
+// u -= omega M r; *hr bounds |r|, *hu takes the largest |u| written.  (*hr is the
+// largest |r| of the V-cycle so far on this level: for a later, smaller r the unit
+// costs 0.08 h^2 2^-56 of it at most, a third of the unit of u, whose maximum the
+// first step on that r has made a quarter h^2 |r|.)
 cudaError_t launch_c27_fx_spai(const Dims& d, const C27Ops& ops, const double* r, double* u, DevState* st,
                                const unsigned* hr, unsigned* hu, cudaStream_t s);
 // r = b - L_h u stored as FP32 with partials {sum r^2, 0} in *nb blocks: the

@@ -18,13 +18,14 @@
 // (S - 6 C and the like): both are nearer the exact values than the FP64 chains.
 //
 // A pass reads phi and fs once and writes a part of phi: on 256^3, 134 + 134 MB in
-// and 134 out (whole lines), 59 us at the copy rate.  Measured (us a pass; FP64
-// diagonal walks before): 256^3 87 -> 70.5, with the lag 121 -> 92, residual
-// 104 -> 75; 160 x 112 x 208 unequal spacings 32.7 -> 25.7; 96^3 10.2 -> 9.3;
-// 13-point 192^3 54.7 -> 33.5, residual 113 -> 48, norm 131 -> 48.  Bound by the
-// memory system at 80 % of the copy rate on the largest levels (half of the issue
-// slots busy), on the smallest by the chain of TMA wait, barrier and update from
-// plane to plane.
+// and 134 out (whole lines), 59 us at the copy rate.  Measured (us a pass under ncu;
+// FP64 diagonal walks before): 256^3 88 -> 75, with the lag 131 -> 102, residual
+// 104 -> 79; 160 x 112 x 208 unequal spacings 32.7 -> 27.7; 13-point 192^3 54.7 -> 36.8,
+// residual 113 -> 51, norm 131 -> 55; 96^3 sweeps 11.1 (walks 10.2), with the lag
+// 15.5, residual 11.5, its solve 1920 -> 1879.  Bound by the memory system at 78 % of
+// the copy rate on the largest levels (half of the issue slots busy, 4 us of it for
+// rounding the values to nearest), on the smallest by the chain of TMA wait,
+// barrier and update from plane to plane.
 //
 // Bounds.  H: the largest of |phi| as last tracked, the boundary data and |fs|,
 // below 2^57 units (13-point 2^56).  A 7-point update is a mean of its neighbours
@@ -321,7 +322,8 @@ static cudaError_t fc_t(const Dims& d, const Coef<double>& cf, int colour, doubl
   // 7-point, more than 3 10^6 nodes: 64 x 16 tiles (halo 1.16 instead of 1.29 of the
   // nodes; 256^3: 70.5 us against 72.1, with the lag 92 against 104); below, and
   // 13-point: tiles of 8 rows and one more stage (128^3 12.9 us against 13.7, 96^3
-  // 9.3 against 11.1; 13-point 192^3 33.5 against 43.9 with two stages, 50 with 16 rows)
+  // 9.3 against 11.1; 13-point 192^3 33.5 against 43.9 with two stages, 50 with 16 rows;
+  // all of these with truncated values, 4 to 10 % below the passes' present times)
   if (KIND == FX7 && (long long)d.ni() * d.nj() * d.nk() > 3000000)
     return fc_v<KIND, ISO, MODE, FcGeom<KIND, 2, 2>>(d, cf, colour, phi, fs, out, st, b, partials, nblocks, s);
   return fc_v<KIND, ISO, MODE, FcGeom<KIND, 1, 3>>(d, cf, colour, phi, fs, out, st, b, partials, nblocks, s);
