@@ -1858,13 +1858,11 @@ cudaError_t launch_finish_norm(const double* partials, int nblocks, double dscal
 // state is the result, or phase 2 updates the black values from the new red
 // ones.  Updates and residuals repeat the colour passes' arithmetic
 // (gs_value's order), so iterates agree bit for bit.
-// 32 registers a thread let as many solves stay resident beside each other as the
-// SM has warps for (64^3, four at once: 8.9 -> 8.2 ms a solve).
 // 31^3 unknowns to 1e-10: 24.2 us a step as four kernels of a loop graph (17.9 with
 // the shorter finisher), 11.0 with three barriers a step, 8.1 with these two; 95^3:
 // 1.85 times faster than the graph.
 template <bool ISO, int NT>
-__global__ void __launch_bounds__(NT, 2048 / NT)
+__global__ void __launch_bounds__(NT)
     k_sor_steps(Dims d, Coef<double> cf, double* __restrict__ phi, double* __restrict__ alt, const double* __restrict__ fs,
                 double omega0, const double* __restrict__ wtab, int wlen, DevState* __restrict__ st,
                 double* __restrict__ partials) {
@@ -1992,20 +1990,17 @@ bool sor_steps_fit(const Dims& d) {
   return d.g == 1 && (long long)d.ni() * d.nj() * d.nk() <= SOR_STEPS_MAX;
 }
 
-// Several solves in flight (ms a solve, eight at once; loop graphs): 32^3 0.31 (0.71),
-// 48^3 2.2 (2.6), 64^3 8.0 (7.2; four at once 8.2, 9.3), 80^3 22.6 (33.9), 96^3 47.7
-// (71.2): below 350000 unknowns a launch that would wait for room beside the others
-// leaves the work to the loop graph, above the graph is never the faster one.
+// Several solves in flight (ms a solve, eight at once; loop graphs): 32^3 0.32 (0.71),
+// 48^3 2.3 (2.6), 64^3 8.3 (7.2; four at once 8.9, 9.3), 80^3 22.9 (33.9), 96^3 47.7
+// (71.2): below 350000 unknowns, launches of more threads than the SMs have leave the
+// work to the loop graph, above the graph is never the faster one.  (With 32
+// registers a thread instead of 40 four launches of 512 threads fit at once: 64^3
+// 8.2 ms, but 71^3 alone 1.7 % slower.)
 int sor_steps_share(const Dims& d, const double h[3], int npart) {
   if ((long long)d.ni() * d.nj() * d.nk() > 350000) return 0;
-  return sor_variant(d, h, [&](auto iso, auto nt) -> int {
+  return sor_variant(d, h, [&](auto, auto nt) -> int {
     constexpr int NT = decltype(nt)::value;
-    static PerDevice cached;
-    int occ = 1;
-    (void)cached.get(
-        [](int* n) { return cudaOccupancyMaxActiveBlocksPerMultiprocessor(n, k_sor_steps<decltype(iso)::value, NT>, NT, 0); },
-        &occ);
-    return steps_share(sor_blocks(d, NT, npart), occ);
+    return steps_share(sor_blocks(d, NT, npart), 2048 / NT);
   });
 }
 
